@@ -290,7 +290,7 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     CK(tmp.alloc(sizeof(uint64_t) * M, s), "alloc");
     CK(cover_emit(lens, n, m, bounds.as<double>(), n_int[0], m == 2 ? n_int[1] : 1,
                   pos.as<int64_t>(), c->keys.as<uint64_t>(), s), "cover_emit");
-    CK(radix_sort_u64(c->keys.as<uint64_t>(), tmp.as<uint64_t>(), M, 32, 32 + bits_for(E), s), "sort");
+    CK(radix_sort_u64(c->keys, tmp, M, 32, 32 + bits_for(E), s), "sort");
     CK(c->elem_off.alloc(sizeof(int64_t) * (E + 1), s), "alloc");
     CK(element_offsets(c->keys.as<uint64_t>(), M, E, c->elem_off.as<int64_t>(), s), "elem_off");
     CK(c->slot_point.alloc(sizeof(int32_t) * M, s), "alloc");
@@ -665,10 +665,8 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         if (PL.n[li] <= 1 || (li == kListSimt && !cross_tc)) continue;
         Buf tmp;
         CK(tmp.alloc(sizeof(uint64_t) * PL.n[li], s), "alloc");
-        uint64_t* keys = PL.list[li].as<uint64_t>();
-        const int tb = bits_for(L.T);
-        CK(radix_sort_u64(keys, tmp.as<uint64_t>(), PL.n[li], 32, 32 + tb, s), "sort pairs");
-        CK(radix_sort_u64(keys, tmp.as<uint64_t>(), PL.n[li], 0, tb, s), "sort pairs");
+        // (an int2 holds a in the low 32 bits of the key, b in the high ones)
+        CK(radix_sort_u64_two(PL.list[li], tmp, PL.n[li], 32, 0, bits_for(L.T), s), "sort pairs");
     }
     // pass 1 flags the screened tile pairs holding a neighbour pair; only
     // those can matter to the union pass
@@ -1119,7 +1117,7 @@ int run_density(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int64_t l
 }
 
 // ------------------------------------------------------------------ nerve
-int nerve_edges(mapper_ctx* ctx, uint64_t* keys2, int64_t Gm, int64_t n_points, int64_t N, mapper_graph_t* g);
+int nerve_edges(mapper_ctx* ctx, Buf& keys2, int64_t Gm, int64_t n_points, int64_t N, mapper_graph_t* g);
 
 int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_graph_t* g)
 {
@@ -1148,12 +1146,12 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
     CK(member_keys(cl->lab.as<int32_t>(), nid.as<int64_t>(), mpos.as<int64_t>(),
                    cov->slot_point.as<int32_t>(), cov->slot_elem.as<int32_t>(), M,
                    keys.as<uint64_t>(), g->node_elem.as<int32_t>(), s), "member keys");
-    CK(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), Gm, 32, 32 + bits_for(N), s), "sort");
+    CK(radix_sort_u64(keys, tmp, Gm, 32, 32 + bits_for(N), s), "sort");
     CK(node_offsets(keys.as<uint64_t>(), Gm, g->node_off.as<int64_t>(), g->node_members.as<int32_t>(),
                     keys2.as<uint64_t>(), s), "node offsets");
     CK(cudaMemcpyAsync(g->node_off.as<int64_t>() + N, &g->Gm, sizeof(int64_t), cudaMemcpyHostToDevice, s),
        "copy");
-    int rc = nerve_edges(ctx, keys2.as<uint64_t>(), Gm, cov->n, N, g);
+    int rc = nerve_edges(ctx, keys2, Gm, cov->n, N, g);
     if (rc) return rc;
     g->stats = cl->stats;
     g->stats.n_nodes = N;
@@ -1164,16 +1162,16 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
 // Nerve edges from the memberships (point << 32 | node) of N nodes (the keys
 // are sorted in place): group by point, emit each point's node pairs, sort,
 // unique. Sets g->edges and g->Eg.
-int nerve_edges(mapper_ctx* ctx, uint64_t* keys2, int64_t Gm, int64_t n_points, int64_t N, mapper_graph_t* g)
+int nerve_edges(mapper_ctx* ctx, Buf& keys2, int64_t Gm, int64_t n_points, int64_t N, mapper_graph_t* g)
 {
     cudaStream_t s = ctx->stream->s;
     Buf tmp;
     CK(tmp.alloc(sizeof(uint64_t) * std::max<int64_t>(Gm, 1), s), "alloc");
-    CK(radix_sort_u64(keys2, tmp.as<uint64_t>(), Gm, 32, 32 + bits_for(n_points), s), "sort");
+    CK(radix_sort_u64(keys2, tmp, Gm, 32, 32 + bits_for(n_points), s), "sort");
     Buf cnt, ppos;
     CK(cnt.alloc(sizeof(int64_t) * Gm, s), "alloc");
     CK(ppos.alloc(sizeof(int64_t) * (Gm + 1), s), "alloc");
-    CK(run_pairs(keys2, Gm, cnt.as<int64_t>(), s), "run pairs");
+    CK(run_pairs(keys2.as<uint64_t>(), Gm, cnt.as<int64_t>(), s), "run pairs");
     CK(exclusive_scan_i64(cnt.as<int64_t>(), ppos.as<int64_t>(), Gm, s), "scan");
     int64_t P = 0;
     CK(cudaMemcpyAsync(&P, ppos.as<int64_t>() + Gm, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "copy");
@@ -1181,10 +1179,9 @@ int nerve_edges(mapper_ctx* ctx, uint64_t* keys2, int64_t Gm, int64_t n_points, 
     Buf pairs, ptmp, flag, upos;
     CK(pairs.alloc(sizeof(uint64_t) * P, s), "alloc");
     CK(ptmp.alloc(sizeof(uint64_t) * P, s), "alloc");
-    CK(emit_pairs(keys2, Gm, ppos.as<int64_t>(), pairs.as<uint64_t>(), s), "emit pairs");
+    CK(emit_pairs(keys2.as<uint64_t>(), Gm, ppos.as<int64_t>(), pairs.as<uint64_t>(), s), "emit pairs");
     const int nb = bits_for(N);
-    CK(radix_sort_u64(pairs.as<uint64_t>(), ptmp.as<uint64_t>(), P, 0, nb, s), "sort");
-    CK(radix_sort_u64(pairs.as<uint64_t>(), ptmp.as<uint64_t>(), P, 32, 32 + nb, s), "sort");
+    CK(radix_sort_u64_two(pairs, ptmp, P, 0, 32, nb, s), "sort");
     CK(flag.alloc(sizeof(int32_t) * P, s), "alloc");
     CK(upos.alloc(sizeof(int64_t) * (P + 1), s), "alloc");
     CK(unique_flags(pairs.as<uint64_t>(), P, flag.as<int32_t>(), s), "unique");
@@ -1773,7 +1770,7 @@ int mapper_nerve_from_nodes(mapper_ctx* ctx, int64_t n_points, int64_t n_nodes, 
     CK(keys2.alloc(sizeof(uint64_t) * std::max<int64_t>(Gm, 1), s), "alloc");
     CK(node_member_keys(g->node_off.as<int64_t>(), n_nodes, Gm, g->node_members.as<int32_t>(),
                         keys2.as<uint64_t>(), s), "member keys");
-    if ((rc = nerve_edges(ctx, keys2.as<uint64_t>(), Gm, n_points, n_nodes, g.get()))) return rc;
+    if ((rc = nerve_edges(ctx, keys2, Gm, n_points, n_nodes, g.get()))) return rc;
     g->stats.n_points = n_points;
     g->stats.n_nodes = n_nodes;
     g->stats.n_edges = g->Eg;

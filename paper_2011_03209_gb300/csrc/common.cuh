@@ -142,10 +142,11 @@ cudaError_t cover_emit(const double* f, int64_t n, int m, const double* bounds, 
 cudaError_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n,
                                       cudaStream_t s);   // out has n+1 entries
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s);
-// Stable LSD radix sort of 64-bit keys on bits [lo_bit, hi_bit). In place
-// (keys) with a scratch buffer of the same size.
-cudaError_t radix_sort_u64(uint64_t* keys, uint64_t* tmp, int64_t n, int lo_bit, int hi_bit,
-                           cudaStream_t s);
+// Stable LSD radix sorts of n 64-bit keys: on bits [lo_bit, hi_bit), or on
+// bits [lo1, lo1 + bits) above bits [lo0, lo0 + bits). tmp: a buffer of at least n keys;
+// the two buffers may come back swapped (the sorted keys are in `keys`).
+cudaError_t radix_sort_u64(Buf& keys, Buf& tmp, int64_t n, int lo_bit, int hi_bit, cudaStream_t s);
+cudaError_t radix_sort_u64_two(Buf& keys, Buf& tmp, int64_t n, int lo0, int lo1, int bits, cudaStream_t s);
 
 // slots of a cover with one element holding every point (slot i = point i)
 cudaError_t whole_cloud_slots(int64_t n, int32_t* slot_point, int32_t* slot_elem, cudaStream_t s);

@@ -272,7 +272,7 @@ cudaError_t balanced_bounds(const double* f, int64_t n, int m, const int32_t* n_
         const int64_t off = j == 0 ? 0 : 2 * (int64_t)n0;
         { order_keys_kernel<<<div_up(n, 256), 256, 0, s>>>(f, n, m, j, keys.as<uint64_t>()); note_launch(); }
         MGB_TRY(cudaGetLastError());
-        MGB_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), n, 0, 64, s));
+        MGB_TRY(radix_sort_u64(keys, tmp, n, 0, 64, s));
         const double* ra = rank_bounds.as<double>() + off;
         { pick_bounds_kernel<<<div_up(nk, 256), 256, 0, s>>>(keys.as<uint64_t>(), n, nk, ra, ra + nk,
                                                             bounds + off, bounds + off + nk); note_launch(); }

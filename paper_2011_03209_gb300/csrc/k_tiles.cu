@@ -1198,7 +1198,7 @@ int build_tiles(const float* X, int64_t n, int32_t d, int64_t ld, int dp, const 
                                           gid.as<int32_t>(), tau2, K, gbits, pbits, keys.as<uint64_t>());
     note_launch();
     TK(cudaGetLastError());
-    TK(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), M, 32, 32 + ebits + gbits + pbits, s));
+    TK(radix_sort_u64(keys, tmp, M, 32, 32 + ebits + gbits + pbits, s));
     TK(flag.alloc(sizeof(int32_t) * M, s));
     TK(segpos.alloc(sizeof(int64_t) * (M + 1), s));
     seg_flag_kernel<<<grid_for(M), 256, 0, s>>>(keys.as<uint64_t>(), M, 32 + pbits, flag.as<int32_t>());
