@@ -233,6 +233,12 @@ int run_lens(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int64_t ld, 
         } else if (kinds[j] == MAPPER_LENS_ECC_INF) {
             const int rc = lens_ecc_inf(X, n, d, ld, lens_dev, m, j, ctx->num_sms, precision != MAPPER_FP32, s);
             if (rc) return rc;
+        } else if (j == 0 && m == 2 && kinds[1] == MAPPER_LENS_PCA) {
+            // two projections in one pass over the rows
+            const double* axes = pca_dev->as<double>() + d;
+            CK(lens_project2(X, n, d, ld, pca_dev->as<double>(), axes + (size_t)d * args[0],
+                             axes + (size_t)d * args[1], lens_dev, s), "lens_project");
+            break;
         } else
             CK(lens_project(X, n, d, ld, pca_dev->as<double>(),
                             pca_dev->as<double>() + (size_t)d * (1 + args[j]), lens_dev, m, j, s),

@@ -113,6 +113,9 @@ cudaError_t lens_linf(const float* X, int64_t n, int32_t d, int64_t ld, double* 
                       cudaStream_t s);
 cudaError_t lens_project(const float* X, int64_t n, int32_t d, int64_t ld, const double* mu,
                          const double* v, double* f, int m, int j, cudaStream_t s);
+// Both columns of a 2D filter of two projections (f: n x 2) in one pass.
+cudaError_t lens_project2(const float* X, int64_t n, int32_t d, int64_t ld, const double* mu, const double* v0,
+                          const double* v1, double* f, cudaStream_t s);
 // Column means of X (FP64, fixed-order block sums): mu[d] on the device.
 cudaError_t column_means(const float* X, int64_t n, int32_t d, int64_t ld, double* mu, cudaStream_t s);
 // Principal axes: mu (d doubles) and K axes (K*d doubles), device outputs.

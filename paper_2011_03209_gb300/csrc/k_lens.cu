@@ -8,9 +8,12 @@
 // expression; the L2 lens rounds the exact sum of squares once. Rows are staged
 // through shared memory so the loads stay coalesced while every thread walks
 // its own row in order.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace mgb {
 
@@ -19,54 +22,85 @@ namespace {
 constexpr int kRows = 128;    // rows per CTA (one thread per row)
 constexpr int kChunk = 32;    // columns staged per step
 
+// (double)x from the bits, in integer instructions (the FP64 pipe of this chip,
+// conversions included, issues two lanes a cycle and SM): for zeros and normal
+// values; `plain` says whether x is one. Kernels ask once for a batch of
+// values and convert the batches that hold another by the conversion.
+__device__ __forceinline__ bool plain(float x)
+{
+    const unsigned t = __float_as_uint(x) & 0x7FFFFFFFu;
+    return t == 0u || t - 0x00800000u < 0x7F000000u;
+}
+
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    const unsigned hi = ((b & 0x7FFFFFFFu) >> 3) + (896u << 20);
+    return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7FFFFFFFu) ? hi : 0u)), (int)(b << 29));
+}
+
 // One CTA = 128 rows. Each warp loads whole 32-column row segments
 // (coalesced); then each thread consumes its row's segment in order.
 // MODE 0: sum x^2 then sqrt (L2). MODE 1: sum (x - mu) v (projection).
-// MODE 2: sum (x - mu)^2 (squared distance to the mean).
+// MODE 2: sum (x - mu)^2 (squared distance to the mean). MODE 3: two
+// projections, sharing x - mu. Bound by the FP64 pipe (MODE 1: subtract,
+// multiply, add per value). 500k x 128, two axes: 0.99 -> 0.74 ms; MODE 2 at 1M
+// x 256: 1.43 -> 0.93 ms (conversions off the FP64 pipe).
 template <int MODE>
 __global__ void __launch_bounds__(kRows) lens_rows_kernel(const float* __restrict__ X, int64_t n,
                                                           int32_t d, int64_t ld,
                                                           const double* __restrict__ mu,
                                                           const double* __restrict__ v,
+                                                          const double* __restrict__ v2,
                                                           double* __restrict__ f, int m, int j)
 {
     __shared__ float tile[kRows][kChunk + 1];
-    __shared__ double smu[kChunk], sv[kChunk];
+    __shared__ double smu[kChunk], sv[kChunk], sv2[kChunk];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t row0 = (int64_t)blockIdx.x * kRows;
-    double acc = 0.0;
+    double acc = 0.0, acc2 = 0.0;
     for (int32_t k0 = 0; k0 < d; k0 += kChunk) {
         const int kc = min(kChunk, d - k0);
-#pragma unroll 4
+        bool all_plain = true;
+#pragma unroll 8
         for (int r = warp; r < kRows; r += kRows / 32) {
             const int64_t row = row0 + r;
             float x = 0.f;
             if (row < n && lane < kc) x = __ldg(X + row * ld + k0 + lane);
             tile[r][lane] = x;
+            all_plain &= plain(x);
         }
         if (MODE >= 1 && tid < kc) {
             smu[tid] = mu[k0 + tid];
-            if (MODE == 1) sv[tid] = v[k0 + tid];
+            if (MODE == 1 || MODE == 3) sv[tid] = v[k0 + tid];
+            if (MODE == 3) sv2[tid] = v2[k0 + tid];
         }
-        __syncthreads();
-        for (int k = 0; k < kc; ++k) {
-            const double x = (double)tile[tid][k];
+        auto add = [&](int k, double x) {
             if (MODE == 0) {
                 // x * x is exact in double (24-bit significands), so one
                 // fused rounding equals the separate multiply and add
                 acc = __fma_rn(x, x, acc);
-            } else if (MODE == 1) {
-                const double t = __dsub_rn(x, smu[k]);
-                acc = __dadd_rn(acc, __dmul_rn(t, sv[k]));
-            } else {
+            } else if (MODE == 2) {
                 const double t = __dsub_rn(x, smu[k]);
                 acc = __fma_rn(t, t, acc);
+            } else {
+                const double t = __dsub_rn(x, smu[k]);
+                acc = __dadd_rn(acc, __dmul_rn(t, sv[k]));
+                if (MODE == 3) acc2 = __dadd_rn(acc2, __dmul_rn(t, sv2[k]));
             }
+        };
+        if (__syncthreads_and(all_plain)) {
+#pragma unroll 8
+            for (int k = 0; k < kc; ++k) add(k, widen(tile[tid][k]));
+        } else {
+            for (int k = 0; k < kc; ++k) add(k, (double)tile[tid][k]);
         }
         __syncthreads();
     }
     const int64_t row = row0 + tid;
-    if (row < n) f[row * m + j] = (MODE == 0) ? __dsqrt_rn(acc) : acc;
+    if (row >= n) return;
+    f[row * m + j] = (MODE == 0) ? __dsqrt_rn(acc) : acc;
+    if (MODE == 3) f[row * m + j + 1] = acc2;
 }
 
 // L2 lens from the exact sum of squares. A float x = m 2^(e-150) (m < 2^24)
@@ -365,106 +399,356 @@ __global__ void __launch_bounds__(256) finite_kernel(const float* __restrict__ X
 }
 
 // --------------------------------------------------------------------- PCA
-// Column means: partial FP64 sums per row block, then a fixed-order reduce
-// (deterministic run to run).
+// Column means: partial FP64 sums per row block, rows in order, then a
+// fixed-order reduce (deterministic run to run). One warp per (32 columns, row
+// block): the sum is a chain of FP64 adds, so the next 32 rows are loaded
+// while the current ones are added, and the columns spread over the SMs (the
+// FP64 pipe takes 16 cycles for a warp's add). 1M x 256: 1.17 -> 0.54 ms.
 constexpr int kMeanRows = 4096;
+constexpr int kMeanAhead = 32;
 
-__global__ void col_partial_sum_kernel(const float* __restrict__ X, int64_t n, int32_t d,
-                                       int64_t ld, double* __restrict__ part)
+__global__ void __launch_bounds__(32) col_partial_sum_kernel(const float* __restrict__ X, int64_t n, int32_t d,
+                                                             int64_t ld, double* __restrict__ part)
 {
+    const int c = min(blockIdx.y * 32 + (int)threadIdx.x, d - 1);  // (lanes past d: the last column again)
     const int64_t r0 = (int64_t)blockIdx.x * kMeanRows;
     const int64_t r1 = min(n, r0 + kMeanRows);
-    for (int c = threadIdx.x; c < d; c += blockDim.x) {
-        double s = 0.0;
-        for (int64_t r = r0; r < r1; ++r) s += (double)X[r * ld + c];
-        part[(int64_t)blockIdx.x * d + c] = s;
+    const float* x = X + r0 * ld + c;
+    const int rows = (int)(r1 - r0);
+    float cur[kMeanAhead], nxt[kMeanAhead];
+#pragma unroll
+    for (int i = 0; i < kMeanAhead; ++i) cur[i] = i < rows ? __ldg(x + i * ld) : 0.f;
+    double s = 0.0;
+    for (int r = 0; r < rows; r += kMeanAhead) {
+#pragma unroll
+        for (int i = 0; i < kMeanAhead; ++i) {
+            const int q = r + kMeanAhead + i;
+            nxt[i] = q < rows ? __ldg(x + q * ld) : 0.f;
+        }
+        bool all_plain = true;
+#pragma unroll
+        for (int i = 0; i < kMeanAhead; ++i) all_plain &= plain(cur[i]);
+        if (__all_sync(0xffffffffu, all_plain)) {                  // (rows past the end add 0)
+#pragma unroll
+            for (int i = 0; i < kMeanAhead; ++i) s += widen(cur[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kMeanAhead; ++i) s += (double)cur[i];
+        }
+#pragma unroll
+        for (int i = 0; i < kMeanAhead; ++i) cur[i] = nxt[i];
     }
+    part[(int64_t)blockIdx.x * d + c] = s;
 }
 
-__global__ void col_mean_kernel(const double* __restrict__ part, int nblk, int32_t d, int64_t n,
-                                double* __restrict__ mu)
+__global__ void __launch_bounds__(32) col_mean_kernel(const double* __restrict__ part, int nblk, int32_t d, int64_t n,
+                                                      double* __restrict__ mu)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= d) return;
     double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[(int64_t)b * d + c];
+#pragma unroll 16
+    for (int b = 0; b < nblk; ++b) s += __ldg(part + (int64_t)b * d + c);
     mu[c] = s / (double)n;
 }
 
-// FP32 covariance tiles: block (ti, tj, chunk) accumulates the 64 x 64 tile
-// (ti, tj), tj >= ti, of sum_p (x_p - mu)(x_p - mu)^T over its row chunk.
-constexpr int kCovT = 64;
-constexpr int kCovRows = 2048;
-
-__global__ void __launch_bounds__(256) cov_partial_kernel(const float* __restrict__ X, int64_t n,
-                                                          int32_t d, int64_t ld,
-                                                          const double* __restrict__ mu,
-                                                          float* __restrict__ part, int ntile)
+// xc = (float)((double)x - mu), the centred rows of the covariance (n x d),
+// without the FP64 pipe (three of its slots a value) for all but a few values:
+// with mu = mh + ml + rest (FP32 parts), x - mh = s + e exactly (two-sum),
+// t = e - ml and s + t = res + r2 exactly, so the true difference is
+// res + r2 + delta, |delta| <= 2^-22 (|t| + |ml|); where that stays strictly
+// inside half an ulp of res (by more than the 2^-53 of a rounding to double),
+// res is the rounding. Otherwise, and for Inf, NaN, powers of two and small
+// values, the FP64 expression itself decides.
+__global__ void __launch_bounds__(256) centre_rows_kernel(const float* __restrict__ X, int64_t n, int32_t d, int64_t ld,
+                                                          const double* __restrict__ mu, float* __restrict__ xc)
 {
-    int ti = 0, tj = 0, t = blockIdx.x;       // decode upper-triangle tile index
-    for (ti = 0; ti < ntile; ++ti) {
-        const int row_len = ntile - ti;
-        if (t < row_len) { tj = ti + t; break; }
-        t -= row_len;
+    extern __shared__ float2 s_mu[];
+    for (int k = threadIdx.x; k < d; k += blockDim.x) {
+        const double m = mu[k];
+        const float mh = (float)m;
+        s_mu[k] = make_float2(mh, (float)(m - (double)mh));
     }
-    const int chunk = blockIdx.y;
-    __shared__ float sa[32][kCovT + 1], sb[32][kCovT + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t r = w0; r < n; r += nw) {
+        const float* x = X + r * ld;
+        float* o = xc + r * d;
+#pragma unroll 4
+        for (int k = lane; k < d; k += 32) {
+            const float v = __ldg(x + k);
+            const float2 m = s_mu[k];
+            const float s = __fsub_rn(v, m.x);
+            const float bb = __fsub_rn(s, v);
+            const float e = __fsub_rn(__fsub_rn(v, __fsub_rn(s, bb)), __fadd_rn(m.x, bb));
+            const float t = __fsub_rn(e, m.y);
+            float res = __fadd_rn(s, t);
+            const float b2 = __fsub_rn(res, s);
+            const float r2 = __fadd_rn(__fsub_rn(s, __fsub_rn(res, b2)), __fsub_rn(t, b2));
+            const unsigned bits = __float_as_uint(res);
+            const unsigned ex = bits & 0x7F800000u;
+            // half an ulp of res, less a 2^-12 part of it
+            const float half = __fmul_rn(__uint_as_float(ex), 5.9604645e-8f * (1.f - 0.000244140625f));
+            const float off = __fmaf_rn(2.3841858e-7f, __fadd_rn(fabsf(t), fabsf(m.y)), fabsf(r2));
+            if (!(off < half) || (bits & 0x7FFFFFu) == 0u || ex < (64u << 23) || ex == 0x7F800000u)
+                res = (float)((double)v - mu[k]);
+            o[k] = res;
+        }
+    }
+}
+
+// FP32 covariance tiles: CTA (tile, chunk) accumulates the 32 x 32 tile
+// (ti, tj), tj >= ti, of sum_p xc_p xc_p^T over its row chunk, each entry an
+// FMA chain over the chunk's rows in order. 64 threads with 4 x 4 entries each:
+// the tiles are small so that a cloud of a hundred thousand rows x 64 columns
+// still fills the SMs (49 chunks x 3 tiles at 100k x 64: 476 -> 89 us with the
+// rows centred once, 26 us; 500k x 128: 1475 -> 390 + 370 us).
+constexpr int kCovT = 32;
+constexpr int kCovRows = 2048;
+constexpr int kCovStep = 32;
+
+__device__ __forceinline__ void cov_tile(int t, int ntile, int* ti, int* tj)
+{
+    int i = 0;
+    while (t >= ntile - i) { t -= ntile - i; ++i; }
+    *ti = i;
+    *tj = i + t;
+}
+
+__global__ void __launch_bounds__(64) cov_partial_kernel(const float* __restrict__ xc, int64_t n, int32_t d,
+                                                         float* __restrict__ part, int ntile)
+{
+    __shared__ __align__(16) float sa[kCovStep][kCovT], sb[kCovStep][kCovT];
+    int ti, tj;
+    cov_tile(blockIdx.x, ntile, &ti, &tj);
+    const int chunk = blockIdx.y, tid = threadIdx.x;
+    const int tx = tid & 7, ty = tid >> 3;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int ca = ti * kCovT + lane, cb = tj * kCovT + lane;
     float acc[4][4] = {};
     const int64_t r0 = (int64_t)chunk * kCovRows, r1 = min(n, r0 + kCovRows);
-    const int ca = ti * kCovT, cb = tj * kCovT;
-    for (int64_t rb = r0; rb < r1; rb += 32) {
-        for (int e = threadIdx.x; e < 32 * kCovT; e += 256) {
-            const int rr = e / kCovT, cc = e % kCovT;
-            const int64_t r = rb + rr;
-            float xa = 0.f, xb = 0.f;
-            if (r < r1) {
-                if (ca + cc < d) xa = (float)((double)X[r * ld + ca + cc] - mu[ca + cc]);
-                if (cb + cc < d) xb = (float)((double)X[r * ld + cb + cc] - mu[cb + cc]);
-            }
-            sa[rr][cc] = xa;
-            sb[rr][cc] = xb;
+    float ra[kCovStep / 2], rb[kCovStep / 2];               // the next step's rows warp, warp + 2, ..
+    auto load = [&](int64_t r) {
+#pragma unroll
+        for (int i = 0; i < kCovStep / 2; ++i) {
+            const int64_t row = r + warp + 2 * i;
+            ra[i] = row < r1 && ca < d ? __ldg(xc + row * d + ca) : 0.f;
+            rb[i] = row < r1 && cb < d ? __ldg(xc + row * d + cb) : 0.f;
+        }
+    };
+    load(r0);
+    for (int64_t r = r0; r < r1; r += kCovStep) {
+#pragma unroll
+        for (int i = 0; i < kCovStep / 2; ++i) {
+            sa[warp + 2 * i][lane] = ra[i];
+            sb[warp + 2 * i][lane] = rb[i];
         }
         __syncthreads();
+        if (r + kCovStep < r1) load(r + kCovStep);
 #pragma unroll 8
-        for (int rr = 0; rr < 32; ++rr) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = sa[rr][ty * 4 + i]; b[i] = sb[rr][tx * 4 + i]; }
+        for (int k = 0; k < kCovStep; ++k) {
+            const float4 a4 = *reinterpret_cast<const float4*>(&sa[k][ty * 4]);
+            const float4 b4 = *reinterpret_cast<const float4*>(&sb[k][tx * 4]);
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[i][k] = fmaf(a[i], b[k], acc[i][k]);
+                for (int q = 0; q < 4; ++q) acc[i][q] = fmaf(a[i], b[q], acc[i][q]);
         }
         __syncthreads();
     }
     float* out = part + ((int64_t)chunk * gridDim.x + blockIdx.x) * kCovT * kCovT;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) out[(ty * 4 + i) * kCovT + tx * 4 + k] = acc[i][k];
+        *reinterpret_cast<float4*>(out + (ty * 4 + i) * kCovT + tx * 4) =
+            make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
 }
 
-__global__ void cov_reduce_kernel(const float* __restrict__ part, int nchunk, int ntile, int32_t d,
-                                  int64_t n, double* __restrict__ C)
+// One thread per entry: the chunks' partials added in order (a chain of FP64
+// adds, the loads ahead of it).
+__global__ void __launch_bounds__(128) cov_reduce_kernel(const float* __restrict__ part, int nchunk, int ntile,
+                                                         int32_t d, int64_t n, double* __restrict__ C)
 {
-    const int tile = blockIdx.x;
-    int ti = 0, tj = 0, t = tile;
-    for (ti = 0; ti < ntile; ++ti) {
-        const int row_len = ntile - ti;
-        if (t < row_len) { tj = ti + t; break; }
-        t -= row_len;
+    const int e = blockIdx.y * blockDim.x + threadIdx.x;
+    int ti, tj;
+    cov_tile(blockIdx.x, ntile, &ti, &tj);
+    const int i = ti * kCovT + e / kCovT, k = tj * kCovT + e % kCovT;
+    if (i >= d || k >= d) return;
+    const int64_t step = (int64_t)gridDim.x * kCovT * kCovT;
+    const float* p = part + (int64_t)blockIdx.x * kCovT * kCovT + e;
+    double s = 0.0;
+#pragma unroll 16
+    for (int c = 0; c < nchunk; ++c) s += (double)__ldg(p + c * step);
+    s /= (double)n;
+    C[(int64_t)i * d + k] = s;
+    C[(int64_t)k * d + i] = s;
+}
+
+// Warp sums of NJ values per lane at once: out of p[j] on 32 lanes, the sum
+// over the lanes of every p[j] in the order of a butterfly (16, 8, 4, 2, 1),
+// returned on the lanes seg_lane<NJ>(j). A butterfly of every value by itself
+// would spend 5 FP64 adds of a whole warp on each; here lanes that have no
+// part in one value's next level carry another value's.
+template <int NJ>
+__device__ __forceinline__ double warp_sums(const double (&p)[NJ], int lane)
+{
+    double q[NJ];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) q[j] = p[j];
+    int o = 16;
+#pragma unroll
+    for (int m = NJ; m > 1; m >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < m / 2; ++i) {
+            const double a = q[2 * i], b = q[2 * i + 1];
+            q[i] = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, o);
+        }
     }
-    const int ntiles = gridDim.x;
-    for (int e = threadIdx.x; e < kCovT * kCovT; e += blockDim.x) {
-        const int i = ti * kCovT + e / kCovT, k = tj * kCovT + e % kCovT;
-        if (i >= d || k >= d) continue;
-        double s = 0.0;
-        for (int c = 0; c < nchunk; ++c) s += (double)part[((int64_t)c * ntiles + tile) * kCovT * kCovT + e];
-        s /= (double)n;
-        C[(int64_t)i * d + k] = s;
-        C[(int64_t)k * d + i] = s;
+    double y = q[0];
+    for (; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+    return y;
+}
+
+template <int NJ>
+__device__ __forceinline__ int seg_lane(int j)
+{
+    int l = 0, o = 16;
+#pragma unroll
+    for (int m = NJ; m > 1; m >>= 1, o >>= 1, j >>= 1)
+        if (j & 1) l |= o;
+    return l;
+}
+
+// sum over the segments (columns 32 j ..) of their warp sums, in order
+template <int NJ>
+__device__ __forceinline__ double vec_sum(const double (&p)[NJ], int lane)
+{
+    const double y = warp_sums<NJ>(p, lane);
+    double t = 0.0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) t += __shfl_sync(0xffffffffu, y, seg_lane<NJ>(j));
+    return t;
+}
+
+// Power iteration (as power_iter_kernel, the same operations in the same
+// order) for d <= 32 NJ <= 256 on a cluster of kPowCluster CTAs. An iteration
+// is a d x d product and a few vector sums, bound by the FP64 pipe of the SMs
+// taking part and by latency: each warp keeps two rows of C in registers, its
+// products go to every CTA's shared memory, one cluster barrier, and the first
+// warp of every CTA does the vector work for itself (lane l holds columns
+// l + 32 j, as the products need them).
+constexpr int kPowCluster = 8;
+
+template <int NJ>
+__global__ void __launch_bounds__(512) power_iter_cluster_kernel(const double* __restrict__ C, int32_t d, int K,
+                                                                 double* __restrict__ axes, int* status)
+{
+    extern __shared__ double s_axes[];                       // K x 32 NJ: the axes found so far
+    __shared__ double s_w[2][32 * NJ], s_v[32 * NJ];
+    __shared__ int s_stop;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int row = 2 * (rank * nwarp + warp);               // the warp's rows row, row + 1
+    double c0[NJ], c1[NJ];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int k = lane + 32 * j;
+        c0[j] = row < d && k < d ? C[(int64_t)row * d + k] : 0.0;
+        c1[j] = row + 1 < d && k < d ? C[(int64_t)(row + 1) * d + k] : 0.0;
     }
+    for (int k = threadIdx.x; k < 64 * NJ; k += blockDim.x) (&s_w[0][0])[k] = 0.0;
+    cluster.sync();                                          // cleared before any CTA writes
+    int not_conv = 0, buf = 0;
+    for (int c = 0; c < K; ++c) {
+        double v[NJ];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int k = lane + 32 * j;
+            v[j] = k < d ? 1.0 + 0.25 * (double)((k * 7919) % 13) : 0.0;
+        }
+        for (int it = 0; it < 2000; ++it, buf ^= 1) {
+            double p[2] = {0.0, 0.0};
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                p[0] = __fma_rn(c0[j], v[j], p[0]);
+                p[1] = __fma_rn(c1[j], v[j], p[1]);
+            }
+            const double y = warp_sums<2>(p, lane);          // lane 0: row, lane 16: row + 1
+            const double w0 = __shfl_sync(0xffffffffu, y, 0), w1 = __shfl_sync(0xffffffffu, y, 16);
+            if (lane < kPowCluster) {
+                double* dst = cluster.map_shared_rank(&s_w[buf][0], lane);
+                if (row < d) dst[row] = w0;
+                if (row + 1 < d) dst[row + 1] = w1;
+            }
+            cluster.sync();
+            if (warp == 0) {
+                double w[NJ], t[NJ];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) w[j] = s_w[buf][lane + 32 * j];
+                for (int q = 0; q < c; ++q) {                // orthogonalise against earlier axes
+                    const double* ax = s_axes + q * 32 * NJ;
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j) t[j] = __dmul_rn(ax[lane + 32 * j], w[j]);
+                    const double proj = vec_sum<NJ>(t, lane);
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j) w[j] = __fma_rn(-proj, ax[lane + 32 * j], w[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) t[j] = __dmul_rn(w[j], w[j]);
+                const double norm = sqrt(vec_sum<NJ>(t, lane));
+                const double inv = norm > 0.0 ? 1.0 / norm : 0.0;
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const double nv = w[j] * inv;
+                    const double dv = nv - v[j];
+                    t[j] = __dmul_rn(dv, dv);
+                    v[j] = nv;
+                    s_v[lane + 32 * j] = nv;
+                }
+                const double diff = vec_sum<NJ>(t, lane);
+                if (lane == 0) s_stop = diff < 1e-14;        // ||dv|| < 1e-7
+            }
+            __syncthreads();
+            const int stop = s_stop;
+            if (warp > 0) {
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) v[j] = s_v[lane + 32 * j];
+            }
+            __syncthreads();
+            if (stop) { buf ^= 1; break; }                   // (the same in every CTA)
+            if (it == 1999) not_conv = 1;
+        }
+        // sign rule: the first entry of largest magnitude is positive
+        if (warp == 0) {
+            double best = -1.0, val = 0.0;
+            int at = 0;
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const int k = lane + 32 * j;
+                if (k < d && fabs(v[j]) > best) { best = fabs(v[j]); val = v[j]; at = k; }
+            }
+            for (int o = 16; o; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, best, o), ov = __shfl_xor_sync(0xffffffffu, val, o);
+                const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+                if (ob > best || (ob == best && oa < at)) { best = ob; val = ov; at = oa; }
+            }
+            const double sign = val < 0.0 ? -1.0 : 1.0;
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const int k = lane + 32 * j;
+                const double a = sign * v[j];
+                s_axes[c * 32 * NJ + k] = k < d ? a : 0.0;
+                if (rank == 0 && k < d) axes[(int64_t)c * d + k] = a;
+            }
+        }
+        __syncthreads();
+    }
+    if (rank == 0 && threadIdx.x == 0) *status = not_conv;
+    cluster.sync();                                          // no CTA leaves while another may write to it
 }
 
 // Power iteration for the top-K eigenvectors of C (d x d, FP64), one CTA.
@@ -565,7 +849,7 @@ cudaError_t lens_l2(const float* X, int64_t n, int32_t d, int64_t ld, double* f,
         const int blocks = (int)std::min<int64_t>(div_up(n, 8 * 32), 152 * 8);
         lens_l2_exact_kernel<false><<<blocks, 256, 0, s>>>(X, n, d, ld, f, m, j, nullptr, 0, nullptr, nullptr);
     } else {
-        lens_rows_kernel<0><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, nullptr, nullptr, f, m, j);
+        lens_rows_kernel<0><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, nullptr, nullptr, nullptr, f, m, j);
     }
     note_launch();
     return cudaGetLastError();
@@ -575,7 +859,15 @@ cudaError_t lens_project(const float* X, int64_t n, int32_t d, int64_t ld, const
                          const double* v, double* f, int m, int j, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    { lens_rows_kernel<1><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu, v, f, m, j); note_launch(); }
+    { lens_rows_kernel<1><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu, v, nullptr, f, m, j); note_launch(); }
+    return cudaGetLastError();
+}
+
+cudaError_t lens_project2(const float* X, int64_t n, int32_t d, int64_t ld, const double* mu, const double* v0,
+                          const double* v1, double* f, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    { lens_rows_kernel<3><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu, v0, v1, f, 2, 0); note_launch(); }
     return cudaGetLastError();
 }
 
@@ -585,8 +877,9 @@ cudaError_t column_means(const float* X, int64_t n, int32_t d, int64_t ld, doubl
     const int nblk = div_up(n, kMeanRows);
     Buf part;
     MGB_TRY(part.alloc(sizeof(double) * (size_t)nblk * d, s));
-    { col_partial_sum_kernel<<<nblk, 256, 0, s>>>(X, n, d, ld, part.as<double>()); note_launch(); }
-    { col_mean_kernel<<<div_up(d, 256), 256, 0, s>>>(part.as<double>(), nblk, d, n, mu); note_launch(); }
+    { col_partial_sum_kernel<<<dim3(nblk, div_up(d, 32)), 32, 0, s>>>(X, n, d, ld, part.as<double>()); note_launch(); }
+    MGB_TRY(cudaGetLastError());
+    { col_mean_kernel<<<div_up(d, 32), 32, 0, s>>>(part.as<double>(), nblk, d, n, mu); note_launch(); }
     return cudaGetLastError();
 }
 
@@ -598,14 +891,11 @@ cudaError_t column_means(const float* X, int64_t n, int32_t d, int64_t ld, doubl
 cudaError_t lens_ecc2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    const int nblk = div_up(n, kMeanRows);
-    Buf part, mu, vpart;
-    MGB_TRY(part.alloc(sizeof(double) * (size_t)nblk * d, s));
+    Buf mu, vpart;
     MGB_TRY(mu.alloc(sizeof(double) * d, s));
     MGB_TRY(vpart.alloc(sizeof(double) * kMeanBlocks, s));
-    { col_partial_sum_kernel<<<nblk, 256, 0, s>>>(X, n, d, ld, part.as<double>()); note_launch(); }
-    { col_mean_kernel<<<div_up(d, 256), 256, 0, s>>>(part.as<double>(), nblk, d, n, mu.as<double>()); note_launch(); }
-    { lens_rows_kernel<2><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu.as<double>(), nullptr, f, m, j);
+    MGB_TRY(column_means(X, n, d, ld, mu.as<double>(), s));
+    { lens_rows_kernel<2><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu.as<double>(), nullptr, nullptr, f, m, j);
       note_launch(); }
     { col_lens_partial_kernel<<<kMeanBlocks, 256, 0, s>>>(f, n, m, j, vpart.as<double>()); note_launch(); }
     { ecc_finish_kernel<<<std::min(div_up(n, 256), 152 * 8), 256, 0, s>>>(f, n, m, j, vpart.as<double>(), kMeanBlocks);
@@ -641,25 +931,60 @@ cudaError_t check_finite(const float* X, int64_t n, int32_t d, int64_t ld, int* 
     return cudaGetLastError();
 }
 
+template <int NJ>
+static cudaError_t power_cluster(const double* C, int32_t d, int K, double* axes, int* status, cudaStream_t s)
+{
+    const size_t smem = sizeof(double) * 32 * NJ * (size_t)K;
+    if (smem > 48 * 1024)
+        MGB_TRY(cudaFuncSetAttribute(power_iter_cluster_kernel<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem));
+    const int rows = div_up(d, kPowCluster);                 // a CTA's rows, two a warp
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kPowCluster);
+    cfg.blockDim = dim3(32u * (unsigned)div_up(rows, 2));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kPowCluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, power_iter_cluster_kernel<NJ>, C, d, K, axes, status);
+}
+
 cudaError_t pca_axes(const float* X, int64_t n, int32_t d, int64_t ld, int K, double* mu,
                      double* axes, int* status, cudaStream_t s)
 {
-    const int nblk = div_up(n, kMeanRows);
-    Buf part;
-    MGB_TRY(part.alloc(sizeof(double) * (size_t)nblk * d, s));
-    { col_partial_sum_kernel<<<nblk, 256, 0, s>>>(X, n, d, ld, part.as<double>()); note_launch(); }
-    { col_mean_kernel<<<div_up(d, 256), 256, 0, s>>>(part.as<double>(), nblk, d, n, mu); note_launch(); }
-    MGB_TRY(cudaGetLastError());
-
+    MGB_TRY(column_means(X, n, d, ld, mu, s));
     const int ntile = div_up(d, kCovT);
     const int ntri = ntile * (ntile + 1) / 2;
     const int nchunk = div_up(n, kCovRows);
-    Buf cpart, C;
+    Buf xc, cpart, C;
+    MGB_TRY(xc.alloc(sizeof(float) * (size_t)n * d, s));
     MGB_TRY(cpart.alloc(sizeof(float) * (size_t)nchunk * ntri * kCovT * kCovT, s));
     MGB_TRY(C.alloc(sizeof(double) * (size_t)d * d, s));
-    { cov_partial_kernel<<<dim3(ntri, nchunk), 256, 0, s>>>(X, n, d, ld, mu, cpart.as<float>(), ntile); note_launch(); }
-    { cov_reduce_kernel<<<ntri, 256, 0, s>>>(cpart.as<float>(), nchunk, ntile, d, n, C.as<double>()); note_launch(); }
+    const size_t mu_smem = sizeof(float2) * (size_t)d;
+    if (mu_smem > 48 * 1024)
+        MGB_TRY(cudaFuncSetAttribute(centre_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mu_smem));
+    centre_rows_kernel<<<(unsigned)std::min<int64_t>(div_up(n, 8), 152 * 8), 256, mu_smem, s>>>(X, n, d, ld, mu,
+                                                                                              xc.as<float>());
     MGB_TRY(cudaGetLastError());
+    cov_partial_kernel<<<dim3(ntri, nchunk), 64, 0, s>>>(xc.as<float>(), n, d, cpart.as<float>(), ntile);
+    MGB_TRY(cudaGetLastError());
+    cov_reduce_kernel<<<dim3(ntri, kCovT * kCovT / 128), 128, 0, s>>>(cpart.as<float>(), nchunk, ntile, d, n,
+                                                                      C.as<double>());
+    note_launch(3);
+    MGB_TRY(cudaGetLastError());
+    // the cluster holds C and the axes on chip; wider clouds or many axes take one CTA
+    if (d <= 256 && (size_t)K * 256 * sizeof(double) <= 160 * 1024) {
+        if (d <= 32) return power_cluster<1>(C.as<double>(), d, K, axes, status, s);
+        if (d <= 64) return power_cluster<2>(C.as<double>(), d, K, axes, status, s);
+        if (d <= 128) return power_cluster<4>(C.as<double>(), d, K, axes, status, s);
+        return power_cluster<8>(C.as<double>(), d, K, axes, status, s);
+    }
     const size_t smem = sizeof(double) * 2 * (size_t)d;
     if (smem > 48 * 1024)
         MGB_TRY(cudaFuncSetAttribute(power_iter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
