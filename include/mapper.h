@@ -344,9 +344,8 @@ int mapper_clusters_copy(const mapper_clusters_t* clusters, int64_t* label, uint
  * single-linkage dendrogram of the element up to height eps. The result is
  * read with mapper_forest_sizes / mapper_forest_copy: edge k joins points
  * u[k] < v[k] of element elem[k] at squared distance d2[k] (the FP64 value of
- * the defining expression); edges come in no particular order (sort by
- * (elem, d2, u, v) for a canonical one). X must be the cloud the cover was
- * built on. MAPPER_EINVAL for eps not finite and > 0, MAPPER_ENONFINITE if X
+ * the defining expression); edges are sorted by (elem, d2, u, v). X must be
+ * the cloud the cover was built on. MAPPER_EINVAL for eps not finite and > 0, MAPPER_ENONFINITE if X
  * holds NaN/Inf. */
 int mapper_single_linkage(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t d, int64_t ld,
                           const mapper_cover_t* cover, double eps, mapper_forest_t** out);

@@ -186,9 +186,7 @@ class Forest(_Handle):
         d2 = np.empty(max(k, 1), dtype=np.float64)
         _capi.check(self._lib.mapper_forest_copy(self.h, _vp(elem.ctypes.data), _vp(u.ctypes.data),
                                                  _vp(v.ctypes.data), _vp(d2.ctypes.data), 0), "mapper_forest_copy")
-        elem, u, v, d2 = elem[:k], u[:k], v[:k], d2[:k]
-        order = np.lexsort((v, u, d2, elem))
-        return dict(elem=elem[order], u=u[order], v=v[order], d2=d2[order])
+        return dict(elem=elem[:k], u=u[:k], v=v[:k], d2=d2[:k])
 
     def cut(self, ctx: "Context", h: float) -> Clusters:
         out = ctypes.c_void_p()

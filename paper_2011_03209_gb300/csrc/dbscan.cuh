@@ -80,6 +80,82 @@ __device__ __forceinline__ float4 pass_ld4(const PassArgs& A, const float* p, in
     return v;
 }
 
+// Packed FP32 pairs (each half rounded as the scalar instruction).
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ void f2_unpack(unsigned long long v, float& lo, float& hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
+// acc += (a + b)^2 per half, one rounding each for the sum and the FMA
+__device__ __forceinline__ void f2_sq_acc(unsigned long long& acc, unsigned long long a, unsigned long long b)
+{
+    unsigned long long t;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(a), "l"(b));
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc) : "l"(t));
+}
+
+constexpr int kSimtK = 32;      // columns staged per step
+constexpr int kSimtPad = 132;   // shared-memory row pitch (floats)
+
+// FP32 sums of squared differences of the rows sa .. sa + 127 and sb .. sb +
+// 127 (rows past na, nb count as zeros) by 256 threads: thread (ty, tx) =
+// (tid / 16, tid % 16) gets rows 4 ty + i, 64 + 4 ty + i - 4 and columns 4 tx
+// + j, 64 + 4 tx + j - 4; columns of a row in order, an FMA each. B is staged
+// negated, so that a difference is a packed add. Bound by the FP32 pipe, which
+// retires a packed instruction at half the rate of a scalar one, so packing
+// saves issue slots, not the pipe (count pass of the 65k x 64 FP32 graph 341 ->
+// 297 us, pivot assignment 102 -> 93).
+__device__ __forceinline__ void simt_tile_sums(const PassArgs& A, int64_t sa, int64_t sb, int na, int nb,
+                                               float (*As)[kSimtPad], float (*Bs)[kSimtPad], float (&acc)[8][8])
+{
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    unsigned long long s[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[i][j] = 0ull;
+    for (int k0 = 0; k0 < A.dp; k0 += kSimtK) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int idx = tid + 256 * v;       // float4 index in the 128 x 32 chunk
+            const int r = idx >> 3, k4 = (idx & 7) * 4;
+            float4 xa = make_float4(0.f, 0.f, 0.f, 0.f), xb = xa;
+            if (r < na) xa = pass_ld4(A, pass_row(A, sa + r), (k0 + k4) >> 2);
+            if (r < nb) xb = pass_ld4(A, pass_row(A, sb + r), (k0 + k4) >> 2);
+            As[k4 + 0][r] = xa.x; As[k4 + 1][r] = xa.y; As[k4 + 2][r] = xa.z; As[k4 + 3][r] = xa.w;
+            Bs[k4 + 0][r] = -xb.x; Bs[k4 + 1][r] = -xb.y; Bs[k4 + 2][r] = -xb.z; Bs[k4 + 3][r] = -xb.w;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int k = 0; k < kSimtK; ++k) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[k][64 + ty * 4]);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[k][tx * 4]);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[k][64 + tx * 4]);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const unsigned long long b[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const unsigned long long aa = f2_pack(a[i], a[i]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) f2_sq_acc(s[i][j], aa, b[j]);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f2_unpack(s[i][j], acc[i][2 * j], acc[i][2 * j + 1]);
+}
+
 // FP32 screen thresholds for eps2 at dimension d: a pair is certainly a
 // neighbour when the FP32 screen value is <= *lo, certainly not when > *hi.
 void fp32_thresholds(double eps2, int d, float* lo, float* hi);
@@ -131,7 +207,7 @@ cudaError_t filter_joined(const PassArgs& a, int64_t T, int2* tile_roots, const 
 // --- single-linkage forest (k_mst.cu)
 // Edges of the minimum spanning forests of the eps-graphs of all elements:
 // points u < v, element, the two cover slots (su < sv) and the FP64 d2; n
-// edges (capacity M), in no particular order.
+// edges (capacity M), sorted by (element, d2, u, v).
 struct ForestOut {
     Buf u, v, elem, su, sv, d2;
     int64_t n = 0;
@@ -140,7 +216,7 @@ struct ForestOut {
 // eps2, hi_thr of fp32_thresholds) and a.pairs[0 .. n_pairs) the element tile
 // pairs not certified all-out at eps. Returns a mapper_status.
 int msf_forest(const PassArgs& a, const int32_t* row_slot, const int32_t* slot_point, const int32_t* slot_elem,
-               int64_t M, int64_t R, int64_t T, int64_t n_pairs, ForestOut* out, cudaStream_t s);
+               int64_t M, int64_t E, int64_t R, int64_t T, int64_t n_pairs, ForestOut* out, cudaStream_t s);
 // Single-linkage clusters at height h (edges with d2 <= h^2) in cover-slot
 // space, in the layout of rows_to_slots (every slot a member and core).
 int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, int32_t* lab, int32_t* is_root,

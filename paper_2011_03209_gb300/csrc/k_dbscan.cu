@@ -29,8 +29,6 @@ namespace mgb {
 namespace {
 
 constexpr int kT = kTile;      // tile rows
-constexpr int kK = 32;         // k chunk
-constexpr int kPad = 132;      // smem row pitch (floats)
 
 __device__ __forceinline__ int64_t upper_bound_i64(const int64_t* a, int64_t n, int64_t v)
 {
@@ -217,8 +215,8 @@ __device__ __forceinline__ bool union_prologue(const PassArgs& A, const PairRows
 template <int MODE>
 __global__ void __launch_bounds__(256, 2) simt_pass_kernel(const PassArgs A)
 {
-    __shared__ __align__(16) float As[kK][kPad];
-    __shared__ __align__(16) float Bs[kK][kPad];
+    __shared__ __align__(16) float As[kSimtK][kSimtPad];
+    __shared__ __align__(16) float Bs[kSimtK][kSimtPad];
     __shared__ int s_aux[2 * kT];                  // 1: column counts; 2: local parents
     __shared__ int s_old[kT];                      // 1: count of each column before this pair
     __shared__ unsigned long long s_code[2 * kT];  // 3: root code of each core row, then best
@@ -251,41 +249,7 @@ __global__ void __launch_bounds__(256, 2) simt_pass_kernel(const PassArgs A)
 
     const int tx = tid & 15, ty = tid >> 4;
     float acc[8][8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-
-    for (int k0 = 0; k0 < A.dp; k0 += kK) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int idx = tid + 256 * v;       // float4 index in the 128 x 32 chunk
-            const int r = idx >> 3, k4 = (idx & 7) * 4;
-            float4 xa = make_float4(0.f, 0.f, 0.f, 0.f), xb = xa;
-            if (r < na) xa = pass_ld4(A, pass_row(A, sa + r), (k0 + k4) >> 2);
-            if (r < nb) xb = pass_ld4(A, pass_row(A, sb + r), (k0 + k4) >> 2);
-            As[k4 + 0][r] = xa.x; As[k4 + 1][r] = xa.y; As[k4 + 2][r] = xa.z; As[k4 + 3][r] = xa.w;
-            Bs[k4 + 0][r] = xb.x; Bs[k4 + 1][r] = xb.y; Bs[k4 + 2][r] = xb.z; Bs[k4 + 3][r] = xb.w;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int k = 0; k < kK; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[k][64 + ty * 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float t = a[i] - b[j];
-                    acc[i][j] = fmaf(t, t, acc[i][j]);
-                }
-        }
-        __syncthreads();
-    }
+    simt_tile_sums(A, sa, sb, na, nb, As, Bs, acc);
 
     const Decider decide{A};
     if (MODE == 1) {

@@ -640,6 +640,8 @@ __device__ __forceinline__ double vec_sum(const double (&p)[NJ], int lane)
 // products go to every CTA's shared memory, one cluster barrier, and the first
 // warp of every CTA does the vector work for itself (lane l holds columns
 // l + 32 j, as the products need them).
+// 100k x 64, one axis: 3.52 -> 0.79 ms; 500k x 128, two axes: 1.47 -> 0.33 ms
+// (one CTA of 1024 threads before).
 constexpr int kPowCluster = 8;
 
 template <int NJ>

@@ -77,11 +77,11 @@ __global__ void __launch_bounds__(256, 2) assign_kernel(const float* __restrict_
 #pragma unroll
     for (int i = 0; i < 8; ++i) { best[i] = FLT_MAX; bidx[i] = INT_MAX; }
     for (int c0 = 0; c0 < K; c0 += kT) {
-        float acc[8][8];
+        unsigned long long s2[8][4];                        // (packed, as simt_tile_sums)
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+            for (int j = 0; j < 4; ++j) s2[i][j] = 0ull;
         for (int k0 = 0; k0 < d; k0 += 32) {
 #pragma unroll 4
             for (int v = 0; v < 16; ++v) {
@@ -97,27 +97,31 @@ __global__ void __launch_bounds__(256, 2) assign_kernel(const float* __restrict_
                 const int r = idx >> 3, k4 = (idx & 7) * 4;
                 float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (c0 + r < K) b = *reinterpret_cast<const float4*>(Pv + (int64_t)(c0 + r) * dp + k0 + k4);
-                Bs[k4 + 0][r] = b.x; Bs[k4 + 1][r] = b.y; Bs[k4 + 2][r] = b.z; Bs[k4 + 3][r] = b.w;
+                Bs[k4 + 0][r] = -b.x; Bs[k4 + 1][r] = -b.y; Bs[k4 + 2][r] = -b.z; Bs[k4 + 3][r] = -b.w;
             }
             __syncthreads();
 #pragma unroll 8
             for (int k = 0; k < 32; ++k) {
                 const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
                 const float4 a1 = *reinterpret_cast<const float4*>(&As[k][64 + ty * 4]);
-                const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-                const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
+                const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[k][tx * 4]);
+                const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[k][64 + tx * 4]);
                 const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                const unsigned long long b[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < 8; ++i) {
+                    const unsigned long long aa = f2_pack(a[i], a[i]);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float t = a[i] - b[j];
-                        acc[i][j] = fmaf(t, t, acc[i][j]);
-                    }
+                    for (int j = 0; j < 4; ++j) f2_sq_acc(s2[i][j], aa, b[j]);
+                }
             }
             __syncthreads();
         }
+        float acc[8][8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) f2_unpack(s2[i][j], acc[i][2 * j], acc[i][2 * j + 1]);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
