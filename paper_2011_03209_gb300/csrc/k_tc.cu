@@ -268,17 +268,67 @@ __device__ __forceinline__ void fma2_inplace(float& u0, float& u1, float m, floa
     asm("mov.b64 {%0, %1}, %2;" : "=f"(u0), "=f"(u1) : "l"(r));
 }
 
-__device__ __forceinline__ float fmax3(float a, float b, float c)
-{
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
 __device__ __forceinline__ float fmin3(float a, float b, float c)
 {
     float r;
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// The signs of u_i - mid as bits (1: negative), and the smallest |u_i - mid|.
+// Two columns per packed add, then one funnel shift and half a three-input
+// minimum per value: 2 instructions where a compare against each of two limits
+// and its bit are 4.
+__device__ __forceinline__ uint32_t sign_bits(const float (&u)[32], float mid, float& nearest)
+{
+    unsigned long long m;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(m) : "f"(-mid));
+    uint32_t bits = 0u;
+    float near = INFINITY;
+#pragma unroll
+    for (int i = 30; i >= 0; i -= 2) {
+        unsigned long long x;
+        float t0, t1;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(u[i]), "f"(u[i + 1]));
+        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(m));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(x));
+        bits = __funnelshift_l(__float_as_uint(t1), bits, 1);
+        bits = __funnelshift_l(__float_as_uint(t0), bits, 1);
+        near = fmin3(near, fabsf(t0), fabsf(t1));
+    }
+    nearest = near;
+    return bits;
+}
+
+// in (u >= k_in) and kept (u >= k_out) bits of a row's 32 screen values. The
+// three-product band is narrow, so most rows have no value in it: with mid
+// between the limits and hb >= k_in - mid, mid - k_out (rounded up),
+// t = fl(u - mid) > hb means u >= k_in and t < -hb means u < k_out (rounding
+// is monotone), so if every |t| passes hb the signs decide every value. Only
+// otherwise (or with limits that are not finite) are both compares made. Count
+// pass of the 500k x 128 2D graph (every block mixed) 18.25 -> 16.60 ms, of four
+// radii at once on 200k x 128 15.6 -> 14.2.
+__device__ __forceinline__ void limit_bits(const float (&u)[32], float k_in, float k_out, uint32_t& in_bits,
+                                           uint32_t& keep_bits)
+{
+    const float mid = 0.5f * k_in + 0.5f * k_out;
+    const float hb = fmaxf(__fsub_ru(k_in, mid), __fsub_ru(mid, k_out));
+    float nearest;
+    in_bits = keep_bits = ~sign_bits(u, mid, nearest);
+    if (!(nearest > hb) || !(k_in < INFINITY)) {
+        in_bits = keep_bits = 0u;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            if (u[i] >= k_in) in_bits |= 1u << i;
+            if (u[i] >= k_out) keep_bits |= 1u << i;
+        }
+    }
+}
+
+__device__ __forceinline__ float fmax3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
 
@@ -1080,10 +1130,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         if (!out && xmin >= k_in) {
                             ib = kb = 0xffffffffu;
                         } else if (!out) {
+                            if constexpr (NS == 3) {
+                                limit_bits(u, k_in, k_out, ib, kb);
+                            } else {
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                if (u[i] >= k_in) ib |= 1u << i;
-                                if (u[i] >= k_out) kb |= 1u << i;
+                                for (int i = 0; i < 32; ++i) {
+                                    if (u[i] >= k_in) ib |= 1u << i;
+                                    if (u[i] >= k_out) kb |= 1u << i;
+                                }
                             }
                         }
                         inb = ib & cand;
@@ -1219,10 +1273,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         fma2_inplace(u[4 * i4 + 0], u[4 * i4 + 1], two, nn.x, nn.y);
                         fma2_inplace(u[4 * i4 + 2], u[4 * i4 + 3], two, nn.z, nn.w);
                     }
+                    if constexpr (NS == 3 && !F) {
+                        limit_bits(u, k_in, k_out, in_bits, keep_bits);
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        if (u[i] >= k_in) in_bits |= 1u << i;
-                        if (u[i] >= k_out) keep_bits |= 1u << i;
+                        for (int i = 0; i < 32; ++i) {
+                            if (u[i] >= k_in) in_bits |= 1u << i;
+                            if (u[i] >= k_out) keep_bits |= 1u << i;
+                        }
                     }
                 }
                 const int left = cur.nb[h] - part * 32;
