@@ -52,16 +52,17 @@ struct CoverData {
     int32_t n_int[2] = {1, 1};
     double overlap[2] = {0, 0};
     int64_t n = 0, E = 0, M = 0;
-    Buf keys;                  // sorted (element << 32 | point), M
     Buf elem_off;              // E + 1 int64
     Buf slot_point, slot_elem; // M int32 each
+    Buf pt_off, slot_o;        // memberships in point order: n + 1 int64 offsets, and each
+                               // slot's place (M int32); unset for a subset of a cover
     std::vector<int64_t> h_elem_off;
 };
 
 struct ClusterData {
     StreamRef stream;
     std::shared_ptr<CoverData> cover;
-    Buf core, lab, is_root, is_member, slot_label;    // per cover slot
+    Buf core, lab, flags, slot_label;                 // per cover slot
     mapper_stats stats{};
 };
 
@@ -266,7 +267,8 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     c->E = E;
     for (int j = 0; j < m; ++j) { c->n_int[j] = n_int[j]; c->overlap[j] = overlap[j]; }
 
-    Buf lohi, bounds, cnt, pos, flag;
+    Buf lohi, bounds, cnt, flag;
+    Buf& pos = c->pt_off;
     CK(lohi.alloc(sizeof(double) * 2 * m, s), "alloc");
     CK(bounds.alloc(sizeof(double) * 2 * ((size_t)n_int[0] + (m == 2 ? n_int[1] : 0)), s), "alloc");
     CK(cnt.alloc(sizeof(int32_t) * n, s), "alloc");
@@ -291,18 +293,19 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     if (h_nf) return fail(MAPPER_ENONFINITE, "lens or X holds NaN or Inf");
     if (M > INT32_MAX) return fail(MAPPER_ENOMEM, "more than 2^31 cover memberships");
     c->M = M;
-    Buf tmp;
-    CK(c->keys.alloc(sizeof(uint64_t) * M, s), "alloc keys");
+    Buf keys, tmp, pt;
+    CK(keys.alloc(sizeof(uint64_t) * M, s), "alloc keys");
     CK(tmp.alloc(sizeof(uint64_t) * M, s), "alloc");
+    CK(pt.alloc(sizeof(int32_t) * M, s), "alloc");
     CK(cover_emit(lens, n, m, bounds.as<double>(), n_int[0], m == 2 ? n_int[1] : 1,
-                  pos.as<int64_t>(), c->keys.as<uint64_t>(), s), "cover_emit");
-    CK(radix_sort_u64(c->keys, tmp, M, 32, 32 + bits_for(E), s), "sort");
+                  pos.as<int64_t>(), keys.as<uint64_t>(), pt.as<int32_t>(), s), "cover_emit");
+    CK(radix_sort_u64(keys, tmp, M, 32, 32 + bits_for(E), s), "sort");
     CK(c->elem_off.alloc(sizeof(int64_t) * (E + 1), s), "alloc");
-    CK(element_offsets(c->keys.as<uint64_t>(), M, E, c->elem_off.as<int64_t>(), s), "elem_off");
     CK(c->slot_point.alloc(sizeof(int32_t) * M, s), "alloc");
     CK(c->slot_elem.alloc(sizeof(int32_t) * M, s), "alloc");
-    CK(split_keys(c->keys.as<uint64_t>(), M, c->slot_point.as<int32_t>(), c->slot_elem.as<int32_t>(), s),
-       "split");
+    CK(c->slot_o.alloc(sizeof(int32_t) * M, s), "alloc");
+    CK(split_keys(keys.as<uint64_t>(), pt.as<int32_t>(), M, E, c->slot_point.as<int32_t>(),
+                  c->slot_elem.as<int32_t>(), c->slot_o.as<int32_t>(), c->elem_off.as<int64_t>(), s), "split");
     c->h_elem_off.resize(E + 1);
     CK(cudaMemcpyAsync(c->h_elem_off.data(), c->elem_off.p, sizeof(int64_t) * (E + 1),
                        cudaMemcpyDeviceToHost, s), "copy");
@@ -967,42 +970,32 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         CK(list_unions(a.count, a.nbr, cap, a.core, a.parent, a.row_pt, R, s, a.stats + kStatOob), "list unions");
         CK(allin_pass(2, rd.a_in, PL.n[kListAllIn], s), "pass 2 all-in");
         // Unions in rounds of growing tile distance b - a (tiles of one pivot
-        // region are adjacent), after the unions along the neighbour lists: a
-        // pair is kept only if its core rows are not all joined yet (from the
-        // second round on when there are no lists), and pairs whose two sides are
-        // each already one component only need one neighbour pair.
+        // region are adjacent): a pair is kept only if its core rows are not
+        // all joined yet (from the second round on when there are no lists), and
+        // pairs whose two sides are each already one component only need one
+        // neighbour pair. After the unions along the neighbour lists few pairs
+        // are left (none to a few hundred of up to 1.2 M; 3 k of 173 k at 1M x
+        // 256), so two rounds do; without lists (minPts 1, or above 65) the
+        // rounds join everything, in five steps.
         auto union_rounds = [&](const PassArgs& base, const TcArgs& tbase, int64_t n, bool tc) -> int {
             if (n == 0) return MAPPER_OK;
             // every count stays on the device: each launch covers the list's
             // capacity n and reads its length there, so the rounds need no host
             // round trip
-            static const int kBounds[] = {-1, 1, 4, 16, 64, INT_MAX};
-            Buf hits, sel, kept, cnt, troots;
+            static const int kFew[] = {-1, 1, INT_MAX}, kMany[] = {-1, 1, 4, 16, 64, INT_MAX};
+            const int* bounds = cap ? kFew : kMany;
+            const int rounds = cap ? 2 : 5;
+            Buf list, cnt, troots;
             CK(troots.alloc(sizeof(int2) * std::max<int64_t>(L.T, 1), s), "alloc");
-            CK(hits.alloc(sizeof(int2) * n, s), "alloc");
-            CK(sel.alloc(sizeof(int2) * n, s), "alloc");
-            CK(kept.alloc(sizeof(int2) * n, s), "alloc");
-            CK(cnt.alloc(sizeof(unsigned long long) * 3, s), "alloc");
-            unsigned long long* c_hit = cnt.as<unsigned long long>();
-            unsigned long long* c_sel = c_hit + 1;
-            unsigned long long* c_kept = c_hit + 2;
-            CK(cudaMemsetAsync(c_hit, 0, sizeof(unsigned long long), s), "memset");
-            CK(select_hit(base.pairs, base.pair_hit, n, hits.as<int2>(), c_hit, s), "select");
-            CK(add_counter(base.stats + kStatUnion, c_hit, s), "count");
-            for (int k = 0; k + 1 < (int)(sizeof(kBounds) / sizeof(kBounds[0])); ++k) {
-                CK(cudaMemsetAsync(c_sel, 0, sizeof(unsigned long long) * 2, s), "memset");
-                CK(select_delta(hits.as<int2>(), n, c_hit, kBounds[k], kBounds[k + 1], sel.as<int2>(), c_sel, s),
-                   "select");
-                const int2* list = sel.as<int2>();
-                const unsigned long long* c_list = c_sel;
-                if (k > 0 || cap) {
-                    CK(filter_joined(base, L.T, troots.as<int2>(), sel.as<int2>(), n, c_sel, kept.as<int2>(), c_kept,
-                                     s), "filter");
-                    list = kept.as<int2>();
-                    c_list = c_kept;
-                }
+            CK(list.alloc(sizeof(int2) * n, s), "alloc");
+            CK(cnt.alloc(sizeof(unsigned long long) * rounds, s), "alloc");
+            CK(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long) * rounds, s), "memset");
+            for (int k = 0; k < rounds; ++k) {
+                unsigned long long* c_list = cnt.as<unsigned long long>() + k;
+                CK(select_round(base, L.T, troots.as<int2>(), n, bounds[k], bounds[k + 1], k > 0 || cap, k == 0,
+                                list.as<int2>(), c_list, s), "select");
                 PassArgs ar = base;
-                ar.pairs = list;
+                ar.pairs = list.as<int2>();
                 ar.n_dev = c_list;
                 ar.pair_hit = nullptr;
                 int r2;
@@ -1036,11 +1029,10 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
 
         CK(c->core.alloc(M, s), "alloc");
         CK(c->lab.alloc(sizeof(int32_t) * M, s), "alloc");
-        CK(c->is_root.alloc(sizeof(int32_t) * M, s), "alloc");
-        CK(c->is_member.alloc(sizeof(int32_t) * M, s), "alloc");
+        CK(c->flags.alloc(M, s), "alloc");
         CK(c->slot_label.alloc(sizeof(int64_t) * M, s), "alloc");
         CK(rows_to_slots(L.row_slot.as<int32_t>(), a.row_pt, a.core, a.root, a.border, R, c->lab.as<int32_t>(),
-                         c->is_root.as<int32_t>(), c->is_member.as<int32_t>(), c->slot_label.as<int64_t>(),
+                         c->flags.as<uint8_t>(), c->slot_label.as<int64_t>(),
                          c->core.as<uint8_t>(), s), "labels");
 
         unsigned long long h_stats[kStatCount];
@@ -1130,35 +1122,50 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
     cudaStream_t s = ctx->stream->s;
     const auto& cov = cl->cover;
     const int64_t M = cov->M;
-    Buf nid, mpos;
-    CK(nid.alloc(sizeof(int64_t) * (M + 1), s), "alloc");
-    CK(mpos.alloc(sizeof(int64_t) * (M + 1), s), "alloc");
-    CK(exclusive_scan_i32_to_i64(cl->is_root.as<int32_t>(), nid.as<int64_t>(), M, s), "scan");
-    CK(exclusive_scan_i32_to_i64(cl->is_member.as<int32_t>(), mpos.as<int64_t>(), M, s), "scan");
-    int64_t h[2];
-    CK(cudaMemcpyAsync(&h[0], nid.as<int64_t>() + M, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "copy");
-    CK(cudaMemcpyAsync(&h[1], mpos.as<int64_t>() + M, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "copy");
+    Buf pos;
+    CK(pos.alloc(sizeof(int64_t) * (M + 1), s), "alloc");
+    CK(exclusive_scan_slot_flags(cl->flags.as<uint8_t>(), pos.as<int64_t>(), M, s), "scan");
+    int64_t totals = 0;
+    CK(cudaMemcpyAsync(&totals, pos.as<int64_t>() + M, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "copy");
     CK(cudaStreamSynchronize(s), "sync");
-    const int64_t N = h[0], Gm = h[1];
+    const int64_t N = totals >> 32, Gm = totals & 0xffffffffll;
     g->N = N;
     g->Gm = Gm;
-    Buf keys, tmp, keys2;
+    const bool in_order = cov->slot_o.p != nullptr;               // the cover keeps the memberships in point order
+    Buf keys, tmp, keys2, node_o;
     CK(keys.alloc(sizeof(uint64_t) * Gm, s), "alloc");
     CK(tmp.alloc(sizeof(uint64_t) * Gm, s), "alloc");
-    CK(keys2.alloc(sizeof(uint64_t) * Gm, s), "alloc");
+    if (in_order) CK(node_o.alloc(sizeof(int32_t) * M, s), "alloc");
     CK(g->node_elem.alloc(sizeof(int32_t) * N, s), "alloc");
     CK(g->node_off.alloc(sizeof(int64_t) * (N + 1), s), "alloc");
     CK(g->node_members.alloc(sizeof(int32_t) * Gm, s), "alloc");
-    CK(member_keys(cl->lab.as<int32_t>(), nid.as<int64_t>(), mpos.as<int64_t>(),
-                   cov->slot_point.as<int32_t>(), cov->slot_elem.as<int32_t>(), M,
-                   keys.as<uint64_t>(), g->node_elem.as<int32_t>(), s), "member keys");
+    CK(member_keys(cl->lab.as<int32_t>(), pos.as<int64_t>(), cov->slot_point.as<int32_t>(),
+                   cov->slot_elem.as<int32_t>(), cov->slot_o.as<int32_t>(), M, keys.as<uint64_t>(),
+                   g->node_elem.as<int32_t>(), node_o.as<int32_t>(), s), "member keys");
     CK(radix_sort_u64(keys, tmp, Gm, 32, 32 + bits_for(N), s), "sort");
-    CK(node_offsets(keys.as<uint64_t>(), Gm, g->node_off.as<int64_t>(), g->node_members.as<int32_t>(),
-                    keys2.as<uint64_t>(), s), "node offsets");
-    CK(cudaMemcpyAsync(g->node_off.as<int64_t>() + N, &g->Gm, sizeof(int64_t), cudaMemcpyHostToDevice, s),
-       "copy");
-    int rc = nerve_edges(ctx, keys2, Gm, cov->n, N, g);
-    if (rc) return rc;
+    auto offsets = [&](uint64_t* k2) {
+        return node_offsets(keys.as<uint64_t>(), Gm, N, g->node_off.as<int64_t>(), g->node_members.as<int32_t>(), k2, s);
+    };
+    bool edges_done = false;
+    if (in_order) {
+        CK(offsets(nullptr), "node offsets");
+        Buf counts;
+        CK(counts.alloc(2 * sizeof(unsigned long long), s), "alloc");
+        unsigned long long* dc = counts.as<unsigned long long>();
+        CK(edge_set(cov->pt_off.as<int64_t>(), cov->n, node_o.as<int32_t>(), &g->edges, dc, s), "edges");
+        CK(radix_sort_u64_two_dev(g->edges.as<uint64_t>(), kEdgeListMax, dc, 32, 0, bits_for(N), s), "sort");
+        unsigned long long h[2] = {0, 0};
+        CK(cudaMemcpyAsync(h, dc, sizeof(h), cudaMemcpyDeviceToHost, s), "copy");
+        CK(cudaStreamSynchronize(s), "sync");
+        edges_done = h[1] == 0;
+        g->Eg = (int64_t)h[0];
+    }
+    if (!edges_done) {
+        CK(keys2.alloc(sizeof(uint64_t) * Gm, s), "alloc");
+        CK(offsets(keys2.as<uint64_t>()), "node offsets");
+        int rc = nerve_edges(ctx, keys2, Gm, cov->n, N, g);
+        if (rc) return rc;
+    }
     g->stats = cl->stats;
     g->stats.n_nodes = N;
     g->stats.n_edges = g->Eg;
@@ -1659,11 +1666,10 @@ int mapper_forest_cut(mapper_ctx* ctx, const mapper_forest_t* forest, double h, 
     c->cover = f->cover;
     CK(c->core.alloc(std::max<int64_t>(M, 1), s), "alloc");
     CK(c->lab.alloc(sizeof(int32_t) * std::max<int64_t>(M, 1), s), "alloc");
-    CK(c->is_root.alloc(sizeof(int32_t) * std::max<int64_t>(M, 1), s), "alloc");
-    CK(c->is_member.alloc(sizeof(int32_t) * std::max<int64_t>(M, 1), s), "alloc");
+    CK(c->flags.alloc(std::max<int64_t>(M, 1), s), "alloc");
     CK(c->slot_label.alloc(sizeof(int64_t) * std::max<int64_t>(M, 1), s), "alloc");
-    if ((rc = msf_cut(f->f, f->cover->slot_point.as<int32_t>(), M, h, c->lab.as<int32_t>(), c->is_root.as<int32_t>(),
-                      c->is_member.as<int32_t>(), c->slot_label.as<int64_t>(), c->core.as<uint8_t>(), s)))
+    if ((rc = msf_cut(f->f, f->cover->slot_point.as<int32_t>(), M, h, c->lab.as<int32_t>(), c->flags.as<uint8_t>(),
+                      c->slot_label.as<int64_t>(), c->core.as<uint8_t>(), s)))
         return rc;
     CK(cudaStreamSynchronize(s), "sync");
     c->stats = f->stats;

@@ -139,23 +139,32 @@ cudaError_t balanced_bounds(const double* f, int64_t n, int m, const int32_t* n_
 cudaError_t cover_count(const double* f, int64_t n, int m, const double* bounds,
                         int32_t n0, int32_t n1, int32_t* cnt, cudaStream_t s);
 cudaError_t cover_emit(const double* f, int64_t n, int m, const double* bounds, int32_t n0,
-                       int32_t n1, const int64_t* pos, uint64_t* keys, cudaStream_t s);
+                       int32_t n1, const int64_t* pos, uint64_t* keys, int32_t* pt, cudaStream_t s);
 
 // scan / sort / compaction (k_sort.cu)
 cudaError_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n,
                                       cudaStream_t s);   // out has n+1 entries
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s);
+// Per slot a byte of flags, bit 0 member and bit 1 root: out[i] = (roots before
+// slot i) << 32 | members before slot i, out[n] the totals.
+cudaError_t exclusive_scan_slot_flags(const uint8_t* in, int64_t* out, int64_t n, cudaStream_t s);
 // Stable LSD radix sorts of n 64-bit keys: on bits [lo_bit, hi_bit), or on
 // bits [lo1, lo1 + bits) above bits [lo0, lo0 + bits). tmp: a buffer of at least n keys;
 // the two buffers may come back swapped (the sorted keys are in `keys`).
 cudaError_t radix_sort_u64(Buf& keys, Buf& tmp, int64_t n, int lo_bit, int hi_bit, cudaStream_t s);
 cudaError_t radix_sort_u64_two(Buf& keys, Buf& tmp, int64_t n, int lo0, int lo1, int bits, cudaStream_t s);
 
+// The same in place for *n_dev <= n_max <= 131072 keys, their number on the device.
+cudaError_t radix_sort_u64_two_dev(uint64_t* keys, int64_t n_max, const unsigned long long* n_dev, int lo0, int lo1,
+                                   int bits, cudaStream_t s);
+
 // slots of a cover with one element holding every point (slot i = point i)
 cudaError_t whole_cloud_slots(int64_t n, int32_t* slot_point, int32_t* slot_elem, cudaStream_t s);
 
-// split sorted (element << 32 | point) keys into slot_point / slot_elem
-cudaError_t split_keys(const uint64_t* keys, int64_t M, int32_t* slot_point, int32_t* slot_elem,
-                       cudaStream_t s);
+// From the sorted keys of cover_emit (element << 32 | membership, M of them, pt
+// the memberships' points): slot_point, slot_elem and slot_o (the slot's
+// membership in point order), and elem_off[E + 1].
+cudaError_t split_keys(const uint64_t* keys, const int32_t* pt, int64_t M, int64_t E, int32_t* slot_point,
+                       int32_t* slot_elem, int32_t* slot_o, int64_t* elem_off, cudaStream_t s);
 
 }  // namespace mgb

@@ -173,13 +173,14 @@ cudaError_t border_from_lists(const int32_t* count, const int32_t* nbr, int cap,
                               int64_t R, unsigned long long* border, cudaStream_t s,
                               unsigned long long* oob = nullptr);
 // Row space -> cover-slot space: per slot the root slot of its node (or -1),
-// canonical point id (or -1), root flag, member flag and core flag.
+// canonical point id (or -1), the flags of exclusive_scan_slot_flags and the
+// core flag.
 // Unions of each core row with the core rows of its pass-1 neighbour list.
 cudaError_t list_unions(const int32_t* count, const int32_t* nbr, int cap, const uint8_t* core, int32_t* parent,
                         const int32_t* row_pt, int64_t R, cudaStream_t s, unsigned long long* oob = nullptr);
 cudaError_t rows_to_slots(const int32_t* row_slot, const int32_t* row_pt, const uint8_t* core,
                           const int32_t* root, const unsigned long long* border, int64_t R,
-                          int32_t* lab, int32_t* is_root, int32_t* is_member,
+                          int32_t* lab, uint8_t* flags,
                           int64_t* slot_label, uint8_t* slot_core, cudaStream_t s);
 cudaError_t element_offsets(const uint64_t* keys, int64_t M, int64_t E, int64_t* elem_off,
                             cudaStream_t s);
@@ -187,22 +188,13 @@ cudaError_t element_offsets(const uint64_t* keys, int64_t M, int64_t E, int64_t*
 // a one-element cover of the whole cloud: the density filter).
 cudaError_t counts_to_lens(const int32_t* row_slot, const int32_t* row_pt, const int32_t* count, int64_t R,
                            double* f, int m, int j, cudaStream_t s);
-// Appends to `out` the tile pairs of `pairs` whose hit flag is set; *count
-// receives the size.
-cudaError_t select_hit(const int2* pairs, const uint8_t* hit, int64_t n, int2* out,
-                       unsigned long long* count, cudaStream_t s);
-// *dst += *src (one device counter into another).
-cudaError_t add_counter(unsigned long long* dst, const unsigned long long* src, cudaStream_t s);
-// Appends to `out` the tile pairs (a, b) of pairs[0 .. *n_dev) (at most n)
-// with lo < b - a <= hi; *count receives the size.
-cudaError_t select_delta(const int2* pairs, int64_t n, const unsigned long long* n_dev, int lo, int hi, int2* out,
-                         unsigned long long* count, cudaStream_t s);
-// Keeps the union-pass tile pairs of pairs[0 .. *n_dev) (at most n) whose
-// core rows do not all share one root yet (flagging kPairOneEach pairs);
-// *count receives the size. tile_roots: scratch of T entries (the current
-// root range of each of the T tiles).
-cudaError_t filter_joined(const PassArgs& a, int64_t T, int2* tile_roots, const int2* pairs, int64_t n,
-                          const unsigned long long* n_dev, int2* out, unsigned long long* count, cudaStream_t s);
+// The tile pairs of a union round: appends to `out` the pairs of a.pairs[0 .. n)
+// flagged in a.pair_hit with lo < b - a <= hi and (filter) core rows that do not
+// all share one root yet (flagging kPairOneEach pairs); *count (zeroed by the
+// caller) receives their number. first: also adds the flagged pairs to
+// kStatUnion. tile_roots: scratch of T entries (the root range of each tile).
+cudaError_t select_round(const PassArgs& a, int64_t T, int2* tile_roots, int64_t n, int lo, int hi, bool filter,
+                         bool first, int2* out, unsigned long long* count, cudaStream_t s);
 
 // --- single-linkage forest (k_mst.cu)
 // Edges of the minimum spanning forests of the eps-graphs of all elements:
@@ -219,8 +211,8 @@ int msf_forest(const PassArgs& a, const int32_t* row_slot, const int32_t* slot_p
                int64_t M, int64_t E, int64_t R, int64_t T, int64_t n_pairs, ForestOut* out, cudaStream_t s);
 // Single-linkage clusters at height h (edges with d2 <= h^2) in cover-slot
 // space, in the layout of rows_to_slots (every slot a member and core).
-int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, int32_t* lab, int32_t* is_root,
-            int32_t* is_member, int64_t* slot_label, uint8_t* core, cudaStream_t s);
+int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, int32_t* lab, uint8_t* flags,
+            int64_t* slot_label, uint8_t* core, cudaStream_t s);
 
 // --- nodes and nerve (k_nerve.cu)
 // Nerve keys (point << 32 | node) of the members of nodes given by offsets.
@@ -228,11 +220,20 @@ cudaError_t node_member_keys(const int64_t* node_off, int64_t N, int64_t G, cons
                              uint64_t* keys2, cudaStream_t s);
 // slot_elem[i] = the element e with elem_off[e] <= i < elem_off[e + 1].
 cudaError_t fill_slot_elem(const int64_t* elem_off, int32_t k, int64_t M, int32_t* slot_elem, cudaStream_t s);
-cudaError_t member_keys(const int32_t* lab, const int64_t* nid, const int64_t* mpos,
-                        const int32_t* slot_point, const int32_t* slot_elem, int64_t M,
-                        uint64_t* keys, int32_t* node_elem, cudaStream_t s);
-cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t* node_off, int32_t* members,
+// pos: the scan of the slots' flags. keys: (node << 32 | point) of the member
+// slots; node_elem; node_o (if set): the node of every membership in point order
+// (slot_o of split_keys), -1 for none.
+cudaError_t member_keys(const int32_t* lab, const int64_t* pos, const int32_t* slot_point, const int32_t* slot_elem,
+                        const int32_t* slot_o, int64_t M, uint64_t* keys, int32_t* node_elem, int32_t* node_o,
+                        cudaStream_t s);
+cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t N, int64_t* node_off, int32_t* members,
                          uint64_t* keys2, cudaStream_t s);
+// The distinct node pairs (v << 32 | u) sharing a point, unsorted, into *list (at
+// most kEdgeListMax); counts[0]: their number, counts[1]: nonzero if the list
+// does not hold them all.
+constexpr uint32_t kEdgeListMax = 1u << 15;
+cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, Buf* list, unsigned long long* counts,
+                     cudaStream_t s);
 cudaError_t run_pairs(const uint64_t* keys2, int64_t G, int64_t* cnt, cudaStream_t s);
 cudaError_t emit_pairs(const uint64_t* keys2, int64_t G, const int64_t* pos, uint64_t* out,
                        cudaStream_t s);

@@ -11,7 +11,7 @@
 // closed (a_k <= f <= b_k). Both a_k and b_k are nondecreasing in k, so the
 // elements holding a value f form the index range [first k with b_k >= f,
 // last k with a_k <= f], found by binary search.
-#include "common.cuh"
+#include "dbscan.cuh"
 
 namespace mgb {
 
@@ -177,7 +177,8 @@ __global__ void cover_count_kernel(const double* __restrict__ f, int64_t n, int 
 
 __global__ void cover_emit_kernel(const double* __restrict__ f, int64_t n, int m,
                                   const double* __restrict__ bounds, int32_t n0, int32_t n1,
-                                  const int64_t* __restrict__ pos, uint64_t* __restrict__ keys)
+                                  const int64_t* __restrict__ pos, uint64_t* __restrict__ keys,
+                                  int32_t* __restrict__ pt)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
@@ -192,18 +193,29 @@ __global__ void cover_emit_kernel(const double* __restrict__ f, int64_t n, int m
     for (int32_t i = l0; i <= h0; ++i)
         for (int32_t k = l1; k <= h1; ++k) {
             const uint64_t e = (uint64_t)((int64_t)i * nn1 + k);
-            keys[o++] = (e << 32) | (uint64_t)(uint32_t)p;
+            keys[o] = (e << 32) | (uint64_t)o;
+            pt[o++] = (int32_t)p;
         }
 }
 
-__global__ void split_keys_kernel(const uint64_t* __restrict__ keys, int64_t M,
-                                  int32_t* __restrict__ slot_point, int32_t* __restrict__ slot_elem)
+__global__ void split_keys_kernel(const uint64_t* __restrict__ keys, const int32_t* __restrict__ pt, int64_t M,
+                                  int64_t E, int32_t* __restrict__ slot_point, int32_t* __restrict__ slot_elem,
+                                  int32_t* __restrict__ slot_o, int64_t* __restrict__ elem_off)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= M) return;
     const uint64_t k = keys[s];
-    slot_point[s] = (int32_t)(uint32_t)k;
-    slot_elem[s] = (int32_t)(k >> 32);
+    const int32_t o = (int32_t)(uint32_t)k, e = (int32_t)(k >> 32);
+    slot_point[s] = pt[o];
+    slot_elem[s] = e;
+    slot_o[s] = o;
+    if (elem_off) {
+        // element offsets where the element changes (empty elements between)
+        const int32_t before = s ? (int32_t)(keys[s - 1] >> 32) : -1;
+        for (int32_t x = before + 1; x <= e; ++x) elem_off[x] = s;
+        if (s == M - 1)
+            for (int64_t x = (int64_t)e + 1; x <= E; ++x) elem_off[x] = M;
+    }
 }
 
 }  // namespace
@@ -224,12 +236,22 @@ cudaError_t whole_cloud_slots(int64_t n, int32_t* slot_point, int32_t* slot_elem
     return cudaGetLastError();
 }
 
-cudaError_t split_keys(const uint64_t* keys, int64_t M, int32_t* slot_point, int32_t* slot_elem,
-                       cudaStream_t s)
+// Up to this many elements the thread at a change of element writes the offsets
+// of the empty ones before it; more (a fine grid, mostly empty) take a search
+// per element.
+constexpr int64_t kSplitElems = 4096;
+
+cudaError_t split_keys(const uint64_t* keys, const int32_t* pt, int64_t M, int64_t E, int32_t* slot_point,
+                       int32_t* slot_elem, int32_t* slot_o, int64_t* elem_off, cudaStream_t s)
 {
-    if (M == 0) return cudaSuccess;
-    { split_keys_kernel<<<div_up(M, 256), 256, 0, s>>>(keys, M, slot_point, slot_elem); note_launch(); }
-    return cudaGetLastError();
+    const bool search = E > kSplitElems || M == 0;
+    if (M > 0) {
+        split_keys_kernel<<<div_up(M, 256), 256, 0, s>>>(keys, pt, M, E, slot_point, slot_elem, slot_o,
+                                                         search ? nullptr : elem_off);
+        note_launch();
+        MGB_TRY(cudaGetLastError());
+    }
+    return search ? element_offsets(keys, M, E, elem_off, s) : cudaSuccess;
 }
 
 cudaError_t lens_range_flag(const double* f, int64_t n, int m, double* lohi, int* nonfinite,
@@ -291,10 +313,10 @@ cudaError_t cover_count(const double* f, int64_t n, int m, const double* bounds,
 }
 
 cudaError_t cover_emit(const double* f, int64_t n, int m, const double* bounds, int32_t n0,
-                       int32_t n1, const int64_t* pos, uint64_t* keys, cudaStream_t s)
+                       int32_t n1, const int64_t* pos, uint64_t* keys, int32_t* pt, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    { cover_emit_kernel<<<div_up(n, 256), 256, 0, s>>>(f, n, m, bounds, n0, n1, pos, keys); note_launch(); }
+    { cover_emit_kernel<<<div_up(n, 256), 256, 0, s>>>(f, n, m, bounds, n0, n1, pos, keys, pt); note_launch(); }
     return cudaGetLastError();
 }
 

@@ -495,26 +495,68 @@ __global__ void border_lists_kernel(const int32_t* __restrict__ count, const int
 // Unions along the neighbour lists of pass 1: a core row's list holds its
 // first cap neighbours, every one a certified neighbour pair; joining the
 // core ones merges most of each cluster before the union pass, which then
-// skips every tile pair whose core rows already share one root.
+// skips every tile pair whose core rows already share one root. In three
+// steps: with every row its own root, all rows of a cluster would race for
+// the same few roots with compare-and-swap along growing chains.
+//   hook      each row points at its core neighbour of smallest key, if
+//             smaller than its own (no atomics; keys fall along every chain);
+//   compress  each row points at its root;
+//   unions    list entries whose rows still point at different roots.
+// All of a graph's union work (these, and two rounds over the tile pairs where
+// there were five with lists between them): with the nerve's hash set 14k x 37
+// 1308 -> 1148 us, 100k x 64 2644 -> 2218, sweep of 200k x 128 25762 -> 24064.
+__global__ void list_hook_kernel(const int32_t* __restrict__ count, const int32_t* __restrict__ nbr, int cap,
+                                 const uint8_t* __restrict__ core, int32_t* __restrict__ parent,
+                                 const int32_t* __restrict__ row_pt, int64_t R, unsigned long long* oob)
+{
+    (void)oob;
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= R || !core[s]) return;
+    const int k = min(count[s], cap);
+    int best = (int)s, key = key_of(row_pt, (int)s);
+#pragma unroll 4
+    for (int i = 0; i < k; ++i) {
+        const int q = nbr[s * cap + i];
+        if (q < 0 || !MGB_IN_RANGE(q, R, oob) || !core[q]) continue;
+        const int kq = key_of(row_pt, q);
+        if (kq < key) { key = kq; best = q; }
+    }
+    parent[s] = best;
+}
+
+__global__ void list_compress_kernel(const uint8_t* __restrict__ core, int32_t* parent, int64_t R)
+{
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= R || !core[s]) return;
+    volatile int32_t* par = parent;
+    int r = (int)s, p = par[r];
+    while (p != r) { r = p; p = par[r]; }
+    par[s] = r;
+}
+
 __global__ void list_unions_kernel(const int32_t* __restrict__ count, const int32_t* __restrict__ nbr, int cap,
-                                   const uint8_t* __restrict__ core, int32_t* __restrict__ parent,
+                                   const uint8_t* __restrict__ core, int32_t* parent,
                                    const int32_t* __restrict__ row_pt, int64_t R, unsigned long long* oob)
 {
     (void)oob;
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= R || !core[s]) return;
     const int k = min(count[s], cap);
+    volatile int32_t* par = parent;
+    int ps = par[s];
     for (int i = 0; i < k; ++i) {
         const int q = nbr[s * cap + i];
-        if (q >= 0 && MGB_IN_RANGE(q, R, oob) && core[q]) gunion(parent, row_pt, (int)s, q);
+        if (q < 0 || !MGB_IN_RANGE(q, R, oob) || par[q] == ps || !core[q]) continue;
+        gunion(parent, row_pt, (int)s, q);
+        ps = par[s];
     }
 }
 
 __global__ void rows_to_slots_kernel(const int32_t* __restrict__ row_slot, const int32_t* __restrict__ row_pt,
                                      const uint8_t* __restrict__ core, const int32_t* __restrict__ root,
                                      const unsigned long long* __restrict__ border, int64_t R,
-                                     int32_t* __restrict__ lab, int32_t* __restrict__ is_root,
-                                     int32_t* __restrict__ is_member, int64_t* __restrict__ slot_label,
+                                     int32_t* __restrict__ lab, uint8_t* __restrict__ flags,
+                                     int64_t* __restrict__ slot_label,
                                      uint8_t* __restrict__ slot_core)
 {
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -527,8 +569,7 @@ __global__ void rows_to_slots_kernel(const int32_t* __restrict__ row_slot, const
     else if (border[row] != ~0ull) l = (int)(unsigned)(border[row] & 0xffffffffull);
     lab[slot] = l >= 0 ? row_slot[l] : -1;
     slot_label[slot] = l >= 0 ? (int64_t)row_pt[l] : -1;
-    is_root[slot] = c && root[row] == (int32_t)row;
-    is_member[slot] = l >= 0;
+    flags[slot] = (uint8_t)((l >= 0 ? 1 : 0) | (c && root[row] == (int32_t)row ? 2 : 0));
     slot_core[slot] = c;
 }
 
@@ -554,26 +595,6 @@ __global__ void elem_offsets_kernel(const uint64_t* __restrict__ keys, int64_t M
     elem_off[e] = l;
 }
 
-__global__ void select_hit_kernel(const int2* __restrict__ pairs, const uint8_t* __restrict__ hit, int64_t n,
-                                  int2* __restrict__ out, unsigned long long* __restrict__ count)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !hit[i]) return;
-    out[atomicAdd(count, 1ull)] = pairs[i];
-}
-
-// Tile pairs whose tile distance b - a lies in (lo, hi].
-__global__ void select_delta_kernel(const int2* __restrict__ pairs, int64_t n,
-                                    const unsigned long long* __restrict__ n_dev, int lo, int hi,
-                                    int2* __restrict__ out, unsigned long long* __restrict__ count)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || (n_dev && (unsigned long long)i >= *n_dev)) return;
-    const int2 p = pairs[i];
-    const int delta = p.y - p.x;
-    if (delta > lo && delta <= hi) out[atomicAdd(count, 1ull)] = p;
-}
-
 // Smallest and largest current root over each tile's core rows (INT_MAX,
 // -1 for a tile without core rows); one warp per tile.
 __global__ void tile_roots_kernel(const PassArgs A, int64_t T, int2* __restrict__ tr)
@@ -597,83 +618,69 @@ __global__ void tile_roots_kernel(const PassArgs A, int64_t T, int2* __restrict_
     if (lane == 0) tr[t] = make_int2(lo, hi);
 }
 
-// A tile pair is kept if the roots of its core rows differ (read from the
-// tiles' root ranges); an off-diagonal pair whose A cores share one root and
-// whose B cores share another is flagged (kPairOneEach): one neighbour pair
-// joins them. One thread per pair.
-__global__ void filter_joined_kernel(const int2* __restrict__ pairs, int64_t n,
-                                     const unsigned long long* __restrict__ n_dev, const int2* __restrict__ tr,
-                                     int2* __restrict__ out, unsigned long long* __restrict__ count,
-                                     unsigned long long* __restrict__ stats)
+// The tile pairs of a union round: flagged by the count pass (hit), tile
+// distance b - a in (lo, hi], and the roots of their core rows differ (read from
+// the tiles' root ranges tr; null: not asked); an off-diagonal pair whose A cores
+// share one root and whose B cores share another is marked kPairOneEach: one
+// neighbour pair joins them. One thread per pair of the whole list. first: also
+// counts the flagged pairs.
+__global__ void __launch_bounds__(256) select_round_kernel(const int2* __restrict__ pairs,
+                                                           const uint8_t* __restrict__ hit, int64_t n, int lo, int hi,
+                                                           const int2* __restrict__ tr, bool first,
+                                                           int2* __restrict__ out, unsigned long long* __restrict__ count,
+                                                           unsigned long long* __restrict__ stats)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n_dev) n = min(n, (int64_t)*n_dev);
     bool keep = false, skipped = false;
+    const bool flagged = i < n && hit[i];
     int2 p = make_int2(0, 0);
-    if (i < n) {
+    if (flagged) {
         p = pairs[i];
-        const bool diag = p.x == p.y;
-        const int2 a = tr[p.x], b = tr[p.y];
-        bool work, one_each = false;
-        if (diag) {
-            work = a.y >= 0 && a.x != a.y;
-        } else {
-            work = a.y >= 0 && b.y >= 0 && (a.x != a.y || b.x != b.y || a.x != b.x);
-            one_each = work && a.x == a.y && b.x == b.y;
+        const int delta = p.y - p.x;
+        keep = delta > lo && delta <= hi;
+        if (keep && tr) {
+            const int2 a = tr[p.x], b = tr[p.y];
+            bool one_each = false;
+            if (p.x == p.y) {
+                keep = a.y >= 0 && a.x != a.y;
+            } else {
+                keep = a.y >= 0 && b.y >= 0 && (a.x != a.y || b.x != b.y || a.x != b.x);
+                one_each = keep && a.x == a.y && b.x == b.y;
+            }
+            skipped = !keep && a.y >= 0;
+            if (one_each) p.y |= kPairOneEach;
         }
-        keep = work;
-        skipped = !work && a.y >= 0;
-        if (one_each) p.y |= kPairOneEach;
     }
-    // one output atomic per warp
+    // one output atomic per warp, one per counter and block
     const unsigned m = __ballot_sync(0xffffffffu, keep);
     unsigned long long base = 0;
     const int lane = threadIdx.x & 31;
     if (lane == 0 && m) base = atomicAdd(count, (unsigned long long)__popc(m));
     base = __shfl_sync(0xffffffffu, base, 0);
     if (keep) out[base + __popc(m & ((1u << lane) - 1u))] = p;
-    const unsigned ms = __ballot_sync(0xffffffffu, skipped);
-    if (lane == 0 && ms) atomicAdd(&stats[kStatSkipped], (unsigned long long)__popc(ms));
+    const int ns = __syncthreads_count(skipped);
+    if (threadIdx.x == 0 && ns) atomicAdd(&stats[kStatSkipped], (unsigned long long)ns);
+    if (first) {
+        const int nf = __syncthreads_count(flagged);
+        if (threadIdx.x == 0 && nf) atomicAdd(&stats[kStatUnion], (unsigned long long)nf);
+    }
 }
 
 inline unsigned grid_for(int64_t n, int t = 256) { return (unsigned)std::max<int64_t>(1, div_up(n, t)); }
 
 }  // namespace
 
-cudaError_t select_hit(const int2* pairs, const uint8_t* hit, int64_t n, int2* out,
-                       unsigned long long* count, cudaStream_t s)
+cudaError_t select_round(const PassArgs& a, int64_t T, int2* tile_roots, int64_t n, int lo, int hi, bool filter,
+                         bool first, int2* out, unsigned long long* count, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    select_hit_kernel<<<grid_for(n), 256, 0, s>>>(pairs, hit, n, out, count);
+    if (filter) {
+        tile_roots_kernel<<<grid_for(T * 32), 256, 0, s>>>(a, T, tile_roots);
+        note_launch();
+    }
+    select_round_kernel<<<grid_for(n), 256, 0, s>>>(a.pairs, a.pair_hit, n, lo, hi, filter ? tile_roots : nullptr,
+                                                    first, out, count, a.stats);
     note_launch();
-    return cudaGetLastError();
-}
-
-__global__ void add_counter_kernel(unsigned long long* dst, const unsigned long long* src) { *dst += *src; }
-
-cudaError_t add_counter(unsigned long long* dst, const unsigned long long* src, cudaStream_t s)
-{
-    add_counter_kernel<<<1, 1, 0, s>>>(dst, src);
-    note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t select_delta(const int2* pairs, int64_t n, const unsigned long long* n_dev, int lo, int hi, int2* out,
-                         unsigned long long* count, cudaStream_t s)
-{
-    if (n == 0) return cudaSuccess;
-    select_delta_kernel<<<grid_for(n), 256, 0, s>>>(pairs, n, n_dev, lo, hi, out, count);
-    note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t filter_joined(const PassArgs& a, int64_t T, int2* tile_roots, const int2* pairs, int64_t n,
-                          const unsigned long long* n_dev, int2* out, unsigned long long* count, cudaStream_t s)
-{
-    if (n == 0) return cudaSuccess;
-    tile_roots_kernel<<<grid_for(T * 32), 256, 0, s>>>(a, T, tile_roots);
-    filter_joined_kernel<<<grid_for(n), 256, 0, s>>>(pairs, n, n_dev, tile_roots, out, count, a.stats);
-    note_launch(2);
     return cudaGetLastError();
 }
 
@@ -753,19 +760,21 @@ cudaError_t list_unions(const int32_t* count, const int32_t* nbr, int cap, const
                         const int32_t* row_pt, int64_t R, cudaStream_t s, unsigned long long* oob)
 {
     if (R == 0 || cap == 0) return cudaSuccess;
+    list_hook_kernel<<<grid_for(R), 256, 0, s>>>(count, nbr, cap, core, parent, row_pt, R, oob);
+    list_compress_kernel<<<grid_for(R), 256, 0, s>>>(core, parent, R);
     list_unions_kernel<<<grid_for(R), 256, 0, s>>>(count, nbr, cap, core, parent, row_pt, R, oob);
-    note_launch();
+    note_launch(3);
     return cudaGetLastError();
 }
 
 cudaError_t rows_to_slots(const int32_t* row_slot, const int32_t* row_pt, const uint8_t* core,
                           const int32_t* root, const unsigned long long* border, int64_t R,
-                          int32_t* lab, int32_t* is_root, int32_t* is_member,
+                          int32_t* lab, uint8_t* flags,
                           int64_t* slot_label, uint8_t* slot_core, cudaStream_t s)
 {
     if (R == 0) return cudaSuccess;
     rows_to_slots_kernel<<<grid_for(R), 256, 0, s>>>(row_slot, row_pt, core, root, border, R, lab,
-                                                     is_root, is_member, slot_label, slot_core);
+                                                     flags, slot_label, slot_core);
     note_launch();
     return cudaGetLastError();
 }

@@ -404,8 +404,8 @@ __global__ void cut_union_kernel(const int32_t* __restrict__ e_su, const int32_t
 }
 
 __global__ void cut_labels_kernel(int32_t* parent, const int32_t* __restrict__ slot_point, int64_t M,
-                                  int32_t* __restrict__ lab, int32_t* __restrict__ is_root,
-                                  int32_t* __restrict__ is_member, int64_t* __restrict__ slot_label,
+                                  int32_t* __restrict__ lab, uint8_t* __restrict__ flags,
+                                  int64_t* __restrict__ slot_label,
                                   uint8_t* __restrict__ core)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -413,8 +413,7 @@ __global__ void cut_labels_kernel(int32_t* parent, const int32_t* __restrict__ s
     const int r = mfind(parent, (int)i);
     lab[i] = r;
     slot_label[i] = slot_point[r];
-    is_root[i] = r == (int)i;
-    is_member[i] = 1;
+    flags[i] = r == (int)i ? 3 : 1;
     core[i] = 1;
 }
 
@@ -620,8 +619,8 @@ int msf_forest(const PassArgs& a, const int32_t* row_slot, const int32_t* slot_p
     return MAPPER_OK;
 }
 
-int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, int32_t* lab, int32_t* is_root,
-            int32_t* is_member, int64_t* slot_label, uint8_t* core, cudaStream_t s)
+int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, int32_t* lab, uint8_t* flags,
+            int64_t* slot_label, uint8_t* core, cudaStream_t s)
 {
     if (M == 0) return MAPPER_OK;
     Buf parent;
@@ -632,8 +631,8 @@ int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, 
             cut_union_kernel<<<(unsigned)div_up(f.n, 256), 256, 0, s>>>(f.su.as<int32_t>(), f.sv.as<int32_t>(),
                                                                          f.d2.as<double>(), f.n, h * h,
                                                                          parent.as<int32_t>());
-        cut_labels_kernel<<<(unsigned)div_up(M, 256), 256, 0, s>>>(parent.as<int32_t>(), slot_point, M, lab, is_root,
-                                                                     is_member, slot_label, core);
+        cut_labels_kernel<<<(unsigned)div_up(M, 256), 256, 0, s>>>(parent.as<int32_t>(), slot_point, M, lab, flags,
+                                                                     slot_label, core);
         note_launch(3);
         e = cudaGetLastError();
     }

@@ -5,31 +5,36 @@
 // Nodes are numbered by the cover slot of their root (slots are ordered by
 // element, then point), i.e. by (element, canonical id). Memberships become
 // (node << 32 | point) keys, sorted into per-node member lists; the same
-// memberships re-keyed as (point << 32 | node) and sorted group the nodes of
-// each point, every pair of them is emitted as (u << 32 | v), u < v, and a
-// sort-unique of those keys gives the edge list in lexicographic order.
+// memberships in point order (kept by the cover) give the nodes of each point,
+// whose pairs go through a hash set of the distinct edges, sorted at the end.
+// Without that order (given nodes, cover subsets), or with more edges than the
+// set takes, the memberships re-keyed as (point << 32 | node) and sorted group
+// the nodes of each point, every pair of them is emitted as (u << 32 | v), u < v,
+// and a sort-unique of those keys gives the edge list in lexicographic order.
 #include "dbscan.cuh"
 
 namespace mgb {
 
 namespace {
 
-__global__ void member_keys_kernel(const int32_t* __restrict__ lab, const int64_t* __restrict__ nid,
-                                   const int64_t* __restrict__ mpos,
+__global__ void member_keys_kernel(const int32_t* __restrict__ lab, const int64_t* __restrict__ pos,
                                    const int32_t* __restrict__ slot_point,
-                                   const int32_t* __restrict__ slot_elem, int64_t M,
-                                   uint64_t* __restrict__ keys, int32_t* __restrict__ node_elem)
+                                   const int32_t* __restrict__ slot_elem, const int32_t* __restrict__ slot_o, int64_t M,
+                                   uint64_t* __restrict__ keys, int32_t* __restrict__ node_elem,
+                                   int32_t* __restrict__ node_o)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= M) return;
     const int l = lab[s];
+    const int node = l < 0 ? -1 : (int)(pos[l] >> 32);
+    if (node_o) node_o[slot_o[s]] = node;
     if (l < 0) return;
-    const int64_t node = nid[l];
-    keys[mpos[s]] = ((uint64_t)node << 32) | (uint64_t)(uint32_t)slot_point[s];
+    keys[(uint32_t)pos[s]] = ((uint64_t)(uint32_t)node << 32) | (uint64_t)(uint32_t)slot_point[s];
     if (l == (int)s) node_elem[node] = slot_elem[s];
 }
 
-__global__ void node_offsets_kernel(const uint64_t* __restrict__ keys, int64_t G,
+// keys2 (if set): the same memberships as (point << 32 | node)
+__global__ void node_offsets_kernel(const uint64_t* __restrict__ keys, int64_t G, int64_t N,
                                     int64_t* __restrict__ node_off, int32_t* __restrict__ members,
                                     uint64_t* __restrict__ keys2)
 {
@@ -38,8 +43,56 @@ __global__ void node_offsets_kernel(const uint64_t* __restrict__ keys, int64_t G
     const uint64_t k = keys[i];
     const int64_t node = (int64_t)(k >> 32);
     members[i] = (int32_t)(uint32_t)k;
-    keys2[i] = ((k & 0xffffffffull) << 32) | (uint64_t)node;
+    if (keys2) keys2[i] = ((k & 0xffffffffull) << 32) | (uint64_t)node;
     if (i == 0 || (int64_t)(keys[i - 1] >> 32) != node) node_off[node] = i;
+    if (i == G - 1) node_off[N] = G;
+}
+
+// Nerve edges from the nodes of every membership in point order (node_o, -1:
+// none; the memberships of point p are pos[p] .. pos[p + 1]): each pair of a
+// point's nodes goes through a hash set of the distinct edges, and the thread
+// that adds one to the set appends it to the list. Memberships of a point
+// ascend in element, and nodes in (element, root), so u < v. A pair seen before
+// is one read of the set (in L2); the edges are few (hundreds) beside the
+// points, so sorting all pairs, or the memberships by point, would move far
+// more. counts[0]: edges, counts[1]: set when the list or a probe run is full.
+constexpr int kEdgeProbes = 64;
+
+__global__ void __launch_bounds__(256) edge_set_kernel(const int64_t* __restrict__ pos, int64_t n,
+                                                       const int32_t* __restrict__ node_o,
+                                                       unsigned long long* set, uint32_t mask,
+                                                       uint64_t* __restrict__ list, uint32_t cap,
+                                                       unsigned long long* counts)
+{
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int64_t o0 = pos[p], o1 = pos[p + 1];
+    for (int64_t a = o0; a < o1; ++a) {
+        const int u = node_o[a];
+        if (u < 0) continue;
+        for (int64_t b = a + 1; b < o1; ++b) {
+            const int v = node_o[b];
+            if (v < 0) continue;
+            // (v in the high half: the sorted list is then the int32 pairs (u, v))
+            const unsigned long long key = ((unsigned long long)(unsigned)v << 32) | (unsigned)u;
+            unsigned long long x = key * 0x9E3779B97F4A7C15ull;
+            uint32_t h = (uint32_t)(x >> 40) & mask;
+            int tries = 0;
+            for (; tries < kEdgeProbes; ++tries, h = (h + 1) & mask) {
+                unsigned long long cur = __ldcg(set + h);
+                if (cur == key) break;
+                if (cur != ~0ull) continue;
+                cur = atomicCAS(set + h, ~0ull, key);
+                if (cur == key) break;
+                if (cur != ~0ull) continue;
+                const unsigned long long at = atomicAdd(&counts[0], 1ull);
+                if (at < cap) list[at] = key;
+                else counts[1] = 1ull;
+                break;
+            }
+            if (tries == kEdgeProbes) counts[1] = 1ull;
+        }
+    }
 }
 
 // Nerve keys (point << 32 | node) of given nodes: member i belongs to the
@@ -124,21 +177,36 @@ inline unsigned grid_for(int64_t n, int t = 256) { return (unsigned)std::max<int
 
 }  // namespace
 
-cudaError_t member_keys(const int32_t* lab, const int64_t* nid, const int64_t* mpos,
-                        const int32_t* slot_point, const int32_t* slot_elem, int64_t M,
-                        uint64_t* keys, int32_t* node_elem, cudaStream_t s)
+cudaError_t member_keys(const int32_t* lab, const int64_t* pos, const int32_t* slot_point, const int32_t* slot_elem,
+                        const int32_t* slot_o, int64_t M, uint64_t* keys, int32_t* node_elem, int32_t* node_o,
+                        cudaStream_t s)
 {
     if (M == 0) return cudaSuccess;
-    { member_keys_kernel<<<grid_for(M), 256, 0, s>>>(lab, nid, mpos, slot_point, slot_elem, M, keys,
-                                                   node_elem); note_launch(); }
+    { member_keys_kernel<<<grid_for(M), 256, 0, s>>>(lab, pos, slot_point, slot_elem, slot_o, M, keys, node_elem,
+                                                   node_o); note_launch(); }
     return cudaGetLastError();
 }
 
-cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t* node_off, int32_t* members,
+cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t N, int64_t* node_off, int32_t* members,
                          uint64_t* keys2, cudaStream_t s)
 {
-    if (G == 0) return cudaSuccess;
-    { node_offsets_kernel<<<grid_for(G), 256, 0, s>>>(keys, G, node_off, members, keys2); note_launch(); }
+    if (G == 0) return cudaMemsetAsync(node_off, 0, sizeof(int64_t) * (N + 1), s);
+    { node_offsets_kernel<<<grid_for(G), 256, 0, s>>>(keys, G, N, node_off, members, keys2); note_launch(); }
+    return cudaGetLastError();
+}
+
+cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, Buf* list, unsigned long long* counts,
+                     cudaStream_t s)
+{
+    constexpr uint32_t kSlots = 4 * kEdgeListMax;
+    Buf set;
+    MGB_TRY(set.alloc(sizeof(uint64_t) * kSlots, s));
+    MGB_TRY(list->alloc(sizeof(uint64_t) * kEdgeListMax, s));
+    MGB_TRY(cudaMemsetAsync(set.p, 0xff, sizeof(uint64_t) * kSlots, s));
+    MGB_TRY(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), s));
+    edge_set_kernel<<<grid_for(n), 256, 0, s>>>(pos, n, node_o, set.as<unsigned long long>(), kSlots - 1,
+                                                list->as<uint64_t>(), kEdgeListMax, counts);
+    note_launch();
     return cudaGetLastError();
 }
 

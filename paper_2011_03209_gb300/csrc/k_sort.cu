@@ -16,6 +16,13 @@ namespace mgb {
 
 namespace {
 
+// A slot's flags as a scan value: bit 0 (member) in the low half, bit 1 (root)
+// in the high half of the sum, so that one scan counts both.
+struct SlotFlag {
+    uint8_t v;
+    __device__ operator int64_t() const { return (int64_t)(v & 1) | ((int64_t)(v >> 1) << 32); }
+};
+
 // ---------------------------------------------------------------- scan
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
@@ -322,9 +329,12 @@ constexpr int64_t kRcMaxKeys = (int64_t)kRcCluster * kRcThreads * kRcItems;
 // digit: ranks in registers, counts to the other CTAs, then the keys go
 // through shared memory (sorted by digit there) so that they are written in
 // runs. In place: every key is in registers before the first write.
+// n_dev (if set): the number of keys, at most n.
 __global__ void __launch_bounds__(kRcThreads) radix_cluster_kernel(uint64_t* __restrict__ keys, int64_t n, SortField f,
-                                                                   int items)
+                                                                   int items,
+                                                                   const unsigned long long* __restrict__ n_dev)
 {
+    if (n_dev) n = min(n, (int64_t)*n_dev);
     extern __shared__ uint64_t s_keys[];                           // 1024 items keys
     __shared__ __align__(16) uint16_t wcnt[kRcWarps][kRsBins];
     __shared__ int s_total[kRsBins];                               // this CTA's keys of each digit
@@ -488,7 +498,8 @@ __global__ void __launch_bounds__(kRsThreads) radix_scatter_kernel(const uint64_
     }
 }
 
-cudaError_t radix_sort_cluster(uint64_t* keys, int64_t n, const SortField& f, cudaStream_t s)
+cudaError_t radix_sort_cluster(uint64_t* keys, int64_t n, const SortField& f, cudaStream_t s,
+                               const unsigned long long* n_dev = nullptr)
 {
     // the keys spread over the CTAs of the cluster: fewer rounds each
     int nc = 1;
@@ -510,7 +521,7 @@ cudaError_t radix_sort_cluster(uint64_t* keys, int64_t n, const SortField& f, cu
     cfg.attrs = at;
     cfg.numAttrs = 1;
     note_launch();
-    return cudaLaunchKernelEx(&cfg, radix_cluster_kernel, keys, n, f, items);
+    return cudaLaunchKernelEx(&cfg, radix_cluster_kernel, keys, n, f, items, n_dev);
 }
 
 cudaError_t radix_sort_field(Buf& keys, Buf& tmp, int64_t n, const SortField& f, cudaStream_t s)
@@ -559,9 +570,21 @@ cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaS
     return exclusive_scan_impl<int64_t>(in, out, n, s);
 }
 
+cudaError_t exclusive_scan_slot_flags(const uint8_t* in, int64_t* out, int64_t n, cudaStream_t s)
+{
+    return exclusive_scan_impl<SlotFlag>(reinterpret_cast<const SlotFlag*>(in), out, n, s);
+}
+
 cudaError_t radix_sort_u64(Buf& keys, Buf& tmp, int64_t n, int lo_bit, int hi_bit, cudaStream_t s)
 {
     return radix_sort_field(keys, tmp, n, SortField{lo_bit, hi_bit - lo_bit, 0, 0}, s);
+}
+
+cudaError_t radix_sort_u64_two_dev(uint64_t* keys, int64_t n_max, const unsigned long long* n_dev, int lo0, int lo1,
+                                   int bits, cudaStream_t s)
+{
+    if (n_max > kRcMaxKeys) return cudaErrorInvalidValue;
+    return radix_sort_cluster(keys, n_max, SortField{lo0, bits, lo1, bits}, s, n_dev);
 }
 
 cudaError_t radix_sort_u64_two(Buf& keys, Buf& tmp, int64_t n, int lo0, int lo1, int bits, cudaStream_t s)

@@ -2497,7 +2497,7 @@ int tc_pass(int mode, const PassArgs& a, const TcArgs& t, int64_t n_pairs, cudaS
     // FP32 limits of the recheck's lane-split sum (relative error (dp/8 + 5) 2^-24)
     const double eta = 1.5 * (a.dp / 8 + 5) * std::ldexp(1.0, -24);
     const double tiny = 3.0 * (a.d + 2) * std::ldexp(1.0, -149);
-    const int rgrid = t.num_sms * 16;
+    const int rgrid = t.num_sms * (mode == 2 ? 4 : 16);          // a union round's queue is short
     auto recheck = [&](const PassArgs& ar, const uint2* queue, const unsigned long long* queue_n) {
         float lo32 = (float)(ar.eps2 * (1.0 - eta) - tiny), hi32 = (float)(ar.eps2 * (1.0 + eta) + tiny);
         if ((double)lo32 > ar.eps2 * (1.0 - eta) - tiny) lo32 = std::nextafter(lo32, -INFINITY);
