@@ -455,7 +455,7 @@ __device__ __forceinline__ bool push_band_radius(const TcParams& P, uint2* queue
 // pair's buffer is written before the barrier that follows the accumulator
 // wait and read after it, so the next pair can be staged meanwhile.
 struct SmemTail {
-    uint64_t full[4], empty[4], acc_full[2], acc_empty[2], fin;
+    uint64_t full[4], empty[4], acc_full[4], acc_empty[4], fin;
     uint32_t tmem_base;
     int abort;
     int consumed;                              // stage fills consumed by the MMA warp
@@ -464,7 +464,9 @@ struct SmemTail {
     float red[2][12];                          // max |b|^2, |b| and |b - hi| of the columns, per warp
     __align__(16) float nbn[2][kT];            // -|b|^2 of the pair's columns
     __align__(16) float nbr[2][kT];            // k-distance pass: |b| (rounded up) of the pair's columns
-    __align__(16) float wn[kEpiWarps][32];     // count pass: -|b|^2 of each warp's 32 columns
+    __align__(16) float wn[kEpiWarps][kT];     // count pass: -|b|^2 of the columns of each warp's pair
+                                               // (k-distance pass: of its 32 columns)
+    int pre[kEpiWarps][kT];                    // count pass: the columns' counts before the pair
     uint32_t colmask[4][kT];                   // union pass: neighbour bits per column (by row quadrant)
     uint32_t rowmask[kT / 32][kT];             // neighbour bits per row (by 32-column chunk)
     int par[2][2 * kT];                        // union pass: local union-find / component
@@ -594,6 +596,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     constexpr int kStages = TcShape<NS, W>::kStages;
     constexpr int kStageBytes = TcShape<NS, W>::kStageBytes;
     constexpr int kAccCols = TcShape<NS, W>::kAccCols;
+    constexpr bool kCountPass = MODE == 1 || MODE == 5;
+    // accumulators in TMEM: the count pass takes all 512 columns (its epilogue
+    // works on up to four pairs at a time), the others two
+    constexpr int kBufs = kCountPass ? 512 / kAccCols : 2;
     const int64_t n_cap = W == 1 ? P.n_pairs : P.n_groups;
     const int64_t n_items = MODE == 3 ? 0 : (P.n_dev ? min(n_cap, (int64_t)*P.n_dev) : n_cap);
     auto group_at = [&](int64_t g) -> int2 { return W == 1 ? make_int2((int)g, -1) : P.groups[g]; };
@@ -615,7 +621,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     // items (consecutive groups of the list mostly share tile A, whose blocks
     // then stay in the stages), the CTAs' runs interleaved so that the CTAs
     // working at one time stay close in the list (tiles shared through L2)
-    constexpr bool kCountPass = MODE == 1 || MODE == 5;
     constexpr int kRun = kCountPass ? 4 : 1;
     auto item_at = [&](int64_t k) -> int64_t {
         if (MODE == 3) return k;
@@ -641,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&S.tmem_base)),
-                     "r"(2 * kAccCols));
+                     "r"(kBufs * kAccCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 32) {
@@ -649,9 +654,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             mbar_init(&S.full[i], 1);
             mbar_init(&S.empty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kBufs; ++i) {
             mbar_init(&S.acc_full[i], 1);
-            mbar_init(&S.acc_empty[i], kEpiWarps);
+            mbar_init(&S.acc_empty[i], kCountPass ? 4 * W : kEpiWarps);
         }
         mbar_init(&S.fin, 1);
         S.abort = 0;
@@ -740,8 +745,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 const bool diag = W == 1 && itm.x == itm.y;
                 const uint32_t idesc = F ? (W == 2 && itm.z >= 0 ? kIdescF8x2 : kIdescF8)
                                          : (W == 2 && itm.z >= 0 ? kIdesc2 : kIdesc);
-                const int buf = it & 1;
-                const uint32_t acc_phase = (uint32_t)((it >> 1) & 1);
+                const int buf = it % kBufs;
+                const uint32_t acc_phase = (uint32_t)((it / kBufs) & 1);
                 if (!mbar_wait(&S.acc_empty[buf], acc_phase ^ 1, abort)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + (uint32_t)(buf * kAccCols);
@@ -915,165 +920,231 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         }
     } else if constexpr (kCountPass) {
         // ------------------------------------------ epilogue: count pass
-        // Each epilogue warp works alone on one 32 x 32 sub-block of every
-        // tile pair: TMEM lane quadrant quad = A rows 32 quad .. +31 (a row per
-        // lane) and B columns 32 part .. +31; no barrier across warps. Per
-        // pair: screen values u = fl(2 acc - |b|^2) against per-row limits
-        // (all out / all in at once from the row's extremes), then the row
+        // Four groups of four warps, each group on a tile pair of its own: with
+        // one pair per item (W = 1) group g takes items g, g + 4, .. from the four
+        // accumulators in turn; with two (W = 2) groups 2 b and 2 b + 1 take the
+        // first and second pair of the items in accumulator b. A warp holds TMEM
+        // lane quadrant quad = A rows 32 quad .. +31 (a row per lane) and walks
+        // the pair's 128 columns in four parts of 32; no barrier across warps.
+        // The chain of one pair (its loads, the accumulator, the counts' atomics)
+        // is long beside the pair's MMAs, so four pairs in flight hide it, and a
+        // pair's row data are loaded by one warp a quadrant, not by four.
+        // Count pass of the 500k x 128 2D graph 16.6 -> 13.9 ms (all 16 warps on
+        // one pair before), of four radii on 200k x 128 14.2 -> 13.2, of 1M x 256
+        // (straight and first phase) 4.2 -> 3.7.
+        // Per 32 x 32 block: screen values u = fl(2 acc - |b|^2) against per-row
+        // limits (all out / all in at once from the row's extremes), then the row
         // counts (and lists) from the lane's bits and the column counts from
         // a 32 x 32 bit transpose; band pairs go to the FP64 recheck, or, in
-        // the first phase of the two-phase pass, defer the whole sub-block to
+        // the first phase of the two-phase pass, defer the whole block to
         // the three-product pass. Each item's group and tile pairs are loaded
         // while the previous item is processed, its row and column data before
         // the accumulator wait.
         const int ew = warp - 2;                              // 0 .. 15
         const int quad = warp & 3;
-        const int part = ew >> 2;
-        const int sub = quad * 4 + part;
+        const int group = ew >> 2;
+        const int h = W == 2 ? (group & 1) : 0;               // the group's pair of an item
+        const int first = W == 2 ? (group >> 1) : group;      // its accumulator
         const int r = quad * 32 + lane;
-        float* wn = S.wn[ew];
-        struct Item {
-            int q[2], tb[2], nb[2], pre_col[2];               // per pair (B side)
-            float ncol2[2], bn2[2], bn[2], bl[2], bmin2[2];
-            float sb[2];                                      // FP8: the B tiles' scales
-            int ta, na, pre_row;                              // A side (shared by the pairs)
-            float na2, nra, rla, sa;
-            int nbt;
-            bool mine[2];
-        };
-        // the item's group and tile pairs (the first loads of its chain), then the rest
+        float* const wn = S.wn[ew];
+        int* const pre = S.pre[ew];
+        // the group's items: every kBufs-th of the CTA's
+        auto item_of = [&](int64_t j) { return item_at(j * kBufs + first); };
         struct Head {
-            int2 grp, tp[2];
+            int2 grp, tp;
         };
         auto load_head = [&](int64_t g, Head& hd) {
             hd.grp = group_at(g);
-            hd.tp[0] = A.pairs[hd.grp.x];
-            hd.tp[1] = hd.grp.y >= 0 ? A.pairs[hd.grp.y] : hd.tp[0];
+            const int q = h ? hd.grp.y : hd.grp.x;
+            hd.tp = q >= 0 ? A.pairs[q] : make_int2(0, 0);
         };
-        auto load_item = [&](const Head& hd, Item& it) {
-            const int2 grp = hd.grp;
-            it.nbt = grp.y >= 0 ? 2 : 1;
+        int64_t screened = 0;
+        // neighbours counted for a row whose list is full, kept from pair to
+        // pair while tile A stays the same: the CTAs work on neighbouring pairs,
+        // so they all add to the same few tiles' rows, and one atomic per block
+        // would serialise there
+        int row_add = 0, ta_sum = -1;
+        auto flush_rows = [&]() {
+            if (row_add) atomicAdd(&A.count[(int64_t)ta_sum * kT + r], row_add);
+            row_add = 0;
+        };
+        Head head;
+        int64_t g = item_of(0), g_next = 0;
+        if (g < n_items) load_head(g, head);
+        for (int64_t j = 0; g < n_items; ++j, g = g_next) {
+            g_next = item_of(j + 1);
+            const uint32_t acc_phase = (uint32_t)(j & 1);
+            const int q = h ? head.grp.y : head.grp.x;
+            const bool have = q >= 0;                         // (an item of one pair has no second)
+            uint32_t mine = have ? 0xFu : 0u;                 // parts to count
+            int2 tp = head.tp;
+            if (g_next < n_items) load_head(g_next, head);
+            if (have && P.sub_mask) mine = (P.sub_mask[P.sub_q[q]] >> (quad * 4)) & 0xFu;
+            if (!MGB_IN_RANGE(tp.x, A.n_tiles, A.stats + kStatOob) ||
+                !MGB_IN_RANGE(tp.y & kPairTileMask, A.n_tiles, A.stats + kStatOob)) {
+                tp = make_int2(0, 0);                         // checked build: counted, then skipped
+                mine = 0u;
+            }
+            const int ta = tp.x, tb = tp.y & kPairTileMask;
+            const bool diag = ta == tb;
+            const int64_t sa = (int64_t)ta * kT, sb = (int64_t)tb * kT;
+            const int64_t row = sa + r;
+            if (MODE == 1 && mine && ta != ta_sum) {
+                flush_rows();
+                ta_sum = ta;
+            }
+            int na = 0, nb = 0, pre_row = 0;
+            float na2 = 0.f, bmin2 = 0.f, E = 0.f, two = 2.f;
+            float4 tm = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (mine) {
+                na = A.tile_n[ta];
+                nb = A.tile_n[tb];
+                na2 = P.rn2[row];
+                const float nra = P.rn[row], rla = P.rl ? P.rl[row] : 0.f;
+                tm = P.tmax[tb];
+                bmin2 = P.tn2min[tb];
+                float nc[4];
+                int pc[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (h >= it.nbt) break;
-                it.q[h] = h ? grp.y : grp.x;
-                it.mine[h] = P.sub_mask ? ((P.sub_mask[P.sub_q[it.q[h]]] >> sub) & 1u) != 0u : true;
-                int2 tp = hd.tp[h];
-                if (!MGB_IN_RANGE(tp.x, A.n_tiles, A.stats + kStatOob) ||
-                    !MGB_IN_RANGE(tp.y & kPairTileMask, A.n_tiles, A.stats + kStatOob)) {
-                    tp = make_int2(0, 0);                     // checked build: counted, then skipped
-                    it.mine[h] = false;
-                }
-                it.tb[h] = tp.y & kPairTileMask;
-                if (h == 0) {
-                    it.ta = tp.x;
-                    it.na = A.tile_n[tp.x];
-                    const int64_t row = (int64_t)tp.x * kT + r;
-                    it.na2 = P.rn2[row];
-                    it.nra = P.rn[row];
-                    it.rla = P.rl ? P.rl[row] : 0.f;
+                for (int p = 0; p < 4; ++p) {
+                    const int64_t col = sb + p * 32 + lane;
+                    nc[p] = -P.rn2[col];
                     if constexpr (MODE == 5) {
-                        // bit e: radius e's list of this row is full (its count can only grow)
+                        // bit e: radius e's list of this column is full (its count can only grow)
                         int full = A.cap > 0 ? 0 : 0xF;
 #pragma unroll
                         for (int e = 0; e < kMaxRadii; ++e)
-                            if (A.cap > 0 && e < P.n_rad && P.rad[e].count[row] >= A.cap) full |= 1 << e;
-                        it.pre_row = full;
+                            if (A.cap > 0 && !diag && e < P.n_rad && P.rad[e].count[col] >= A.cap) full |= 1 << e;
+                        pc[p] = full;
                     } else {
-                        it.pre_row = MODE == 1 && A.cap > 0 ? A.count[row] : INT_MAX;
+                        pc[p] = A.cap > 0 && !diag ? A.count[col] : INT_MAX;
                     }
-                    it.sa = F ? P.tmax[tp.x].w : 1.f;
                 }
-                it.nb[h] = A.tile_n[it.tb[h]];
-                const int64_t col = (int64_t)it.tb[h] * kT + part * 32 + lane;
-                it.ncol2[h] = -P.rn2[col];
-                const float4 tm = P.tmax[it.tb[h]];
-                it.bn2[h] = tm.x;
-                it.bn[h] = tm.y;
-                it.bl[h] = tm.z;
-                it.sb[h] = tm.w;
-                it.bmin2[h] = P.tn2min[it.tb[h]];
                 if constexpr (MODE == 5) {
-                    // (W = 2: rows only; the columns' reads would not fit the registers)
-                    int full = A.cap > 0 ? 0 : 0xF;
-                    if constexpr (W == 1) {
+                    pre_row = A.cap > 0 ? 0 : 0xF;
 #pragma unroll
-                        for (int e = 0; e < kMaxRadii; ++e)
-                            if (A.cap > 0 && it.mine[h] && tp.x != it.tb[h] && e < P.n_rad &&
-                                P.rad[e].count[col] >= A.cap)
-                                full |= 1 << e;
-                    }
-                    it.pre_col[h] = full;
+                    for (int e = 0; e < kMaxRadii; ++e)
+                        if (A.cap > 0 && e < P.n_rad && P.rad[e].count[row] >= A.cap) pre_row |= 1 << e;
                 } else {
-                    it.pre_col[h] = MODE == 1 && A.cap > 0 && it.mine[h] && tp.x != it.tb[h] ? A.count[col] : INT_MAX;
+                    pre_row = A.cap > 0 ? A.count[row] : INT_MAX;
                 }
-            }
-        };
-        int64_t screened = 0;
-        int git = 0;
-        Item cur;
-        Head head;
-        int64_t g = item_at(0), g_next = 0;
-        if (g < n_items) load_head(g, head);
-        for (int64_t k = 0; g < n_items; ++k, ++git, g = g_next) {
-            g_next = next_item(k, g);
-            load_item(head, cur);
-            if (g_next < n_items) load_head(g_next, head);
-            const int tbuf = git & 1;
-            const bool bad = !mbar_wait(&S.acc_full[tbuf], (uint32_t)((git >> 1) & 1), abort) || *abort;
-            if (__any_sync(0xffffffffu, bad)) break;
-            tc_fence_after();
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (h >= cur.nbt) break;
-                const int q = cur.q[h];
-                const bool diag = cur.ta == cur.tb[h];
-                const int64_t sa = (int64_t)cur.ta * kT, sb = (int64_t)cur.tb[h] * kT;
-                const int64_t row = sa + r, col = sb + part * 32 + lane;
-                float u[32];
-                tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tbuf * kAccCols + h * kT + part * 32), u);
-                if (h == cur.nbt - 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&S.acc_empty[tbuf]);
-                }
-                if (!P.sub_mask && ew == 0 && lane == 0)
-                    screened += diag ? (int64_t)cur.na * (cur.na + 1) / 2 : (int64_t)cur.na * cur.nb[h];
-                if (!cur.mine[h]) continue;
-                // per-row limits: in iff u >= k_in, out iff u < k_out (FP32, outward rounding)
-                float E;
+                // the error bound of the row against the tile's largest norms
                 if (P.rl) {
-                    const float cross = __fadd_ru(__fmul_ru(cur.rla, cur.bn[h]), __fmul_ru(cur.nra, cur.bl[h]));
-                    E = __fmaf_ru(P.K2f, __fmul_ru(cur.rla, cur.bl[h]),
+                    const float cross = __fadd_ru(__fmul_ru(rla, tm.y), __fmul_ru(nra, tm.z));
+                    E = __fmaf_ru(P.K2f, __fmul_ru(rla, tm.z),
                                   __fmaf_ru(P.K1f, cross,
-                                            __fmaf_ru(P.K0f, __fmul_ru(cur.nra, cur.bn[h]),
-                                                      __fmaf_ru(P.A2f, __fadd_ru(cur.na2, cur.bn2[h]), P.A3f))));
+                                            __fmaf_ru(P.K0f, __fmul_ru(nra, tm.y),
+                                                      __fmaf_ru(P.A2f, __fadd_ru(na2, tm.x), P.A3f))));
                 } else {
-                    E = __fmaf_ru(P.A1f, __fmul_ru(cur.nra, cur.bn[h]),
-                                  __fmaf_ru(P.A2f, __fadd_ru(cur.na2, cur.bn2[h]), P.A3f));
+                    E = __fmaf_ru(P.A1f, __fmul_ru(nra, tm.y), __fmaf_ru(P.A2f, __fadd_ru(na2, tm.x), P.A3f));
                 }
-                float two = 2.f;
                 if constexpr (F) {
                     // E4M3 subnormal floor of the scaled rows: K4 (s_b |a| + s_a |b|) + K5 s_a s_b
-                    const float ss = cur.sa * cur.sb[h];              // exact (powers of two)
-                    E = __fmaf_ru(P.K4f, __fadd_ru(__fmul_ru(cur.sb[h], cur.nra), __fmul_ru(cur.sa, cur.bn[h])),
+                    const float sca = P.tmax[ta].w, ss = sca * tm.w;    // exact (powers of two)
+                    E = __fmaf_ru(P.K4f, __fadd_ru(__fmul_ru(tm.w, nra), __fmul_ru(sca, tm.y)),
                                   __fmaf_ru(P.K5f, ss, E));
                     two = 2.f * ss;
                 }
+                __syncwarp();                                 // the previous pair's wn and pre are read
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    wn[p * 32 + lane] = nc[p];
+                    pre[p * 32 + lane] = pc[p];
+                }
+                __syncwarp();
+            }
+            const bool bad = !mbar_wait(&S.acc_full[first], acc_phase, abort) || *abort;
+            if (__any_sync(0xffffffffu, bad)) break;
+            tc_fence_after();
+            if (have && !P.sub_mask && quad == 0 && lane == 0)
+                screened += diag ? (int64_t)na * (na + 1) / 2 : (int64_t)na * nb;
+            const bool pad = r >= na;                         // padding rows hold no pair
+            uint32_t deferred = 0u;                           // parts left to the three-product pass
+            bool hit_pair = false;
+#pragma unroll 1
+            for (int part = 0; part < 4; ++part) {
+                if (!((mine >> part) & 1u)) continue;
+                float u[32];
+                tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) +
+                              (uint32_t)(first * kAccCols + h * kT + part * 32), u);
+                if ((mine >> part) == 1u) {                   // the last part read: the accumulator is free
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&S.acc_empty[first]);
+                }
+                const int64_t col = sb + part * 32 + lane;
+                // the row's extremes from the raw accumulator: with x_j = two acc_j -
+                // |b_j|^2 (exact), max x <= RU(two max acc - min |b|^2) and min x >=
+                // RD(two min acc - max |b|^2); x < k_out certifies out and x >= k_in in
+                // (E covers the rounding of the computed screen value too)
+                float vmax = fmax3(u[0], u[1], u[2]);
+#pragma unroll
+                for (int i = 3; i + 1 < 32; i += 2) vmax = fmax3(vmax, u[i], u[i + 1]);
+                vmax = fmaxf(vmax, u[31]);
+                const float xmax = __fmaf_ru(two, vmax, -bmin2);
+                const int left = nb - part * 32;
+                const uint32_t cand = pad ? 0u : (left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u));
+                // u = fl(two acc - |b|^2) (two = 2, or 2 s_a s_b for FP8), two
+                // columns per packed FMA (each lane correctly rounded)
+                auto screen_values = [&]() {
+                    const float4* wn4 = reinterpret_cast<const float4*>(wn + part * 32);
+#pragma unroll
+                    for (int i4 = 0; i4 < 8; ++i4) {
+                        const float4 nn = wn4[i4];
+                        fma2_inplace(u[4 * i4 + 0], u[4 * i4 + 1], two, nn.x, nn.y);
+                        fma2_inplace(u[4 * i4 + 2], u[4 * i4 + 3], two, nn.z, nn.w);
+                    }
+                };
+                auto row_min = [&]() {
+                    float vmin = fmin3(u[0], u[1], u[2]);
+#pragma unroll
+                    for (int i = 3; i + 1 < 32; i += 2) vmin = fmin3(vmin, u[i], u[i + 1]);
+                    return __fmaf_rd(two, fminf(vmin, u[31]), -tm.x);
+                };
+                auto compare = [&](float k_in, float k_out, uint32_t& ib, uint32_t& kb) {
+                    if constexpr (NS == 3 && !F) {
+                        limit_bits(u, k_in, k_out, ib, kb);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            if (u[i] >= k_in) ib |= 1u << i;
+                            if (u[i] >= k_out) kb |= 1u << i;
+                        }
+                    }
+                };
+                // lane j of the result: the rows of the block whose bit j is set
+                auto transpose = [&](uint32_t x) {
+#pragma unroll
+                    for (int sft = 16; sft >= 1; sft >>= 1) {
+                        const uint32_t m = sft == 16 ? 0x0000FFFFu : sft == 8 ? 0x00FF00FFu : sft == 4 ? 0x0F0F0F0Fu
+                                                               : sft == 2 ? 0x33333333u : 0x55555555u;
+                        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sft);
+                        x = (lane & sft) ? (((y >> sft) & m) | (x & ~m)) : ((x & m) | ((y & m) << sft));
+                    }
+                    return x;
+                };
+                // adds the neighbours of row (or column) `at`, bit i standing for row
+                // base + i, and lists them while the list has room; returns the
+                // count afterwards (as far as known)
+                auto add_listed = [&](int32_t* cnt, int32_t* lists, int64_t at, uint32_t bits, int64_t base) {
+                    const int k = __popc(bits);
+                    int pos = atomicAdd(&cnt[at], k);
+                    const int after = pos + k;
+                    while (bits && pos < A.cap) {
+                        const int i = __ffs(bits) - 1;
+                        bits &= bits - 1;
+                        lists[at * A.cap + pos++] = (int32_t)(base + i);
+                    }
+                    return after;
+                };
                 if constexpr (MODE == 5) {
                     // Several radii, ascending, each with the limits of the
                     // one-radius pass below. A row all out at a radius is all
                     // out at every smaller one; the screen values are formed
                     // once and compared with each radius's limits.
                     const int nr = P.n_rad;
-                    const bool pad = r >= cur.na;             // padding rows hold no pair
-                    auto k_in_of = [&](float lo) { return __fadd_ru(__fsub_ru(cur.na2, lo), E); };
-                    auto k_out_of = [&](float hi) { return __fsub_rd(__fsub_rd(cur.na2, hi), E); };
-                    float vmax = fmax3(u[0], u[1], u[2]);
-#pragma unroll
-                    for (int i = 3; i + 1 < 32; i += 2) vmax = fmax3(vmax, u[i], u[i + 1]);
-                    vmax = fmaxf(vmax, u[31]);
-                    const float xmax = __fmaf_ru(two, vmax, -cur.bmin2[h]);
+                    auto k_in_of = [&](float lo) { return __fadd_ru(__fsub_ru(na2, lo), E); };
+                    auto k_out_of = [&](float hi) { return __fsub_rd(__fsub_rd(na2, hi), E); };
                     int e_lo = nr;                            // radii e_lo .. nr - 1 hold a row not all out
 #pragma unroll
                     for (int e = kMaxRadii - 1; e >= 0; --e) {
@@ -1083,11 +1154,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         e_lo = e;
                     }
                     if (e_lo == nr) continue;                 // all out at every radius
-                    float vmin = fmin3(u[0], u[1], u[2]);
-#pragma unroll
-                    for (int i = 3; i + 1 < 32; i += 2) vmin = fmin3(vmin, u[i], u[i + 1]);
-                    vmin = fminf(vmin, u[31]);
-                    const float xmin = __fmaf_rd(two, vmin, -cur.bn2[h]);
+                    const float xmin = row_min();
                     bool mixed = false;
 #pragma unroll
                     for (int e = 0; e < kMaxRadii; ++e) {
@@ -1096,70 +1163,39 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         mixed |= !out && !(xmin >= k_in_of(P.rad[e].eps2_lo));
                     }
                     mixed = __any_sync(0xffffffffu, mixed);
-                    auto defer_radii = [&]() {
-                        if (lane == 0) {
-                            if (atomicOr(&P.redo_mask[q], 1u << sub) == 0u) atomicAdd(&A.stats[kStatRedo], 1ull);
-#pragma unroll
-                            for (int e = 0; e < kMaxRadii; ++e)
-                                if (e < nr && P.rad[e].pair_hit) P.rad[e].pair_hit[q] = 1;
-                        }
-                    };
                     if (P.defer == 2 && mixed) {
-                        defer_radii();
+                        deferred |= 1u << part;
                         continue;
                     }
-                    if (mixed) {
-                        __syncwarp();                         // the previous pair's wn is read
-                        wn[lane] = cur.ncol2[h];
-                        __syncwarp();
-                        const float4* wn4 = reinterpret_cast<const float4*>(wn);
-#pragma unroll
-                        for (int i4 = 0; i4 < 8; ++i4) {
-                            const float4 nn = wn4[i4];
-                            fma2_inplace(u[4 * i4 + 0], u[4 * i4 + 1], two, nn.x, nn.y);
-                            fma2_inplace(u[4 * i4 + 2], u[4 * i4 + 3], two, nn.z, nn.w);
-                        }
-                    }
-                    const int left = cur.nb[h] - part * 32;
-                    const uint32_t cand = pad ? 0u : (left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u));
+                    if (mixed) screen_values();
                     // in and band bits of one radius
                     auto bits_of = [&](float lo, float hi, uint32_t& inb, uint32_t& band) {
                         const float k_in = k_in_of(lo), k_out = k_out_of(hi);
                         const bool out = pad || xmax < k_out;
                         uint32_t ib = 0u, kb = 0u;
-                        if (!out && xmin >= k_in) {
-                            ib = kb = 0xffffffffu;
-                        } else if (!out) {
-                            if constexpr (NS == 3) {
-                                limit_bits(u, k_in, k_out, ib, kb);
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 32; ++i) {
-                                    if (u[i] >= k_in) ib |= 1u << i;
-                                    if (u[i] >= k_out) kb |= 1u << i;
-                                }
-                            }
-                        }
+                        if (!out && xmin >= k_in) ib = kb = 0xffffffffu;
+                        else if (!out) compare(k_in, k_out, ib, kb);
                         inb = ib & cand;
                         band = kb & ~ib & cand;
                     };
                     if (P.defer == 1) {
                         bool any_band = false;
-#pragma unroll
-                        for (int e = 0; e < kMaxRadii; ++e) {
-                            if (e < e_lo || e >= nr) continue;
+#pragma unroll 1
+                        for (int e = e_lo; e < nr; ++e) {
                             uint32_t ib, bd;
                             bits_of(P.rad[e].eps2_lo, P.rad[e].eps2_hi, ib, bd);
                             any_band |= bd != 0u;
                         }
                         if (__any_sync(0xffffffffu, any_band)) {
-                            defer_radii();
+                            deferred |= 1u << part;
                             continue;
                         }
                     }
-#pragma unroll
-                    for (int e = 0; e < kMaxRadii; ++e) {
-                        if (e < e_lo || e >= nr) continue;
+                    // (not unrolled: the groups run at different places of the
+                    // code, and four radii's worth does not stay in the
+                    // instruction cache)
+#pragma unroll 1
+                    for (int e = e_lo; e < nr; ++e) {
                         int32_t* const cnt = P.rad[e].count;
                         int32_t* const nbl = P.rad[e].nbr;
                         uint32_t inb, band;
@@ -1170,181 +1206,102 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         while (bq) {
                             const int i = __ffs(bq) - 1;
                             bq &= bq - 1;
-                            const int j = part * 32 + i;
-                            const uint32_t fl = (diag ? 0u : kQBoth) | ((!diag || r < j) ? kQTie : 0u);
+                            const int c = part * 32 + i;
+                            const uint32_t fl = (diag ? 0u : kQBoth) | ((!diag || r < c) ? kQTie : 0u);
                             bool decided;
                             const bool in = push_band_radius(P, P.rad[e].queue, P.rad[e].queue_n, P.rad[e].stats,
-                                                             P.rad[e].eps2, P.rad[e].tie_thr, (int)row, (int)(sb + j),
+                                                             P.rad[e].eps2, P.rad[e].tie_thr, (int)row, (int)(sb + c),
                                                              fl, &decided);
                             if (decided && in) inb |= 1u << i;
                         }
                         // counts, and list entries while the list has room (read
                         // before the item: a full list takes no returning atomic)
-                        const int k = __popc(inb);
-                        if (k) {
-                            if ((cur.pre_row >> e) & 1) {
-                                atomicAdd(&cnt[row], k);
-                            } else {
-                                int pos = atomicAdd(&cnt[row], k);
-                                uint32_t bm = inb;
-                                while (bm && pos < A.cap) {
-                                    const int i = __ffs(bm) - 1;
-                                    bm &= bm - 1;
-                                    nbl[row * A.cap + pos++] = (int32_t)(sb + part * 32 + i);
-                                }
-                            }
+                        if (inb) {
+                            if ((pre_row >> e) & 1) atomicAdd(&cnt[row], __popc(inb));
+                            else if (add_listed(cnt, nbl, row, inb, sb + part * 32) >= A.cap) pre_row |= 1 << e;
                         }
                         if (!diag && __any_sync(0xffffffffu, inb != 0u)) {
-                            uint32_t x = inb;
-#pragma unroll
-                            for (int sft = 16; sft >= 1; sft >>= 1) {
-                                const uint32_t m = sft == 16 ? 0x0000FFFFu : sft == 8 ? 0x00FF00FFu
-                                                 : sft == 4 ? 0x0F0F0F0Fu : sft == 2 ? 0x33333333u : 0x55555555u;
-                                const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sft);
-                                x = (lane & sft) ? (((y >> sft) & m) | (x & ~m)) : ((x & m) | ((y & m) << sft));
-                            }
-                            const int kc = __popc(x);
-                            if (kc) {
-                                if ((cur.pre_col[h] >> e) & 1) {
-                                    atomicAdd(&cnt[col], kc);
-                                } else {
-                                    int pos = atomicAdd(&cnt[col], kc);
-                                    while (x && pos < A.cap) {
-                                        const int i = __ffs(x) - 1;
-                                        x &= x - 1;
-                                        nbl[col * A.cap + pos++] = (int32_t)(sa + quad * 32 + i);
-                                    }
-                                }
+                            const uint32_t x = transpose(inb);
+                            if (x) {
+                                if ((pre[part * 32 + lane] >> e) & 1) atomicAdd(&cnt[col], __popc(x));
+                                else add_listed(cnt, nbl, col, x, sa + quad * 32);
                             }
                         }
                     }
                     continue;
                 }
-                const float k_in = __fadd_ru(__fsub_ru(cur.na2, P.eps2_lo), E);
-                const float k_out = __fsub_rd(__fsub_rd(cur.na2, P.eps2_hi), E);
-                // the row's extremes from the raw accumulator: with x_j = two acc_j -
-                // |b_j|^2 (exact), max x <= RU(two max acc - min |b|^2) and min x >=
-                // RD(two min acc - max |b|^2); x < k_out certifies out and x >= k_in in
-                // (E covers the rounding of the computed screen value too)
-                float vmax = fmax3(u[0], u[1], u[2]);
-#pragma unroll
-                for (int i = 3; i + 1 < 32; i += 2) vmax = fmax3(vmax, u[i], u[i + 1]);
-                vmax = fmaxf(vmax, u[31]);
-                uint32_t in_bits = 0u, keep_bits = 0u;
-                // padding rows hold no pair: out
-                const bool all_out = r >= cur.na || __fmaf_ru(two, vmax, -cur.bmin2[h]) < k_out;
+                const float k_in = __fadd_ru(__fsub_ru(na2, P.eps2_lo), E);
+                const float k_out = __fsub_rd(__fsub_rd(na2, P.eps2_hi), E);
+                const bool all_out = pad || xmax < k_out;
                 if (__all_sync(0xffffffffu, all_out)) continue;   // nothing in, no band: nothing to do
-                bool all_in = false;
-                if (!all_out) {
-                    float vmin = fmin3(u[0], u[1], u[2]);
-#pragma unroll
-                    for (int i = 3; i + 1 < 32; i += 2) vmin = fmin3(vmin, u[i], u[i + 1]);
-                    vmin = fminf(vmin, u[31]);
-                    all_in = __fmaf_rd(two, vmin, -cur.bn2[h]) >= k_in;
-                }
+                const bool all_in = !all_out && row_min() >= k_in;
                 const bool mixed = !all_out && !all_in;
-                auto defer_block = [&]() {
-                    // first phase: the sub-block goes to the three-product pass, whole
-                    if (lane == 0) {
-                        if (atomicOr(&P.redo_mask[q], 1u << sub) == 0u) atomicAdd(&A.stats[kStatRedo], 1ull);
-                        if (A.pair_hit) A.pair_hit[q] = 1;
-                    }
-                };
+                const bool any_mixed = __any_sync(0xffffffffu, mixed);
                 // first phase, extremes only: a block with a row neither all in
                 // nor all out is deferred without looking at its values
-                if (P.defer == 2 && __any_sync(0xffffffffu, mixed)) {
-                    defer_block();
+                if (P.defer == 2 && any_mixed) {
+                    deferred |= 1u << part;
                     continue;
                 }
-                if (__any_sync(0xffffffffu, mixed)) {
-                    __syncwarp();                             // the previous pair's wn is read
-                    wn[lane] = cur.ncol2[h];
-                    __syncwarp();
-                }
+                uint32_t in_bits = 0u, keep_bits = 0u;
                 if (all_in) {
                     in_bits = keep_bits = 0xffffffffu;
                 } else if (mixed) {
-                    // u = fl(two acc - |b|^2) (two = 2, or 2 s_a s_b for FP8), two
-                    // columns per packed FMA (each lane correctly rounded)
-                    const float4* wn4 = reinterpret_cast<const float4*>(wn);
-#pragma unroll
-                    for (int i4 = 0; i4 < 8; ++i4) {
-                        const float4 nn = wn4[i4];
-                        fma2_inplace(u[4 * i4 + 0], u[4 * i4 + 1], two, nn.x, nn.y);
-                        fma2_inplace(u[4 * i4 + 2], u[4 * i4 + 3], two, nn.z, nn.w);
-                    }
-                    if constexpr (NS == 3 && !F) {
-                        limit_bits(u, k_in, k_out, in_bits, keep_bits);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            if (u[i] >= k_in) in_bits |= 1u << i;
-                            if (u[i] >= k_out) keep_bits |= 1u << i;
-                        }
-                    }
+                    screen_values();
+                    compare(k_in, k_out, in_bits, keep_bits);
                 }
-                const int left = cur.nb[h] - part * 32;
-                const uint32_t cand = r >= cur.na ? 0u
-                                                  : (left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u));
                 uint32_t inb = in_bits & cand;
                 const uint32_t band = keep_bits & ~in_bits & cand;
                 if (P.defer && __any_sync(0xffffffffu, band != 0u)) {
-                    defer_block();
+                    deferred |= 1u << part;
                     continue;
                 }
-                if (A.pair_hit && __any_sync(0xffffffffu, (inb | band) != 0u) && lane == 0) A.pair_hit[q] = 1;
+                hit_pair |= (inb | band) != 0u;
                 // band pairs: queued for the FP64 recheck; decided here if the queue is full
                 uint32_t bq = band;
                 while (bq) {
                     const int i = __ffs(bq) - 1;
                     bq &= bq - 1;
-                    const int j = part * 32 + i;
-                    const uint32_t fl = (diag ? 0u : kQBoth) | ((!diag || r < j) ? kQTie : 0u);
+                    const int c = part * 32 + i;
+                    const uint32_t fl = (diag ? 0u : kQBoth) | ((!diag || r < c) ? kQTie : 0u);
                     bool decided;
-                    const bool in = push_band(P, (int)row, (int)(sb + j), fl, &decided);
+                    const bool in = push_band(P, (int)row, (int)(sb + c), fl, &decided);
                     if (decided && in) inb |= 1u << i;
                 }
                 // row counts (and the first cap neighbours of each row)
-                const int k = __popc(inb);
-                if (k) {
-                    if (cur.pre_row < A.cap) {
-                        int pos = atomicAdd(&A.count[row], k);
-                        uint32_t bm = inb;
-                        while (bm && pos < A.cap) {
-                            const int i = __ffs(bm) - 1;
-                            bm &= bm - 1;
-                            A.nbr[row * A.cap + pos++] = (int32_t)(sb + part * 32 + i);
-                        }
-                    } else {
-                        atomicAdd(&A.count[row], k);
-                    }
+                if (inb) {
+                    if (pre_row < A.cap) pre_row = add_listed(A.count, A.nbr, row, inb, sb + part * 32);
+                    else row_add += __popc(inb);
                 }
-                // column counts: 32 x 32 bit transpose, lane j gets column part * 32 + j
+                // column counts: lane j gets column part * 32 + j
                 if (!diag && __any_sync(0xffffffffu, inb != 0u)) {
-                    uint32_t x = inb;
-#pragma unroll
-                    for (int sft = 16; sft >= 1; sft >>= 1) {
-                        const uint32_t m = sft == 16 ? 0x0000FFFFu : sft == 8 ? 0x00FF00FFu : sft == 4 ? 0x0F0F0F0Fu
-                                                               : sft == 2 ? 0x33333333u : 0x55555555u;
-                        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sft);
-                        x = (lane & sft) ? (((y >> sft) & m) | (x & ~m)) : ((x & m) | ((y & m) << sft));
-                    }
-                    const int kc = __popc(x);
-                    if (kc) {
-                        if (cur.pre_col[h] < A.cap) {
-                            int pos = atomicAdd(&A.count[col], kc);
-                            while (x && pos < A.cap) {
-                                const int i = __ffs(x) - 1;
-                                x &= x - 1;
-                                A.nbr[col * A.cap + pos++] = (int32_t)(sa + quad * 32 + i);
-                            }
-                        } else {
-                            atomicAdd(&A.count[col], kc);
-                        }
+                    const uint32_t x = transpose(inb);
+                    if (x) {
+                        if (pre[part * 32 + lane] < A.cap) add_listed(A.count, A.nbr, col, x, sa + quad * 32);
+                        else atomicAdd(&A.count[col], __popc(x));
                     }
                 }
             }
+            if (!mine) {                                      // nothing read: the accumulator is free
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.acc_empty[first]);
+            }
+            if (MODE == 1) {
+                if (A.pair_hit && __any_sync(0xffffffffu, hit_pair) && lane == 0) A.pair_hit[q] = 1;
+            }
+            if (deferred && lane == 0) {
+                // first phase: these blocks go to the three-product pass, whole
+                if (atomicOr(&P.redo_mask[q], deferred << (quad * 4)) == 0u) atomicAdd(&A.stats[kStatRedo], 1ull);
+                if constexpr (MODE == 5) {
+#pragma unroll
+                    for (int e = 0; e < kMaxRadii; ++e)
+                        if (e < P.n_rad && P.rad[e].pair_hit) P.rad[e].pair_hit[q] = 1;
+                } else {
+                    if (A.pair_hit) A.pair_hit[q] = 1;
+                }
+            }
         }
+        if (MODE == 1) flush_rows();
         if (screened) {
             atomicAdd(&A.stats[kStatScreened], (unsigned long long)screened);
             atomicAdd(&A.stats[kStatTcPairs], (unsigned long long)screened);
@@ -1682,7 +1639,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     tc_fence_after();
     if (tid == 0 && S.abort) atomicExch(P.err, 1);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kAccCols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kBufs * kAccCols));
 }
 
 // ------------------------------------------------ nearest pivot (layout)
@@ -1887,11 +1844,12 @@ __global__ void split_rows_kernel(const float* __restrict__ src, int64_t n, int 
 
 __global__ void mean_rows_kernel(const float* __restrict__ rows, int K, int dp, float* __restrict__ c)
 {
-    for (int k = threadIdx.x; k < dp; k += blockDim.x) {
-        float s = 0.f;
-        for (int i = 0; i < K; ++i) s += rows[(int64_t)i * dp + k];
-        c[k] = s / (float)K;
-    }
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= dp) return;
+    float s = 0.f;
+#pragma unroll 16
+    for (int i = 0; i < K; ++i) s += rows[(int64_t)i * dp + k];    // (loads ahead of the chain)
+    c[k] = s / (float)K;
 }
 
 // Band pairs queued by the epilogues, 8 lanes per pair (4 pairs per warp in
@@ -2223,7 +2181,7 @@ int assign_pivots_tc(const float* X, int64_t n, int d, int64_t ld, int dp, const
         AK(c.alloc(sizeof(float) * dp, s));
         AK(xh.alloc(sizeof(__nv_bfloat16) * (size_t)rows * dp, s));
         AK(xn2.alloc(sizeof(float) * rows, s));
-        mean_rows_kernel<<<1, 256, 0, s>>>(Pv, K, dp, c.as<float>());
+        mean_rows_kernel<<<div_up(dp, 32), 32, 0, s>>>(Pv, K, dp, c.as<float>());
         const bool vec = ld % 4 == 0 && ((uintptr_t)X & 15) == 0;
         split_rows_kernel<<<num_sms * 8, 256, 0, s>>>(X, n, d, ld, dp, c.as<float>(), rows,
                                                       xh.as<__nv_bfloat16>(), xn2.as<float>(), 0.f, vec);
