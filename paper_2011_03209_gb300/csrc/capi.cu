@@ -189,7 +189,7 @@ int run_density(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int64_t l
 
 int run_lens(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int64_t ld, int32_t m,
              const int32_t* kinds, const int32_t* args, const double* lens_param, int32_t precision,
-             double* lens_dev, Buf* pca_dev, int64_t* n_pca, PivotSet* split = nullptr)
+             double* lens_dev, Buf* pca_dev, int64_t* n_pca, PivotSet* split = nullptr, int* finite_flag = nullptr)
 {
     cudaStream_t s = ctx->stream->s;
     int K = 0;
@@ -225,7 +225,7 @@ int run_lens(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int64_t ld, 
         else if (kinds[j] == MAPPER_LENS_COORD)
             CK(lens_coord(X, n, ld, args[j], lens_dev, m, j, s), "lens_coord");
         else if (kinds[j] == MAPPER_LENS_ECC)
-            CK(lens_ecc2(X, n, d, ld, lens_dev, m, j, s), "lens_ecc2");
+            CK(lens_ecc2(X, n, d, ld, lens_dev, m, j, s, finite_flag), "lens_ecc2");
         else if (kinds[j] == MAPPER_LENS_LINF)
             CK(lens_linf(X, n, d, ld, lens_dev, m, j, s), "lens_linf");
         else if (kinds[j] == MAPPER_LENS_DENSITY) {
@@ -340,7 +340,7 @@ constexpr double kPhase1Cost = 0.55;
 constexpr double kTwoPhaseGain = 0.97;
 
 int sample_deferral(const mapper_ctx* ctx, const PassArgs& a, const TcArgs& first, int64_t n_pairs, int64_t R,
-                    int cap, cudaStream_t s, double* frac, const uint8_t* bins = nullptr,
+                    int cap, cudaStream_t s, double* frac, const TileLayout* L = nullptr, double eps = 0.0,
                     unsigned long long* h_bins = nullptr)
 {
     (void)ctx;
@@ -393,10 +393,12 @@ int sample_deferral(const mapper_ctx* ctx, const PassArgs& a, const TcArgs& firs
     if ((rc = tc_pass(ts.n_radii > 0 ? 5 : 1, as, ts, n_s, s))) return rc;
     unsigned long long h_redo = 0;
     int h_err = 0;
-    Buf bc;
-    if (bins && h_bins) {
+    Buf bc, bins;
+    if (L && h_bins) {
+        CK(bins.alloc(n_s, s), "alloc");
         CK(bc.alloc(sizeof(unsigned long long) * 2 * kPairBins, s), "alloc");
-        CK(sample_bins(mask.as<uint32_t>(), n_s, bins, stride, bc.as<unsigned long long>(), s), "sample bins");
+        CK(pair_bins(*L, sp.as<int2>(), n_s, a.dp, eps, bins.as<uint8_t>(), s), "pair bins");
+        CK(sample_bins(mask.as<uint32_t>(), n_s, bins.as<uint8_t>(), bc.as<unsigned long long>(), s), "sample bins");
         CK(cudaMemcpyAsync(h_bins, bc.p, sizeof(unsigned long long) * 2 * kPairBins, cudaMemcpyDeviceToHost, s),
            "copy");
     }
@@ -772,14 +774,9 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         double f = 0.0;
         const int64_t n = PL.n[kListTC];
         const bool per_bin = !f8;
-        Buf bins;
         unsigned long long h_bins[2 * kPairBins] = {};
-        if (per_bin) {
-            CK(bins.alloc(n, s), "alloc");
-            CK(pair_bins(L, PL.list[kListTC].as<int2>(), n, dp, eps_max, bins.as<uint8_t>(), s), "pair bins");
-        }
         if ((rc = sample_deferral(ctx, a_tc, with_radii(f8 ? t8 : t, false, true), n, R, cap, s, &f,
-                                  per_bin ? bins.as<uint8_t>() : nullptr, per_bin ? h_bins : nullptr)))
+                                  per_bin ? &L : nullptr, eps_max, per_bin ? h_bins : nullptr)))
             return rc;
         st.pass1_sample_deferred = f;
         uint8_t chosen[kPairBins] = {};
@@ -800,8 +797,11 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
             two_phase = false;
         }
         if (any) {
-            // the chosen bins' pairs first (list order kept within each part)
-            Buf dchosen, part, pos;
+            // the chosen bins' pairs first (list order kept within each part);
+            // only now does every pair need its bin
+            Buf bins, dchosen, part, pos;
+            CK(bins.alloc(n, s), "alloc");
+            CK(pair_bins(L, PL.list[kListTC].as<int2>(), n, dp, eps_max, bins.as<uint8_t>(), s), "pair bins");
             CK(dchosen.alloc(kPairBins, s), "alloc");
             CK(part.alloc(sizeof(int2) * n, s), "alloc");
             CK(cudaMemcpyAsync(dchosen.p, chosen, kPairBins, cudaMemcpyHostToDevice, s), "copy");
@@ -967,7 +967,8 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         Timer pr(ctx->timing, s);
         CK(core_flags(a.count, R, min_pts, rd.core.as<uint8_t>(), a.parent, a.border, a.stats, s), "core");
         pr.mark();                                                // 0
-        CK(list_unions(a.count, a.nbr, cap, a.core, a.parent, a.row_pt, R, s, a.stats + kStatOob), "list unions");
+        CK(list_unions(a.count, a.nbr, cap, a.core, a.parent, rd.root.as<int32_t>(), a.row_pt, R, s,
+                       a.stats + kStatOob), "list unions");
         CK(allin_pass(2, rd.a_in, PL.n[kListAllIn], s), "pass 2 all-in");
         // Unions in rounds of growing tile distance b - a (tiles of one pivot
         // region are adjacent): a pair is kept only if its core rows are not
@@ -1465,9 +1466,13 @@ int mapper_lens_ex(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t d, in
     Buf flag, pca;
     CK(flag.alloc(sizeof(int), s), "alloc");
     CK(cudaMemsetAsync(flag.p, 0, sizeof(int), s), "memset");
-    CK(check_finite(X_dev, n, d, ld, flag.as<int>(), s), "finite");
+    // the eccentricity's column sums read every value: they check X on the way
+    bool checked = false;
+    for (int j = 0; j < m; ++j) checked |= kinds[j] == MAPPER_LENS_ECC;
+    if (!checked) CK(check_finite(X_dev, n, d, ld, flag.as<int>(), s), "finite");
     int64_t n_pca = 0;
-    if ((rc = run_lens(ctx, X_dev, n, d, ld, m, kinds, args, lens_param, precision, lens_dev, &pca, &n_pca)))
+    if ((rc = run_lens(ctx, X_dev, n, d, ld, m, kinds, args, lens_param, precision, lens_dev, &pca, &n_pca, nullptr,
+                       flag.as<int>())))
         return rc;
     int h_nf = 0;
     CK(cudaMemcpyAsync(&h_nf, flag.p, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");

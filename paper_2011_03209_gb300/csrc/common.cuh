@@ -78,8 +78,9 @@ struct Buf {
 // lens (k_lens.cu)
 cudaError_t lens_l2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j,
                     cudaStream_t s);
+// flag (if set): set to 1 if a value of X is NaN or Inf (as check_finite)
 cudaError_t lens_ecc2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j,
-                      cudaStream_t s);
+                      cudaStream_t s, int* flag = nullptr);
 // k-th nearest-neighbour distances of q query rows (device indices) over all
 // n rows, the row itself first; out: q doubles on the device. Returns a
 // mapper_status (k in [1, min(16, n)]).

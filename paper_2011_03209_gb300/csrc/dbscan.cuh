@@ -176,8 +176,10 @@ cudaError_t border_from_lists(const int32_t* count, const int32_t* nbr, int cap,
 // canonical point id (or -1), the flags of exclusive_scan_slot_flags and the
 // core flag.
 // Unions of each core row with the core rows of its pass-1 neighbour list.
+// root: scratch of R entries.
 cudaError_t list_unions(const int32_t* count, const int32_t* nbr, int cap, const uint8_t* core, int32_t* parent,
-                        const int32_t* row_pt, int64_t R, cudaStream_t s, unsigned long long* oob = nullptr);
+                        int32_t* root, const int32_t* row_pt, int64_t R, cudaStream_t s,
+                        unsigned long long* oob = nullptr);
 cudaError_t rows_to_slots(const int32_t* row_slot, const int32_t* row_pt, const uint8_t* core,
                           const int32_t* root, const unsigned long long* border, int64_t R,
                           int32_t* lab, uint8_t* flags,
@@ -320,11 +322,11 @@ int classify_pairs(const TileLayout& L, const float* X, int64_t ld, int d, int d
 constexpr int kPairBins = 64;
 cudaError_t pair_bins(const TileLayout& L, const int2* pairs, int64_t n, int dp, double eps, uint8_t* bin,
                       cudaStream_t s);
-// Tally of a sample of the list (sample pair j = list pair j * stride, mask[j]
-// its first phase's deferred blocks): cnt[2 b] sampled pairs of bin b,
-// cnt[2 b + 1] of them that deferred a block (2 kPairBins counters, zeroed here).
-cudaError_t sample_bins(const uint32_t* mask, int64_t n_s, const uint8_t* bin, int64_t stride,
-                        unsigned long long* cnt, cudaStream_t s);
+// Tally of sampled pairs (mask[j] pair j's first phase's deferred blocks, bin[j]
+// its bin): cnt[2 b] sampled pairs of bin b, cnt[2 b + 1] of them that deferred a
+// block (2 kPairBins counters, zeroed here).
+cudaError_t sample_bins(const uint32_t* mask, int64_t n_s, const uint8_t* bin, unsigned long long* cnt,
+                        cudaStream_t s);
 // Stable partition of pairs[0 .. n): those whose bin is chosen (chosen: kPairBins
 // bytes on the device) first, then the rest, into out; *pos receives [n + 1]
 // int64 with their number at pos[n].

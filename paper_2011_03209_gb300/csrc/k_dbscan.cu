@@ -501,6 +501,8 @@ __global__ void border_lists_kernel(const int32_t* __restrict__ count, const int
 //   hook      each row points at its core neighbour of smallest key, if
 //             smaller than its own (no atomics; keys fall along every chain);
 //   compress  each row points at its root;
+//   (large)   roots hook on the smallest root their rows' neighbours have, and
+//             compress again, a few times;
 //   unions    list entries whose rows still point at different roots.
 // All of a graph's union work (these, and two rounds over the tile pairs where
 // there were five with lists between them): with the nerve's hash set 14k x 37
@@ -532,6 +534,31 @@ __global__ void list_compress_kernel(const uint8_t* __restrict__ core, int32_t* 
     int r = (int)s, p = par[r];
     while (p != r) { r = p; p = par[r]; }
     par[s] = r;
+}
+
+// Each row points its root at the smallest root among its core neighbours', if
+// smaller. Plain stores: of several rows of one tree any may win (each is a
+// certified neighbour tree of smaller key), what is lost is joined later.
+__global__ void list_hook_roots_kernel(const int32_t* __restrict__ count, const int32_t* __restrict__ nbr, int cap,
+                                       const uint8_t* __restrict__ core, int32_t* parent,
+                                       const int32_t* __restrict__ root, const int32_t* __restrict__ row_pt, int64_t R,
+                                       unsigned long long* oob)
+{
+    (void)oob;
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= R || !core[s]) return;
+    const int k = min(count[s], cap);
+    const int rs = root[s];
+    int best = rs, key = key_of(row_pt, rs);
+    for (int i = 0; i < k; ++i) {
+        const int q = nbr[s * cap + i];
+        if (q < 0 || !MGB_IN_RANGE(q, R, oob)) continue;
+        const int rq = root[q];
+        if (rq == rs || rq == best || !core[q]) continue;
+        const int kq = key_of(row_pt, rq);
+        if (kq < key) { key = kq; best = rq; }
+    }
+    if (best != rs) *(volatile int32_t*)&parent[rs] = best;
 }
 
 __global__ void list_unions_kernel(const int32_t* __restrict__ count, const int32_t* __restrict__ nbr, int cap,
@@ -756,14 +783,24 @@ cudaError_t border_from_lists(const int32_t* count, const int32_t* nbr, int cap,
     return cudaGetLastError();
 }
 
+constexpr int64_t kHookRows = 1 << 17;
+
 cudaError_t list_unions(const int32_t* count, const int32_t* nbr, int cap, const uint8_t* core, int32_t* parent,
-                        const int32_t* row_pt, int64_t R, cudaStream_t s, unsigned long long* oob)
+                        int32_t* root, const int32_t* row_pt, int64_t R, cudaStream_t s, unsigned long long* oob)
 {
     if (R == 0 || cap == 0) return cudaSuccess;
     list_hook_kernel<<<grid_for(R), 256, 0, s>>>(count, nbr, cap, core, parent, row_pt, R, oob);
     list_compress_kernel<<<grid_for(R), 256, 0, s>>>(core, parent, R);
+    // many rows: the trees of one hook (about ten rows each) would still race
+    // for the roots of large clusters
+    const int rounds = R >= kHookRows ? 2 : 0;
+    for (int k = 0; k < rounds; ++k) {
+        MGB_TRY(cudaMemcpyAsync(root, parent, sizeof(int32_t) * R, cudaMemcpyDeviceToDevice, s));
+        list_hook_roots_kernel<<<grid_for(R), 256, 0, s>>>(count, nbr, cap, core, parent, root, row_pt, R, oob);
+        list_compress_kernel<<<grid_for(R), 256, 0, s>>>(core, parent, R);
+    }
     list_unions_kernel<<<grid_for(R), 256, 0, s>>>(count, nbr, cap, core, parent, row_pt, R, oob);
-    note_launch(3);
+    note_launch(3 + 2 * rounds);
     return cudaGetLastError();
 }
 

@@ -21,6 +21,7 @@ namespace {
 
 constexpr int kRows = 128;    // rows per CTA (one thread per row)
 constexpr int kChunk = 32;    // columns staged per step
+constexpr int kMeanRows = 4096;   // rows per partial column sum
 
 // (double)x from the bits, in integer instructions (the FP64 pipe of this chip,
 // conversions included, issues two lanes a cycle and SM): for zeros and normal
@@ -42,10 +43,8 @@ __device__ __forceinline__ double widen(float x)
 // One CTA = 128 rows. Each warp loads whole 32-column row segments
 // (coalesced); then each thread consumes its row's segment in order.
 // MODE 0: sum x^2 then sqrt (L2). MODE 1: sum (x - mu) v (projection).
-// MODE 2: sum (x - mu)^2 (squared distance to the mean). MODE 3: two
-// projections, sharing x - mu. Bound by the FP64 pipe (MODE 1: subtract,
-// multiply, add per value). 500k x 128, two axes: 0.99 -> 0.74 ms; MODE 2 at 1M
-// x 256: 1.43 -> 0.93 ms (conversions off the FP64 pipe).
+// MODE 3: two projections, sharing x - mu. Bound by the FP64 pipe (MODE 1: subtract,
+// multiply, add per value). 500k x 128, two axes: 0.99 -> 0.63 ms.
 template <int MODE>
 __global__ void __launch_bounds__(kRows) lens_rows_kernel(const float* __restrict__ X, int64_t n,
                                                           int32_t d, int64_t ld,
@@ -80,9 +79,6 @@ __global__ void __launch_bounds__(kRows) lens_rows_kernel(const float* __restric
                 // x * x is exact in double (24-bit significands), so one
                 // fused rounding equals the separate multiply and add
                 acc = __fma_rn(x, x, acc);
-            } else if (MODE == 2) {
-                const double t = __dsub_rn(x, smu[k]);
-                acc = __fma_rn(t, t, acc);
             } else {
                 const double t = __dsub_rn(x, smu[k]);
                 acc = __dadd_rn(acc, __dmul_rn(t, sv[k]));
@@ -144,7 +140,7 @@ __device__ __forceinline__ unsigned long long mad_wide(uint32_t a, unsigned long
 
 constexpr int kL2Per = 8;                     // values per lane per 256-column chunk
 
-// lane l takes columns k0 + 8 l .. k0 + 8 l + 7 of the chunk (two 16-byte
+// lane l of a row's lanes takes columns k0 + 8 l .. k0 + 8 l + 7 (two 16-byte
 // loads when the row allows; the exact sum does not depend on the order)
 __device__ __forceinline__ void l2_load(const float* __restrict__ x, int k0, int d, int lane, unsigned* v, bool vec)
 {
@@ -194,51 +190,67 @@ __device__ __forceinline__ int lane_emax(const unsigned* v, int* raw)
     return min(el, 254);
 }
 
-// A warp sums 32 rows in turn (all lanes on one row), lane i keeps row i's
-// sum, and the 32 double conversions and square roots then run side by side.
+// G lanes take a row (8 columns each; G = 32 walks longer rows in chunks of
+// 256), so a warp sums 32 / G rows at a time, `iters` (at most G) times over; lane
+// i then holds the sum of the warp's row i, and the double conversions and
+// square roots run side by side. Bound by integer instructions on long rows
+// (2.2 TB/s at 1M x 256), by the chain of one row after another in a warp
+// where there are few: with all lanes on one row and 32 rows a warp, 14k x 37
+// took 61 us, now 11.
 // SPLIT: the same pass also writes the rows for the pivot assignment, x - c
 // rounded to BF16 (pitch dp, zero padded) and |x - c|^2 in FP32.
-template <bool SPLIT>
+template <bool SPLIT, int G>
 __global__ void __launch_bounds__(256) lens_l2_exact_kernel(const float* __restrict__ X, int64_t n, int32_t d,
-                                                            int64_t ld, double* __restrict__ f, int m, int j,
+                                                            int64_t ld, int iters, double* __restrict__ f, int m, int j,
                                                             const float* __restrict__ c, int dp,
                                                             __nv_bfloat16* __restrict__ xh, float* __restrict__ xn2)
 {
+    constexpr int kPar = 32 / G;                                   // rows at a time
     const int lane = threadIdx.x & 31;
+    const int sub = lane & (G - 1), grp = lane / G;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const bool one_chunk = d <= 32 * kL2Per;
+    const bool one_chunk = G < 32 || d <= 32 * kL2Per;             // (G < 32: d <= 8 G)
     const bool vec = ld % 4 == 0 && ((uintptr_t)X & 15) == 0;
-    for (int64_t r0 = warp * 32; r0 < n; r0 += nwarp * 32) {
+    const int per_warp = kPar * iters;
+    for (int64_t r0 = warp * per_warp; r0 < n; r0 += nwarp * per_warp) {
         unsigned long long my_hi = 0ull, my_lo = 0ull;
         int my_emax = 1;
         unsigned my_special = 0u;
-        const int rows = n - r0 < 32 ? (int)(n - r0) : 32;
-        for (int i = 0; i < rows; ++i) {
-            const float* x = X + (r0 + i) * ld;
+        const int rows = n - r0 < per_warp ? (int)(n - r0) : per_warp;
+        for (int i = 0; i < iters; ++i) {
+            const bool live = i * kPar + grp < rows;
+            const int64_t row = r0 + (live ? i * kPar + grp : 0);
+            const float* x = X + row * ld;
             unsigned v[kL2Per];
             int emax = 1, raw_max = 0;
-            for (int k0 = 0; k0 < d; k0 += 32 * kL2Per) {
-                l2_load(x, k0, d, lane, v, vec);
+            for (int k0 = 0; k0 < d; k0 += G * kL2Per) {
+                l2_load(x, k0, d, sub, v, vec);
                 int raw;
                 emax = max(emax, lane_emax(v, &raw));
                 raw_max = max(raw_max, raw);
             }
-            emax = __reduce_max_sync(0xffffffffu, emax);
+            if (G == 32) {
+                emax = __reduce_max_sync(0xffffffffu, emax);
+            } else {
+#pragma unroll
+                for (int o = G / 2; o; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+            }
             unsigned special = 0u;                                 // 1: an Inf, 2: a NaN
             if (__any_sync(0xffffffffu, raw_max == 255)) {
-                for (int k0 = 0; k0 < d; k0 += 32 * kL2Per) {
-                    l2_load(x, k0, d, lane, v, vec);
+                for (int k0 = 0; k0 < d; k0 += G * kL2Per) {
+                    l2_load(x, k0, d, sub, v, vec);
 #pragma unroll
                     for (int t = 0; t < kL2Per; ++t)
                         if (((v[t] >> 23) & 0xFFu) == 0xFFu) special |= (v[t] & 0x7FFFFFu) ? 2u : 1u;
                 }
-                special = __reduce_or_sync(0xffffffffu, special);
+#pragma unroll
+                for (int o = G / 2; o; o >>= 1) special |= __shfl_xor_sync(0xffffffffu, special, o);
             }
             unsigned long long hi = 0ull, lo = 0ull;
             float n2 = 0.f;
-            for (int k0 = 0; k0 < d && !special; k0 += 32 * kL2Per) {
-                if (!one_chunk) l2_load(x, k0, d, lane, v, vec);
+            for (int k0 = 0; k0 < d && !special; k0 += G * kL2Per) {
+                if (!one_chunk) l2_load(x, k0, d, sub, v, vec);
                 int raw;
                 const int el = lane_emax(v, &raw);
                 unsigned long long s1 = 0ull, s2 = 0ull;
@@ -262,15 +274,15 @@ __global__ void __launch_bounds__(256) lens_l2_exact_kernel(const float* __restr
                 add128_shifted(hi, lo, s1, 52 - 2 * (emax - el));
                 add128_shifted(hi, lo, s2, 38 - 2 * (emax - el));
                 if constexpr (SPLIT) {
-                    const int col0 = k0 + kL2Per * lane;
+                    const int col0 = k0 + kL2Per * sub;
                     float a[kL2Per];
 #pragma unroll
                     for (int t = 0; t < kL2Per; ++t) {
                         a[t] = col0 + t < d ? __uint_as_float(v[t]) - c[col0 + t] : 0.f;
                         n2 = fmaf(a[t], a[t], n2);
                     }
-                    __nv_bfloat16* dst = xh + (r0 + i) * dp + col0;
-                    if (col0 + kL2Per <= dp) {
+                    __nv_bfloat16* dst = xh + row * dp + col0;
+                    if (live && col0 + kL2Per <= dp) {
                         uint32_t w[4];
 #pragma unroll
                         for (int t = 0; t < kL2Per; t += 2) {
@@ -278,23 +290,30 @@ __global__ void __launch_bounds__(256) lens_l2_exact_kernel(const float* __restr
                             w[t >> 1] = *reinterpret_cast<const uint32_t*>(&h);
                         }
                         *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-                    } else {
+                    } else if (live) {
                         for (int t = 0; t < kL2Per && col0 + t < dp; ++t) dst[t] = __float2bfloat16_rn(a[t]);
                     }
                 }
             }
             if constexpr (SPLIT) {
 #pragma unroll
-                for (int o = 16; o; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-                if (lane == 0) xn2[r0 + i] = n2;
+                for (int o = G / 2; o; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+                if (sub == 0 && live) xn2[row] = n2;
             }
 #pragma unroll
-            for (int o = 16; o; o >>= 1) {
+            for (int o = G / 2; o; o >>= 1) {
                 const unsigned long long oh = __shfl_xor_sync(0xffffffffu, hi, o);
                 const unsigned long long ol = __shfl_xor_sync(0xffffffffu, lo, o);
                 add128(hi, lo, oh, ol);
             }
-            if (lane == i) {
+            if (kPar > 1) {                                        // lane l: the sum of group l % kPar
+                const int src = (lane & (kPar - 1)) * G;
+                hi = __shfl_sync(0xffffffffu, hi, src);
+                lo = __shfl_sync(0xffffffffu, lo, src);
+                emax = __shfl_sync(0xffffffffu, emax, src);
+                special = __shfl_sync(0xffffffffu, special, src);
+            }
+            if (lane / kPar == i) {
                 my_hi = hi;
                 my_lo = lo;
                 my_emax = emax;
@@ -303,6 +322,184 @@ __global__ void __launch_bounds__(256) lens_l2_exact_kernel(const float* __restr
         }
         if (lane < rows) f[(r0 + lane) * m + j] = l2_finish(my_hi, my_lo, my_emax, my_special);
     }
+}
+
+// Enough warps for the chip first (a row at a time each), then rows per warp.
+template <bool SPLIT, int G>
+cudaError_t launch_l2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j, const float* c, int dp,
+                      void* xh, float* xn2, cudaStream_t s)
+{
+    constexpr int kPar = 32 / G;
+    constexpr int64_t kWarps = 152 * 8 * 8;
+    const int iters = (int)std::max<int64_t>(1, std::min<int64_t>(G, n / (kWarps * kPar)));
+    const int blocks = (int)std::min<int64_t>(div_up(n, 8 * kPar * iters), 152 * 8);
+    lens_l2_exact_kernel<SPLIT, G><<<blocks, 256, 0, s>>>(X, n, d, ld, iters, f, m, j, c, dp,
+                                                          static_cast<__nv_bfloat16*>(xh), xn2);
+    note_launch();
+    return cudaGetLastError();
+}
+
+template <bool SPLIT>
+cudaError_t launch_l2_by_width(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j,
+                               const float* c, int dp, void* xh, float* xn2, cudaStream_t s)
+{
+    if (d <= 4 * kL2Per) return launch_l2<SPLIT, 4>(X, n, d, ld, f, m, j, c, dp, xh, xn2, s);
+    if (d <= 8 * kL2Per) return launch_l2<SPLIT, 8>(X, n, d, ld, f, m, j, c, dp, xh, xn2, s);
+    if (d <= 16 * kL2Per) return launch_l2<SPLIT, 16>(X, n, d, ld, f, m, j, c, dp, xh, xn2, s);
+    return launch_l2<SPLIT, 32>(X, n, d, ld, f, m, j, c, dp, xh, xn2, s);
+}
+
+// a + b = s + e exactly (FP32)
+__device__ __forceinline__ float two_sum(float a, float b, float& e)
+{
+    const float s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+
+// Column sums of a row block for the eccentricity, as col_partial_sum_kernel,
+// but in FP32 expansions: (s, e, e2) with s + e + e2 the sum up to 2^-70 of its
+// magnitude, so the FP64 pipe sees three conversions a column instead of an add
+// a value, and the rows of a block split over the warps of a CTA (their sums
+// added in order). A batch holding a value of magnitude above 2^100 or below
+// 2^-80 (whose roundings might fall outside FP32) takes FP64 adds. *flag: set if
+// a value is NaN or Inf. One CTA per (32 columns, row block).
+constexpr int kEccWarps = 8;
+
+__device__ __forceinline__ bool mid_range(float x)      // zero, or 2^-80 <= |x| < 2^100
+{
+    const unsigned t = __float_as_uint(x) & 0x7FFFFFFFu;
+    return t == 0u || t - (47u << 23) < (180u << 23);
+}
+
+__global__ void __launch_bounds__(32 * kEccWarps) col_sum_exp_kernel(const float* __restrict__ X, int64_t n, int32_t d,
+                                                                     int64_t ld, double* __restrict__ part, int* flag)
+{
+    __shared__ double s_sum[kEccWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = min((int)blockIdx.y * 32 + lane, d - 1);         // (lanes past d: the last column again)
+    const int64_t r0 = (int64_t)blockIdx.x * kMeanRows;
+    const int rows = (int)min((int64_t)kMeanRows, n - r0);
+    const float* x = X + r0 * ld + c;
+    float s = 0.f, e = 0.f, e2 = 0.f;
+    double wide = 0.0;
+    bool bad = false;
+    for (int r = warp * 16; r < rows; r += kEccWarps * 16) {
+        float v[16];
+        bool mid = true;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = r + i < rows ? __ldg(x + (int64_t)(r + i) * ld) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) mid &= mid_range(v[i]);
+        if (__all_sync(0xffffffffu, mid)) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                float a, b;
+                s = two_sum(s, v[i], a);
+                e = two_sum(e, a, b);
+                e2 = __fadd_rn(e2, b);
+            }
+        } else {
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i) {
+                wide += (double)v[i];
+                bad |= !isfinite(v[i]);
+            }
+        }
+    }
+    s_sum[warp][lane] = wide + ((double)s + ((double)e + (double)e2));
+    if (__syncthreads_or(bad) && flag && threadIdx.x == 0) atomicOr(flag, 1);
+    if (warp == 0 && blockIdx.y * 32 + lane < d) {
+        double t = 0.0;
+        for (int w = 0; w < kEccWarps; ++w) t += s_sum[w][lane];
+        part[(int64_t)blockIdx.x * d + c] = t;
+    }
+}
+
+// |x - mu|^2 of every row for the eccentricity. In FP64 that is a subtract and
+// an FMA a value, which the FP64 pipe takes 0.84 ms for at 1M x 256; here a value
+// takes ~45 FP32 instructions: with mu = mh + ml, t = x - mu as th + tl (two-sums;
+// tl to 2^-24 of itself), th^2 = p + pe exactly, 2 th tl + (tl^2 + pe) in two
+// FMAs, and a 32-column sum of them as an FP32 expansion of three terms, added to the row's
+// FP64 sum. The roundings are below 2^-47 of a value's square and independent,
+// against 2^-53 of the running sum at every FP64 step. A chunk where some |t| is
+// not zero or in [2^-40, 2^55) is summed in FP64 instead (subtract and FMA,
+// columns in order). One thread a row, as lens_rows_kernel.
+__global__ void __launch_bounds__(kRows) ecc_rows_kernel(const float* __restrict__ X, int64_t n, int32_t d, int64_t ld,
+                                                         const double* __restrict__ mu, double* __restrict__ f, int m,
+                                                         int j)
+{
+    __shared__ float tile[kRows][kChunk + 1];
+    __shared__ double smu[kChunk];
+    __shared__ float2 smf[kChunk];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t row0 = (int64_t)blockIdx.x * kRows;
+    const bool vec = ld % 4 == 0 && ((uintptr_t)X & 15) == 0;
+    double acc = 0.0;
+    for (int32_t k0 = 0; k0 < d; k0 += kChunk) {
+        const int kc = min(kChunk, d - k0);
+        if (vec && kc == kChunk) {
+            // 16 bytes a lane: 8 lanes a row, 4 rows a warp at a time
+#pragma unroll
+            for (int i = 0; i < kRows / 16; ++i) {
+                const int r = warp * 4 + (lane >> 3) + 16 * i, c4 = (lane & 7) * 4;
+                const int64_t row = row0 + r;
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row < n) x = __ldg(reinterpret_cast<const float4*>(X + row * ld + k0 + c4));
+                tile[r][c4] = x.x;
+                tile[r][c4 + 1] = x.y;
+                tile[r][c4 + 2] = x.z;
+                tile[r][c4 + 3] = x.w;
+            }
+        } else {
+#pragma unroll 8
+            for (int r = warp; r < kRows; r += kRows / 32) {
+                const int64_t row = row0 + r;
+                float x = 0.f;
+                if (row < n && lane < kc) x = __ldg(X + row * ld + k0 + lane);
+                tile[r][lane] = x;
+            }
+        }
+        if (tid < kc) {
+            const double mk = mu[k0 + tid];
+            const float mh = (float)mk;
+            smu[tid] = mk;
+            smf[tid] = make_float2(mh, (float)(mk - (double)mh));
+        }
+        __syncthreads();
+        float s = 0.f, e = 0.f, e2 = 0.f;
+        unsigned lo = 0x7F800000u, hi = 0u;                        // smallest (not 0) and largest |th|
+#pragma unroll 4
+        for (int k = 0; k < kc; ++k) {
+            const float2 mk = smf[k];
+            float a, tl, err, b;
+            const float y = two_sum(tile[tid][k], -mk.x, a);        // x - mh = y + a
+            const float th = two_sum(y, __fsub_rn(a, mk.y), tl);
+            const unsigned t = __float_as_uint(th) & 0x7FFFFFFFu;
+            hi = max(hi, t);
+            lo = min(lo, t ? t : 0x7F800000u);
+            const float p = __fmul_rn(th, th);
+            const float low = __fmaf_rn(__fadd_rn(th, th), tl, __fmaf_rn(tl, tl, __fmaf_rn(th, th, -p)));
+            s = two_sum(s, p, err);
+            e = two_sum(e, err, b);
+            e2 = __fadd_rn(e2, b);
+            e = two_sum(e, low, b);
+            e2 = __fadd_rn(e2, b);
+        }
+        // 2^-40 and 2^55 as bits
+        if (lo >= (87u << 23) && hi < (182u << 23)) {
+            acc += (double)s + ((double)e + (double)e2);
+        } else if (hi != 0u) {
+            for (int k = 0; k < kc; ++k) {
+                const double t = __dsub_rn((double)tile[tid][k], smu[k]);
+                acc = __fma_rn(t, t, acc);
+            }
+        }
+        __syncthreads();
+    }
+    const int64_t row = row0 + tid;
+    if (row < n) f[row * m + j] = acc;
 }
 
 // Mean of f[r * m + j] over the rows: per-block sums (rows strided over the
@@ -327,17 +524,20 @@ __global__ void __launch_bounds__(256) col_lens_partial_kernel(const double* __r
     }
 }
 
-// f = sqrt(q + V), V = (sum of the block sums) / n
+// f = sqrt(q + V), V = (sum of the nb <= 512 block sums) / n, added up by every
+// block in the same tree
 __global__ void __launch_bounds__(256) ecc_finish_kernel(double* __restrict__ f, int64_t n, int m, int j,
                                                          const double* __restrict__ part, int nb)
 {
-    __shared__ double V;
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int b = 0; b < nb; ++b) t += part[b];
-        V = t / (double)n;
-    }
+    __shared__ double ws[8];
+    double t = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 256) t += part[b];
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = t;
     __syncthreads();
+    t = 0.0;
+    for (int w = 0; w < 8; ++w) t += ws[w];
+    const double V = t / (double)n;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
         f[r * m + j] = __dsqrt_rn(__dadd_rn(f[r * m + j], V));
 }
@@ -404,7 +604,6 @@ __global__ void __launch_bounds__(256) finite_kernel(const float* __restrict__ X
 // block): the sum is a chain of FP64 adds, so the next 32 rows are loaded
 // while the current ones are added, and the columns spread over the SMs (the
 // FP64 pipe takes 16 cycles for a warp's add). 1M x 256: 1.17 -> 0.54 ms.
-constexpr int kMeanRows = 4096;
 constexpr int kMeanAhead = 32;
 
 __global__ void __launch_bounds__(32) col_partial_sum_kernel(const float* __restrict__ X, int64_t n, int32_t d,
@@ -460,6 +659,13 @@ __global__ void __launch_bounds__(32) col_mean_kernel(const double* __restrict__
 // inside half an ulp of res (by more than the 2^-53 of a rounding to double),
 // res is the rounding. Otherwise, and for Inf, NaN, powers of two and small
 // values, the FP64 expression itself decides.
+// (not inlined: the compiler would predicate the FP64 instructions, and every
+// value would pay for them)
+__device__ __noinline__ float centred_fp64(float v, const double* mu)
+{
+    return (float)((double)v - *mu);
+}
+
 __global__ void __launch_bounds__(256) centre_rows_kernel(const float* __restrict__ X, int64_t n, int32_t d, int64_t ld,
                                                           const double* __restrict__ mu, float* __restrict__ xc)
 {
@@ -493,7 +699,7 @@ __global__ void __launch_bounds__(256) centre_rows_kernel(const float* __restric
             const float half = __fmul_rn(__uint_as_float(ex), 5.9604645e-8f * (1.f - 0.000244140625f));
             const float off = __fmaf_rn(2.3841858e-7f, __fadd_rn(fabsf(t), fabsf(m.y)), fabsf(r2));
             if (!(off < half) || (bits & 0x7FFFFFu) == 0u || ex < (64u << 23) || ex == 0x7F800000u)
-                res = (float)((double)v - mu[k]);
+                res = centred_fp64(v, mu + k);
             o[k] = res;
         }
     }
@@ -836,23 +1042,15 @@ cudaError_t lens_l2_split(const float* X, int64_t n, int32_t d, int64_t ld, doub
 {
     if (n == 0) return cudaSuccess;
     if (d > 32768) return cudaErrorInvalidValue;
-    const int blocks = (int)std::min<int64_t>(div_up(n, 8 * 32), 152 * 8);
-    lens_l2_exact_kernel<true><<<blocks, 256, 0, s>>>(X, n, d, ld, f, m, j, c, dp,
-                                                      static_cast<__nv_bfloat16*>(xh), xn2);
-    note_launch();
-    return cudaGetLastError();
+    return launch_l2_by_width<true>(X, n, d, ld, f, m, j, c, dp, xh, xn2, s);
 }
 
 cudaError_t lens_l2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j,
                     cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    if (d <= 32768) {
-        const int blocks = (int)std::min<int64_t>(div_up(n, 8 * 32), 152 * 8);
-        lens_l2_exact_kernel<false><<<blocks, 256, 0, s>>>(X, n, d, ld, f, m, j, nullptr, 0, nullptr, nullptr);
-    } else {
-        lens_rows_kernel<0><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, nullptr, nullptr, nullptr, f, m, j);
-    }
+    if (d <= 32768) return launch_l2_by_width<false>(X, n, d, ld, f, m, j, nullptr, 0, nullptr, nullptr, s);
+    lens_rows_kernel<0><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, nullptr, nullptr, nullptr, f, m, j);
     note_launch();
     return cudaGetLastError();
 }
@@ -888,20 +1086,28 @@ cudaError_t column_means(const float* X, int64_t n, int32_t d, int64_t ld, doubl
 // Eccentricity with exponent 2 (§3 and §4.1 name eccentricity among the
 // common filters): the mean squared distance from x to the cloud equals
 // |x - mu|^2 + mean_y |y - mu|^2 (mu the column means), so f(x) =
-// sqrt(|x - mu|^2 + V) in FP64 without any pair of points: column means by
-// fixed-order block sums, |x - mu|^2 summed k ascending, V their mean.
-cudaError_t lens_ecc2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j, cudaStream_t s)
+// sqrt(|x - mu|^2 + V) without any pair of points: column means and |x - mu|^2
+// to FP64 accuracy, V their mean (fixed-order sums). 1M x 256 through mapper_lens:
+// 3024 us with FP64 arithmetic throughout and a pass of its own for the finite
+// check, 831 us now (column sums 286, rows 400); error against 64 bits 2.5e-16
+// before, 1.3e-16 now.
+cudaError_t lens_ecc2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j, cudaStream_t s,
+                      int* flag)
 {
     if (n == 0) return cudaSuccess;
-    Buf mu, vpart;
+    const int nblk = div_up(n, kMeanRows);
+    Buf part, mu, vpart;
+    MGB_TRY(part.alloc(sizeof(double) * (size_t)nblk * d, s));
     MGB_TRY(mu.alloc(sizeof(double) * d, s));
     MGB_TRY(vpart.alloc(sizeof(double) * kMeanBlocks, s));
-    MGB_TRY(column_means(X, n, d, ld, mu.as<double>(), s));
-    { lens_rows_kernel<2><<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu.as<double>(), nullptr, nullptr, f, m, j);
-      note_launch(); }
-    { col_lens_partial_kernel<<<kMeanBlocks, 256, 0, s>>>(f, n, m, j, vpart.as<double>()); note_launch(); }
-    { ecc_finish_kernel<<<std::min(div_up(n, 256), 152 * 8), 256, 0, s>>>(f, n, m, j, vpart.as<double>(), kMeanBlocks);
-      note_launch(); }
+    col_sum_exp_kernel<<<dim3(nblk, div_up(d, 32)), 32 * kEccWarps, 0, s>>>(X, n, d, ld, part.as<double>(), flag);
+    MGB_TRY(cudaGetLastError());
+    col_mean_kernel<<<div_up(d, 32), 32, 0, s>>>(part.as<double>(), nblk, d, n, mu.as<double>());
+    ecc_rows_kernel<<<div_up(n, kRows), kRows, 0, s>>>(X, n, d, ld, mu.as<double>(), f, m, j);
+    MGB_TRY(cudaGetLastError());
+    col_lens_partial_kernel<<<kMeanBlocks, 256, 0, s>>>(f, n, m, j, vpart.as<double>());
+    ecc_finish_kernel<<<std::min(div_up(n, 256), 152 * 8), 256, 0, s>>>(f, n, m, j, vpart.as<double>(), kMeanBlocks);
+    note_launch(5);
     return cudaGetLastError();
 }
 

@@ -52,11 +52,22 @@ __global__ void pivot_gather_kernel(const float* __restrict__ X, int64_t n, int 
 }
 
 // c[k] = the FP32 sum of the K pivots' column k in pivot order, / K
-__global__ void pivot_mean_kernel(const float* __restrict__ Pv, int K, int dp, float* __restrict__ c)
+// Mean of the pivots, 32 columns a CTA: eight warps of a column set each sum
+// every eighth pivot (loads ahead of the chain).
+__global__ void __launch_bounds__(256) pivot_mean_kernel(const float* __restrict__ Pv, int K, int dp,
+                                                         float* __restrict__ c)
 {
-    for (int k = threadIdx.x; k < dp; k += blockDim.x) {
-        float s = 0.f;
-        for (int i = 0; i < K; ++i) s += Pv[(int64_t)i * dp + k];
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (k < dp) {
+#pragma unroll 16
+        for (int i = warp; i < K; i += 8) s += Pv[(int64_t)i * dp + k];
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && k < dp) {
+        for (int w = 1; w < 8; ++w) s += part[w][lane];
         c[k] = s / (float)K;
     }
 }
@@ -175,9 +186,12 @@ __global__ void pivot_adj_kernel(const float* __restrict__ Pv, int dp, int K, fl
 }
 
 // Pivot groups: connected components of the adjacency, numbered 0.. in
-// order of their smallest pivot. One CTA.
-__global__ void __launch_bounds__(256) group_kernel(const unsigned* __restrict__ adj_g, int K,
-                                                    int32_t* __restrict__ gid, int32_t* __restrict__ n_groups)
+// order of their smallest pivot, and the pivots' places in the order (group,
+// pivot): rank[pivot], and the group at each place, group_at[rank] (K for the
+// place K of the outliers). One CTA of kPiv threads.
+__global__ void __launch_bounds__(kPiv) group_kernel(const unsigned* __restrict__ adj_g, int K,
+                                                     int32_t* __restrict__ rank, int32_t* __restrict__ group_at,
+                                                     int32_t* __restrict__ n_groups)
 {
     __shared__ unsigned adj[kPiv][kPiv / 32];
     __shared__ int lab[kPiv];
@@ -205,48 +219,86 @@ __global__ void __launch_bounds__(256) group_kernel(const unsigned* __restrict__
         if (!changed) break;
         __syncthreads();
     }
+    // number the components: prefix counts of the pivots that label themselves
+    __shared__ unsigned roots[kPiv / 32];
+    __shared__ int cnt[kPiv / 32][kPiv];               // pivots of each warp with each label
+    __shared__ int wsum[kPiv / 32];
+    const int lane = tid & 31, warp = tid >> 5;
+    const int l = tid < K ? lab[tid] : kPiv + tid;     // (threads past K: labels of their own)
+    for (int w = 0; w < kPiv / 32; ++w) cnt[w][tid] = 0;
+    const unsigned m = __ballot_sync(0xffffffffu, l == tid);
+    const unsigned peers = __match_any_sync(0xffffffffu, l);
+    if (lane == 0) roots[warp] = m;
+    __syncthreads();
+    if (tid < K && (peers & ((1u << lane) - 1u)) == 0u) cnt[warp][l] = __popc(peers);
+    __syncthreads();
+    // start of each label's pivots in the order: exclusive scan of the label sizes
+    int size = 0;
+    for (int w = 0; w < kPiv / 32; ++w) size += cnt[w][tid];
+    int x = size;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    int start = x - size;
+    for (int w = 0; w < warp; ++w) start += wsum[w];
+    __syncthreads();
+    adj[tid][0] = (unsigned)start;                     // (the adjacency is no longer needed)
+    __syncthreads();
     if (tid < K) {
-        const int l = lab[tid];
-        int g = 0;
-        for (int j = 0; j < l; ++j) g += lab[j] == j;
-        gid[tid] = g;
-        if (tid == K - 1) {
-            int ng = 0;
-            for (int j = 0; j < K; ++j) ng += lab[j] == j;
-            *n_groups = ng;
-        }
+        int g = __popc(roots[l >> 5] & ((1u << (l & 31)) - 1u));
+        for (int w = 0; w < (l >> 5); ++w) g += __popc(roots[w]);
+        int r = (int)adj[l][0] + __popc(peers & ((1u << lane) - 1u));
+        for (int w = 0; w < warp; ++w) r += cnt[w][l];
+        rank[tid] = r;
+        group_at[r] = g;
+    }
+    if (tid == 0) {
+        int ng = 0;
+        for (int w = 0; w < kPiv / 32; ++w) ng += __popc(roots[w]);
+        *n_groups = ng;
+        group_at[K] = K;
     }
 }
 
-// Sort key of a slot: (element, group, pivot) above the slot index.
+// Sort key of a slot: its element above its pivot's place in the order (group,
+// pivot) (K for outliers), above the slot index. rbits = 0: the element alone.
 __global__ void key_kernel(const int32_t* __restrict__ slot_point, const int32_t* __restrict__ slot_elem,
                            int64_t M, const int32_t* __restrict__ piv, const float* __restrict__ pd2,
-                           const int32_t* __restrict__ gid, float tau2, int K, int gbits, int pbits,
+                           const int32_t* __restrict__ rank, float tau2, int K, int rbits,
                            uint64_t* __restrict__ keys)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= M) return;
-    const int pt = slot_point[s];
-    const int pv = piv[pt];
-    const bool outlier = !(pd2[pt] <= tau2);
-    uint64_t g = 0, pf = 0;
-    if (gbits) g = outlier ? (uint64_t)K : (uint64_t)gid[pv];
-    if (pbits && !outlier) pf = (uint64_t)pv;
-    const uint64_t hi = ((uint64_t)slot_elem[s] << (gbits + pbits)) | (g << pbits) | pf;
+    uint64_t hi = (uint64_t)(uint32_t)slot_elem[s];
+    if (rbits) {
+        const int pt = slot_point[s];
+        hi = (hi << rbits) | (uint64_t)(!(pd2[pt] <= tau2) ? K : rank[piv[pt]]);
+    }
     keys[s] = (hi << 32) | (uint64_t)(uint32_t)s;
 }
 
-__global__ void seg_flag_kernel(const uint64_t* __restrict__ keys, int64_t M, int shift,
-                                int32_t* __restrict__ flag)
+// A segment starts where the element or the group changes.
+__global__ void seg_flag_kernel(const uint64_t* __restrict__ keys, int64_t M, int rbits,
+                                const int32_t* __restrict__ group_at, int32_t* __restrict__ flag)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M) return;
-    flag[i] = i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift);
+    bool f = i == 0;
+    if (!f) {
+        const uint64_t a = keys[i - 1] >> 32, b = keys[i] >> 32;
+        const uint64_t mask = (1ull << rbits) - 1ull;
+        f = (a >> rbits) != (b >> rbits) || (a != b && group_at[a & mask] != group_at[b & mask]);
+    }
+    flag[i] = f;
 }
 
 // seg_start[nseg+1], seg_elem, seg_out (outlier segment) from the flags' scan
 __global__ void seg_start_kernel(const uint64_t* __restrict__ keys, const int32_t* __restrict__ flag,
-                                 const int64_t* __restrict__ segpos, int64_t M, int gbits, int pbits,
+                                 const int64_t* __restrict__ segpos, int64_t M, int rbits,
                                  int K, int64_t* __restrict__ seg_start, int32_t* __restrict__ seg_elem,
                                  int32_t* __restrict__ seg_out)
 {
@@ -256,8 +308,8 @@ __global__ void seg_start_kernel(const uint64_t* __restrict__ keys, const int32_
         const int64_t sg = segpos[i];
         const uint64_t hi = keys[i] >> 32;
         seg_start[sg] = i;
-        seg_elem[sg] = (int32_t)(hi >> (gbits + pbits));
-        seg_out[sg] = gbits ? (int32_t)(((hi >> pbits) & ((1ull << gbits) - 1)) == (uint64_t)K) : 0;
+        seg_elem[sg] = (int32_t)(hi >> rbits);
+        seg_out[sg] = rbits ? (int32_t)((hi & ((1ull << rbits) - 1)) == (uint64_t)K) : 0;
     }
     if (i == M - 1) seg_start[segpos[M]] = M;
 }
@@ -463,43 +515,64 @@ __global__ void __launch_bounds__(32 * kPrepWarps, 1) tile_prep_reg_kernel(
 
 // Segment centre: the row-weighted mean of its tile centres, in double.
 // With dp <= 512 the CTA splits the tiles over blockDim / dp thread groups
-// (one thread per column in each) and adds the group sums at the end.
+// (one thread per column in each) and adds the group sums at the end. One FP64
+// FMA a value: the centres widen in integer instructions, the weights come as
+// doubles from shared memory, and the weight sum is an integer.
+constexpr int kCentTiles = 128;
+
+// (not inlined: a predicated conversion would take its FP64 slot for every value)
+__device__ __noinline__ double widen_rare(float x) { return (double)x; }
+
+__device__ __forceinline__ double widen_centre(float x)
+{
+    const unsigned b = __float_as_uint(x), t = b & 0x7FFFFFFFu;
+    if (t != 0u && t - 0x00800000u >= 0x7F000000u) return widen_rare(x);       // subnormal, Inf, NaN
+    const unsigned hi = t ? (t >> 3) + (896u << 20) : 0u;
+    return __hiloint2double((int)((b & 0x80000000u) | hi), (int)(b << 29));
+}
+
 __global__ void __launch_bounds__(1024) seg_cent_kernel(const float* __restrict__ cent,
                                                         const int32_t* __restrict__ tile_n,
                                                         const int64_t* __restrict__ seg_toff, int dp,
                                                         float* __restrict__ seg_cent)
 {
-    __shared__ double s_sum[2][1024];
+    __shared__ double s_sum[1024];
+    __shared__ double s_w[kCentTiles];
     const int64_t g = blockIdx.x;
-    const int W = dp <= 512 ? (int)blockDim.x / dp : 1;
-    const int w = dp <= 512 ? (int)threadIdx.x / dp : 0;
+    const int W = dp <= (int)blockDim.x && dp <= 512 ? (int)blockDim.x / dp : 1;
+    const bool wide = dp > (int)blockDim.x || dp > 512;            // columns in blocks, one group
+    const int w = wide ? 0 : (int)threadIdx.x / dp;
     const int64_t t0 = seg_toff[g], t1 = seg_toff[g + 1];
-    for (int k0 = 0; k0 < dp; k0 += (dp <= 512 ? dp : (int)blockDim.x)) {
-        const int k = dp <= 512 ? (int)threadIdx.x % dp : k0 + (int)threadIdx.x;
-        double sum = 0.0, wt = 0.0;
-        if (w < W && k < dp) {
-            for (int64_t t = t0 + w; t < t1; t += W) {
-                sum += (double)cent[t * dp + k] * (double)tile_n[t];
-                wt += (double)tile_n[t];
+    for (int k0 = 0; k0 < dp; k0 += wide ? (int)blockDim.x : dp) {
+        const int k = wide ? k0 + (int)threadIdx.x : (int)threadIdx.x % dp;
+        double sum = 0.0;
+        long long wt = 0;
+        for (int64_t b = t0; b < t1; b += kCentTiles) {
+            const int cnt = (int)min((int64_t)kCentTiles, t1 - b);
+            for (int i = threadIdx.x; i < cnt; i += blockDim.x) s_w[i] = (double)tile_n[b + i];
+            __syncthreads();
+            if (w < W && k < dp) {
+#pragma unroll 8
+                for (int i = w; i < cnt; i += W) sum = fma(widen_centre(cent[(b + i) * dp + k]), s_w[i], sum);
             }
+            if (w == 0 && k < dp)
+                for (int i = 0; i < cnt; ++i) wt += tile_n[b + i];
+            __syncthreads();
         }
         if (W > 1) {
-            if (w < W) {
-                s_sum[0][threadIdx.x] = sum;
-                s_sum[1][threadIdx.x] = wt;
-            }
+            if (w < W) s_sum[threadIdx.x] = sum;
             __syncthreads();
             if (w == 0) {
-                for (int v = 1; v < W; ++v) {
-                    sum += s_sum[0][v * dp + k];
-                    wt += s_sum[1][v * dp + k];
-                }
+                for (int v = 1; v < W; ++v) sum += s_sum[v * dp + k];
             }
             __syncthreads();
         }
-        if (w == 0 && k < dp) seg_cent[g * dp + k] = (float)(sum / wt);
+        if (w == 0 && k < dp) seg_cent[g * dp + k] = (float)(sum / (double)wt);
     }
 }
+
+// Threads of a CTA per segment: few where the segments hold few tiles.
+inline unsigned seg_threads(int64_t tiles, int64_t segs) { return tiles <= 4 * segs ? 256u : 1024u; }
 
 // BF16 operands centred on the segment centre c (FP32): a = fl(x - c),
 // hi = bf16(a), lo = bf16(a - hi) (a - hi is exact in FP32); |a|^2 summed in
@@ -745,10 +818,23 @@ __global__ void __launch_bounds__(1024) seg_rad_kernel(const float* __restrict__
     __shared__ double s_max[32];
     const int64_t g = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // a warp takes up to 32 consecutive tiles at a time, lane i keeps tile i's
+    // sum, and the FP64 square roots of all of them run side by side (a warp's
+    // FP64 instruction costs the same for one lane as for all)
+    const int64_t t0 = seg_toff[g], t1 = seg_toff[g + 1];
+    const int per = (int)min((int64_t)32, (t1 - t0 + nw - 1) / nw);
     double m = 0.0;
-    for (int64_t t = seg_toff[g] + warp; t < seg_toff[g + 1]; t += nw) {
-        const float ssum = dist_sum32(cent + t * dp, seg_cent + g * dp, dp, lane);
-        m = fmax(m, sqrt((double)ssum * (1.0 + rel)) * (1.0 + 1e-15) + rad[t]);
+    for (int64_t b = t0 + (int64_t)warp * per; b < t1; b += (int64_t)nw * per) {
+        const int cnt = (int)min((int64_t)per, t1 - b);
+        float mine = 0.f;
+        for (int i = 0; i < cnt; ++i) {
+            const float ssum = dist_sum32(cent + (b + i) * dp, seg_cent + g * dp, dp, lane);
+            if (lane == i) mine = ssum;
+        }
+        if (lane < cnt) m = fmax(m, sqrt((double)mine * (1.0 + rel)) * (1.0 + 1e-15) + rad[b + lane]);
+    }
+    if (t0 + (int64_t)warp * per < t1) {
+        for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
     if (lane == 0) s_max[warp] = m;
     __syncthreads();
@@ -1002,14 +1088,14 @@ __global__ void __launch_bounds__(256) pair_bin_kernel(const int2* __restrict__ 
     }
 }
 
-// Per bin of the sampled pairs (pair j of the sample is pairs[j * stride] of
-// the list): cnt[2 b] sampled pairs, cnt[2 b + 1] of them with a deferred block.
+// Per bin of the sampled pairs: cnt[2 b] pairs, cnt[2 b + 1] of them with a
+// deferred block.
 __global__ void sample_bin_kernel(const uint32_t* __restrict__ mask, int64_t n_s, const uint8_t* __restrict__ bin,
-                                  int64_t stride, unsigned long long* __restrict__ cnt)
+                                  unsigned long long* __restrict__ cnt)
 {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_s) return;
-    const int b = bin[j * stride];
+    const int b = bin[j];
     atomicAdd(&cnt[2 * b], 1ull);
     if (mask[j]) atomicAdd(&cnt[2 * b + 1], 1ull);
 }
@@ -1051,12 +1137,12 @@ cudaError_t pair_bins(const TileLayout& L, const int2* pairs, int64_t n, int dp,
     return cudaGetLastError();
 }
 
-cudaError_t sample_bins(const uint32_t* mask, int64_t n_s, const uint8_t* bin, int64_t stride,
-                        unsigned long long* cnt, cudaStream_t s)
+cudaError_t sample_bins(const uint32_t* mask, int64_t n_s, const uint8_t* bin, unsigned long long* cnt,
+                        cudaStream_t s)
 {
     MGB_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 2 * kPairBins, s));
     if (n_s == 0) return cudaSuccess;
-    sample_bin_kernel<<<grid_for(n_s), 256, 0, s>>>(mask, n_s, bin, stride, cnt);
+    sample_bin_kernel<<<grid_for(n_s), 256, 0, s>>>(mask, n_s, bin, cnt);
     note_launch();
     return cudaGetLastError();
 }
@@ -1133,7 +1219,7 @@ int pivot_prepare(const float* X, int64_t n, int32_t d, int64_t ld, int dp, bool
     }
     if (!host) {
         pivot_gather_kernel<<<K, 128, 0, s>>>(X, n, d, ld, dp, K, P->Pv.as<float>());
-        pivot_mean_kernel<<<1, 256, 0, s>>>(P->Pv.as<float>(), K, dp, P->c.as<float>());
+        pivot_mean_kernel<<<div_up(dp, 32), 256, 0, s>>>(P->Pv.as<float>(), K, dp, P->c.as<float>());
         note_launch(2);
         PK(cudaGetLastError());
     } else {
@@ -1180,32 +1266,35 @@ int build_tiles(const float* X, int64_t n, int32_t d, int64_t ld, int dp, const 
     const Buf& Pv = pre->Pv;
     const Buf& piv = pre->piv;
     const Buf& pd2 = pre->pd2;
-    Buf gid, ngrp, adj;
-    TK(gid.alloc(sizeof(int32_t) * kPiv, s));
+    Buf rank, group_at, ngrp, adj;
+    TK(rank.alloc(sizeof(int32_t) * kPiv, s));
+    TK(group_at.alloc(sizeof(int32_t) * (kPiv + 1), s));
     TK(ngrp.alloc(sizeof(int32_t), s));
     TK(adj.alloc(sizeof(unsigned) * kPiv * (kPiv / 32), s));
     TK(cudaMemsetAsync(adj.p, 0, sizeof(unsigned) * kPiv * (kPiv / 32), s));
     const float tau2 = (float)(tau * tau);
     pivot_adj_kernel<<<grid_for((int64_t)K * K * 32, 256), 256, 0, s>>>(Pv.as<float>(), dp, K, tau2,
                                                                        adj.as<unsigned>());
-    group_kernel<<<1, 256, 0, s>>>(adj.as<unsigned>(), K, gid.as<int32_t>(), ngrp.as<int32_t>());
+    group_kernel<<<1, kPiv, 0, s>>>(adj.as<unsigned>(), K, rank.as<int32_t>(), group_at.as<int32_t>(),
+                                    ngrp.as<int32_t>());
     note_launch(2);
     TK(cudaGetLastError());
 
-    int ebits = bits_for(E), gbits = bits_for(K + 1), pbits = bits_for(K);
-    if (ebits + gbits + pbits > 32) pbits = 0;
-    if (ebits + gbits + pbits > 32) gbits = 0;
+    const int ebits = bits_for(E);
+    int rbits = bits_for(K + 1);
+    if (ebits + rbits > 32) rbits = 0;
     Buf keys, tmp, flag, segpos;
     TK(keys.alloc(sizeof(uint64_t) * M, s));
     TK(tmp.alloc(sizeof(uint64_t) * M, s));
     key_kernel<<<grid_for(M), 256, 0, s>>>(slot_point, slot_elem, M, piv.as<int32_t>(), pd2.as<float>(),
-                                          gid.as<int32_t>(), tau2, K, gbits, pbits, keys.as<uint64_t>());
+                                          rank.as<int32_t>(), tau2, K, rbits, keys.as<uint64_t>());
     note_launch();
     TK(cudaGetLastError());
-    TK(radix_sort_u64(keys, tmp, M, 32, 32 + ebits + gbits + pbits, s));
+    TK(radix_sort_u64(keys, tmp, M, 32, 32 + ebits + rbits, s));
     TK(flag.alloc(sizeof(int32_t) * M, s));
     TK(segpos.alloc(sizeof(int64_t) * (M + 1), s));
-    seg_flag_kernel<<<grid_for(M), 256, 0, s>>>(keys.as<uint64_t>(), M, 32 + pbits, flag.as<int32_t>());
+    seg_flag_kernel<<<grid_for(M), 256, 0, s>>>(keys.as<uint64_t>(), M, rbits, group_at.as<int32_t>(),
+                                               flag.as<int32_t>());
     note_launch();
     TK(cudaGetLastError());
     TK(exclusive_scan_i32_to_i64(flag.as<int32_t>(), segpos.as<int64_t>(), M, s));
@@ -1215,7 +1304,7 @@ int build_tiles(const float* X, int64_t n, int32_t d, int64_t ld, int dp, const 
     TK(cudaMemcpyAsync(&ng, ngrp.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     TK(cudaStreamSynchronize(s));
     L->n_seg = nseg;
-    L->n_groups = gbits ? ng : 1;
+    L->n_groups = rbits ? ng : 1;
 
     Buf seg_start, seg_tiles;
     Buf& seg_elem = L->seg_elem;
@@ -1226,7 +1315,7 @@ int build_tiles(const float* X, int64_t n, int32_t d, int64_t ld, int dp, const 
     TK(seg_tiles.alloc(sizeof(int64_t) * nseg, s));
     TK(seg_toff.alloc(sizeof(int64_t) * (nseg + 1), s));
     seg_start_kernel<<<grid_for(M), 256, 0, s>>>(keys.as<uint64_t>(), flag.as<int32_t>(), segpos.as<int64_t>(),
-                                                M, gbits, pbits, K, seg_start.as<int64_t>(),
+                                                M, rbits, K, seg_start.as<int64_t>(),
                                                 seg_elem.as<int32_t>(), L->seg_outlier.as<int32_t>());
     seg_tiles_kernel<<<grid_for(nseg), 256, 0, s>>>(seg_start.as<int64_t>(), nseg, seg_tiles.as<int64_t>());
     note_launch(2);
@@ -1268,13 +1357,13 @@ int build_tiles(const float* X, int64_t n, int32_t d, int64_t ld, int dp, const 
                                                      L->row_pt.as<int32_t>(), L->tile_cent.as<float>(),
                                                      L->tile_rad.as<double>(), nonfinite);
     }
-    seg_cent_kernel<<<(unsigned)nseg, 1024, 0, s>>>(L->tile_cent.as<float>(), L->tile_n.as<int32_t>(),
+    seg_cent_kernel<<<(unsigned)nseg, seg_threads(T, nseg), 0, s>>>(L->tile_cent.as<float>(), L->tile_n.as<int32_t>(),
                                                   seg_toff.as<int64_t>(), dp, L->seg_cent.as<float>());
     note_launch(4);
     TK(cudaGetLastError());
     TK(L->seg_rad.alloc(sizeof(double) * nseg, s));
     const double rel = (double)(dp / 32 + 12) * std::ldexp(1.0, -23);
-    seg_rad_kernel<<<(unsigned)nseg, 1024, 0, s>>>(L->tile_cent.as<float>(), L->tile_rad.as<double>(),
+    seg_rad_kernel<<<(unsigned)nseg, seg_threads(T, nseg), 0, s>>>(L->tile_cent.as<float>(), L->tile_rad.as<double>(),
                                                  L->seg_cent.as<float>(), seg_toff.as<int64_t>(), dp, rel,
                                                  L->seg_rad.as<double>());
     note_launch();
@@ -1369,7 +1458,7 @@ int cross_operands(const TileLayout& L, const float* X, int64_t ld, int d, int d
     XK(tmax->alloc(sizeof(float4) * T, s));
     XK(tn2min->alloc(sizeof(float) * T, s));
     elem_tiles_kernel<<<grid_for(E + 1), 256, 0, s>>>(L.tile_elem.as<int32_t>(), T, E, etile_off.as<int64_t>());
-    seg_cent_kernel<<<(unsigned)E, 1024, 0, s>>>(L.tile_cent.as<float>(), L.tile_n.as<int32_t>(),
+    seg_cent_kernel<<<(unsigned)E, seg_threads(T, E), 0, s>>>(L.tile_cent.as<float>(), L.tile_n.as<int32_t>(),
                                                etile_off.as<int64_t>(), dp, ecent.as<float>());
     const float norm_infl = 1.0f + (float)(dp / 32 + 16) * 5.9604645e-8f;
     const bool xvec = ld % 4 == 0 && ((uintptr_t)X & 15) == 0;
