@@ -21,6 +21,7 @@ namespace mgb {
 
 thread_local std::string g_last_error;
 thread_local int64_t g_launches = 0;
+thread_local void* g_pinned = nullptr;
 void set_error(const std::string& msg) { g_last_error = msg; }
 
 }  // namespace mgb
@@ -57,12 +58,20 @@ struct CoverData {
     Buf pt_off, slot_o;        // memberships in point order: n + 1 int64 offsets, and each
                                // slot's place (M int32); unset for a subset of a cover
     std::vector<int64_t> h_elem_off;
+    void* offsets_at = nullptr;  // h_elem_off on its way through page-locked scratch
+    void take_offsets()                // after a wait for the stream
+    {
+        if (offsets_at) memcpy(h_elem_off.data(), offsets_at, sizeof(int64_t) * h_elem_off.size());
+        offsets_at = nullptr;
+    }
 };
 
 struct ClusterData {
     StreamRef stream;
     std::shared_ptr<CoverData> cover;
     Buf core, lab, flags, slot_label;                 // per cover slot
+    Buf node_pos;                                     // scan of the flags, if done with the clustering (M + 1)
+    int64_t node_totals = 0;                          //   and its last entry
     mapper_stats stats{};
 };
 
@@ -71,6 +80,7 @@ struct ClusterData {
 struct mapper_ctx {
     int device = 0;
     StreamRef stream;
+    void* pinned = nullptr;                    // page-locked scratch for read-backs (kPinBytes)
     size_t budget = 0;
     bool timing = false;
     int num_sms = 152;
@@ -171,6 +181,7 @@ int check_ctx(mapper_ctx* ctx)
 {
     if (!ctx) return fail(MAPPER_EINVAL, "null context");
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
+    g_pinned = ctx->pinned;
     return MAPPER_OK;
 }
 
@@ -287,9 +298,10 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     CK(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), pos.as<int64_t>(), n, s), "scan");
     int64_t M = 0;
     int h_nf = 0;
-    CK(cudaMemcpyAsync(&M, pos.as<int64_t>() + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "copy");
-    CK(cudaMemcpyAsync(&h_nf, nf, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
-    CK(cudaStreamSynchronize(s), "sync");
+    Readback rb(s);
+    CK(rb.get(&M, pos.as<int64_t>() + n, sizeof(int64_t)), "copy");
+    CK(rb.get(&h_nf, nf, sizeof(int)), "copy");
+    CK(rb.wait(), "sync");
     if (h_nf) return fail(MAPPER_ENONFINITE, "lens or X holds NaN or Inf");
     if (M > INT32_MAX) return fail(MAPPER_ENOMEM, "more than 2^31 cover memberships");
     c->M = M;
@@ -306,10 +318,17 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     CK(c->slot_o.alloc(sizeof(int32_t) * M, s), "alloc");
     CK(split_keys(keys.as<uint64_t>(), pt.as<int32_t>(), M, E, c->slot_point.as<int32_t>(),
                   c->slot_elem.as<int32_t>(), c->slot_o.as<int32_t>(), c->elem_off.as<int64_t>(), s), "split");
+    // the host's copy of the offsets lands with the next wait (take_offsets)
+    // where it fits the page-locked scratch
     c->h_elem_off.resize(E + 1);
-    CK(cudaMemcpyAsync(c->h_elem_off.data(), c->elem_off.p, sizeof(int64_t) * (E + 1),
-                       cudaMemcpyDeviceToHost, s), "copy");
-    CK(cudaStreamSynchronize(s), "sync");
+    const size_t bytes = sizeof(int64_t) * (E + 1);
+    if (g_pinned && bytes <= kPinBytes - Readback::kSmall) {
+        c->offsets_at = static_cast<char*>(g_pinned) + Readback::kSmall;
+        CK(cudaMemcpyAsync(c->offsets_at, c->elem_off.p, bytes, cudaMemcpyDeviceToHost, s), "copy");
+    } else {
+        CK(cudaMemcpyAsync(c->h_elem_off.data(), c->elem_off.p, bytes, cudaMemcpyDeviceToHost, s), "copy");
+        CK(cudaStreamSynchronize(s), "sync");
+    }
     *out = c;
     return MAPPER_OK;
 }
@@ -394,18 +413,17 @@ int sample_deferral(const mapper_ctx* ctx, const PassArgs& a, const TcArgs& firs
     unsigned long long h_redo = 0;
     int h_err = 0;
     Buf bc, bins;
+    Readback rb(s);
     if (L && h_bins) {
         CK(bins.alloc(n_s, s), "alloc");
         CK(bc.alloc(sizeof(unsigned long long) * 2 * kPairBins, s), "alloc");
         CK(pair_bins(*L, sp.as<int2>(), n_s, a.dp, eps, bins.as<uint8_t>(), s), "pair bins");
         CK(sample_bins(mask.as<uint32_t>(), n_s, bins.as<uint8_t>(), bc.as<unsigned long long>(), s), "sample bins");
-        CK(cudaMemcpyAsync(h_bins, bc.p, sizeof(unsigned long long) * 2 * kPairBins, cudaMemcpyDeviceToHost, s),
-           "copy");
+        CK(rb.get(h_bins, bc.p, sizeof(unsigned long long) * 2 * kPairBins), "copy");
     }
-    CK(cudaMemcpyAsync(&h_redo, st.as<unsigned long long>() + kStatRedo, sizeof(h_redo), cudaMemcpyDeviceToHost, s),
-       "copy");
-    CK(cudaMemcpyAsync(&h_err, err.p, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
-    CK(cudaStreamSynchronize(s), "sync");
+    CK(rb.get(&h_redo, st.as<unsigned long long>() + kStatRedo, sizeof(h_redo)), "copy");
+    CK(rb.get(&h_err, err.p, sizeof(int)), "copy");
+    CK(rb.wait(), "sync");
     if (h_err) return fail(MAPPER_ETIMEOUT, "a tensor-core pass gave up waiting on a barrier (phase sample)");
     *frac = (double)h_redo / (double)n_s;
     return MAPPER_OK;
@@ -566,12 +584,6 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
     st.n_points = n;
     st.n_elements = E;
     st.n_members = M;
-    double s2 = 0.0;
-    for (int64_t e = 0; e < E; ++e) {
-        const double ne = (double)(cov->h_elem_off[e + 1] - cov->h_elem_off[e]);
-        s2 += ne * ne;
-    }
-    st.sum_ni2 = s2;
 
     // per radius: outputs, counters and the pass arguments
     struct Radius {
@@ -605,6 +617,13 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         if (rc) return rc;
         layout = &own;
     }
+    cov->take_offsets();                                          // (the layout's sizes were waited for)
+    double s2 = 0.0;
+    for (int64_t e = 0; e < E; ++e) {
+        const double ne = (double)(cov->h_elem_off[e + 1] - cov->h_elem_off[e]);
+        s2 += ne * ne;
+    }
+    st.sum_ni2 = s2;
     // FP8 screen: E4M3 operands with per-tile scales beside the BF16 ones (the
     // union pass and the second phase of the count pass stay in BF16)
     const bool f8 = precision == MAPPER_FP8;
@@ -954,7 +973,6 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         return MAPPER_OK;
     }
     unsigned long long h_shared[kStatCount] = {};
-    if (K > 1) CK(cudaMemcpyAsync(h_shared, shared_stats.p, sizeof(h_shared), cudaMemcpyDeviceToHost, s), "copy");
     float ms_count = 0.f;
     bool have_ms_count = false;
     for (int e = 0; e < K; ++e) {
@@ -1036,12 +1054,18 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
                          c->flags.as<uint8_t>(), c->slot_label.as<int64_t>(),
                          c->core.as<uint8_t>(), s), "labels");
 
+        // the nerve's sizes come with the same wait
+        CK(c->node_pos.alloc(sizeof(int64_t) * (M + 1), s), "alloc");
+        CK(exclusive_scan_slot_flags(c->flags.as<uint8_t>(), c->node_pos.as<int64_t>(), M, s), "scan");
         unsigned long long h_stats[kStatCount];
         int h_nf = 0;
-        CK(cudaMemcpyAsync(h_stats, a.stats, sizeof(h_stats), cudaMemcpyDeviceToHost, s), "copy");
-        CK(cudaMemcpyAsync(&h_nf, nf, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
-        if (use_tc) CK(cudaMemcpyAsync(&h_err, tc_err.p, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");
-        CK(cudaStreamSynchronize(s), "sync");
+        Readback rb(s);
+        CK(rb.get(h_stats, a.stats, sizeof(h_stats)), "copy");
+        CK(rb.get(&h_nf, nf, sizeof(int)), "copy");
+        if (use_tc) CK(rb.get(&h_err, tc_err.p, sizeof(int)), "copy");
+        CK(rb.get(&c->node_totals, c->node_pos.as<int64_t>() + M, sizeof(int64_t)), "copy");
+        if (K > 1 && e == 0) CK(rb.get(h_shared, shared_stats.p, sizeof(h_shared)), "copy");
+        CK(rb.wait(), "sync");
         if (h_nf) return fail(MAPPER_ENONFINITE, "X holds NaN or Inf");
         if (h_err) return fail(MAPPER_ETIMEOUT, "a tensor-core pass gave up waiting on a barrier");
         // the count pass's counters (kept apart when there are several radii)
@@ -1123,12 +1147,16 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
     cudaStream_t s = ctx->stream->s;
     const auto& cov = cl->cover;
     const int64_t M = cov->M;
-    Buf pos;
-    CK(pos.alloc(sizeof(int64_t) * (M + 1), s), "alloc");
-    CK(exclusive_scan_slot_flags(cl->flags.as<uint8_t>(), pos.as<int64_t>(), M, s), "scan");
-    int64_t totals = 0;
-    CK(cudaMemcpyAsync(&totals, pos.as<int64_t>() + M, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "copy");
-    CK(cudaStreamSynchronize(s), "sync");
+    Buf own_pos;
+    int64_t totals = cl->node_totals;
+    if (!cl->node_pos.p) {
+        CK(own_pos.alloc(sizeof(int64_t) * (M + 1), s), "alloc");
+        CK(exclusive_scan_slot_flags(cl->flags.as<uint8_t>(), own_pos.as<int64_t>(), M, s), "scan");
+        Readback rb(s);
+        CK(rb.get(&totals, own_pos.as<int64_t>() + M, sizeof(int64_t)), "copy");
+        CK(rb.wait(), "sync");
+    }
+    const Buf& pos = cl->node_pos.p ? cl->node_pos : own_pos;
     const int64_t N = totals >> 32, Gm = totals & 0xffffffffll;
     g->N = N;
     g->Gm = Gm;
@@ -1156,8 +1184,9 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
         CK(edge_set(cov->pt_off.as<int64_t>(), cov->n, node_o.as<int32_t>(), &g->edges, dc, s), "edges");
         CK(radix_sort_u64_two_dev(g->edges.as<uint64_t>(), kEdgeListMax, dc, 32, 0, bits_for(N), s), "sort");
         unsigned long long h[2] = {0, 0};
-        CK(cudaMemcpyAsync(h, dc, sizeof(h), cudaMemcpyDeviceToHost, s), "copy");
-        CK(cudaStreamSynchronize(s), "sync");
+        Readback rb(s);
+        CK(rb.get(h, dc, sizeof(h)), "copy");
+        CK(rb.wait(), "sync");
         edges_done = h[1] == 0;
         g->Eg = (int64_t)h[0];
     }
@@ -1211,11 +1240,17 @@ int nerve_edges(mapper_ctx* ctx, Buf& keys2, int64_t Gm, int64_t n_points, int64
     return MAPPER_OK;
 }
 
+// Queues a copy to the caller's memory; copies_done waits for all of them.
 int copy_out(void* dst, const void* src, size_t bytes, int on_device, cudaStream_t s)
 {
     if (!dst || bytes == 0) return MAPPER_OK;
     CK(cudaMemcpyAsync(dst, src, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s),
        "copy out");
+    return MAPPER_OK;
+}
+
+int copies_done(cudaStream_t s)
+{
     CK(cudaStreamSynchronize(s), "sync");
     return MAPPER_OK;
 }
@@ -1342,6 +1377,10 @@ int mapper_create(mapper_ctx** out, int device, size_t hbm_budget_bytes, void* c
         ctx->stream->owned = true;
     }
     CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device), "attr");
+    if (cudaMallocHost(&ctx->pinned, kPinBytes) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->pinned = nullptr;                 // (read-backs then go to pageable memory)
+    }
 
     // keep freed scratch in the pool between calls
     cudaMemPool_t pool;
@@ -1360,6 +1399,8 @@ void mapper_destroy(mapper_ctx* ctx)
     cudaSetDevice(ctx->device);
     if (ctx->stream && ctx->stream->s) cudaStreamSynchronize(ctx->stream->s);
     tune_cache_save(ctx);
+    if (ctx->pinned) cudaFreeHost(ctx->pinned);
+    if (g_pinned == ctx->pinned) g_pinned = nullptr;
     delete ctx;
 }
 
@@ -1493,6 +1534,8 @@ static int cover_call(mapper_ctx* ctx, const double* lens_dev, int64_t n, int32_
     if (n < 1 || n > INT32_MAX) return fail(MAPPER_EINVAL, "n must be in [1, 2^31)");
     std::shared_ptr<CoverData> c;
     if ((rc = run_cover(ctx, lens_dev, n, m, n_intervals, overlap, &c, nullptr, balanced != 0))) return rc;
+    CK(cudaStreamSynchronize(ctx->stream->s), "sync");
+    c->take_offsets();
     auto h = new mapper_cover_t;
     h->c = c;
     *out = h;
@@ -1528,7 +1571,8 @@ int mapper_cover_copy(const mapper_cover_t* cover, int64_t* elem_offsets, int32_
     cudaStream_t s = h->c->stream->s;
     int rc = copy_out(elem_offsets, h->c->elem_off.p, sizeof(int64_t) * (h->c->E + 1), on_device, s);
     if (rc) return rc;
-    return copy_out(elem_points, h->c->slot_point.p, sizeof(int32_t) * h->c->M, on_device, s);
+    if ((rc = copy_out(elem_points, h->c->slot_point.p, sizeof(int32_t) * h->c->M, on_device, s))) return rc;
+    return elem_offsets || elem_points ? copies_done(s) : MAPPER_OK;
 }
 
 int mapper_cluster(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t d, int64_t ld,
@@ -1557,7 +1601,8 @@ int mapper_clusters_copy(const mapper_clusters_t* clusters, int64_t* label, uint
     const int64_t M = h->c->cover->M;
     int rc = copy_out(label, h->c->slot_label.p, sizeof(int64_t) * M, on_device, s);
     if (rc) return rc;
-    return copy_out(core, h->c->core.p, M, on_device, s);
+    if ((rc = copy_out(core, h->c->core.p, M, on_device, s))) return rc;
+    return label || core ? copies_done(s) : MAPPER_OK;
 }
 
 int mapper_single_linkage(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t d, int64_t ld,
@@ -1838,7 +1883,8 @@ int mapper_knn_distance(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t 
                           ctx->knn_info);
     }
     if (rc) return rc;
-    return copy_out(out, od.p, sizeof(double) * q, !is_host_pointer(out), s);
+    if ((rc = copy_out(out, od.p, sizeof(double) * q, !is_host_pointer(out), s))) return rc;
+    return copies_done(s);
 }
 
 // Host rows to the device (xdev, n x d). When every lens of p is row-local
@@ -2162,7 +2208,8 @@ int mapper_graph_copy(const mapper_graph_t* g, int64_t* node_offsets, int32_t* n
     if ((rc = copy_out(node_offsets, h->node_off.p, sizeof(int64_t) * (h->N + 1), on_device, s))) return rc;
     if ((rc = copy_out(node_members, h->node_members.p, sizeof(int32_t) * h->Gm, on_device, s))) return rc;
     if ((rc = copy_out(node_elem, h->node_elem.p, sizeof(int32_t) * h->N, on_device, s))) return rc;
-    return copy_out(edges, h->edges.p, sizeof(int32_t) * 2 * h->Eg, on_device, s);
+    if ((rc = copy_out(edges, h->edges.p, sizeof(int32_t) * 2 * h->Eg, on_device, s))) return rc;
+    return node_offsets || node_members || node_elem || edges ? copies_done(s) : MAPPER_OK;
 }
 
 int mapper_graph_lens(const mapper_graph_t* g, double* lens, double* pca, int64_t* n_pca, int on_device)
@@ -2174,7 +2221,8 @@ int mapper_graph_lens(const mapper_graph_t* g, double* lens, double* pca, int64_
     if (lens && !h->lens.p) return fail(MAPPER_EINVAL, "graph was built from a given cover; no lens stored");
     int rc = copy_out(lens, h->lens.p, sizeof(double) * h->n * h->m, on_device, s);
     if (rc) return rc;
-    return copy_out(pca, h->pca.p, sizeof(double) * h->n_pca, on_device, s);
+    if ((rc = copy_out(pca, h->pca.p, sizeof(double) * h->n_pca, on_device, s))) return rc;
+    return lens || pca ? copies_done(s) : MAPPER_OK;
 }
 
 const mapper_cover_t* mapper_graph_cover(const mapper_graph_t* g)

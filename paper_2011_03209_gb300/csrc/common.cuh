@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <string>
 
@@ -72,6 +73,47 @@ struct Buf {
         bytes = 0;
     }
     template <class T> T* as() const { return static_cast<T*>(p); }
+};
+
+// Page-locked host scratch of the calling thread's context (kPinBytes), set by
+// every entry point; null outside one.
+constexpr size_t kPinBytes = 64 << 10;
+extern thread_local void* g_pinned;
+
+// A few device values for the host with one wait: get() queues the copies
+// (through the page-locked scratch: a copy to pageable memory is a wait of its
+// own), wait() synchronises the stream once and fills the destinations.
+// A copy and a wait cost the host 8 to 9 us, and the device idles meanwhile: a
+// graph has 6 of them where it had 11 (with the sizes of a layout and of the
+// nerve taken together), 5k x 8 945 -> 758 us, 13.7k x 37 1097 -> 847.
+struct Readback {
+    explicit Readback(cudaStream_t stream) : s(stream) {}
+    cudaError_t get(void* dst, const void* src, size_t bytes)
+    {
+        const size_t at = (used + 15) & ~size_t(15);
+        if (!g_pinned || n == kMax || at + bytes > kSmall)
+            return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s);
+        item[n++] = {dst, at, bytes};
+        used = at + bytes;
+        return cudaMemcpyAsync(static_cast<char*>(g_pinned) + at, src, bytes, cudaMemcpyDeviceToHost, s);
+    }
+    cudaError_t wait()
+    {
+        const cudaError_t e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess)
+            for (int i = 0; i < n; ++i) memcpy(item[i].dst, static_cast<char*>(g_pinned) + item[i].at, item[i].bytes);
+        n = 0;
+        used = 0;
+        return e;
+    }
+    static constexpr size_t kSmall = 8 << 10;      // the scratch's part for these
+    static constexpr int kMax = 8;
+
+private:
+    struct Item { void* dst; size_t at, bytes; } item[kMax];
+    cudaStream_t s;
+    int n = 0;
+    size_t used = 0;
 };
 
 // ------------------------------------------------------------------ kernels

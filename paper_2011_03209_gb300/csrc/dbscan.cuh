@@ -259,6 +259,9 @@ struct TileLayout {
     Buf seg_outlier;             // [n_seg] int32: 1 if the segment holds outliers
     Buf seg_elem;                // [n_seg] int32 element of each segment
     Buf seg_toff;                // [n_seg + 1] int64 first tile of each segment
+    Buf eseg_off;                // [E + 1] int64 first segment of each element
+    Buf blk_off;                 // [n_seg + 1] int64 blocks of tiles before each segment (classification)
+    int64_t n_cand = 0;          // tile pairs of all elements
     Buf seg_rad;                 // [n_seg] FP64 upper bound of its rows' distance to its centre
     Buf Ah, Al;                  // [R x dp] BF16 centred rows (hi and lo parts)
     Buf rn2, rn;                 // [R] FP32 |a|^2 and |a| (rounded up)
@@ -283,6 +286,7 @@ struct PairLists {
 struct PivotSet {
     int K = 0;
     Buf Pv, piv, pd2;
+    Buf err;                     // int: set if the tensor-core assignment gave up waiting (read by build_tiles)
     // set by pivot_prepare: the pivots' centre c and the points' split for
     // the tensor-core assignment (written by the lens pass, lens_l2_split)
     bool split = false;

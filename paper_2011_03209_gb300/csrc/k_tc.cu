@@ -2157,11 +2157,11 @@ int tc_groups_dev(const int2* pairs, int64_t n, const unsigned long long* n_dev,
 }
 
 int assign_pivots_tc(const float* X, int64_t n, int d, int64_t ld, int dp, const float* Pv, int K,
-                     int num_sms, int32_t* piv, float* pd2, cudaStream_t s, const PivotSplit* pre)
+                     int num_sms, int32_t* piv, float* pd2, cudaStream_t s, Buf* err, const PivotSplit* pre)
 {
     if (K > kPivN) { set_error("assign_pivots_tc: more than 256 pivots"); return MAPPER_EINVAL; }
     const int64_t n_tiles = (n + kT - 1) / kT, rows = n_tiles * kT;
-    Buf c, xh, xn2, ph, pn2, err;
+    Buf c, xh, xn2, ph, pn2;
 #define AK(expr)                                                                         \
     do {                                                                                 \
         cudaError_t e_ = (expr);                                                         \
@@ -2172,8 +2172,8 @@ int assign_pivots_tc(const float* X, int64_t n, int d, int64_t ld, int dp, const
     } while (0)
     AK(ph.alloc(sizeof(__nv_bfloat16) * (size_t)kPivN * dp, s));
     AK(pn2.alloc(sizeof(float) * kPivN, s));
-    AK(err.alloc(sizeof(int), s));
-    AK(cudaMemsetAsync(err.p, 0, sizeof(int), s));
+    AK(err->alloc(sizeof(int), s));
+    AK(cudaMemsetAsync(err->p, 0, sizeof(int), s));
     const float* cc = pre ? pre->c : nullptr;
     const void* xhp = pre ? pre->xh : nullptr;
     const float* xn2p = pre ? pre->xn2 : nullptr;
@@ -2207,17 +2207,13 @@ int assign_pivots_tc(const float* X, int64_t n, int d, int64_t ld, int dp, const
     p.pn2 = pn2.as<float>();
     p.piv = piv;
     p.pd2 = pd2;
-    p.err = err.as<int>();
+    p.err = err->as<int>();
     const int smem = kAsgStages * kAsgStageBytes + (int)sizeof(AsgTail) + 1024;
     AK(cudaFuncSetAttribute(assign_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     assign_tc_kernel<<<(int)std::min<int64_t>(n_tiles, num_sms), 192, smem, s>>>(mxh, mph, p);
     note_launch();
     AK(cudaGetLastError());
-    int h_err = 0;
-    AK(cudaMemcpyAsync(&h_err, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    AK(cudaStreamSynchronize(s));
 #undef AK
-    if (h_err) { set_error("pivot assignment gave up waiting on a barrier"); return MAPPER_ETIMEOUT; }
     return MAPPER_OK;
 }
 

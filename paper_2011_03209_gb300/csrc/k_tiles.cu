@@ -32,6 +32,7 @@ namespace mgb {
 namespace {
 
 constexpr int kPiv = 256;      // most pivots
+constexpr int kClsA = 8;
 constexpr int kT = kTile;
 
 inline unsigned grid_for(int64_t n, int t = 256) { return (unsigned)std::max<int64_t>(1, div_up(n, t)); }
@@ -276,7 +277,8 @@ __global__ void key_kernel(const int32_t* __restrict__ slot_point, const int32_t
     uint64_t hi = (uint64_t)(uint32_t)slot_elem[s];
     if (rbits) {
         const int pt = slot_point[s];
-        hi = (hi << rbits) | (uint64_t)(!(pd2[pt] <= tau2) ? K : rank[piv[pt]]);
+        const int pv = min(max(piv[pt], 0), K - 1);      // (unset if the assignment timed out)
+        hi = (hi << rbits) | (uint64_t)(!(pd2[pt] <= tau2) ? K : rank[pv]);
     }
     keys[s] = (hi << 32) | (uint64_t)(uint32_t)s;
 }
@@ -320,6 +322,100 @@ __global__ void seg_tiles_kernel(const int64_t* __restrict__ seg_start, int64_t 
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= nseg) return;
     seg_tiles[g] = (seg_start[g + 1] - seg_start[g] + kT - 1) / kT;
+}
+
+// *pairs += the element tile pairs n (n + 1) / 2 of all elements.
+__global__ void __launch_bounds__(256) cand_count_kernel(const int64_t* __restrict__ eseg_off,
+                                                         const int64_t* __restrict__ seg_toff, int64_t E,
+                                                         unsigned long long* pairs)
+{
+    unsigned long long c = 0;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t n = seg_toff[eseg_off[e + 1]] - seg_toff[eseg_off[e]];
+        c += (unsigned long long)(n * (n + 1) / 2);
+    }
+    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(pairs, c);
+}
+
+// The sizes of a layout in one CTA, with their number of segments on the
+// device: tiles before every segment (seg_toff), blocks of kClsA tiles before
+// every segment (blk_off, see classify_blk_kernel), first segment of every
+// element (eseg_off[E + 1]), and out = (segments, tiles, element tile pairs).
+// One launch and one read-back where a scan per array would take a launch or two
+// each and the host three round trips. Covers of more than kLayoutElems elements
+// (fine grids, mostly empty) take those.
+constexpr int kLayoutThreads = 1024;
+constexpr int64_t kLayoutElems = 16384;
+
+__global__ void __launch_bounds__(kLayoutThreads) layout_sizes_kernel(
+    const int64_t* __restrict__ n_seg, const int64_t* __restrict__ seg_start, const int32_t* __restrict__ seg_elem,
+    int64_t E, int64_t* __restrict__ seg_toff, int64_t* __restrict__ blk_off, int64_t* __restrict__ eseg_off,
+    int64_t* __restrict__ out)
+{
+    __shared__ int64_t s_warp[kLayoutThreads / 32];
+    __shared__ int64_t s_pairs[kLayoutThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t S = *n_seg;
+    int64_t carry = 0;                                   // blocks << 32 | tiles so far
+    for (int64_t b = 0; b < S; b += kLayoutThreads) {
+        const int64_t g = b + tid;
+        int64_t v = 0;
+        if (g < S) {
+            const int64_t tiles = (seg_start[g + 1] - seg_start[g] + kT - 1) / kT;
+            v = tiles | (((tiles + kClsA - 1) / kClsA) << 32);
+            const int32_t e = seg_elem[g], before = g ? seg_elem[g - 1] : -1;
+            for (int32_t x = before + 1; x <= e; ++x) eseg_off[x] = g;
+            if (g == S - 1)
+                for (int64_t x = (int64_t)e + 1; x <= E; ++x) eseg_off[x] = S;
+        }
+        int64_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        if (warp == 0) {
+            int64_t w = s_warp[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t y = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += y;
+            }
+            s_warp[lane] = w;
+        }
+        __syncthreads();
+        const int64_t at = carry + (warp ? s_warp[warp - 1] : 0) + x - v;
+        if (g < S) {
+            seg_toff[g] = at & 0xffffffffll;
+            blk_off[g] = at >> 32;
+        }
+        carry += s_warp[kLayoutThreads / 32 - 1];
+        __syncthreads();
+    }
+    if (S == 0)
+        for (int64_t x = tid; x <= E; x += kLayoutThreads) eseg_off[x] = 0;
+    if (tid == 0) {
+        seg_toff[S] = carry & 0xffffffffll;
+        blk_off[S] = carry >> 32;
+    }
+    __syncthreads();                                     // the CTA's own global writes are visible to it
+    int64_t pairs = 0;
+    for (int64_t e = tid; e < E; e += kLayoutThreads) {
+        const int64_t n = seg_toff[eseg_off[e + 1]] - seg_toff[eseg_off[e]];
+        pairs += n * (n + 1) / 2;
+    }
+    for (int o = 16; o; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+    if (lane == 0) s_pairs[warp] = pairs;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kLayoutThreads / 32; ++w) pairs += s_pairs[w];
+        out[0] = S;
+        out[1] = carry & 0xffffffffll;
+        out[2] = pairs;
+    }
 }
 
 __global__ void row_map_kernel(const uint64_t* __restrict__ keys, const int64_t* __restrict__ segpos,
@@ -785,14 +881,6 @@ __global__ void elem_tiles_kernel(const int32_t* __restrict__ tile_elem, int64_t
     etile_off[e] = l;
 }
 
-__global__ void cand_count_kernel(const int64_t* __restrict__ etile_off, int64_t E, int64_t* __restrict__ cnt)
-{
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= E) return;
-    const int64_t T = etile_off[e + 1] - etile_off[e];
-    cnt[e] = T * (T + 1) / 2;
-}
-
 // Upper bound of the distance between two centres from an FP32 sum of
 // squares s: the sum of d rounded squares of rounded differences (lane
 // partials, then a shuffle tree) is within (d/32 + 12) 2^-23 of the exact one.
@@ -919,7 +1007,6 @@ constexpr int kMaxSegList = 1024;
 // lane keeps the kClsA sums itself (a sequential FMA chain over dp columns:
 // the true squared distance lies in [ssum c_lo, ssum c_hi]). CTA c takes block c of the blocks of kClsA tiles
 // that blk_off (exclusive prefix of ceil(tiles / kClsA) per segment) numbers.
-constexpr int kClsA = 8;
 
 __global__ void __launch_bounds__(256) classify_blk_kernel(const int64_t* __restrict__ blk_off, int64_t n_seg,
                                                            const int64_t* __restrict__ eseg_off,
@@ -1183,7 +1270,7 @@ int pivot_assign(const float* X, int64_t n, int32_t d, int64_t ld, int dp, bool 
     if (bf16) {
         const PivotSplit pre{P->c.as<float>(), P->xh.p, P->xn2.as<float>()};
         const int rc = assign_pivots_tc(X, n, d, ld, dp, P->Pv.as<float>(), K, num_sms, P->piv.as<int32_t>(),
-                                        P->pd2.as<float>(), s, P->split ? &pre : nullptr);
+                                        P->pd2.as<float>(), s, &P->err, P->split ? &pre : nullptr);
         if (rc) return rc;
     } else {
         assign_kernel<<<grid_for(n, kT), 256, 0, s>>>(X, n, d, ld, P->Pv.as<float>(), dp, K, P->piv.as<int32_t>(),
@@ -1298,32 +1385,74 @@ int build_tiles(const float* X, int64_t n, int32_t d, int64_t ld, int dp, const 
     note_launch();
     TK(cudaGetLastError());
     TK(exclusive_scan_i32_to_i64(flag.as<int32_t>(), segpos.as<int64_t>(), M, s));
-    int64_t nseg = 0;
-    int32_t ng = 0;
-    TK(cudaMemcpyAsync(&nseg, segpos.as<int64_t>() + M, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TK(cudaMemcpyAsync(&ng, ngrp.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    TK(cudaStreamSynchronize(s));
-    L->n_seg = nseg;
-    L->n_groups = rbits ? ng : 1;
-
-    Buf seg_start, seg_tiles;
+    // at most one segment per membership, and per element and group
+    const int64_t seg_max = std::min<int64_t>(std::max<int64_t>(M, 1), E * (int64_t)(K + 1));
+    Buf seg_start, sizes;
     Buf& seg_elem = L->seg_elem;
     Buf& seg_toff = L->seg_toff;
-    TK(seg_start.alloc(sizeof(int64_t) * (nseg + 1), s));
-    TK(seg_elem.alloc(sizeof(int32_t) * nseg, s));
-    TK(L->seg_outlier.alloc(sizeof(int32_t) * nseg, s));
-    TK(seg_tiles.alloc(sizeof(int64_t) * nseg, s));
-    TK(seg_toff.alloc(sizeof(int64_t) * (nseg + 1), s));
+    TK(seg_start.alloc(sizeof(int64_t) * (seg_max + 1), s));
+    TK(seg_elem.alloc(sizeof(int32_t) * seg_max, s));
+    TK(L->seg_outlier.alloc(sizeof(int32_t) * seg_max, s));
+    TK(seg_toff.alloc(sizeof(int64_t) * (seg_max + 1), s));
+    TK(L->blk_off.alloc(sizeof(int64_t) * (seg_max + 1), s));
+    TK(L->eseg_off.alloc(sizeof(int64_t) * (E + 1), s));
+    TK(sizes.alloc(sizeof(int64_t) * 3, s));
     seg_start_kernel<<<grid_for(M), 256, 0, s>>>(keys.as<uint64_t>(), flag.as<int32_t>(), segpos.as<int64_t>(),
                                                 M, rbits, K, seg_start.as<int64_t>(),
                                                 seg_elem.as<int32_t>(), L->seg_outlier.as<int32_t>());
-    seg_tiles_kernel<<<grid_for(nseg), 256, 0, s>>>(seg_start.as<int64_t>(), nseg, seg_tiles.as<int64_t>());
-    note_launch(2);
+    note_launch();
     TK(cudaGetLastError());
-    TK(exclusive_scan_i64(seg_tiles.as<int64_t>(), seg_toff.as<int64_t>(), nseg, s));
-    int64_t T = 0;
-    TK(cudaMemcpyAsync(&T, seg_toff.as<int64_t>() + nseg, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TK(cudaStreamSynchronize(s));
+    int64_t h_sizes[3] = {0, 0, 0};
+    int32_t ng = 0, assign_err = 0;
+    const bool small = E <= kLayoutElems;
+    if (small) {
+        layout_sizes_kernel<<<1, kLayoutThreads, 0, s>>>(segpos.as<int64_t>() + M, seg_start.as<int64_t>(),
+                                                         seg_elem.as<int32_t>(), E, seg_toff.as<int64_t>(),
+                                                         L->blk_off.as<int64_t>(), L->eseg_off.as<int64_t>(),
+                                                         sizes.as<int64_t>());
+        note_launch();
+        TK(cudaGetLastError());
+    }
+    {
+        Readback rb(s);
+        TK(rb.get(h_sizes, small ? sizes.p : segpos.as<int64_t>() + M, sizeof(int64_t) * (small ? 3 : 1)));
+        TK(rb.get(&ng, ngrp.p, sizeof(int32_t)));
+        if (pre->err.p) TK(rb.get(&assign_err, pre->err.p, sizeof(int32_t)));
+        TK(rb.wait());
+    }
+    if (!small) {
+        const int64_t S = h_sizes[0];
+        Buf cnt;
+        TK(cnt.alloc(sizeof(int64_t) * std::max<int64_t>(S, 1), s));
+        TK(cudaMemsetAsync(sizes.p, 0, sizeof(int64_t) * 3, s));
+        if (S > 0) {
+            seg_tiles_kernel<<<grid_for(S), 256, 0, s>>>(seg_start.as<int64_t>(), S, cnt.as<int64_t>());
+            TK(cudaGetLastError());
+        }
+        TK(exclusive_scan_i64(cnt.as<int64_t>(), seg_toff.as<int64_t>(), S, s));
+        if (S > 0) {
+            seg_blocks_kernel<<<grid_for(S), 256, 0, s>>>(seg_toff.as<int64_t>(), S, cnt.as<int64_t>());
+            TK(cudaGetLastError());
+        }
+        TK(exclusive_scan_i64(cnt.as<int64_t>(), L->blk_off.as<int64_t>(), S, s));
+        elem_segs_kernel<<<grid_for(E + 1), 256, 0, s>>>(seg_elem.as<int32_t>(), S, E, L->eseg_off.as<int64_t>());
+        cand_count_kernel<<<std::min(grid_for(E), 152u * 8u), 256, 0, s>>>(
+            L->eseg_off.as<int64_t>(), seg_toff.as<int64_t>(), E, sizes.as<unsigned long long>() + 2);
+        note_launch(4);
+        TK(cudaGetLastError());
+        Readback rb(s);
+        TK(rb.get(h_sizes + 1, seg_toff.as<int64_t>() + S, sizeof(int64_t)));
+        TK(rb.get(h_sizes + 2, sizes.as<int64_t>() + 2, sizeof(int64_t)));
+        TK(rb.wait());
+    }
+    if (assign_err) {
+        set_error("pivot assignment gave up waiting on a barrier");
+        return MAPPER_ETIMEOUT;
+    }
+    const int64_t nseg = h_sizes[0], T = h_sizes[1];
+    L->n_seg = nseg;
+    L->n_groups = rbits ? ng : 1;
+    L->n_cand = h_sizes[2];
     L->T = T;
     L->R = T * kT;
     const int64_t R = L->R;
@@ -1477,35 +1606,13 @@ int classify_pairs(const TileLayout& L, const float* X, int64_t ld, int d, int d
                    PairLists* P, cudaStream_t s, double eps_all_in)
 {
     if (!(eps_all_in > 0.0)) eps_all_in = eps;
-    Buf etile_off, cnt, cand_off, counts, eseg_off;
-    TK(etile_off.alloc(sizeof(int64_t) * (E + 1), s));
-    TK(eseg_off.alloc(sizeof(int64_t) * (E + 1), s));
-    TK(cnt.alloc(sizeof(int64_t) * std::max<int64_t>(E, 1), s));
-    TK(cand_off.alloc(sizeof(int64_t) * (E + 1), s));
+    const int64_t C = L.n_cand;
+    const Buf &eseg_off = L.eseg_off, &blk_off = L.blk_off;
+    Buf counts;
     TK(counts.alloc(sizeof(unsigned long long) * 4, s));
     TK(cudaMemsetAsync(counts.p, 0, sizeof(unsigned long long) * 4, s));
-    elem_tiles_kernel<<<grid_for(E + 1), 256, 0, s>>>(L.tile_elem.as<int32_t>(), L.T, E, etile_off.as<int64_t>());
-    elem_segs_kernel<<<grid_for(E + 1), 256, 0, s>>>(L.seg_elem.as<int32_t>(), L.n_seg, E, eseg_off.as<int64_t>());
-    cand_count_kernel<<<grid_for(E), 256, 0, s>>>(etile_off.as<int64_t>(), E, cnt.as<int64_t>());
-    note_launch(3);
-    TK(cudaGetLastError());
-    TK(exclusive_scan_i64(cnt.as<int64_t>(), cand_off.as<int64_t>(), E, s));
-    int64_t C = 0;
-    TK(cudaMemcpyAsync(&C, cand_off.as<int64_t>() + E, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TK(cudaStreamSynchronize(s));
     P->n_candidates = C;
     for (int k = 0; k < kListCount; ++k) TK(P->list[k].alloc(sizeof(int2) * std::max<int64_t>(C, 1), s));
-    // blocks of kClsA tiles A per segment for classify_blk_kernel
-    Buf blk_cnt, blk_off;
-    TK(blk_cnt.alloc(sizeof(int64_t) * std::max<int64_t>(L.n_seg, 1), s));
-    TK(blk_off.alloc(sizeof(int64_t) * (L.n_seg + 1), s));
-    if (L.n_seg > 0) {
-        seg_blocks_kernel<<<grid_for(L.n_seg), 256, 0, s>>>(L.seg_toff.as<int64_t>(), L.n_seg,
-                                                            blk_cnt.as<int64_t>());
-        note_launch();
-        TK(cudaGetLastError());
-    }
-    TK(exclusive_scan_i64(blk_cnt.as<int64_t>(), blk_off.as<int64_t>(), L.n_seg, s));
     const unsigned cls_grid = (unsigned)(div_up(L.T, kClsA) + L.n_seg);
     const size_t cls_smem = sizeof(float) * kClsA * dp;
     if (cls_smem > 48 * 1024)
@@ -1535,8 +1642,12 @@ int classify_pairs(const TileLayout& L, const float* X, int64_t ld, int d, int d
         if (rc) return rc;
     }
     unsigned long long h[4] = {0, 0, 0, 0};
-    TK(cudaMemcpyAsync(h, counts.p, sizeof(h), cudaMemcpyDeviceToHost, s));
-    TK(cudaStreamSynchronize(s));
+    auto read_counts = [&]() -> cudaError_t {
+        Readback rb(s);
+        MGB_TRY(rb.get(h, counts.p, sizeof(h)));
+        return rb.wait();
+    };
+    TK(read_counts());
     // Many mixed pairs across segments (a cover element holding scattered
     // points): bound the outlier tiles' distance to every segment of their
     // element and classify again, certifying more pairs all-out.
@@ -1553,8 +1664,7 @@ int classify_pairs(const TileLayout& L, const float* X, int64_t ld, int d, int d
         TK(cudaMemsetAsync(counts.p, 0, sizeof(unsigned long long) * 4, s));
         const int rc = classify(tsm.as<float>(), smax);
         if (rc) return rc;
-        TK(cudaMemcpyAsync(h, counts.p, sizeof(h), cudaMemcpyDeviceToHost, s));
-        TK(cudaStreamSynchronize(s));
+        TK(read_counts());
     }
     for (int k = 0; k < kListCount; ++k) P->n[k] = (int64_t)h[k];
     P->n_out = (int64_t)h[3];
