@@ -276,7 +276,7 @@ def mapper_lens(ctx: Context, X, kinds, args, lens_param=None, precision: int = 
     a = (ctypes.c_int32 * m)(*args)
     lp = (ctypes.c_double * m)(*[float(r) for r in lens_param]) if lens_param is not None else None
     npca = d * (1 + max([arg for kind, arg in zip(kinds, args) if kind == LENS_PCA], default=-1))
-    pca = np.empty(max(npca, 1), dtype=np.float64)
+    pca = np.empty(npca + d, dtype=np.float64)     # the call writes the mean and every axis up to the highest
     _capi.check(ctx._lib.mapper_lens_ex(ctx.h, p, n, d, ld, m, k, a, lp, int(precision), _vp(out.data_ptr()),
                                         _vp(pca.ctypes.data) if npca > d else None), "mapper_lens")
     return out, (pca[:npca] if npca > d else None)
