@@ -6,6 +6,7 @@
 // key on its high field only keeps the low field's incoming order.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "common.cuh"
@@ -212,7 +213,7 @@ cudaError_t exclusive_scan_impl(const T* in, int64_t* out, int64_t n, cudaStream
 //                     holds the keys in registers, the CTAs exchange their
 //                     digit counts through distributed shared memory, and the
 //                     cluster barrier separates the digits;
-//   n <= kRsSelfTiles tiles of kRsTile: two launches a digit (counts per
+//   up to kRsSelfTiles tiles (4.2M keys): two launches a digit (counts per
 //                     tile; then every CTA adds up the counts of the tiles
 //                     before it, ranks its keys and writes them in runs);
 //   more              the counts are scanned by launches in between (every
@@ -398,35 +399,46 @@ __global__ void __launch_bounds__(kRcThreads) radix_cluster_kernel(uint64_t* __r
 }
 
 // ---- two launches a digit
-constexpr int kRsThreads = 512;
+constexpr int kRsThreads = 1024;
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsItems = 16;                         // rounds per warp
-constexpr int kRsTile = kRsThreads * kRsItems;       // 8192 keys per CTA
+constexpr int kRsItems = 8;                          // most rounds per warp
 constexpr int64_t kRsSelfTiles = 512;
+constexpr int64_t kRsFill = 152;                     // CTAs that fill the chip
 
+// A CTA's tile is kRsThreads * items keys: as few rounds as fill the chip once,
+// because a CTA's time is the chain of its rounds (with 16 rounds in 512 threads
+// a digit of 330k keys took 13 + 14 us on 41 CTAs, of 1.25M 13 + 19 on 153).
 // SELF: hist[block * 256 + digit] (int32); else offs[digit * nblocks + block]
 // (int64), the layout that one scan turns into output offsets.
 template <bool SELF>
 __global__ void __launch_bounds__(kRsThreads) radix_hist_kernel(const uint64_t* __restrict__ keys, int64_t n,
-                                                                SortField f, int shift, uint32_t mask,
+                                                                SortField f, int shift, uint32_t mask, int items,
                                                                 void* __restrict__ hist)
 {
     __shared__ int cnt[kRsBins];
-    for (int b = threadIdx.x; b < kRsBins; b += kRsThreads) cnt[b] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRsTile;
+    if (threadIdx.x < kRsBins) cnt[threadIdx.x] = 0;
+    const int64_t base = (int64_t)blockIdx.x * kRsThreads * items;
     const int lane = threadIdx.x & 31;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < kRsTile; i += kRsThreads) {
-        const int64_t idx = base + i;
+    uint64_t key[kRsItems];
+#pragma unroll
+    for (int r = 0; r < kRsItems; ++r) {
+        const int64_t idx = base + (int64_t)r * kRsThreads + threadIdx.x;
+        key[r] = r < items && idx < n ? keys[idx] : 0ull;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRsItems; ++r) {
+        if (r >= items) break;                                     // uniform
+        const int64_t idx = base + (int64_t)r * kRsThreads + threadIdx.x;
         // one shared-memory atomic per distinct digit of the warp: runs of
         // equal digits (nearly sorted input) would serialise
-        const int dg = idx < n ? digit_of(keys[idx], f, shift, mask) : -1;
+        const int dg = idx < n ? digit_of(key[r], f, shift, mask) : -1;
         const unsigned peers = __match_any_sync(0xffffffffu, dg);
         if (dg >= 0 && (peers & ((1u << lane) - 1u)) == 0) atomicAdd(&cnt[dg], __popc(peers));
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < kRsBins; b += kRsThreads) {
+    if (threadIdx.x < kRsBins) {
+        const int b = threadIdx.x;
         if (SELF) static_cast<int32_t*>(hist)[(int64_t)blockIdx.x * kRsBins + b] = cnt[b];
         else static_cast<int64_t*>(hist)[(int64_t)b * gridDim.x + blockIdx.x] = cnt[b];
     }
@@ -435,54 +447,66 @@ __global__ void __launch_bounds__(kRsThreads) radix_hist_kernel(const uint64_t* 
 template <bool SELF>
 __global__ void __launch_bounds__(kRsThreads) radix_scatter_kernel(const uint64_t* __restrict__ in,
                                                                    uint64_t* __restrict__ out, int64_t n, SortField f,
-                                                                   int shift, uint32_t mask,
+                                                                   int shift, uint32_t mask, int items,
                                                                    const void* __restrict__ hist)
 {
-    extern __shared__ uint64_t s_keys[];                           // kRsTile keys
+    extern __shared__ uint64_t s_keys[];                           // the tile's keys
     __shared__ __align__(16) uint16_t wcnt[kRsWarps][kRsBins];
     __shared__ int s_total[kRsBins], s_local[kRsBins];
     __shared__ int64_t s_out[kRsBins];
-    __shared__ int s_part[2][2][kRsBins];
+    __shared__ int s_part[2][4][kRsBins];
     __shared__ int s_warp[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t base = (int64_t)blockIdx.x * kRsTile;
-    const int here = (int)min((int64_t)kRsTile, n - base);
+    const int64_t base = (int64_t)blockIdx.x * kRsThreads * items;
+    const int here = (int)min((int64_t)kRsThreads * items, n - base);
+    const int w0 = warp * 32 * items;                              // the warp's first key of the tile
     uint64_t key[kRsItems];
     int at[kRsItems];
 #pragma unroll
     for (int r = 0; r < kRsItems; ++r) {
-        const int i = warp * 32 * kRsItems + r * 32 + lane;
-        key[r] = i < here ? in[base + i] : 0ull;
-        at[r] = i < here ? digit_of(key[r], f, shift, mask) : -1;
+        const int i = w0 + r * 32 + lane;
+        const bool valid = r < items && i < here;
+        key[r] = valid ? in[base + i] : 0ull;
+        at[r] = valid ? digit_of(key[r], f, shift, mask) : -1;
     }
     if (SELF) {
-        // two threads a digit, each over half of the tiles
+        // four threads a digit, each over a quarter of the tiles
         const int32_t* h = static_cast<const int32_t*>(hist);
-        const int b = tid & (kRsBins - 1), half = tid >> 8;
+        const int b = tid & (kRsBins - 1), q = tid >> 8;
         const int nb = (int)gridDim.x, me = (int)blockIdx.x;
         int all = 0, before = 0;
 #pragma unroll 8
-        for (int t = half; t < nb; t += 2) {
+        for (int t = q; t < nb; t += 4) {
             const int v = __ldg(h + (int64_t)t * kRsBins + b);
             all += v;
             if (t < me) before += v;
         }
-        s_part[0][half][b] = all;
-        s_part[1][half][b] = before;
+        s_part[0][q][b] = all;
+        s_part[1][q][b] = before;
     }
     for (int e = lane; e < kRsBins / 2; e += 32) reinterpret_cast<uint32_t*>(wcnt[warp])[e] = 0u;
     __syncwarp();
-    warp_rank<kRsItems>(at, kRsItems, wcnt[warp]);
+    warp_rank<kRsItems>(at, items, wcnt[warp]);
     __syncthreads();
     warp_prefixes<kRsWarps>(wcnt, s_total);
     __syncthreads();
     const int mine = tid < kRsBins ? s_total[tid] : 0;
     const int local = scan256(mine, s_warp);
-    int start = 0;
-    if (SELF) start = scan256(tid < kRsBins ? s_part[0][0][tid] + s_part[0][1][tid] : 0, s_warp);
+    int start = 0, before = 0;
+    if (SELF) {
+        int all = 0;
+        if (tid < kRsBins) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                all += s_part[0][q][tid];
+                before += s_part[1][q][tid];
+            }
+        }
+        start = scan256(all, s_warp);
+    }
     if (tid < kRsBins) {
         s_local[tid] = local;
-        s_out[tid] = (SELF ? (int64_t)start + s_part[1][0][tid] + s_part[1][1][tid]
+        s_out[tid] = (SELF ? (int64_t)start + before
                            : static_cast<const int64_t*>(hist)[(int64_t)tid * gridDim.x + blockIdx.x]) - local;
     }
     __syncthreads();
@@ -529,27 +553,30 @@ cudaError_t radix_sort_field(Buf& keys, Buf& tmp, int64_t n, const SortField& f,
     const int width = f.w0 + f.w1;
     if (n <= 1 || width <= 0) return cudaSuccess;
     if (n <= kRcMaxKeys) return radix_sort_cluster(keys.as<uint64_t>(), n, f, s);
-    const int64_t nb = div_up(n, kRsTile);
+    const int items = (int)std::min<int64_t>(kRsItems, div_up(n, (int64_t)kRsThreads * kRsFill));
+    const int tile = kRsThreads * items;
+    const int64_t nb = div_up(n, tile);
     const bool self = nb <= kRsSelfTiles;
     Buf hist, offs;
     MGB_TRY(hist.alloc((self ? sizeof(int32_t) : sizeof(int64_t)) * kRsBins * nb, s));
     if (!self) MGB_TRY(offs.alloc(sizeof(int64_t) * (kRsBins * nb + 1), s));
-    const size_t smem = sizeof(uint64_t) * kRsTile;
-    if (self) MGB_TRY(cudaFuncSetAttribute(radix_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    else MGB_TRY(cudaFuncSetAttribute(radix_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = sizeof(uint64_t) * tile, most = sizeof(uint64_t) * kRsThreads * kRsItems;
+    if (self) MGB_TRY(cudaFuncSetAttribute(radix_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    else MGB_TRY(cudaFuncSetAttribute(radix_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     for (int shift = 0; shift < width; shift += 8) {
         const uint32_t mask = width - shift < 8 ? (1u << (width - shift)) - 1u : 255u;
         const uint64_t* src = keys.as<uint64_t>();
         uint64_t* dst = tmp.as<uint64_t>();
+        const unsigned g = (unsigned)nb;
         if (self) {
-            radix_hist_kernel<true><<<(unsigned)nb, kRsThreads, 0, s>>>(src, n, f, shift, mask, hist.p);
+            radix_hist_kernel<true><<<g, kRsThreads, 0, s>>>(src, n, f, shift, mask, items, hist.p);
             MGB_TRY(cudaGetLastError());
-            radix_scatter_kernel<true><<<(unsigned)nb, kRsThreads, smem, s>>>(src, dst, n, f, shift, mask, hist.p);
+            radix_scatter_kernel<true><<<g, kRsThreads, smem, s>>>(src, dst, n, f, shift, mask, items, hist.p);
         } else {
-            radix_hist_kernel<false><<<(unsigned)nb, kRsThreads, 0, s>>>(src, n, f, shift, mask, hist.p);
+            radix_hist_kernel<false><<<g, kRsThreads, 0, s>>>(src, n, f, shift, mask, items, hist.p);
             MGB_TRY(cudaGetLastError());
             MGB_TRY(exclusive_scan_i64(hist.as<int64_t>(), offs.as<int64_t>(), kRsBins * nb, s));
-            radix_scatter_kernel<false><<<(unsigned)nb, kRsThreads, smem, s>>>(src, dst, n, f, shift, mask, offs.p);
+            radix_scatter_kernel<false><<<g, kRsThreads, smem, s>>>(src, dst, n, f, shift, mask, items, offs.p);
         }
         note_launch(2);
         MGB_TRY(cudaGetLastError());
