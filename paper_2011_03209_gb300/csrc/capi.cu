@@ -486,7 +486,10 @@ int tune_pass1(mapper_ctx* ctx, const PassArgs& a, const TcArgs& t, int64_t n_pa
     ts.redo_mask = mask.as<uint32_t>();
     ts.sub_mask = nullptr;
     ts.sub_q = nullptr;
-    // each shape twice, alternating; the faster of each counts
+    // Each shape twice, alternating; the faster of each counts. Before a long
+    // pass the counts are cleared once only: its first pairs fill the rows'
+    // lists (returning atomics), but most find the rows' counts done.
+    const bool warm = n_pairs >= (int64_t)ctx->num_sms * 256;
     constexpr int kRuns = 4;
     cudaEvent_t ev[2 * kRuns] = {};
     struct Guard {
@@ -496,8 +499,10 @@ int tune_pass1(mapper_ctx* ctx, const PassArgs& a, const TcArgs& t, int64_t n_pa
     for (int i = 0; i < 2 * kRuns; ++i) CK(cudaEventCreate(&ev[i]), "event");
     for (int run = 0; run < kRuns; ++run) {
         const int v = run & 1;
-        CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * R, s), "memset");
-        if (cap) CK(cudaMemsetAsync(nbr.p, 0xff, sizeof(int32_t) * (size_t)R * cap, s), "memset");
+        if (run == 0 || !warm) {
+            CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * R, s), "memset");
+            if (cap) CK(cudaMemsetAsync(nbr.p, 0xff, sizeof(int32_t) * (size_t)R * cap, s), "memset");
+        }
         CK(cudaMemsetAsync(hit.p, 0, n_t, s), "memset");
         CK(cudaMemsetAsync(st.p, 0, sizeof(unsigned long long) * kStatCount, s), "memset");
         if (t.defer) CK(cudaMemsetAsync(mask.p, 0, sizeof(uint32_t) * n_t, s), "memset");
@@ -680,6 +685,7 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         a.count = rd.count.as<int32_t>();
         a.nbr = rd.nbr.as<int32_t>();
         a.cap = cap;
+        a.need = counts_out ? INT_MAX : min_pts;
         a.core = rd.core.as<uint8_t>();
         a.parent = rd.parent.as<int32_t>();
         a.root = rd.root.as<int32_t>();

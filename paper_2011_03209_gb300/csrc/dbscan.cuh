@@ -50,6 +50,9 @@ struct PassArgs {
     int32_t* count;              // pass 1 output, per row
     int32_t* nbr;                // pass 1: first `cap` neighbour rows of each row
     int cap;                     //   (0: no lists)
+    int need = INT_MAX;          // pass 1: a count of at least this many is not needed exactly (more
+                                 //   may stay uncounted): minPts, which decides the core flag and
+                                 //   is above every list; INT_MAX: exact counts
     uint8_t* pair_hit;           // pass 1 (explicit mode, optional): set to 1 for each tile
                                  //   pair with a neighbour pair, or one left to the recheck
     const uint8_t* core;         // passes 2, 3

@@ -14,10 +14,11 @@
 //
 // Kernel layout (one CTA per SM, persistent over a static share of the tile
 // pairs): warp 0 issues TMA loads of 64-column K blocks (128-byte swizzle)
-// into a ring of smem stages; warp 1 issues the MMAs into one of two TMEM
-// accumulators (128 x 128 FP32 each); 16 warps read the accumulator back
-// with tcgen05.ld (four warps per TMEM lane quadrant, each thread one row and
-// 32 columns) and run the pass epilogue, branch-free per pair:
+// into a ring of smem stages; warp 1 issues the MMAs into the TMEM
+// accumulators (128 x 128 or 128 x 256 FP32 each; the count pass fills all 512
+// columns with them); 16 warps read the accumulators back with tcgen05.ld
+// (four warps per TMEM lane quadrant, a row per thread) and run the pass
+// epilogue:
 //   pass 1: neighbour counts of rows and columns (and neighbour lists),
 //   pass 2: unions of core-core neighbour pairs.
 // Every mbarrier wait is bounded in time; a wait that runs out sets an error
@@ -300,6 +301,24 @@ __device__ __forceinline__ uint32_t sign_bits(const float (&u)[32], float mid, f
     return bits;
 }
 
+// The smallest |u_i - mid| alone.
+__device__ __forceinline__ float nearest_of(const float (&u)[32], float mid)
+{
+    unsigned long long m;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(m) : "f"(-mid));
+    float near = INFINITY;
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+        unsigned long long x;
+        float t0, t1;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(u[i]), "f"(u[i + 1]));
+        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(m));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(x));
+        near = fmin3(near, fabsf(t0), fabsf(t1));
+    }
+    return near;
+}
+
 // in (u >= k_in) and kept (u >= k_out) bits of a row's 32 screen values. The
 // three-product band is narrow, so most rows have no value in it: with mid
 // between the limits and hb >= k_in - mid, mid - k_out (rounded up),
@@ -323,6 +342,14 @@ __device__ __forceinline__ void limit_bits(const float (&u)[32], float k_in, flo
             if (u[i] >= k_out) keep_bits |= 1u << i;
         }
     }
+}
+
+// Whether a row's 32 values all lie outside the band, as limit_bits proves it.
+__device__ __forceinline__ bool no_band(const float (&u)[32], float k_in, float k_out)
+{
+    const float mid = 0.5f * k_in + 0.5f * k_out;
+    const float hb = fmaxf(__fsub_ru(k_in, mid), __fsub_ru(mid, k_out));
+    return nearest_of(u, mid) > hb && k_in < INFINITY;
 }
 
 __device__ __forceinline__ float fmax3(float a, float b, float c)
@@ -431,6 +458,25 @@ __device__ __forceinline__ bool push_band(const TcParams& P, int ra, int rb, uin
     return d2 <= A.eps2;
 }
 
+// A band pair that found the queue full after its block was counted: decided by
+// the defining expression and counted (and listed) for its rows.
+__device__ __noinline__ void band_here(const TcParams& P, uint2 e)
+{
+    const PassArgs& A = P.A;
+    const int ra = (int)e.x, rb = (int)(e.y & 0x3fffffffu);
+    const uint32_t flags = e.y >> 30;
+    const double d2 = exact_sqdist(pass_row(A, ra), pass_row(A, rb), A.d);
+    atomicAdd(&A.stats[kStatBand], 1ull);
+    if ((flags & kQTie) && fabs(d2 - A.eps2) <= A.tie_thr) atomicAdd(&A.stats[kStatTies], 1ull);
+    if (!(d2 <= A.eps2)) return;
+    const int pa = atomicAdd(&A.count[ra], 1);
+    if (pa < A.cap) A.nbr[(int64_t)ra * A.cap + pa] = rb;
+    if (flags & kQBoth) {
+        const int pb = atomicAdd(&A.count[rb], 1);
+        if (pb < A.cap) A.nbr[(int64_t)rb * A.cap + pb] = ra;
+    }
+}
+
 // The same for radius e of a count pass over several radii.
 __device__ __forceinline__ bool push_band_radius(const TcParams& P, uint2* queue, unsigned long long* queue_n,
                                                  unsigned long long* stats, double eps2, double tie_thr, int ra,
@@ -454,8 +500,11 @@ __device__ __forceinline__ bool push_band_radius(const TcParams& P, uint2* queue
 // Per-pair epilogue data is double-buffered (index: pair counter & 1): a
 // pair's buffer is written before the barrier that follows the accumulator
 // wait and read after it, so the next pair can be staged meanwhile.
+constexpr int kMaxSlots = 6;
+constexpr int kBandList = 32;                 // band pairs that a warp of the count pass collects
+constexpr int kRunLog = 4, kRunMax = 1 << kRunLog;   // count pass: most items of a run
 struct SmemTail {
-    uint64_t full[4], empty[4], acc_full[4], acc_empty[4], fin;
+    uint64_t full[kMaxSlots], empty[kMaxSlots], acc_full[4], acc_empty[4], fin;
     uint32_t tmem_base;
     int abort;
     int consumed;                              // stage fills consumed by the MMA warp
@@ -467,6 +516,7 @@ struct SmemTail {
     __align__(16) float wn[kEpiWarps][kT];     // count pass: -|b|^2 of the columns of each warp's pair
                                                // (k-distance pass: of its 32 columns)
     int pre[kEpiWarps][kT];                    // count pass: the columns' counts before the pair
+    uint2 band[kEpiWarps][kBandList];          // count pass: each warp's band pairs on their way to the queue
     uint32_t colmask[4][kT];                   // union pass: neighbour bits per column (by row quadrant)
     uint32_t rowmask[kT / 32][kT];             // neighbour bits per row (by 32-column chunk)
     int par[2][2 * kT];                        // union pass: local union-find / component
@@ -582,6 +632,10 @@ struct TcShape {
     static constexpr int kStages = W == 1 ? (NS == 1 ? 4 : 3) : (NS == 1 ? 4 : 2);
     static constexpr int kStageBytes = kOps * kBlk;
     static constexpr int kAccCols = W * kT;               // TMEM columns of one accumulator
+    // count pass, W = 1, NS = 3: slots of one K block of one tile (hi, lo), A's and B's apart
+    static constexpr int kSlots = 6;
+    static constexpr int kSlotBytes = 2 * kBlk;
+    static_assert(kStages <= kMaxSlots && kSlots <= kMaxSlots, "barriers");
 };
 
 // W = 1: one tile pair per work item. W = 2: a group of one or two tile
@@ -600,12 +654,24 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     // accumulators in TMEM: the count pass takes all 512 columns (its epilogue
     // works on up to four pairs at a time), the others two
     constexpr int kBufs = kCountPass ? 512 / kAccCols : 2;
+    // Operand slots of their own for A and B (count pass, W = 1, three products):
+    // the pairs of a run mostly share tile A, whose K blocks stay in their slots
+    // while only B streams. [0, a_slots) A, the rest B. A whole tile of A is kept
+    // if that leaves three slots for B (up to 192 columns), with a slot to load
+    // the next run's ahead where there is room; wider rows stream both (at 256
+    // columns A kept beside two slots for B took 1.99 ms where streaming both
+    // takes 1.81). Four radii on 200k x 128: 13.2 -> 12.3 ms with A kept.
+    constexpr bool kSplit = kCountPass && W == 1 && NS == 3;
+    constexpr int kSlots = TcShape<NS, W>::kSlots, kSlotBytes = TcShape<NS, W>::kSlotBytes;
+    const bool keep_a = P.nkb <= kSlots - 3;
+    const int a_slots = keep_a ? min(P.nkb + 1, kSlots / 2) : kSlots / 2;
+    const int b_slots = kSlots - a_slots;
     const int64_t n_cap = W == 1 ? P.n_pairs : P.n_groups;
     const int64_t n_items = MODE == 3 ? 0 : (P.n_dev ? min(n_cap, (int64_t)*P.n_dev) : n_cap);
     auto group_at = [&](int64_t g) -> int2 { return W == 1 ? make_int2((int)g, -1) : P.groups[g]; };
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    SmemTail& S = *reinterpret_cast<SmemTail*>(smem + kStages * kStageBytes);
+    SmemTail& S = *reinterpret_cast<SmemTail*>(smem + (kSplit ? kSlots * kSlotBytes : kStages * kStageBytes));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const PassArgs& A = P.A;
     volatile int* abort = &S.abort;
@@ -617,19 +683,27 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
     const int64_t g_begin = MODE == 3 ? 0 : blockIdx.x;
     const int64_t g_step = MODE == 3 ? 1 : gridDim.x;
     const int64_t g_end = MODE == 3 ? (kq_bhi > kq_ch * P.kq_ct ? (kq_bhi - kq_ch * P.kq_ct + 1) / 2 : 0) : n_items;
-    // the k-th work item of this CTA. Count pass: runs of kRun consecutive
+    // the k-th work item of this CTA. Count pass: runs of 2^run consecutive
     // items (consecutive groups of the list mostly share tile A, whose blocks
-    // then stay in the stages), the CTAs' runs interleaved so that the CTAs
-    // working at one time stay close in the list (tiles shared through L2)
-    constexpr int kRun = kCountPass ? 4 : 1;
+    // then stay in shared memory), the CTAs' runs interleaved so that the CTAs
+    // working at one time stay close in the list (tiles shared through L2).
+    // At least 16 runs a CTA where there are as many items, so that the last
+    // ones leave few CTAs idle (runs of four everywhere left most CTAs without
+    // work on a few hundred pairs).
+    int run = 0;
+    if constexpr (kCountPass) {
+        const int64_t per = n_items / ((int64_t)gridDim.x * 16);
+        run = per >= kRunMax ? kRunLog : per > 1 ? 31 - __clz((int)per) : 0;
+    }
     auto item_at = [&](int64_t k) -> int64_t {
         if (MODE == 3) return k;
-        return ((k / kRun) * (int64_t)gridDim.x + blockIdx.x) * kRun + (k % kRun);
+        if (!kCountPass) return blockIdx.x + k * (int64_t)gridDim.x;
+        return (((k >> run) * (int64_t)gridDim.x + blockIdx.x) << run) + (k & ((1 << run) - 1));
     };
     // item_at(k + 1) from g = item_at(k)
     auto next_item = [&](int64_t k, int64_t g) -> int64_t {
-        if (kRun == 1) return g + g_step;
-        return ((k + 1) % kRun) ? g + 1 : g + ((int64_t)gridDim.x - 1) * kRun + 1;
+        if (!kCountPass) return g + g_step;
+        return ((k + 1) & ((1 << run) - 1)) ? g + 1 : g + (((int64_t)gridDim.x - 1) << run) + 1;
     };
     // tiles of item g: (A, B0, B1 or -1)
     auto item = [&](int64_t g) -> int3 {
@@ -650,7 +724,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 32) {
-        for (int i = 0; i < kStages; ++i) {
+        for (int i = 0; i < (kSplit ? kSlots : kStages); ++i) {
             mbar_init(&S.full[i], 1);
             mbar_init(&S.empty[i], 1);
         }
@@ -670,7 +744,52 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 
     if (warp == 0) {
         // ---------------------------------------------------- TMA producer
-        if (lane == 0) {
+        if constexpr (kSplit) {
+            if (lane == 0) {
+                int fa = 0, fb = 0;                                 // fills issued (A, B)
+                int sa = 0, sb = 0;                                 // the next fill's slot
+                uint32_t pa = 0, pb = 0;                            // and its parity
+                int held = -1;                                      // the tile in A's slots
+                for (int64_t k = 0, g = item_at(0); g < g_end && !*abort; g = next_item(k, g), ++k) {
+                    const int3 itm = item(g);
+                    const bool load_a = !(keep_a && itm.x == held), load_b = itm.x != itm.y;
+                    held = itm.x;
+                    for (int kb = 0; kb < P.nkb; ++kb) {
+                        if (load_a) {
+                            if (!mbar_wait(&S.empty[sa], pa ^ 1, abort)) break;
+                            unsigned char* st = smem + sa * kSlotBytes;
+                            mbar_expect_tx(&S.full[sa], (uint32_t)kSlotBytes);
+                            tma_load(st, &mAh, kb * kKB, itm.x * kT, &S.full[sa]);
+                            if (NS == 3) tma_load(st + kBlk, &mAl, kb * kKB, itm.x * kT, &S.full[sa]);
+                            ++fa;
+                            if (++sa == a_slots) { sa = 0; pa ^= 1; }
+                        }
+                        if (load_b) {
+                            const int slot = a_slots + sb;
+                            if (!mbar_wait(&S.empty[slot], pb ^ 1, abort)) break;
+                            unsigned char* st = smem + slot * kSlotBytes;
+                            mbar_expect_tx(&S.full[slot], (uint32_t)kSlotBytes);
+                            tma_load(st, &mAh, kb * kKB, itm.y * kT, &S.full[slot]);
+                            if (NS == 3) tma_load(st + kBlk, &mAl, kb * kKB, itm.y * kT, &S.full[slot]);
+                            ++fb;
+                            if (++sb == b_slots) { sb = 0; pb ^= 1; }
+                        }
+                    }
+                }
+                // on abort: let the copies already issued land before the CTA
+                // exits (a slot's last fill; those before it were consumed)
+                if (*abort) {
+                    volatile int dummy = 0;
+                    for (int i = 0; i < kSlots; ++i) {
+                        const int n = i < a_slots ? a_slots : b_slots, fills = i < a_slots ? fa : fb;
+                        const int at = i < a_slots ? i : i - a_slots;
+                        if (fills <= at) continue;
+                        const int last = fills - 1 - (fills - 1 - at) % n;
+                        mbar_wait(&S.full[i], (uint32_t)((last / n) & 1), &dummy);
+                    }
+                }
+            }
+        } else if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
             int issued = 0;
@@ -680,7 +799,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
 #pragma unroll
             for (int i = 0; i < (kCountPass ? kStages : 1); ++i) tag[i] = -1;
             constexpr int nA = NS == 3 ? 2 : 1;                 // A blocks per stage (hi, lo)
-            for (int64_t k = 0, g = kRun == 1 ? g_begin : item_at(0); g < g_end && !*abort; g = next_item(k, g), ++k) {
+            for (int64_t k = 0, g = kCountPass ? item_at(0) : g_begin; g < g_end && !*abort; g = next_item(k, g), ++k) {
                 const int3 itm = item(g);
                 const int2 tp = make_int2(itm.x, itm.y);
                 const bool diag = W == 1 && tp.x == tp.y;
@@ -735,11 +854,76 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         }
     } else if (warp == 1) {
         // ---------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        if constexpr (kSplit) {
+            if (lane == 0) {
+                constexpr uint32_t idesc = F ? kIdescF8 : kIdesc;
+                int a0 = 0, sb = 0;                                 // slots of the run's first A block, of the next B
+                uint32_t a0p = 0, pb = 0;                           // their fills' parities
+                int it = 0;
+                int64_t g = item_at(0), g_next = 0;
+                int3 itm = g < g_end ? item(g) : make_int3(-1, -1, -1);
+                for (int64_t k = 0; g < g_end && !*abort; g = g_next, ++k, ++it) {
+                    g_next = next_item(k, g);
+                    const int3 next = g_next < g_end ? item(g_next) : make_int3(-1, -1, -1);
+                    const bool more = keep_a && next.x == itm.x;    // A's blocks stay
+                    const bool diag = itm.x == itm.y;
+                    const int buf = it % kBufs;
+                    const uint32_t acc_phase = (uint32_t)((it / kBufs) & 1);
+                    if (!mbar_wait(&S.acc_empty[buf], acc_phase ^ 1, abort)) break;
+                    tc_fence_after();
+                    const uint32_t d_tmem = tmem + (uint32_t)(buf * kAccCols);
+                    int sa = a0;
+                    uint32_t pa = a0p;
+                    bool ok = true;
+                    for (int kb = 0; kb < P.nkb; ++kb) {
+                        const int slot_b = a_slots + sb;
+                        if (!mbar_wait(&S.full[sa], pa, abort)) { ok = false; break; }
+                        if (!diag && !mbar_wait(&S.full[slot_b], pb, abort)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t ah = su32(smem + sa * kSlotBytes), al = ah + kBlk;
+                        const uint32_t bh = diag ? ah : su32(smem + slot_b * kSlotBytes), bl = bh + kBlk;
+#pragma unroll
+                        for (int j = 0; j < kKB / 16; ++j) {
+                            const uint32_t acc0 = (kb | j) ? 1u : 0u;
+                            if constexpr (F) {
+                                mma_f8_id(d_tmem, smem_desc(ah + 32 * j), smem_desc(bh + 32 * j), idesc, acc0);
+                                if (NS == 3) {
+                                    mma_f8_id(d_tmem, smem_desc(ah + 32 * j), smem_desc(bl + 32 * j), idesc, 1u);
+                                    mma_f8_id(d_tmem, smem_desc(al + 32 * j), smem_desc(bh + 32 * j), idesc, 1u);
+                                }
+                            } else {
+                                mma_bf16_id(d_tmem, smem_desc(ah + 32 * j), smem_desc(bh + 32 * j), idesc, acc0);
+                                if (NS == 3) {
+                                    mma_bf16_id(d_tmem, smem_desc(ah + 32 * j), smem_desc(bl + 32 * j), idesc, 1u);
+                                    mma_bf16_id(d_tmem, smem_desc(al + 32 * j), smem_desc(bh + 32 * j), idesc, 1u);
+                                }
+                            }
+                        }
+                        if (!more) mma_commit(&S.empty[sa]);
+                        if (++sa == a_slots) { sa = 0; pa ^= 1; }
+                        if (!diag) {
+                            mma_commit(&S.empty[slot_b]);
+                            if (++sb == b_slots) { sb = 0; pb ^= 1; }
+                        }
+                    }
+                    if (!ok) break;
+                    mma_commit(&S.acc_full[buf]);
+                    if (!more) {
+                        a0 = sa;
+                        a0p = pa;
+                    }
+                    itm = next;
+                }
+                // all MMAs issued by this thread have completed once `fin` flips
+                mma_commit(&S.fin);
+                volatile int dummy = 0;
+                mbar_wait(&S.fin, 0, &dummy);
+            }
+        } else if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
-            for (int64_t k = 0, g = kRun == 1 ? g_begin : item_at(0); g < g_end && !*abort;
+            for (int64_t k = 0, g = kCountPass ? item_at(0) : g_begin; g < g_end && !*abort;
                  g = next_item(k, g), ++k, ++it) {
                 const int3 itm = item(g);
                 const bool diag = W == 1 && itm.x == itm.y;
@@ -929,9 +1113,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         // The chain of one pair (its loads, the accumulator, the counts' atomics)
         // is long beside the pair's MMAs, so four pairs in flight hide it, and a
         // pair's row data are loaded by one warp a quadrant, not by four.
-        // Count pass of the 500k x 128 2D graph 16.6 -> 13.9 ms (all 16 warps on
-        // one pair before), of four radii on 200k x 128 14.2 -> 13.2, of 1M x 256
-        // (straight and first phase) 4.2 -> 3.7.
         // Per 32 x 32 block: screen values u = fl(2 acc - |b|^2) against per-row
         // limits (all out / all in at once from the row's extremes), then the row
         // counts (and lists) from the lane's bits and the column counts from
@@ -940,6 +1121,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         // the three-product pass. Each item's group and tile pairs are loaded
         // while the previous item is processed, its row and column data before
         // the accumulator wait.
+        // What the counts are for is the core flag (count >= minPts) and the lists
+        // of rows below it, so a row or column whose count, read before the item,
+        // has reached PassArgs::need is not counted any more (counts only grow):
+        // most rows of a cluster are done after a few pairs, and their blocks need
+        // neither transpose nor atomics, only the check for band pairs.
+        // At 500k x 128 (every block mixed, 1.165 M pairs; the MMAs alone take 6.9
+        // ms at N = 256 and 11.5 at N = 128, whose operands fill the shared-memory
+        // bandwidth): all 16 warps on one pair 16.6 ms, a group a pair 13.3; blocks
+        // after a mixed one taken as mixed and bytes transposed by permutes 12.8;
+        // band pairs collected (a slot taken per block was a returning atomic that
+        // the warp waited for) 12.3; finished counts left out 10.2. Four radii on
+        // 200k x 128 14.2 -> 13.2 -> 9.8; 1M x 256 (straight and first phase) 2.9
+        // -> 2.6.
         const int ew = warp - 2;                              // 0 .. 15
         const int quad = warp & 3;
         const int group = ew >> 2;
@@ -963,10 +1157,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         // pair while tile A stays the same: the CTAs work on neighbouring pairs,
         // so they all add to the same few tiles' rows, and one atomic per block
         // would serialise there
+        bool was_mixed = false;                               // the warp's last block
         int row_add = 0, ta_sum = -1;
         auto flush_rows = [&]() {
             if (row_add) atomicAdd(&A.count[(int64_t)ta_sum * kT + r], row_add);
             row_add = 0;
+        };
+        // The band pairs go to the queue kBandList at a time: a slot taken for each
+        // block that holds one is a returning atomic that the warp waits for.
+        int n_band = 0;
+        auto band_any = [&](uint32_t band) { return MODE == 1 && __any_sync(0xffffffffu, band != 0u); };
+        auto flush_band = [&]() {
+            if (n_band == 0) return;
+            unsigned long long at = 0ull;
+            if (lane == 0) at = atomicAdd(P.queue_n, (unsigned long long)n_band);
+            at = __shfl_sync(0xffffffffu, at, 0) + lane;
+            __syncwarp();
+            if (lane < n_band) {
+                const uint2 e = S.band[ew][lane];
+                if (at < P.queue_cap) P.queue[at] = e;
+                else band_here(P, e);
+            }
+            __syncwarp();
+            n_band = 0;
         };
         Head head;
         int64_t g = item_of(0), g_next = 0;
@@ -994,6 +1207,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 ta_sum = ta;
             }
             int na = 0, nb = 0, pre_row = 0;
+            // counts that are known to be large enough (PassArgs::need): of all the
+            // warp's rows, of all columns of a part (MODE 5: a bit per radius)
+            uint32_t rows_done = 0u, cols_done = 0u;
             float na2 = 0.f, bmin2 = 0.f, E = 0.f, two = 2.f;
             float4 tm = make_float4(0.f, 0.f, 0.f, 0.f);
             if (mine) {
@@ -1005,28 +1221,33 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 bmin2 = P.tn2min[tb];
                 float nc[4];
                 int pc[4];
+                cols_done = 0u;
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const int64_t col = sb + p * 32 + lane;
                     nc[p] = -P.rn2[col];
                     if constexpr (MODE == 5) {
-                        // bit e: radius e's list of this column is full (its count can only grow)
-                        int full = A.cap > 0 ? 0 : 0xF;
+                        // bit e: this column's count at radius e is done (it can only grow)
+                        int done = diag || p * 32 + lane >= nb ? 0xF : 0;
 #pragma unroll
                         for (int e = 0; e < kMaxRadii; ++e)
-                            if (A.cap > 0 && !diag && e < P.n_rad && P.rad[e].count[col] >= A.cap) full |= 1 << e;
-                        pc[p] = full;
+                            if (!diag && e < P.n_rad && P.rad[e].count[col] >= A.need) done |= 1 << e;
+                        pc[p] = done;
+                        cols_done |= __reduce_and_sync(0xffffffffu, (uint32_t)done) << (4 * p);
                     } else {
-                        pc[p] = A.cap > 0 && !diag ? A.count[col] : INT_MAX;
+                        pc[p] = diag || p * 32 + lane >= nb ? INT_MAX : A.count[col];
+                        if (__all_sync(0xffffffffu, pc[p] >= A.need)) cols_done |= 1u << p;
                     }
                 }
                 if constexpr (MODE == 5) {
-                    pre_row = A.cap > 0 ? 0 : 0xF;
+                    pre_row = r >= na ? 0xF : 0;
 #pragma unroll
                     for (int e = 0; e < kMaxRadii; ++e)
-                        if (A.cap > 0 && e < P.n_rad && P.rad[e].count[row] >= A.cap) pre_row |= 1 << e;
+                        if (e < P.n_rad && P.rad[e].count[row] >= A.need) pre_row |= 1 << e;
+                    rows_done = __reduce_and_sync(0xffffffffu, (uint32_t)pre_row);
                 } else {
-                    pre_row = A.cap > 0 ? A.count[row] : INT_MAX;
+                    pre_row = r >= na ? INT_MAX : A.count[row] + row_add;
+                    rows_done = __all_sync(0xffffffffu, pre_row >= A.need) ? 1u : 0u;
                 }
                 // the error bound of the row against the tile's largest norms
                 if (P.rl) {
@@ -1061,13 +1282,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             const bool pad = r >= na;                         // padding rows hold no pair
             uint32_t deferred = 0u;                           // parts left to the three-product pass
             bool hit_pair = false;
+            uint32_t hit_rad = 0u;                            // MODE 5: the radii whose pair is flagged
+            uint32_t todo = mine;
 #pragma unroll 1
-            for (int part = 0; part < 4; ++part) {
-                if (!((mine >> part) & 1u)) continue;
+            while (todo) {
+                const int part = __ffs(todo) - 1;
+                todo &= todo - 1u;
                 float u[32];
                 tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) +
                               (uint32_t)(first * kAccCols + h * kT + part * 32), u);
-                if ((mine >> part) == 1u) {                   // the last part read: the accumulator is free
+                if (!todo) {                   // the last part read: the accumulator is free
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&S.acc_empty[first]);
@@ -1077,11 +1301,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 // |b_j|^2 (exact), max x <= RU(two max acc - min |b|^2) and min x >=
                 // RD(two min acc - max |b|^2); x < k_out certifies out and x >= k_in in
                 // (E covers the rounding of the computed screen value too)
-                float vmax = fmax3(u[0], u[1], u[2]);
+                auto row_max = [&]() {
+                    float vmax = fmax3(u[0], u[1], u[2]);
 #pragma unroll
-                for (int i = 3; i + 1 < 32; i += 2) vmax = fmax3(vmax, u[i], u[i + 1]);
-                vmax = fmaxf(vmax, u[31]);
-                const float xmax = __fmaf_ru(two, vmax, -bmin2);
+                    for (int i = 3; i + 1 < 32; i += 2) vmax = fmax3(vmax, u[i], u[i + 1]);
+                    return __fmaf_ru(two, fmaxf(vmax, u[31]), -bmin2);
+                };
                 const int left = nb - part * 32;
                 const uint32_t cand = pad ? 0u : (left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u));
                 // u = fl(two acc - |b|^2) (two = 2, or 2 s_a s_b for FP8), two
@@ -1114,12 +1339,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 };
                 // lane j of the result: the rows of the block whose bit j is set
                 auto transpose = [&](uint32_t x) {
+                    uint32_t y = __shfl_xor_sync(0xffffffffu, x, 16);
+                    x = __byte_perm(x, y, (lane & 16) ? 0x3276u : 0x5410u);
+                    y = __shfl_xor_sync(0xffffffffu, x, 8);
+                    x = __byte_perm(x, y, (lane & 8) ? 0x3715u : 0x6240u);
 #pragma unroll
-                    for (int sft = 16; sft >= 1; sft >>= 1) {
-                        const uint32_t m = sft == 16 ? 0x0000FFFFu : sft == 8 ? 0x00FF00FFu : sft == 4 ? 0x0F0F0F0Fu
-                                                               : sft == 2 ? 0x33333333u : 0x55555555u;
-                        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sft);
-                        x = (lane & sft) ? (((y >> sft) & m) | (x & ~m)) : ((x & m) | ((y & m) << sft));
+                    for (int sft = 4; sft >= 1; sft >>= 1) {
+                        // keep the bits of m (of ~m in the upper lane), take the
+                        // others from the partner, rotated into place
+                        const uint32_t m = sft == 4 ? 0x0F0F0F0Fu : sft == 2 ? 0x33333333u : 0x55555555u;
+                        const uint32_t keep = (lane & sft) ? ~m : m;
+                        y = __shfl_xor_sync(0xffffffffu, x, sft);
+                        y = __funnelshift_l(y, y, (lane & sft) ? 32 - sft : sft);
+                        x = (x & keep) | (y & ~keep);
                     }
                     return x;
                 };
@@ -1143,6 +1375,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     // out at every smaller one; the screen values are formed
                     // once and compared with each radius's limits.
                     const int nr = P.n_rad;
+                    const float xmax = row_max();
                     auto k_in_of = [&](float lo) { return __fadd_ru(__fsub_ru(na2, lo), E); };
                     auto k_out_of = [&](float hi) { return __fsub_rd(__fsub_rd(na2, hi), E); };
                     int e_lo = nr;                            // radii e_lo .. nr - 1 hold a row not all out
@@ -1198,10 +1431,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     for (int e = e_lo; e < nr; ++e) {
                         int32_t* const cnt = P.rad[e].count;
                         int32_t* const nbl = P.rad[e].nbr;
+                        const bool done = ((rows_done & (cols_done >> (4 * part))) >> e) & 1u;
+                        if (NS == 3 && !F && done && ((hit_rad >> e) & 1u) && left >= 32) {
+                            // nothing to count, and the pair is flagged: only a band pair matters
+                            const float k_in = k_in_of(P.rad[e].eps2_lo), k_out = k_out_of(P.rad[e].eps2_hi);
+                            const bool sure = pad || xmax < k_out || xmin >= k_in || no_band(u, k_in, k_out);
+                            if (__all_sync(0xffffffffu, sure)) continue;
+                        }
                         uint32_t inb, band;
                         bits_of(P.rad[e].eps2_lo, P.rad[e].eps2_hi, inb, band);
                         if (!__any_sync(0xffffffffu, (inb | band) != 0u)) continue;
-                        if (lane == 0 && P.rad[e].pair_hit) P.rad[e].pair_hit[q] = 1;
+                        if (!((hit_rad >> e) & 1u) && lane == 0 && P.rad[e].pair_hit) P.rad[e].pair_hit[q] = 1;
+                        hit_rad |= 1u << e;
                         uint32_t bq = band;
                         while (bq) {
                             const int i = __ffs(bq) - 1;
@@ -1214,17 +1455,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                                                              fl, &decided);
                             if (decided && in) inb |= 1u << i;
                         }
-                        // counts, and list entries while the list has room (read
-                        // before the item: a full list takes no returning atomic)
-                        if (inb) {
-                            if ((pre_row >> e) & 1) atomicAdd(&cnt[row], __popc(inb));
-                            else if (add_listed(cnt, nbl, row, inb, sb + part * 32) >= A.cap) pre_row |= 1 << e;
+                        // counts and list entries of the rows and columns whose
+                        // counts are not done
+                        if (inb && !((pre_row >> e) & 1)) {
+                            if (add_listed(cnt, nbl, row, inb, sb + part * 32) >= A.need) pre_row |= 1 << e;
                         }
-                        if (!diag && __any_sync(0xffffffffu, inb != 0u)) {
-                            const uint32_t x = transpose(inb);
-                            if (x) {
-                                if ((pre[part * 32 + lane] >> e) & 1) atomicAdd(&cnt[col], __popc(x));
-                                else add_listed(cnt, nbl, col, x, sa + quad * 32);
+                        if (!((cols_done >> (4 * part + e)) & 1u)) {
+                            const uint32_t open = inb & __ballot_sync(0xffffffffu, !((pre[part * 32 + lane] >> e) & 1));
+                            if (__any_sync(0xffffffffu, open != 0u)) {
+                                const uint32_t x = transpose(open);
+                                if (x) add_listed(cnt, nbl, col, x, sa + quad * 32);
                             }
                         }
                     }
@@ -1232,23 +1472,42 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 }
                 const float k_in = __fadd_ru(__fsub_ru(na2, P.eps2_lo), E);
                 const float k_out = __fsub_rd(__fsub_rd(na2, P.eps2_hi), E);
-                const bool all_out = pad || xmax < k_out;
-                if (__all_sync(0xffffffffu, all_out)) continue;   // nothing in, no band: nothing to do
-                const bool all_in = !all_out && row_min() >= k_in;
-                const bool mixed = !all_out && !all_in;
-                const bool any_mixed = __any_sync(0xffffffffu, mixed);
-                // first phase, extremes only: a block with a row neither all in
-                // nor all out is deferred without looking at its values
-                if (P.defer == 2 && any_mixed) {
-                    deferred |= 1u << part;
-                    continue;
+                // After a mixed block most blocks of a run are mixed too, and the
+                // extremes would only cost their 32 instructions (the first
+                // phase's rule needs them).
+                const bool assume = NS == 3 && !F && P.defer == 0 && was_mixed;
+                const bool cols_open = !((cols_done >> part) & 1u);
+                bool formed = false;                          // u holds the screen values
+                // nothing to count, and the pair is flagged: only a band pair matters
+                if (assume && rows_done && !cols_open && hit_pair && left >= 32) {
+                    screen_values();
+                    if (__all_sync(0xffffffffu, pad || no_band(u, k_in, k_out))) continue;
+                    formed = true;
+                }
+                bool all_in = false, mixed = !pad;
+                if (!assume) {
+                    const bool all_out = pad || row_max() < k_out;
+                    if (__all_sync(0xffffffffu, all_out)) continue;   // nothing in, no band: nothing to do
+                    all_in = !all_out && row_min() >= k_in;
+                    mixed = !all_out && !all_in;
+                    was_mixed = __any_sync(0xffffffffu, mixed);
+                    // first phase, extremes only: a block with a row neither all in
+                    // nor all out is deferred without looking at its values
+                    if (P.defer == 2 && was_mixed) {
+                        deferred |= 1u << part;
+                        continue;
+                    }
                 }
                 uint32_t in_bits = 0u, keep_bits = 0u;
                 if (all_in) {
                     in_bits = keep_bits = 0xffffffffu;
                 } else if (mixed) {
-                    screen_values();
+                    if (!formed) screen_values();
                     compare(k_in, k_out, in_bits, keep_bits);
+                }
+                if (assume) {
+                    was_mixed = __any_sync(0xffffffffu, (in_bits != 0u && in_bits != 0xffffffffu) || keep_bits != in_bits);
+                    if (!__any_sync(0xffffffffu, keep_bits != 0u)) continue;
                 }
                 uint32_t inb = in_bits & cand;
                 const uint32_t band = keep_bits & ~in_bits & cand;
@@ -1256,9 +1515,31 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     deferred |= 1u << part;
                     continue;
                 }
-                hit_pair |= (inb | band) != 0u;
+                hit_pair |= __any_sync(0xffffffffu, (inb | band) != 0u);
                 // band pairs: queued for the FP64 recheck; decided here if the queue is full
                 uint32_t bq = band;
+                if (band_any(band)) {
+                    const int n = __popc(band);
+                    int at = n;                                // inclusive prefix over the lanes
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, at, o);
+                        if (lane >= o) at += y;
+                    }
+                    const int total = __shfl_sync(0xffffffffu, at, 31);
+                    if (n_band + total > kBandList) flush_band();
+                    if (n_band + total <= kBandList) {
+                        at += n_band - n;
+                        while (bq) {
+                            const int i = __ffs(bq) - 1;
+                            bq &= bq - 1;
+                            const int c = part * 32 + i;
+                            const uint32_t fl = (diag ? 0u : kQBoth) | ((!diag || r < c) ? kQTie : 0u);
+                            S.band[ew][at++] = make_uint2((uint32_t)row, (uint32_t)(sb + c) | (fl << 30));
+                        }
+                        n_band += total;
+                    }
+                }
                 while (bq) {
                     const int i = __ffs(bq) - 1;
                     bq &= bq - 1;
@@ -1269,16 +1550,20 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     if (decided && in) inb |= 1u << i;
                 }
                 // row counts (and the first cap neighbours of each row)
-                if (inb) {
+                if (inb && pre_row < A.need) {
                     if (pre_row < A.cap) pre_row = add_listed(A.count, A.nbr, row, inb, sb + part * 32);
                     else row_add += __popc(inb);
                 }
                 // column counts: lane j gets column part * 32 + j
-                if (!diag && __any_sync(0xffffffffu, inb != 0u)) {
-                    const uint32_t x = transpose(inb);
-                    if (x) {
-                        if (pre[part * 32 + lane] < A.cap) add_listed(A.count, A.nbr, col, x, sa + quad * 32);
-                        else atomicAdd(&A.count[col], __popc(x));
+                if (cols_open) {
+                    const int had = pre[part * 32 + lane];
+                    const uint32_t open = inb & __ballot_sync(0xffffffffu, had < A.need);
+                    if (__any_sync(0xffffffffu, open != 0u)) {
+                        const uint32_t x = transpose(open);
+                        if (x) {
+                            if (had < A.cap) add_listed(A.count, A.nbr, col, x, sa + quad * 32);
+                            else atomicAdd(&A.count[col], __popc(x));
+                        }
                     }
                 }
             }
@@ -1287,7 +1572,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 if (lane == 0) mbar_arrive(&S.acc_empty[first]);
             }
             if (MODE == 1) {
-                if (A.pair_hit && __any_sync(0xffffffffu, hit_pair) && lane == 0) A.pair_hit[q] = 1;
+                if (A.pair_hit && hit_pair && lane == 0) A.pair_hit[q] = 1;
             }
             if (deferred && lane == 0) {
                 // first phase: these blocks go to the three-product pass, whole
@@ -1301,7 +1586,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 }
             }
         }
-        if (MODE == 1) flush_rows();
+        if (MODE == 1) {
+            flush_rows();
+            flush_band();
+        }
         if (screened) {
             atomicAdd(&A.stats[kStatScreened], (unsigned long long)screened);
             atomicAdd(&A.stats[kStatTcPairs], (unsigned long long)screened);
@@ -1980,18 +2268,21 @@ bool make_map(CUtensorMap* m, const void* ptr, int64_t rows, int dp, int box_row
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NS, int W>
+template <int NS, int MODE, int W>
 constexpr int smem_bytes()
 {
-    return TcShape<NS, W>::kStages * TcShape<NS, W>::kStageBytes + (int)sizeof(SmemTail) + 1024;
+    using T = TcShape<NS, W>;
+    const bool split = (MODE == 1 || MODE == 5) && W == 1 && NS == 3;
+    return (split ? T::kSlots * T::kSlotBytes : T::kStages * T::kStageBytes) + (int)sizeof(SmemTail) + 1024;
 }
-static_assert(smem_bytes<3, 1>() <= 232448 && smem_bytes<1, 1>() <= 232448, "shared memory");
-static_assert(smem_bytes<3, 2>() <= 232448 && smem_bytes<1, 2>() <= 232448, "shared memory");
+static_assert(smem_bytes<3, 1, 1>() <= 232448 && smem_bytes<1, 1, 1>() <= 232448, "shared memory");
+static_assert(smem_bytes<3, 2, 1>() <= 232448 && smem_bytes<1, 2, 1>() <= 232448, "shared memory");
+static_assert(smem_bytes<3, 1, 2>() <= 232448 && smem_bytes<1, 1, 2>() <= 232448, "shared memory");
 
 template <int NS, int MODE, int W, int F = 0>
 cudaError_t launch(const CUtensorMap& mh, const CUtensorMap& ml, const TcParams& p, int grid, cudaStream_t s)
 {
-    const int smem = smem_bytes<NS, W>();
+    const int smem = smem_bytes<NS, MODE, W>();
     cudaError_t e =
         cudaFuncSetAttribute(tc_kernel<NS, MODE, W, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

@@ -86,3 +86,58 @@ def test_eccentricity_rejects_non_finite_values(ctx, bad, d):
     X[331, d // 2] = bad
     with pytest.raises(mg.MapperError):
         mg.mapper_lens(ctx, _device(X), (mg.LENS_ECC,), (0,))
+
+
+def _graph(ctx, Xd, nint, ov, eps, min_pts, prec):
+    g = mg.mapper_graph(ctx, Xd, mg.params((mg.LENS_COORD,), (0,), (nint,), (ov,), eps, min_pts, prec))
+    return g.numpy(), g.stats()
+
+
+# counts stop at minPts once they are known to reach it; lists hold up to 64
+@pytest.mark.parametrize("min_pts", [1, 2, 64, 65, 66, 300])
+@pytest.mark.parametrize("tile_n", [128, 256])
+def test_core_flags_at_the_limits_of_the_counts(min_pts, tile_n):
+    rng = np.random.default_rng(min_pts)
+    c = rng.standard_normal((5, 24)) * 4
+    X = (c[rng.integers(0, 5, 3000)] + rng.standard_normal((3000, 24)) * rng.choice([0.3, 1.0], (3000, 1))).astype(np.float32)
+    with mg.Context(0) as ctx:
+        ctx.set_pass1_tile_n(tile_n)
+        g = mg.mapper_graph(ctx, _device(X), mg.params((mg.LENS_COORD,), (0,), (3,), (0.3,), 3.5, min_pts, mg.BF16))
+        got, core = g.numpy(), g.clusters().numpy(len(g.cover().numpy()[1]))[1]
+        lens, _ = g.lens(len(X), 1)
+    ref = oracle.mapper_graph(X, lens, (3,), (0.3,), 3.5, min_pts)
+    assert np.array_equal(core, ref["core"])
+    for k in ("node_offsets", "node_members", "node_elem", "edges"):
+        assert np.array_equal(np.asarray(got[k]), np.asarray(ref[k])), k
+
+
+# every squared distance is an integer and eps^2 is one of them: whole blocks
+# of band pairs, and near ties that have to be counted
+def test_blocks_of_band_pairs(ctx):
+    X = np.random.default_rng(3).integers(0, 2, (2000, 16)).astype(np.float32)
+    got, st = _graph(ctx, _device(X), 2, 0.3, 2.0, 40, mg.BF16)
+    lens = X[:, :1].astype(np.float64)
+    ref = oracle.mapper_graph(X, lens, (2,), (0.3,), 2.0, 40)
+    assert st["near_ties"] == ref["near_ties"] > 0
+    for k in ("node_offsets", "node_members", "node_elem", "edges"):
+        assert np.array_equal(np.asarray(got[k]), np.asarray(ref[k])), k
+
+
+# columns in K blocks of 64: A's tile kept whole (1 to 3 blocks) or streamed
+@pytest.mark.parametrize("d", [40, 64, 100, 192, 250, 257, 400])
+@pytest.mark.parametrize("n", [1500, 14_000])
+def test_three_products_at_every_depth(d, n):
+    rng = np.random.default_rng(d)
+    c = rng.standard_normal((12, d)) * 0.6
+    X = (c[rng.integers(0, 12, n)] + rng.standard_normal((n, d))).astype(np.float32)
+    eps = float(np.sqrt(2.0 * d) * 0.98)
+    with mg.Context(0) as ctx:
+        Xd = _device(X)
+        ref, rs = _graph(ctx, Xd, 2, 0.2, eps, 10, mg.FP32)
+        for tile_n in (128, 256):
+            ctx.set_pass1_tile_n(tile_n)
+            ctx.set_pass1_screen(2)
+            got, st = _graph(ctx, Xd, 2, 0.2, eps, 10, mg.BF16)
+            assert st["n_core"] == rs["n_core"]
+            for k in ref:
+                assert np.array_equal(np.asarray(got[k]), np.asarray(ref[k])), (tile_n, k)
