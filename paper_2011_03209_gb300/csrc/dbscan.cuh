@@ -166,6 +166,8 @@ void fp32_thresholds(double eps2, int d, float* lo, float* hi);
 // --- screening passes (k_dbscan.cu)
 cudaError_t simt_pass(int mode, const PassArgs& a, int64_t n_pairs, cudaStream_t s);
 cudaError_t allin_pass(int mode, const PassArgs& a, int64_t n_pairs, cudaStream_t s);
+// mode 2 once the neighbour lists have joined most rows (tile_roots: scratch, [T])
+cudaError_t allin_unions(const PassArgs& a, int64_t n_pairs, int64_t T, int2* tile_roots, cudaStream_t s);
 cudaError_t core_flags(const int32_t* count, int64_t R, int32_t min_pts, uint8_t* core,
                        int32_t* parent, unsigned long long* border, unsigned long long* stats,
                        cudaStream_t s);

@@ -406,17 +406,18 @@ __global__ void __launch_bounds__(256) allin_kernel(const PassArgs A)
     const bool valid = side_b ? (!P.diag && x < P.nb) : x < P.na;
     const int64_t row = side_b ? P.sb + x : P.sa + x;
     if (MODE == 1) {
-        if (!valid) return;
+        if (tid == 0) {
+            const int64_t pairs = P.diag ? (int64_t)P.na * (P.na + 1) / 2 : (int64_t)P.na * P.nb;
+            atomicAdd(&A.stats[kStatScreened], (unsigned long long)pairs);
+        }
+        // (a count that is large enough already stays as it is: no returning atomic)
+        if (!valid || A.count[row] >= A.need) return;
         const int k = side_b ? P.na : (P.diag ? P.na : P.nb);
         const int old = atomicAdd(&A.count[row], k);
         if (A.cap > 0 && old < A.cap) {
             const int64_t other = side_b ? P.sa : (P.diag ? P.sa : P.sb);
             for (int i = 0; i < k && old + i < A.cap; ++i)
                 A.nbr[row * A.cap + old + i] = (int32_t)(other + i);
-        }
-        if (tid == 0) {
-            const int64_t pairs = P.diag ? (int64_t)P.na * (P.na + 1) / 2 : (int64_t)P.na * P.nb;
-            atomicAdd(&A.stats[kStatScreened], (unsigned long long)pairs);
         }
     } else if (MODE == 2) {
         if (!union_prologue(A, P, s_core, s_mm)) return;
@@ -693,6 +694,56 @@ __global__ void __launch_bounds__(256) select_round_kernel(const int2* __restric
     }
 }
 
+// The unions of all-in tile pairs after those along the neighbour lists, in two
+// launches: the diagonal pairs (a tile's rows join row by row, a warp a tile),
+// then, with the tiles' root ranges tr read again, the others, of which nearly
+// all are joined or have one root on each side: a union by one thread. A CTA per
+// pair that looked up all its rows' roots took 0.18 ms for 48 k pairs at 1M x 256,
+// these two launches and their tile roots 0.06.
+__global__ void __launch_bounds__(256) allin_unions_kernel(const PassArgs A, int64_t n, bool diagonal,
+                                                           const int2* __restrict__ tr)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    int2 p = make_int2(0, 0);
+    bool open = false, joined = false;
+    if (i < n) {
+        p = A.pairs[i];
+        p.y &= kPairTileMask;
+        if ((p.x == p.y) == diagonal && MGB_IN_RANGE(p.x, A.n_tiles, A.stats + kStatOob) &&
+            MGB_IN_RANGE(p.y, A.n_tiles, A.stats + kStatOob)) {
+            const int2 a = tr[p.x], b = tr[p.y];
+            const bool cores = a.y >= 0 && b.y >= 0;
+            open = cores && (a.x != a.y || b.x != b.y || a.x != b.x);
+            joined = cores && !open;
+            if (open && a.x == a.y && b.x == b.y) {
+                gunion(A.parent, A.row_pt, a.x, b.x);
+                open = false;
+            }
+        }
+    }
+    const int nj = __syncthreads_count(joined);
+    if (threadIdx.x == 0 && nj) atomicAdd(&A.stats[kStatSkipped], (unsigned long long)nj);
+    unsigned todo = __ballot_sync(0xffffffffu, open);
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int ta = __shfl_sync(0xffffffffu, p.x, src), tb = __shfl_sync(0xffffffffu, p.y, src);
+        int first = -1;                                    // the pair's first core row
+        for (int side = 0; side < (ta == tb ? 1 : 2); ++side) {
+            const int t = side ? tb : ta, nt = A.tile_n[t];
+            for (int x0 = 0; x0 < nt; x0 += 32) {
+                const int row = t * kT + x0 + lane;
+                const bool c = x0 + lane < nt && A.core[row];
+                const unsigned m = __ballot_sync(0xffffffffu, c);
+                if (!m) continue;
+                if (first < 0) first = t * kT + x0 + __ffs(m) - 1;
+                if (c && row != first) gunion(A.parent, A.row_pt, row, first);
+            }
+        }
+    }
+}
+
 inline unsigned grid_for(int64_t n, int t = 256) { return (unsigned)std::max<int64_t>(1, div_up(n, t)); }
 
 }  // namespace
@@ -708,6 +759,17 @@ cudaError_t select_round(const PassArgs& a, int64_t T, int2* tile_roots, int64_t
     select_round_kernel<<<grid_for(n), 256, 0, s>>>(a.pairs, a.pair_hit, n, lo, hi, filter ? tile_roots : nullptr,
                                                     first, out, count, a.stats);
     note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t allin_unions(const PassArgs& a, int64_t n, int64_t T, int2* tile_roots, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    for (int off = 0; off < 2; ++off) {
+        tile_roots_kernel<<<grid_for(T * 32), 256, 0, s>>>(a, T, tile_roots);
+        allin_unions_kernel<<<grid_for(n), 256, 0, s>>>(a, n, off == 0, tile_roots);
+    }
+    note_launch(4);
     return cudaGetLastError();
 }
 

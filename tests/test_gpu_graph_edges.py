@@ -141,3 +141,20 @@ def test_three_products_at_every_depth(d, n):
             assert st["n_core"] == rs["n_core"]
             for k in ref:
                 assert np.array_equal(np.asarray(got[k]), np.asarray(ref[k])), (tile_n, k)
+
+
+# more than 8192 all-in tile pairs, in tiles that are one component and tiles
+# that are not
+@pytest.mark.parametrize("prec", [mg.FP32, mg.BF16])
+def test_many_all_in_pairs(ctx, prec):
+    rng = np.random.default_rng(11)
+    X = np.concatenate([rng.normal(0, 0.01, (22_000, 4)), rng.normal(0, 0.01, (900, 4)) + 3.0,
+                        rng.uniform(-4, 6, (400, 4))]).astype(np.float32)
+    X = X[rng.permutation(len(X))]
+    prm = mg.params((mg.LENS_COORD,), (0,), (1,), (0.0,), 1.0, 5, prec)
+    g = mg.mapper_graph(ctx, _device(X), prm)
+    assert g.stats()["tile_pairs_in"] >= 8192
+    got = g.numpy()
+    ref = oracle.mapper_graph(X, X[:, :1].astype(np.float64), (1,), (0.0,), 1.0, 5)
+    for k in ("node_offsets", "node_members", "node_elem", "edges"):
+        assert np.array_equal(np.asarray(got[k]), np.asarray(ref[k])), k
