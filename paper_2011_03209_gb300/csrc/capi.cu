@@ -340,9 +340,14 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
 // that defer a block, two phases cost about T1 + f T3 and one phase T3 (T1,
 // T3: the one- and three-product passes over the list; T1 ~ 0.6 T3 at d =
 // 256), so a call takes one phase when f exceeds kDeferMax. Lists shorter
-// than kSampleMinPairs keep two phases.
+// than kSampleMinPairs are not sampled: they keep two phases, except that
+// with the BF16 first phase lists of at most kShortBlocks pairs times K blocks of
+// 64 columns take one. The phase would save at most 0.45 T3 there (~2.5 ns a
+// pair and K block, 20 us at the limit); its list and second launch cost about
+// eight short kernels: 5k x 8 742 -> 703 us, 13.7k x 37 881 -> 838 in one phase.
 constexpr double kDeferMax = 0.35;
 constexpr int64_t kSampleMinPairs = 8192;
+constexpr int64_t kShortBlocks = 8192;
 // Within a two-phase pass (MAPPER_BF16), the sample also decides per bin of
 // the tile-pair statistic (pair_bins): a pair skipping the first phase saves
 // its one-product screen (~0.55 T3/pair) and costs a three-product screen
@@ -837,6 +842,10 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
             CK(cudaStreamSynchronize(s), "sync");
         }
     }
+    const int64_t n_screened = PL.n[kListTC] + (cross_tc ? PL.n[kListSimt] : 0);
+    if (ctx->screen_mode == 0 && !f8 && n_screened < kSampleMinPairs &&
+        n_screened * ((dp + 63) / 64) <= kShortBlocks)
+        two_phase = false;
     st.tile_pairs_direct = n_direct;
     st.pass1_phases = use_tc ? (two_phase ? 2 : 1) : 0;
     Buf redo, redo_mask, redo_q;
