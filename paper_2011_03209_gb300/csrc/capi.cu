@@ -1017,16 +1017,18 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         // pairs whose two sides are each already one component only need one
         // neighbour pair. After the unions along the neighbour lists few pairs
         // are left (none to a few hundred of up to 1.2 M; 3 k of 173 k at 1M x
-        // 256), so two rounds do; without lists (minPts 1, or above 65) the
-        // rounds join everything, in five steps.
+        // 256), so two rounds do, and one on short lists (a round is four
+        // launches: 5k x 8 702 -> 685 us, 13.7k x 37 832 -> 813); without lists
+        // (minPts 1, or above 65) the rounds join everything, in five steps.
         auto union_rounds = [&](const PassArgs& base, const TcArgs& tbase, int64_t n, bool tc) -> int {
             if (n == 0) return MAPPER_OK;
             // every count stays on the device: each launch covers the list's
             // capacity n and reads its length there, so the rounds need no host
             // round trip
-            static const int kFew[] = {-1, 1, INT_MAX}, kMany[] = {-1, 1, 4, 16, 64, INT_MAX};
-            const int* bounds = cap ? kFew : kMany;
-            const int rounds = cap ? 2 : 5;
+            static const int kOne[] = {-1, INT_MAX}, kFew[] = {-1, 1, INT_MAX}, kMany[] = {-1, 1, 4, 16, 64, INT_MAX};
+            const bool few = n < kSampleMinPairs;
+            const int* bounds = cap ? (few ? kOne : kFew) : kMany;
+            const int rounds = cap ? (few ? 1 : 2) : 5;
             Buf list, cnt, troots;
             CK(troots.alloc(sizeof(int2) * std::max<int64_t>(L.T, 1), s), "alloc");
             CK(list.alloc(sizeof(int2) * n, s), "alloc");
