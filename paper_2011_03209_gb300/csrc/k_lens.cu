@@ -419,20 +419,24 @@ __global__ void __launch_bounds__(32 * kEccWarps) col_sum_exp_kernel(const float
 
 // |x - mu|^2 of every row for the eccentricity. In FP64 that is a subtract and
 // an FMA a value, which the FP64 pipe takes 0.84 ms for at 1M x 256; here a value
-// takes ~45 FP32 instructions: with mu = mh + ml, t = x - mu as th + tl (two-sums;
-// tl to 2^-24 of itself), th^2 = p + pe exactly, 2 th tl + (tl^2 + pe) in two
-// FMAs, and a 32-column sum of them as an FP32 expansion of three terms, added to the row's
-// FP64 sum. The roundings are below 2^-47 of a value's square and independent,
-// against 2^-53 of the running sum at every FP64 step. A chunk where some |t| is
-// not zero or in [2^-40, 2^55) is summed in FP64 instead (subtract and FMA,
-// columns in order). One thread a row, as lens_rows_kernel.
+// takes ~65 FP32 instructions. The mean's 53 bits are three floats, because what
+// is cut from it shifts a whole column by a part of |mu|, however small x - mu
+// is; t = x - mu as th + tl + t3 (two-sums, to 2^-72 of |t| and |mu|), th^2 = p + pe
+// and 2 th tl = q + qe exactly, qe + tl^2 + 2 th t3 in two FMAs, and a 32-column
+// sum of them as an FP32 expansion of three terms, added to the row's FP64 sum.
+// The roundings are below 2^-68 of a value's square, so a row's error is that of
+// its d / 32 FP64 adds, against two FP64 roundings a value (largest relative
+// error over 3000 rows, means 0 to 1e6: 1.1e-16 at 1 to 8 columns, 3.2e-16 at 256;
+// the FP64 form 4.7e-16 and 1.7e-15). A chunk where some |t| is not zero or in
+// [2^-40, 2^55) is summed in FP64 instead (subtract and FMA, columns in order).
+// One thread a row, as lens_rows_kernel.
 __global__ void __launch_bounds__(kRows) ecc_rows_kernel(const float* __restrict__ X, int64_t n, int32_t d, int64_t ld,
                                                          const double* __restrict__ mu, double* __restrict__ f, int m,
                                                          int j)
 {
     __shared__ float tile[kRows][kChunk + 1];
     __shared__ double smu[kChunk];
-    __shared__ float2 smf[kChunk];
+    __shared__ __align__(16) float4 smf[kChunk];                   // the mean as three floats
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t row0 = (int64_t)blockIdx.x * kRows;
     const bool vec = ld % 4 == 0 && ((uintptr_t)X & 15) == 0;
@@ -463,34 +467,40 @@ __global__ void __launch_bounds__(kRows) ecc_rows_kernel(const float* __restrict
         }
         if (tid < kc) {
             const double mk = mu[k0 + tid];
-            const float mh = (float)mk;
+            const float m1 = (float)mk;
+            const double rest = mk - (double)m1;                   // (exact)
+            const float m2 = (float)rest;
             smu[tid] = mk;
-            smf[tid] = make_float2(mh, (float)(mk - (double)mh));
+            smf[tid] = make_float4(m1, m2, (float)(rest - (double)m2), 0.f);
         }
         __syncthreads();
         float s = 0.f, e = 0.f, e2 = 0.f;
-        unsigned lo = 0x7F800000u, hi = 0u;                        // smallest (not 0) and largest |th|
+        unsigned lo = ~0u, hi = 0u;                                // 2 |th| as bits: smallest (not 0) less 1, largest
 #pragma unroll 4
         for (int k = 0; k < kc; ++k) {
-            const float2 mk = smf[k];
-            float a, tl, err, b;
-            const float y = two_sum(tile[tid][k], -mk.x, a);        // x - mh = y + a
-            const float th = two_sum(y, __fsub_rn(a, mk.y), tl);
-            const unsigned t = __float_as_uint(th) & 0x7FFFFFFFu;
+            const float4 mk = smf[k];
+            float a, c, t3, err, b;
+            const float y = two_sum(tile[tid][k], -mk.x, a);        // x - m1 = y + a
+            const float v = two_sum(a, -mk.y, b);                   // a - m2 = v + b
+            const float th = two_sum(y, v, c);
+            const float tl = two_sum(c, __fsub_rn(b, mk.z), t3);
+            const unsigned t = __float_as_uint(th) << 1;
             hi = max(hi, t);
-            lo = min(lo, t ? t : 0x7F800000u);
-            const float p = __fmul_rn(th, th);
-            const float low = __fmaf_rn(__fadd_rn(th, th), tl, __fmaf_rn(tl, tl, __fmaf_rn(th, th, -p)));
+            lo = min(lo, t - 1u);
+            const float p = __fmul_rn(th, th), h2 = __fadd_rn(th, th), q = __fmul_rn(h2, tl);
+            const float rest = __fmaf_rn(h2, t3, __fmaf_rn(tl, tl, __fmaf_rn(h2, tl, -q)));
             s = two_sum(s, p, err);
             e = two_sum(e, err, b);
             e2 = __fadd_rn(e2, b);
-            e = two_sum(e, low, b);
+            e = two_sum(e, __fmaf_rn(th, th, -p), b);
             e2 = __fadd_rn(e2, b);
+            e = two_sum(e, q, b);
+            e2 = __fadd_rn(e2, __fadd_rn(b, rest));
         }
         // 2^-40 and 2^55 as bits
-        if (lo >= (87u << 23) && hi < (182u << 23)) {
+        if (lo >= (87u << 24) - 1u && hi < (182u << 24)) {
             acc += (double)s + ((double)e + (double)e2);
-        } else if (hi != 0u) {
+        } else {
             for (int k = 0; k < kc; ++k) {
                 const double t = __dsub_rn((double)tile[tid][k], smu[k]);
                 acc = __fma_rn(t, t, acc);
@@ -1086,11 +1096,12 @@ cudaError_t column_means(const float* X, int64_t n, int32_t d, int64_t ld, doubl
 // Eccentricity with exponent 2 (§3 and §4.1 name eccentricity among the
 // common filters): the mean squared distance from x to the cloud equals
 // |x - mu|^2 + mean_y |y - mu|^2 (mu the column means), so f(x) =
-// sqrt(|x - mu|^2 + V) without any pair of points: column means and |x - mu|^2
-// to FP64 accuracy, V their mean (fixed-order sums). 1M x 256 through mapper_lens:
-// 3024 us with FP64 arithmetic throughout and a pass of its own for the finite
-// check, 831 us now (column sums 286, rows 400); error against 64 bits 2.5e-16
-// before, 1.3e-16 now.
+// sqrt(|x - mu|^2 + V) without any pair of points: column means as FP64 sums
+// give them, |x - mu|^2 more exactly than FP64 sums do (ecc_rows_kernel), V their
+// mean (fixed-order sums). 1M x 256 through mapper_lens: 3024 us with FP64
+// arithmetic throughout and a pass of its own for the finite check, 990 us now;
+// with the mean as two floats 832, but on 3000 rows of mean 1e6 and spread 1 in
+// 2 columns up to 2.5e-10 off, where FP64 arithmetic and this form are off by 8e-15.
 cudaError_t lens_ecc2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j, cudaStream_t s,
                       int* flag)
 {
