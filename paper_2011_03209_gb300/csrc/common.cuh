@@ -116,6 +116,23 @@ private:
     size_t used = 0;
 };
 
+// Before a launch with `smem` bytes of dynamic shared memory: lets the kernel
+// take all that a CTA can have beside its own arrays. The 48 KB that need no
+// leave are for both together (kernels that come here keep less than 8 KB of
+// their own). Always the same limit: one that follows the call's size could be
+// lowered by another thread between this and the launch.
+template <class K>
+inline cudaError_t allow_smem(K* kernel, size_t smem)
+{
+    if (smem <= (40 << 10)) return cudaSuccess;
+    constexpr int kMostSmem = 232448;                          // 227 KB
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kMostSmem - (int)a.sharedSizeBytes);
+}
+
 // ------------------------------------------------------------------ kernels
 // lens (k_lens.cu)
 cudaError_t lens_l2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j,

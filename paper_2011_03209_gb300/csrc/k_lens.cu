@@ -1154,9 +1154,7 @@ template <int NJ>
 static cudaError_t power_cluster(const double* C, int32_t d, int K, double* axes, int* status, cudaStream_t s)
 {
     const size_t smem = sizeof(double) * 32 * NJ * (size_t)K;
-    if (smem > 48 * 1024)
-        MGB_TRY(cudaFuncSetAttribute(power_iter_cluster_kernel<NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+    MGB_TRY(allow_smem(power_iter_cluster_kernel<NJ>, smem));
     const int rows = div_up(d, kPowCluster);                 // a CTA's rows, two a warp
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kPowCluster);
@@ -1186,8 +1184,7 @@ cudaError_t pca_axes(const float* X, int64_t n, int32_t d, int64_t ld, int K, do
     MGB_TRY(cpart.alloc(sizeof(float) * (size_t)nchunk * ntri * kCovT * kCovT, s));
     MGB_TRY(C.alloc(sizeof(double) * (size_t)d * d, s));
     const size_t mu_smem = sizeof(float2) * (size_t)d;
-    if (mu_smem > 48 * 1024)
-        MGB_TRY(cudaFuncSetAttribute(centre_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mu_smem));
+    MGB_TRY(allow_smem(centre_rows_kernel, mu_smem));
     centre_rows_kernel<<<(unsigned)std::min<int64_t>(div_up(n, 8), 152 * 8), 256, mu_smem, s>>>(X, n, d, ld, mu,
                                                                                               xc.as<float>());
     MGB_TRY(cudaGetLastError());
@@ -1205,9 +1202,7 @@ cudaError_t pca_axes(const float* X, int64_t n, int32_t d, int64_t ld, int K, do
         return power_cluster<8>(C.as<double>(), d, K, axes, status, s);
     }
     const size_t smem = sizeof(double) * 2 * (size_t)d;
-    if (smem > 48 * 1024)
-        MGB_TRY(cudaFuncSetAttribute(power_iter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+    MGB_TRY(allow_smem(power_iter_kernel, smem));
     { power_iter_kernel<<<1, 1024, smem, s>>>(C.as<double>(), d, K, axes, status); note_launch(); }
     return cudaGetLastError();
 }

@@ -1615,8 +1615,7 @@ int classify_pairs(const TileLayout& L, const float* X, int64_t ld, int d, int d
     for (int k = 0; k < kListCount; ++k) TK(P->list[k].alloc(sizeof(int2) * std::max<int64_t>(C, 1), s));
     const unsigned cls_grid = (unsigned)(div_up(L.T, kClsA) + L.n_seg);
     const size_t cls_smem = sizeof(float) * kClsA * dp;
-    if (cls_smem > 48 * 1024)
-        TK(cudaFuncSetAttribute(classify_blk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cls_smem));
+    TK(allow_smem(classify_blk_kernel, cls_smem));
     // segment distances: lane partial sums and a shuffle tree (dist_sum32);
     // tile distances: one FMA chain over dp columns
     const double rel = (double)(dp / 32 + 12) * std::ldexp(1.0, -23);
