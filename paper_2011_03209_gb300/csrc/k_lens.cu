@@ -721,6 +721,10 @@ __global__ void __launch_bounds__(256) centre_rows_kernel(const float* __restric
 // the tiles are small so that a cloud of a hundred thousand rows x 64 columns
 // still fills the SMs (49 chunks x 3 tiles at 100k x 64: 476 -> 89 us with the
 // rows centred once, 26 us; 500k x 128: 1475 -> 390 + 370 us).
+// The centred rows take at most kCentredBytes at a time, so that no second cloud
+// stands beside a large one (600k x 256 held 658 MB of scratch), and
+// 500k x 128 is still one block of large launches.
+constexpr size_t kCentredBytes = size_t(256) << 20;
 constexpr int kCovT = 32;
 constexpr int kCovRows = 2048;
 constexpr int kCovStep = 32;
@@ -1179,20 +1183,28 @@ cudaError_t pca_axes(const float* X, int64_t n, int32_t d, int64_t ld, int K, do
     const int ntile = div_up(d, kCovT);
     const int ntri = ntile * (ntile + 1) / 2;
     const int nchunk = div_up(n, kCovRows);
+    // the centred rows in blocks of whole chunks, at most kCentredBytes at a time
+    const int64_t fit = (int64_t)(kCentredBytes / (sizeof(float) * (size_t)d)) / kCovRows * kCovRows;
+    const int64_t block = std::min<int64_t>(n, std::max<int64_t>(fit, kCovRows));
     Buf xc, cpart, C;
-    MGB_TRY(xc.alloc(sizeof(float) * (size_t)n * d, s));
+    MGB_TRY(xc.alloc(sizeof(float) * (size_t)block * d, s));
     MGB_TRY(cpart.alloc(sizeof(float) * (size_t)nchunk * ntri * kCovT * kCovT, s));
     MGB_TRY(C.alloc(sizeof(double) * (size_t)d * d, s));
     const size_t mu_smem = sizeof(float2) * (size_t)d;
     MGB_TRY(allow_smem(centre_rows_kernel, mu_smem));
-    centre_rows_kernel<<<(unsigned)std::min<int64_t>(div_up(n, 8), 152 * 8), 256, mu_smem, s>>>(X, n, d, ld, mu,
-                                                                                              xc.as<float>());
-    MGB_TRY(cudaGetLastError());
-    cov_partial_kernel<<<dim3(ntri, nchunk), 64, 0, s>>>(xc.as<float>(), n, d, cpart.as<float>(), ntile);
-    MGB_TRY(cudaGetLastError());
+    for (int64_t r0 = 0; r0 < n; r0 += block) {
+        const int64_t rows = std::min<int64_t>(block, n - r0);
+        centre_rows_kernel<<<(unsigned)std::min<int64_t>(div_up(rows, 8), 152 * 8), 256, mu_smem, s>>>(
+            X + r0 * ld, rows, d, ld, mu, xc.as<float>());
+        MGB_TRY(cudaGetLastError());
+        cov_partial_kernel<<<dim3(ntri, div_up(rows, kCovRows)), 64, 0, s>>>(
+            xc.as<float>(), rows, d, cpart.as<float>() + r0 / kCovRows * (int64_t)ntri * kCovT * kCovT, ntile);
+        note_launch(2);
+        MGB_TRY(cudaGetLastError());
+    }
     cov_reduce_kernel<<<dim3(ntri, kCovT * kCovT / 128), 128, 0, s>>>(cpart.as<float>(), nchunk, ntile, d, n,
                                                                       C.as<double>());
-    note_launch(3);
+    note_launch();
     MGB_TRY(cudaGetLastError());
     // the cluster holds C and the axes on chip; wider clouds or many axes take one CTA
     if (d <= 256 && (size_t)K * 256 * sizeof(double) <= 160 * 1024) {

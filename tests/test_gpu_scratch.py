@@ -1,0 +1,63 @@
+"""Device memory that calls take from the stream-ordered pool, read from the
+pool's own counters."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+mg = pytest.importorskip("paper_2011_03209_gb300")
+
+pytestmark = pytest.mark.gpu
+
+USED_CURRENT, USED_HIGH = 7, 8                              # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH
+
+
+class Pool:
+    """The device's default pool (torch's own tensors are not in it)."""
+
+    def __init__(self):
+        torch.cuda.init()
+        self.cu = ctypes.CDLL("libcuda.so.1")
+        dev, self.pool = ctypes.c_int(), ctypes.c_void_p()
+        assert self.cu.cuDeviceGet(ctypes.byref(dev), 0) == 0
+        assert self.cu.cuDeviceGetDefaultMemPool(ctypes.byref(self.pool), dev) == 0
+
+    def get(self, attr):
+        v = ctypes.c_uint64()
+        assert self.cu.cuMemPoolGetAttribute(self.pool, attr, ctypes.byref(v)) == 0
+        return v.value
+
+    def peak_of(self, call):
+        """The most that `call` holds beyond what is held before it."""
+        torch.cuda.synchronize()
+        before = self.get(USED_CURRENT)
+        zero = ctypes.c_uint64(0)
+        assert self.cu.cuMemPoolSetAttribute(self.pool, USED_HIGH, ctypes.byref(zero)) == 0
+        out = call()
+        torch.cuda.synchronize()
+        return self.get(USED_HIGH) - before, out
+
+
+def _device(X):
+    Xd = torch.from_numpy(np.ascontiguousarray(X)).to("cuda:0")
+    torch.cuda.synchronize()
+    return Xd
+
+
+def test_principal_axes_keep_no_second_cloud():
+    n, d = 600_000, 256
+    X = torch.randn((n, d), device="cuda:0", generator=torch.Generator("cuda:0").manual_seed(1))
+    X[:, 3] *= 4.0
+    pool = Pool()
+    with mg.Context(0) as ctx:
+        peak, (f, _) = pool.peak_of(lambda: mg.mapper_lens(ctx, X, (mg.LENS_PCA,), (0,)))
+        got = f[:, 0].cpu().numpy()
+    # 256 MiB of centred rows, 44 MB of partial tiles (the cloud: 614 MB)
+    assert peak < 400e6, peak
+    # the axis is column 3 but for the sample's correlations with it (4 / sqrt(n) in
+    # all, over the eigenvalues' gap of 15: less than 0.03 of the projections' size)
+    x3 = X[:, 3].double().cpu().numpy()
+    assert np.abs(np.corrcoef(got, x3)[0, 1]) > 0.999
