@@ -1684,7 +1684,7 @@ int mapper_single_linkage(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_
     h->cover = cov;
     h->eps = eps;
     if ((rc = msf_forest(a, L.row_slot.as<int32_t>(), cov->slot_point.as<int32_t>(), cov->slot_elem.as<int32_t>(),
-                         cov->M, cov->E, L.R, L.T, np, &h->f, s)))
+                         cov->M, cov->E, L.R, L.T, np, ctx->budget ? std::max<size_t>(ctx->budget / 4, 1) : 0, &h->f, s)))
         return rc;
     int h_nf = 0;
     CK(cudaMemcpyAsync(&h_nf, flag.p, sizeof(int), cudaMemcpyDeviceToHost, s), "copy");

@@ -213,9 +213,11 @@ struct ForestOut {
 };
 // a: the rows of a tile layout (G or X via row_pt, dp, d, tile_n, row_pt,
 // eps2, hi_thr of fp32_thresholds) and a.pairs[0 .. n_pairs) the element tile
-// pairs not certified all-out at eps. Returns a mapper_status.
+// pairs not certified all-out at eps. queue_bytes: the most that the queue of
+// candidate pairs may take (0: no limit). Returns a mapper_status.
 int msf_forest(const PassArgs& a, const int32_t* row_slot, const int32_t* slot_point, const int32_t* slot_elem,
-               int64_t M, int64_t E, int64_t R, int64_t T, int64_t n_pairs, ForestOut* out, cudaStream_t s);
+               int64_t M, int64_t E, int64_t R, int64_t T, int64_t n_pairs, size_t queue_bytes, ForestOut* out,
+               cudaStream_t s);
 // Single-linkage clusters at height h (edges with d2 <= h^2) in cover-slot
 // space, in the layout of rows_to_slots (every slot a member and core).
 int msf_cut(const ForestOut& f, const int32_t* slot_point, int64_t M, double h, int32_t* lab, uint8_t* flags,

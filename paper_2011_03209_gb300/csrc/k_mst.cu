@@ -506,7 +506,8 @@ cudaError_t sort_forest(ForestOut* out, int64_t M, int64_t E, double eps2, cudaS
 }  // namespace
 
 int msf_forest(const PassArgs& a, const int32_t* row_slot, const int32_t* slot_point, const int32_t* slot_elem,
-               int64_t M, int64_t E, int64_t R, int64_t T, int64_t n_pairs, ForestOut* out, cudaStream_t s)
+               int64_t M, int64_t E, int64_t R, int64_t T, int64_t n_pairs, size_t queue_bytes,
+               ForestOut* out, cudaStream_t s)
 {
 #define MK(expr)                                                                   \
     do {                                                                           \
@@ -542,9 +543,17 @@ int msf_forest(const PassArgs& a, const int32_t* row_slot, const int32_t* slot_p
     unsigned long long* oob = n_edges + 5;
     MK(cudaMemsetAsync(counts.p, 0, sizeof(unsigned long long) * 6, s));
     // every row queues its nearest so far, a few times over (about log(tile
-    // pairs of its element) each)
-    const unsigned long long queue_cap = 8ull * (unsigned long long)R;
-    MK(queue.alloc(sizeof(int4) * queue_cap, s));
+    // pairs of its element) each). That is 128 bytes a row, so the queue keeps to
+    // queue_bytes and takes what can be had: a round that overflows it (at worst
+    // all of them) is screened twice.
+    unsigned long long queue_cap = 8ull * (unsigned long long)R;
+    if (queue_bytes) queue_cap = std::min<unsigned long long>(queue_cap, queue_bytes / sizeof(int4));
+    for (;; queue_cap /= 2) {
+        const cudaError_t e = queue.alloc(sizeof(int4) * queue_cap, s);
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || queue_cap == 0) MK(e);
+        cudaGetLastError();
+    }
     const unsigned gR = (unsigned)div_up(R, 256);
     msf_init_kernel<<<gR, 256, 0, s>>>(row_slot, R, parent.as<int32_t>(), slot_row.as<int32_t>());
     MK(cudaGetLastError());

@@ -61,3 +61,26 @@ def test_principal_axes_keep_no_second_cloud():
     # all, over the eigenvalues' gap of 15: less than 0.03 of the projections' size)
     x3 = X[:, 3].double().cpu().numpy()
     assert np.abs(np.corrcoef(got, x3)[0, 1]) > 0.999
+
+
+def _forest(budget, X, eps):
+    with mg.Context(0, hbm_budget=budget) as ctx:
+        Xd = _device(X)
+        lens, _ = mg.mapper_lens(ctx, Xd, (mg.LENS_COORD,), (0,))
+        cover = mg.mapper_cover(ctx, lens, (4,), (0.2,))
+        peak, f = Pool().peak_of(lambda: mg.mapper_single_linkage(ctx, Xd, cover, eps))
+        return peak, f.numpy()
+
+
+# the budgets give the queue a quarter: 4 MB of the 6 to 7 MB that 8 entries a row
+# would take, 64 KB, 15 entries, none
+@pytest.mark.parametrize("budget", [16 << 20, 256 << 10, 999, 1])
+def test_forest_queue_keeps_to_the_budget(budget):
+    X = np.random.default_rng(2).standard_normal((40_000, 3)).astype(np.float32)
+    free, want = _forest(0, X, 0.08)
+    assert len(want["u"]) > 1000
+    peak, got = _forest(budget, X, 0.08)
+    for k in want:
+        assert np.array_equal(got[k], want[k]), k
+    queue = 128 * 40_000
+    assert peak <= free - (queue - budget / 4) + 4096, (peak, free)
