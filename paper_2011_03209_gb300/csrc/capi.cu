@@ -1203,17 +1203,22 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
     bool edges_done = false;
     if (in_order) {
         CK(offsets(nullptr), "node offsets");
-        Buf counts;
+        Buf counts, list;
         CK(counts.alloc(2 * sizeof(unsigned long long), s), "alloc");
         unsigned long long* dc = counts.as<unsigned long long>();
-        CK(edge_set(cov->pt_off.as<int64_t>(), cov->n, node_o.as<int32_t>(), &g->edges, dc, s), "edges");
-        CK(radix_sort_u64_two_dev(g->edges.as<uint64_t>(), kEdgeListMax, dc, 32, 0, bits_for(N), s), "sort");
+        CK(edge_set(cov->pt_off.as<int64_t>(), cov->n, node_o.as<int32_t>(), &list, dc, s), "edges");
+        CK(radix_sort_u64_two_dev(list.as<uint64_t>(), kEdgeListMax, dc, 32, 0, bits_for(N), s), "sort");
         unsigned long long h[2] = {0, 0};
         Readback rb(s);
         CK(rb.get(h, dc, sizeof(h)), "copy");
         CK(rb.wait(), "sync");
         edges_done = h[1] == 0;
-        g->Eg = (int64_t)h[0];
+        if (edges_done) {                                          // (the graph keeps the edges, not the list)
+            const size_t bytes = sizeof(int32_t) * 2 * (size_t)h[0];
+            g->Eg = (int64_t)h[0];
+            CK(g->edges.alloc(bytes, s), "alloc");
+            if (bytes) CK(cudaMemcpyAsync(g->edges.p, list.p, bytes, cudaMemcpyDeviceToDevice, s), "copy edges");
+        }
     }
     if (!edges_done) {
         CK(keys2.alloc(sizeof(uint64_t) * Gm, s), "alloc");

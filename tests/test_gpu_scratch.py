@@ -84,3 +84,25 @@ def test_forest_queue_keeps_to_the_budget(budget):
         assert np.array_equal(got[k], want[k]), k
     queue = 128 * 40_000
     assert peak <= free - (queue - budget / 4) + 4096, (peak, free)
+
+
+def test_a_graph_keeps_its_edges_only():
+    X = np.random.default_rng(3).standard_normal((500, 3)).astype(np.float32)
+    prm = mg.params((mg.LENS_COORD,), (0,), (8,), (0.3,), 0.8, 3, mg.FP32)
+    pool = Pool()
+    with mg.Context(0) as ctx:
+        Xd = _device(X)
+        graphs = [mg.mapper_graph(ctx, Xd, prm)]
+        torch.cuda.synchronize()
+        before = pool.get(USED_CURRENT)
+        graphs += [mg.mapper_graph(ctx, Xd, prm) for _ in range(32)]
+        torch.cuda.synchronize()
+        kept = (pool.get(USED_CURRENT) - before) / 32
+        got = graphs[-1].numpy()
+        lens, _ = graphs[-1].lens(500, 1)
+        del graphs
+    assert len(got["edges"]) > 0
+    # 700 memberships of 50 bytes and 500 points of 16 in 20 arrays, each rounded up to 512
+    assert kept < 64 << 10, kept
+    ref = oracle.mapper_graph(X, lens, (8,), (0.3,), 0.8, 3)
+    assert np.array_equal(got["edges"], ref["edges"])
