@@ -55,7 +55,10 @@ __global__ void node_offsets_kernel(const uint64_t* __restrict__ keys, int64_t G
 // ascend in element, and nodes in (element, root), so u < v. A pair seen before
 // is one read of the set (in L2); the edges are few (hundreds) beside the
 // points, so sorting all pairs, or the memberships by point, would move far
-// more. counts[0]: edges, counts[1]: set when the list or a probe run is full.
+// more. counts[0]: edges, counts[1]: set when the list or a probe run is full. A
+// thread stops at the first pair it has no place for, and one that starts later
+// at once (a read of the flag at every membership, all of one address, cost more
+// than it saved: nerve of 868k memberships and 1.0 M edges 0.85 -> 1.35 ms).
 constexpr int kEdgeProbes = 64;
 
 __global__ void __launch_bounds__(256) edge_set_kernel(const int64_t* __restrict__ pos, int64_t n,
@@ -65,7 +68,7 @@ __global__ void __launch_bounds__(256) edge_set_kernel(const int64_t* __restrict
                                                        unsigned long long* counts)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
+    if (p >= n || __ldcg(counts + 1)) return;
     const int64_t o0 = pos[p], o1 = pos[p + 1];
     for (int64_t a = o0; a < o1; ++a) {
         const int u = node_o[a];
@@ -86,11 +89,17 @@ __global__ void __launch_bounds__(256) edge_set_kernel(const int64_t* __restrict
                 if (cur == key) break;
                 if (cur != ~0ull) continue;
                 const unsigned long long at = atomicAdd(&counts[0], 1ull);
-                if (at < cap) list[at] = key;
-                else counts[1] = 1ull;
+                if (at >= cap) {
+                    counts[1] = 1ull;
+                    return;
+                }
+                list[at] = key;
                 break;
             }
-            if (tries == kEdgeProbes) counts[1] = 1ull;
+            if (tries == kEdgeProbes) {
+                counts[1] = 1ull;
+                return;
+            }
         }
     }
 }
