@@ -204,17 +204,18 @@ cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t N, int64_t* no
     return cudaGetLastError();
 }
 
-cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, Buf* list, unsigned long long* counts,
-                     cudaStream_t s)
+cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, int64_t cap, Buf* list,
+                     unsigned long long* counts, cudaStream_t s)
 {
+    if (cap > kEdgeListMax) return cudaErrorInvalidValue;
     constexpr uint32_t kSlots = 4 * kEdgeListMax;
     Buf set;
     MGB_TRY(set.alloc(sizeof(uint64_t) * kSlots, s));
-    MGB_TRY(list->alloc(sizeof(uint64_t) * kEdgeListMax, s));
+    MGB_TRY(list->alloc(sizeof(uint64_t) * cap, s));
     MGB_TRY(cudaMemsetAsync(set.p, 0xff, sizeof(uint64_t) * kSlots, s));
     MGB_TRY(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), s));
     edge_set_kernel<<<grid_for(n), 256, 0, s>>>(pos, n, node_o, set.as<unsigned long long>(), kSlots - 1,
-                                                list->as<uint64_t>(), kEdgeListMax, counts);
+                                                list->as<uint64_t>(), (uint32_t)cap, counts);
     note_launch();
     return cudaGetLastError();
 }

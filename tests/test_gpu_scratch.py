@@ -86,9 +86,11 @@ def test_forest_queue_keeps_to_the_budget(budget):
     assert peak <= free - (queue - budget / 4) + 4096, (peak, free)
 
 
-def test_a_graph_keeps_its_edges_only():
-    X = np.random.default_rng(3).standard_normal((500, 3)).astype(np.float32)
-    prm = mg.params((mg.LENS_COORD,), (0,), (8,), (0.3,), 0.8, 3, mg.FP32)
+# about 20 nodes, whose edges the list has room for in little space, and about 300
+@pytest.mark.parametrize("n,nint", [(500, 8), (3000, 150)])
+def test_a_graph_keeps_its_edges_only(n, nint):
+    X = np.random.default_rng(3).standard_normal((n, 3)).astype(np.float32)
+    prm = mg.params((mg.LENS_COORD,), (0,), (nint,), (0.3,), 0.8, 3, mg.FP32)
     pool = Pool()
     with mg.Context(0) as ctx:
         Xd = _device(X)
@@ -99,10 +101,11 @@ def test_a_graph_keeps_its_edges_only():
         torch.cuda.synchronize()
         kept = (pool.get(USED_CURRENT) - before) / 32
         got = graphs[-1].numpy()
-        lens, _ = graphs[-1].lens(500, 1)
+        lens, _ = graphs[-1].lens(n, 1)
         del graphs
     assert len(got["edges"]) > 0
-    # 700 memberships of 50 bytes and 500 points of 16 in 20 arrays, each rounded up to 512
-    assert kept < 64 << 10, kept
-    ref = oracle.mapper_graph(X, lens, (8,), (0.3,), 0.8, 3)
+    # 1.4 memberships a point of 50 bytes and 16 bytes a point, in some 20 arrays of
+    # whole kilobytes; a list of up to 16 KB
+    assert kept < 100 * n + (40 << 10), kept
+    ref = oracle.mapper_graph(X, lens, (nint,), (0.3,), 0.8, 3)
     assert np.array_equal(got["edges"], ref["edges"])
