@@ -55,8 +55,8 @@ struct CoverData {
     int64_t n = 0, E = 0, M = 0;
     Buf elem_off;              // E + 1 int64
     Buf slot_point, slot_elem; // M int32 each
-    Buf pt_off, slot_o;        // memberships in point order: n + 1 int64 offsets, and each
-                               // slot's place (M int32); unset for a subset of a cover
+    Buf pt, slot_o;            // memberships in point order: their points, and each slot's
+                               // place (M int32 each); unset for a subset of a cover
     std::vector<int64_t> h_elem_off;
     void* offsets_at = nullptr;  // h_elem_off on its way through page-locked scratch
     void take_offsets()                // after a wait for the stream
@@ -278,8 +278,7 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     c->E = E;
     for (int j = 0; j < m; ++j) { c->n_int[j] = n_int[j]; c->overlap[j] = overlap[j]; }
 
-    Buf lohi, bounds, cnt, flag;
-    Buf& pos = c->pt_off;
+    Buf lohi, bounds, cnt, pos, flag;
     CK(lohi.alloc(sizeof(double) * 2 * m, s), "alloc");
     CK(bounds.alloc(sizeof(double) * 2 * ((size_t)n_int[0] + (m == 2 ? n_int[1] : 0)), s), "alloc");
     CK(cnt.alloc(sizeof(int32_t) * n, s), "alloc");
@@ -305,7 +304,8 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
     if (h_nf) return fail(MAPPER_ENONFINITE, "lens or X holds NaN or Inf");
     if (M > INT32_MAX) return fail(MAPPER_ENOMEM, "more than 2^31 cover memberships");
     c->M = M;
-    Buf keys, tmp, pt;
+    Buf keys, tmp;
+    Buf& pt = c->pt;
     CK(keys.alloc(sizeof(uint64_t) * M, s), "alloc keys");
     CK(tmp.alloc(sizeof(uint64_t) * M, s), "alloc");
     CK(pt.alloc(sizeof(int32_t) * M, s), "alloc");
@@ -1207,7 +1207,7 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
         CK(counts.alloc(2 * sizeof(unsigned long long), s), "alloc");
         unsigned long long* dc = counts.as<unsigned long long>();
         const int64_t cap = std::min<int64_t>(kEdgeListMax, std::max<int64_t>(1, N * (N - 1) / 2));
-        CK(edge_set(cov->pt_off.as<int64_t>(), cov->n, node_o.as<int32_t>(), cap, &list, dc, s), "edges");
+        CK(edge_set(cov->pt.as<int32_t>(), M, node_o.as<int32_t>(), cap, &list, dc, s), "edges");
         CK(radix_sort_u64_two_dev(list.as<uint64_t>(), cap, dc, 32, 0, bits_for(N), s), "sort");
         unsigned long long h[2] = {0, 0};
         Readback rb(s);

@@ -237,11 +237,12 @@ cudaError_t member_keys(const int32_t* lab, const int64_t* pos, const int32_t* s
                         cudaStream_t s);
 cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t N, int64_t* node_off, int32_t* members,
                          uint64_t* keys2, cudaStream_t s);
-// The distinct node pairs (v << 32 | u) sharing a point, unsorted, into *list (at
+// From the points pt (ascending) and nodes node_o of M memberships in point order:
+// the distinct node pairs (v << 32 | u) sharing a point, unsorted, into *list (at
 // most cap <= kEdgeListMax); counts[0]: their number, counts[1]: nonzero if the list
 // does not hold them all.
 constexpr uint32_t kEdgeListMax = 1u << 15;
-cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, int64_t cap, Buf* list,
+cudaError_t edge_set(const int32_t* pt, int64_t M, const int32_t* node_o, int64_t cap, Buf* list,
                      unsigned long long* counts, cudaStream_t s);
 cudaError_t run_pairs(const uint64_t* keys2, int64_t G, int64_t* cnt, cudaStream_t s);
 cudaError_t emit_pairs(const uint64_t* keys2, int64_t G, const int64_t* pos, uint64_t* out,

@@ -49,57 +49,63 @@ __global__ void node_offsets_kernel(const uint64_t* __restrict__ keys, int64_t G
 }
 
 // Nerve edges from the nodes of every membership in point order (node_o, -1:
-// none; the memberships of point p are pos[p] .. pos[p + 1]): each pair of a
-// point's nodes goes through a hash set of the distinct edges, and the thread
-// that adds one to the set appends it to the list. Memberships of a point
-// ascend in element, and nodes in (element, root), so u < v. A pair seen before
-// is one read of the set (in L2); the edges are few (hundreds) beside the
-// points, so sorting all pairs, or the memberships by point, would move far
-// more. counts[0]: edges, counts[1]: set when the list or a probe run is full. A
-// thread stops at the first pair it has no place for, and one that starts later
-// at once (a read of the flag at every membership, all of one address, cost more
-// than it saved: nerve of 868k memberships and 1.0 M edges 0.85 -> 1.35 ms).
+// none; pt: the memberships' points): each pair of a point's nodes goes through a
+// hash set of the distinct edges, and the thread that adds one to the set
+// appends it to the list. A thread takes a membership against the later ones of
+// its point (a thread a point walked all k (k - 1) / 2 pairs of a point in k
+// elements by itself: 2000 points in 255 elements with 0.996 overlap 24 ms of
+// nerve, now 0.5). Memberships of a point ascend in element, and nodes in
+// (element, root), so u < v. A pair seen before is one read of the set (in L2);
+// the edges are few (hundreds) beside the points, so sorting all pairs, or the
+// memberships by point, would move far more. counts[0]: edges, counts[1]: set when
+// the list or a probe run is full. A CTA's threads stop at the first pair that it
+// has no place for, and a CTA that starts later at once (a read of the flag at
+// every membership, all of one address, cost more than it saved: nerve of 868k
+// memberships and 1.0 M edges 0.85 -> 1.35 ms).
 constexpr int kEdgeProbes = 64;
 
-__global__ void __launch_bounds__(256) edge_set_kernel(const int64_t* __restrict__ pos, int64_t n,
+__global__ void __launch_bounds__(256) edge_set_kernel(const int32_t* __restrict__ pt, int64_t M,
                                                        const int32_t* __restrict__ node_o,
                                                        unsigned long long* set, uint32_t mask,
                                                        uint64_t* __restrict__ list, uint32_t cap,
                                                        unsigned long long* counts)
 {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n || __ldcg(counts + 1)) return;
-    const int64_t o0 = pos[p], o1 = pos[p + 1];
-    for (int64_t a = o0; a < o1; ++a) {
-        const int u = node_o[a];
-        if (u < 0) continue;
-        for (int64_t b = a + 1; b < o1; ++b) {
-            const int v = node_o[b];
-            if (v < 0) continue;
-            // (v in the high half: the sorted list is then the int32 pairs (u, v))
-            const unsigned long long key = ((unsigned long long)(unsigned)v << 32) | (unsigned)u;
-            unsigned long long x = key * 0x9E3779B97F4A7C15ull;
-            uint32_t h = (uint32_t)(x >> 40) & mask;
-            int tries = 0;
-            for (; tries < kEdgeProbes; ++tries, h = (h + 1) & mask) {
-                unsigned long long cur = __ldcg(set + h);
-                if (cur == key) break;
-                if (cur != ~0ull) continue;
-                cur = atomicCAS(set + h, ~0ull, key);
-                if (cur == key) break;
-                if (cur != ~0ull) continue;
-                const unsigned long long at = atomicAdd(&counts[0], 1ull);
-                if (at >= cap) {
-                    counts[1] = 1ull;
-                    return;
-                }
-                list[at] = key;
-                break;
-            }
-            if (tries == kEdgeProbes) {
+    __shared__ volatile int s_full;                  // counts[1] as the CTA knows it
+    if (threadIdx.x == 0) s_full = __ldcg(counts + 1) != 0ull;
+    __syncthreads();
+    const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= M || s_full) return;
+    const int u = node_o[a], p = pt[a];
+    if (u < 0) return;
+    for (int64_t b = a + 1; b < M && pt[b] == p; ++b) {
+        const int v = node_o[b];
+        if (v < 0) continue;
+        // (v in the high half: the sorted list is then the int32 pairs (u, v))
+        const unsigned long long key = ((unsigned long long)(unsigned)v << 32) | (unsigned)u;
+        unsigned long long x = key * 0x9E3779B97F4A7C15ull;
+        uint32_t h = (uint32_t)(x >> 40) & mask;
+        int tries = 0;
+        for (; tries < kEdgeProbes; ++tries, h = (h + 1) & mask) {
+            unsigned long long cur = __ldcg(set + h);
+            if (cur == key) break;
+            if (cur != ~0ull) continue;
+            if (s_full) return;
+            cur = atomicCAS(set + h, ~0ull, key);
+            if (cur == key) break;
+            if (cur != ~0ull) continue;
+            const unsigned long long at = atomicAdd(&counts[0], 1ull);
+            if (at >= cap) {
+                s_full = 1;
                 counts[1] = 1ull;
                 return;
             }
+            list[at] = key;
+            break;
+        }
+        if (tries == kEdgeProbes) {
+            s_full = 1;
+            counts[1] = 1ull;
+            return;
         }
     }
 }
@@ -204,7 +210,7 @@ cudaError_t node_offsets(const uint64_t* keys, int64_t G, int64_t N, int64_t* no
     return cudaGetLastError();
 }
 
-cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, int64_t cap, Buf* list,
+cudaError_t edge_set(const int32_t* pt, int64_t M, const int32_t* node_o, int64_t cap, Buf* list,
                      unsigned long long* counts, cudaStream_t s)
 {
     if (cap > kEdgeListMax) return cudaErrorInvalidValue;
@@ -214,7 +220,7 @@ cudaError_t edge_set(const int64_t* pos, int64_t n, const int32_t* node_o, int64
     MGB_TRY(list->alloc(sizeof(uint64_t) * cap, s));
     MGB_TRY(cudaMemsetAsync(set.p, 0xff, sizeof(uint64_t) * kSlots, s));
     MGB_TRY(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), s));
-    edge_set_kernel<<<grid_for(n), 256, 0, s>>>(pos, n, node_o, set.as<unsigned long long>(), kSlots - 1,
+    edge_set_kernel<<<grid_for(M), 256, 0, s>>>(pt, M, node_o, set.as<unsigned long long>(), kSlots - 1,
                                                 list->as<uint64_t>(), (uint32_t)cap, counts);
     note_launch();
     return cudaGetLastError();

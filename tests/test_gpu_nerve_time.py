@@ -37,3 +37,12 @@ def test_more_edges_than_the_set_holds():
     ms, edges = _nerve_ms(X, (30, 30), (0.9, 0.9), 0.4, 3)
     assert edges > 32768
     assert ms < 10.0, ms
+
+
+def test_points_in_many_elements():
+    # up to 250 elements a point, 31k pairs each; all of at most 32385 edges. A
+    # thread a point took 20 ms and more
+    X = np.random.default_rng(6).uniform(-1, 1, (2000, 3)).astype(np.float32)
+    ms, edges = _nerve_ms(X, (255,), (0.996,), 0.5, 3)
+    assert 20_000 < edges <= 32768
+    assert ms < 6.0, ms
