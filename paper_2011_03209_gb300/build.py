@@ -46,7 +46,7 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
     odir, lib = (CHECKED_BUILD, CHECKED_LIB) if checked else (BUILD, LIB)
     os.makedirs(odir, exist_ok=True)
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [os.path.join(INCLUDE, "mapper.h")]
+    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(INCLUDE, "mapper.h")]
     flags = FLAGS + (["-DMAPPER_BOUNDS_CHECK"] if checked else [])
     objs = []
     jobs = []

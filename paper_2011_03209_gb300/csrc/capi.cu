@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/mapper.h"
+#include "copies.h"
 #include "dbscan.cuh"
 #include "tc.cuh"
 
@@ -1275,19 +1276,20 @@ int nerve_edges(mapper_ctx* ctx, Buf& keys2, int64_t Gm, int64_t n_points, int64
     return MAPPER_OK;
 }
 
-// Queues a copy to the caller's memory; copies_done waits for all of them.
-int copy_out(void* dst, const void* src, size_t bytes, int on_device, cudaStream_t s)
+// Copies arrays of a result to the caller's memory, complete when it returns.
+int copies_out(std::initializer_list<CopyOut> items, int on_device, cudaStream_t s)
 {
-    if (!dst || bytes == 0) return MAPPER_OK;
-    CK(cudaMemcpyAsync(dst, src, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s),
-       "copy out");
-    return MAPPER_OK;
-}
-
-int copies_done(cudaStream_t s)
-{
-    CK(cudaStreamSynchronize(s), "sync");
-    return MAPPER_OK;
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    return copy_all(
+        items,
+        [&](const CopyOut& c) -> int {
+            CK(cudaMemcpyAsync(c.dst, c.src, c.bytes, kind, s), "copy out");
+            return MAPPER_OK;
+        },
+        [&]() -> int {
+            CK(cudaStreamSynchronize(s), "sync");
+            return MAPPER_OK;
+        });
 }
 
 bool is_host_pointer(const void* p)
@@ -1604,10 +1606,8 @@ int mapper_cover_copy(const mapper_cover_t* cover, int64_t* elem_offsets, int32_
     auto* h = handle_as<mapper_cover_t>(cover, kKindCover);
     if (!h) return fail(MAPPER_EINVAL, "not a cover handle");
     cudaStream_t s = h->c->stream->s;
-    int rc = copy_out(elem_offsets, h->c->elem_off.p, sizeof(int64_t) * (h->c->E + 1), on_device, s);
-    if (rc) return rc;
-    if ((rc = copy_out(elem_points, h->c->slot_point.p, sizeof(int32_t) * h->c->M, on_device, s))) return rc;
-    return elem_offsets || elem_points ? copies_done(s) : MAPPER_OK;
+    return copies_out({{elem_offsets, h->c->elem_off.p, sizeof(int64_t) * (h->c->E + 1)},
+                       {elem_points, h->c->slot_point.p, sizeof(int32_t) * h->c->M}}, on_device, s);
 }
 
 int mapper_cluster(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t d, int64_t ld,
@@ -1634,10 +1634,7 @@ int mapper_clusters_copy(const mapper_clusters_t* clusters, int64_t* label, uint
     if (!h) return fail(MAPPER_EINVAL, "not a clusters handle");
     cudaStream_t s = h->c->stream->s;
     const int64_t M = h->c->cover->M;
-    int rc = copy_out(label, h->c->slot_label.p, sizeof(int64_t) * M, on_device, s);
-    if (rc) return rc;
-    if ((rc = copy_out(core, h->c->core.p, M, on_device, s))) return rc;
-    return label || core ? copies_done(s) : MAPPER_OK;
+    return copies_out({{label, h->c->slot_label.p, sizeof(int64_t) * M}, {core, h->c->core.p, (size_t)M}}, on_device, s);
 }
 
 int mapper_single_linkage(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t d, int64_t ld,
@@ -1727,13 +1724,10 @@ int mapper_forest_copy(const mapper_forest_t* forest, int32_t* elem, int32_t* u,
     if (!h) return fail(MAPPER_EINVAL, "bad forest handle");
     cudaStream_t s = h->stream->s;
     const size_t n = (size_t)h->f.n;
-    int rc;
-    if (elem && (rc = copy_out(elem, h->f.elem.p, sizeof(int32_t) * n, on_device, s))) return rc;
-    if (u && (rc = copy_out(u, h->f.u.p, sizeof(int32_t) * n, on_device, s))) return rc;
-    if (v && (rc = copy_out(v, h->f.v.p, sizeof(int32_t) * n, on_device, s))) return rc;
-    if (d2 && (rc = copy_out(d2, h->f.d2.p, sizeof(double) * n, on_device, s))) return rc;
-    CK(cudaStreamSynchronize(s), "sync");
-    return MAPPER_OK;
+    return copies_out({{elem, h->f.elem.p, sizeof(int32_t) * n},
+                       {u, h->f.u.p, sizeof(int32_t) * n},
+                       {v, h->f.v.p, sizeof(int32_t) * n},
+                       {d2, h->f.d2.p, sizeof(double) * n}}, on_device, s);
 }
 
 int mapper_forest_cut(mapper_ctx* ctx, const mapper_forest_t* forest, double h, mapper_clusters_t** out)
@@ -1918,8 +1912,7 @@ int mapper_knn_distance(mapper_ctx* ctx, const float* X_dev, int64_t n, int32_t 
                           ctx->knn_info);
     }
     if (rc) return rc;
-    if ((rc = copy_out(out, od.p, sizeof(double) * q, !is_host_pointer(out), s))) return rc;
-    return copies_done(s);
+    return copies_out({{out, od.p, sizeof(double) * q}}, !is_host_pointer(out), s);
 }
 
 // Host rows to the device (xdev, n x d). When every lens of p is row-local
@@ -2239,12 +2232,10 @@ int mapper_graph_copy(const mapper_graph_t* g, int64_t* node_offsets, int32_t* n
     auto* h = handle_as<mapper_graph_t>(g, kKindGraph);
     if (!h) return fail(MAPPER_EINVAL, "not a graph handle");
     cudaStream_t s = h->stream->s;
-    int rc;
-    if ((rc = copy_out(node_offsets, h->node_off.p, sizeof(int64_t) * (h->N + 1), on_device, s))) return rc;
-    if ((rc = copy_out(node_members, h->node_members.p, sizeof(int32_t) * h->Gm, on_device, s))) return rc;
-    if ((rc = copy_out(node_elem, h->node_elem.p, sizeof(int32_t) * h->N, on_device, s))) return rc;
-    if ((rc = copy_out(edges, h->edges.p, sizeof(int32_t) * 2 * h->Eg, on_device, s))) return rc;
-    return node_offsets || node_members || node_elem || edges ? copies_done(s) : MAPPER_OK;
+    return copies_out({{node_offsets, h->node_off.p, sizeof(int64_t) * (h->N + 1)},
+                       {node_members, h->node_members.p, sizeof(int32_t) * h->Gm},
+                       {node_elem, h->node_elem.p, sizeof(int32_t) * h->N},
+                       {edges, h->edges.p, sizeof(int32_t) * 2 * h->Eg}}, on_device, s);
 }
 
 int mapper_graph_lens(const mapper_graph_t* g, double* lens, double* pca, int64_t* n_pca, int on_device)
@@ -2254,10 +2245,8 @@ int mapper_graph_lens(const mapper_graph_t* g, double* lens, double* pca, int64_
     if (n_pca) *n_pca = h->n_pca;
     cudaStream_t s = h->stream->s;
     if (lens && !h->lens.p) return fail(MAPPER_EINVAL, "graph was built from a given cover; no lens stored");
-    int rc = copy_out(lens, h->lens.p, sizeof(double) * h->n * h->m, on_device, s);
-    if (rc) return rc;
-    if ((rc = copy_out(pca, h->pca.p, sizeof(double) * h->n_pca, on_device, s))) return rc;
-    return lens || pca ? copies_done(s) : MAPPER_OK;
+    return copies_out({{lens, h->lens.p, sizeof(double) * h->n * h->m},
+                       {pca, h->pca.p, sizeof(double) * h->n_pca}}, on_device, s);
 }
 
 const mapper_cover_t* mapper_graph_cover(const mapper_graph_t* g)
