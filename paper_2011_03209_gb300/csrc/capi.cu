@@ -60,6 +60,11 @@ struct CoverData {
                                // place (M int32 each); unset for a subset of a cover
     std::vector<int64_t> h_elem_off;
     void* offsets_at = nullptr;  // h_elem_off on its way through page-locked scratch
+    // (a call that gives up before take_offsets leaves no copy on its way into the scratch)
+    ~CoverData()
+    {
+        if (offsets_at) cudaStreamSynchronize(stream->s);
+    }
     void take_offsets()                // after a wait for the stream
     {
         if (offsets_at) memcpy(h_elem_off.data(), offsets_at, sizeof(int64_t) * h_elem_off.size());

@@ -88,6 +88,11 @@ extern thread_local void* g_pinned;
 // nerve taken together), 5k x 8 945 -> 758 us, 13.7k x 37 1097 -> 847.
 struct Readback {
     explicit Readback(cudaStream_t stream) : s(stream) {}
+    Readback(const Readback&) = delete;
+    Readback& operator=(const Readback&) = delete;
+    // (a call that gives up between get() and wait() leaves no copy on its way into
+    // the scratch: the next call may use another stream)
+    ~Readback() { if (n) cudaStreamSynchronize(s); }
     cudaError_t get(void* dst, const void* src, size_t bytes)
     {
         const size_t at = (used + 15) & ~size_t(15);
