@@ -1344,16 +1344,20 @@ const char* mapper_strerror(int status)
 namespace {
 
 // Persistent autotuner choices: a text file named by MAPPER_TUNE_CACHE, a
-// header line with the device name and SM count, then one "key tile_n" line
+// header line with the count pass's revision, the device name and the SM count
+// (choices timed on another kernel say nothing about this one: raise the
+// revision with every change of the kernel's speed), then one "key tile_n" line
 // per tuned (row pitch, format, products) key. Read when a context is
 // created on the same kind of device; the context's choices are merged in
 // and the file replaced (write to a temporary, then rename) when it is
 // destroyed. Without the variable nothing is read or written.
+constexpr int kCountPassRevision = 2;
+
 std::string tune_cache_header(int device)
 {
     cudaDeviceProp prop{};
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return std::string();
-    return std::string("mapper-tune-v1 ") + prop.name + " sms=" + std::to_string(prop.multiProcessorCount);
+    return "mapper-tune-v1 count-pass-" + std::to_string(kCountPassRevision) + " " + prop.name + " sms=" + std::to_string(prop.multiProcessorCount);
 }
 
 void tune_cache_load(mapper_ctx* ctx)
