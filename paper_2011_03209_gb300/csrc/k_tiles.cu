@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "../../include/mapper.h"
+#include "pivot_mean.h"
 #include "tc.cuh"
 
 namespace mgb {
@@ -52,25 +53,16 @@ __global__ void pivot_gather_kernel(const float* __restrict__ X, int64_t n, int 
     for (int j = threadIdx.x; j < dp; j += blockDim.x) Pv[(int64_t)k * dp + j] = j < d ? X[p * ld + j] : 0.f;
 }
 
-// c[k] = the FP32 sum of the K pivots' column k in pivot order, / K
-// Mean of the pivots, 32 columns a CTA: eight warps of a column set each sum
-// every eighth pivot (loads ahead of the chain).
-__global__ void __launch_bounds__(256) pivot_mean_kernel(const float* __restrict__ Pv, int K, int dp,
-                                                         float* __restrict__ c)
+// Mean of the pivots, 32 columns a CTA: a warp a part of each column's sum
+// (loads ahead of the chain).
+__global__ void __launch_bounds__(32 * kMeanParts) pivot_mean_kernel(const float* __restrict__ Pv, int K, int dp,
+                                                                     float* __restrict__ c)
 {
-    __shared__ float part[8][32];
+    __shared__ float part[kMeanParts][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
-    float s = 0.f;
-    if (k < dp) {
-#pragma unroll 16
-        for (int i = warp; i < K; i += 8) s += Pv[(int64_t)i * dp + k];
-    }
-    part[warp][lane] = s;
+    part[warp][lane] = k < dp ? pivot_part(Pv, K, dp, k, warp) : 0.f;
     __syncthreads();
-    if (warp == 0 && k < dp) {
-        for (int w = 1; w < 8; ++w) s += part[w][lane];
-        c[k] = s / (float)K;
-    }
+    if (warp == 0 && k < dp) c[k] = mean_of_parts(&part[0][lane], 32, K);
 }
 
 // Nearest pivot of every point (FP32 distances; ties to the lower index).
@@ -1306,7 +1298,7 @@ int pivot_prepare(const float* X, int64_t n, int32_t d, int64_t ld, int dp, bool
     }
     if (!host) {
         pivot_gather_kernel<<<K, 128, 0, s>>>(X, n, d, ld, dp, K, P->Pv.as<float>());
-        pivot_mean_kernel<<<div_up(dp, 32), 256, 0, s>>>(P->Pv.as<float>(), K, dp, P->c.as<float>());
+        pivot_mean_kernel<<<div_up(dp, 32), 32 * kMeanParts, 0, s>>>(P->Pv.as<float>(), K, dp, P->c.as<float>());
         note_launch(2);
         PK(cudaGetLastError());
     } else {
@@ -1316,11 +1308,7 @@ int pivot_prepare(const float* X, int64_t n, int32_t d, int64_t ld, int dp, bool
             const float* x = X + ((int64_t)k * n / K) * ld;
             for (int j = 0; j < d; ++j) pv[(size_t)k * dp + j] = x[j];
         }
-        for (int j = 0; j < dp; ++j) {
-            float sum = 0.f;
-            for (int k = 0; k < K; ++k) sum += pv[(size_t)k * dp + j];
-            c[j] = sum / (float)K;
-        }
+        pivot_mean_host(pv.data(), K, dp, c.data());
         PK(cudaMemcpyAsync(P->Pv.p, pv.data(), sizeof(float) * pv.size(), cudaMemcpyHostToDevice, s));
         PK(cudaMemcpyAsync(P->c.p, c.data(), sizeof(float) * dp, cudaMemcpyHostToDevice, s));
         PK(cudaStreamSynchronize(s));                  // the host vectors go out of scope
