@@ -521,37 +521,6 @@ struct MergeArgs {
 };
 constexpr int kF = 8;                // FP64 candidates per query sent to the shared list
 
-// FP32 sum of squared differences of two rows, the warp together: lane l
-// takes columns l, l + 32, .. (vec4: 4 l .. 4 l + 3, + 128, ..) in order with
-// FMAs, then the 32 partial sums meet in a butterfly. A term passes at most
-// ceil(d / 128) 4 + 5 roundings (d + 5 for any d), which the merge's eta covers.
-__device__ __forceinline__ float warp_sqdist_f32(const float* __restrict__ x, const float* __restrict__ y, int d,
-                                                 bool vec4, int lane)
-{
-    float s = 0.f;
-    if (vec4) {
-        for (int k = lane * 4; k < d; k += 128) {
-            const float4 p = *reinterpret_cast<const float4*>(x + k), r = __ldg(reinterpret_cast<const float4*>(y + k));
-            float t = p.x - r.x;
-            s = fmaf(t, t, s);
-            t = p.y - r.y;
-            s = fmaf(t, t, s);
-            t = p.z - r.z;
-            s = fmaf(t, t, s);
-            t = p.w - r.w;
-            s = fmaf(t, t, s);
-        }
-    } else {
-        for (int k = lane; k < d; k += 32) {
-            const float t = x[k] - __ldg(y + k);
-            s = fmaf(t, t, s);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-}
-
 template <bool FAR, int SRC>
 __global__ void __launch_bounds__(256) knn_merge_tc_kernel(const MergeArgs a)
 {

@@ -246,17 +246,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v)
-{
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // u = fl(m u + n) for two columns at once (packed FMA, each lane correctly
 // rounded as fmaf).
 __device__ __forceinline__ void fma2_inplace(float& u0, float& u1, float m, float n0, float n1)
@@ -1600,18 +1589,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         // = A rows 32(w & 3) .. +31 and the 32 kChunks columns of part
         // (w - 2) / 4. Each pair's norms and core flags are loaded one pair
         // ahead.
+        static_assert(MODE == 2, "the other passes have their own epilogues");
         const int et = tid - 64;                              // 0 .. kEpiThreads-1
         const int quad = warp & 3;
         const int half = (warp - 2) >> 2;                     // column part
         const int r = quad * 32 + lane;                       // accumulator row = A-tile row
         struct Pre {
             int2 tp;
-            bool one_each;                                    // union pass: see kPairOneEach
+            bool one_each;                                    // see kPairOneEach
             int na, nb;
             float na2, nra, rla;                              // row r
             float c2, c1, c3;                                 // column et (et < 128)
-            bool core_et;                                     // union pass: row et of A | B
-            int count_et;                                     // count pass: count of row / column et
+            bool core_et;                                     // row et of A | B
         };
         auto prefetch = [&](int64_t q, Pre& f) {
             f.tp = A.pairs[q];
@@ -1631,13 +1620,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 f.c1 = P.rn[sb + et];
                 f.c3 = P.rl ? P.rl[sb + et] : 0.f;
             }
-            if (MODE == 2) {
-                const bool diag = f.tp.x == f.tp.y;
-                f.core_et = et < kT ? (et < f.na && A.core[sa + et])
-                                    : (et < 2 * kT && !diag && et - kT < f.nb && A.core[sb + et - kT]);
-            } else if (et < 2 * kT) {
-                f.count_et = et < kT ? A.count[sa + et] : A.count[sb + et - kT];
-            }
+            const bool diag = f.tp.x == f.tp.y;
+            f.core_et = et < kT ? (et < f.na && A.core[sa + et])
+                                : (et < 2 * kT && !diag && et - kT < f.nb && A.core[sb + et - kT]);
         };
         // work items in turn, each one or (W = 2) two pairs: `it` counts pairs
         // (staging buffers), `git` items (TMEM accumulators)
@@ -1647,9 +1632,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
         int h = 0;                                            // pair of the item
         if (g < n_items) prefetch(grp.x, cur);
         int it = 0, git = 0;
-        int64_t screened = 0;
         while (g < n_items) {
-            const int64_t q = h ? grp.y : grp.x;
             const bool last_sub = h == 1 || grp.y < 0;
             int64_t g_next = g;
             int h_next = 1;
@@ -1661,7 +1644,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             }
             const int2 tp = cur.tp;
             const bool diag = tp.x == tp.y;
-            const bool one_each = MODE == 2 && cur.one_each;
+            const bool one_each = cur.one_each;
             const int na = cur.na, nb = cur.nb;
             const int64_t sa = (int64_t)tp.x * kT, sb = (int64_t)tp.y * kT;
             const int buf = it & 1;
@@ -1669,7 +1652,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             const uint32_t acc_phase = (uint32_t)((git >> 1) & 1);
             const bool valid_r = r < na;
             const float na2 = cur.na2, nra = cur.nra, rla = cur.rla;
-            const int pre_count = cur.count_et;
 
             // (1) stage this pair's column data (and core rows, roots) in buffer `buf`
             if (et < kT) {
@@ -1686,7 +1668,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     S.red[buf][8 + (et >> 5)] = m3;
                 }
             }
-            if (MODE == 2 && et < 2 * kT) {
+            if (et < 2 * kT) {
                 const bool cc = cur.core_et;
                 S.core[buf][et] = cc;
                 S.par[buf][et] = et;
@@ -1696,11 +1678,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                 if (lane == 0 && (diag ? et < kT : et >= kT)) S.colcore[buf][(et & (kT - 1)) >> 5] = m;
                 if (et == 0) { S.s_mm[buf][0] = INT_MAX; S.s_mm[buf][1] = -1; }
             }
-            if (MODE == 2) {
-                if (et == 0) S.edges[buf] = 0;
-                epi_sync();                                     // s_mm, edges initialised
-            }
-            if (MODE == 2 && et < 2 * kT && cur.core_et) {
+            if (et == 0) S.edges[buf] = 0;
+            epi_sync();                                       // s_mm, edges initialised
+            if (et < 2 * kT && cur.core_et) {
                 const int rr = gfind(A.parent, (int)(et < kT ? sa + et : sb + et - kT));
                 S.groot[buf][et] = rr;
                 atomicMin(&S.s_mm[buf][0], rr);
@@ -1731,12 +1711,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             }
             const float k_in = __fadd_ru(__fsub_ru(na2, P.eps2_lo), E);
             const float k_out = __fsub_rd(__fsub_rd(na2, P.eps2_hi), E);
-            bool work = true;
-            if (MODE == 2) {
-                work = S.s_mm[buf][1] >= 0 && S.s_mm[buf][0] != S.s_mm[buf][1];
-                if (!work && S.s_mm[buf][1] >= 0 && et == 0) atomicAdd(&A.stats[kStatSkipped], 1ull);
-            }
-            const bool core_r = MODE == 2 && S.core[buf][r];
+            const bool work = S.s_mm[buf][1] >= 0 && S.s_mm[buf][0] != S.s_mm[buf][1];
+            if (!work && S.s_mm[buf][1] >= 0 && et == 0) atomicAdd(&A.stats[kStatSkipped], 1ull);
+            const bool core_r = S.core[buf][r];
 
             // (4) accumulator rows -> neighbour bits
             uint32_t inb[kChunks], band[kChunks];
@@ -1764,22 +1741,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                         if (u >= k_out) keep_bits |= 1u << i;
                     }
                 }
-                // candidate columns: valid (and core-core, upper triangle for unions)
+                // candidate columns: valid and core-core
                 const int left = nb - c * 32;
                 uint32_t cand = !valid_r ? 0u : (left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u));
+                cand = (work && core_r) ? cand & S.colcore[buf][c] : 0u;
                 uint32_t cand_band = cand;
-                if (MODE == 2) {
-                    cand = (work && core_r) ? cand & S.colcore[buf][c] : 0u;
-                    cand_band = cand;
-                    if (diag) {                                       // band pairs once: j > r
-                        const int lo = r + 1 - c * 32;
-                        cand_band &= lo <= 0 ? 0xffffffffu : (lo >= 32 ? 0u : ~((1u << lo) - 1u));
-                    }
+                if (diag) {                                   // band pairs once: j > r
+                    const int lo = r + 1 - c * 32;
+                    cand_band &= lo <= 0 ? 0xffffffffu : (lo >= 32 ? 0u : ~((1u << lo) - 1u));
                 }
                 inb[c2] = in_bits & cand;
                 band[c2] = keep_bits & ~in_bits & cand_band;
                 S.rowmask[c][r] = inb[c2];
-                if (MODE == 2 && inb[c2]) atomicAdd(&S.edges[buf], __popc(inb[c2]));
+                if (inb[c2]) atomicAdd(&S.edges[buf], __popc(inb[c2]));
                 if (!diag) {
                     // 32 x 32 bit transpose across the warp: lane k gets column c*32+k
                     uint32_t x = inb[c2];
@@ -1808,71 +1782,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
                     const int i = __ffs(b) - 1;
                     b &= b - 1;
                     const int j = (half * kChunks + c2) * 32 + i;
-                    const uint32_t fl = MODE == 1 ? ((diag ? 0u : kQBoth) | ((!diag || r < j) ? kQTie : 0u)) : 0u;
                     bool decided;
-                    const bool in = push_band(P, (int)(sa + r), (int)(sb + j), fl, &decided);
-                    if (decided && in) {
-                        if (MODE == 1) {
-                            int old = atomicAdd(&A.count[sa + r], 1);
-                            if (A.cap > 0 && old < A.cap) A.nbr[(sa + r) * A.cap + old] = (int32_t)(sb + j);
-                            if (!diag) {
-                                old = atomicAdd(&A.count[sb + j], 1);
-                                if (A.cap > 0 && old < A.cap) A.nbr[(sb + j) * A.cap + old] = (int32_t)(sa + r);
-                            }
-                        } else {
-                            gunion(A.parent, A.row_pt, (int)(sa + r), (int)(sb + j));
-                        }
-                    }
+                    const bool in = push_band(P, (int)(sa + r), (int)(sb + j), 0u, &decided);
+                    if (decided && in) gunion(A.parent, A.row_pt, (int)(sa + r), (int)(sb + j));
                 }
             }
 
-            // (6) counts and lists, or unions
-            if (MODE == 1) {
-                // one thread per row (et < 128) and per column (128 <= et < 256) adds the
-                // pair's neighbours to the count; lists are written only while a count may
-                // still be below cap (the count read one pair ahead is a lower bound)
-                int k = 0;
-                uint32_t any_band = 0u;
-#pragma unroll
-                for (int c2 = 0; c2 < kChunks; ++c2) {
-                    k += __popc(inb[c2]);
-                    any_band |= band[c2];
-                }
-                const bool hit = epi_sync_or(k > 0 || any_band != 0u);
-                if (et == 0 && hit && A.pair_hit) A.pair_hit[q] = 1;
-                const bool is_row = et < kT, is_col = !diag && et >= kT && et < 2 * kT;
-                if (is_row || is_col) {
-                    const int x = is_row ? et : et - kT;
-                    const int64_t row = (is_row ? sa : sb) + x;
-                    const int64_t other = is_row ? sb : sa;
-                    int tot = 0;
-                    if (is_row) {
-#pragma unroll
-                        for (int w = 0; w < kT / 32; ++w) tot += __popc(S.rowmask[w][x]);
-                    } else {
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) tot += __popc(S.colmask[w][x]);
-                    }
-                    if (tot > 0) {
-                        if (pre_count >= A.cap) {
-                            atomicAdd(&A.count[row], tot);          // no list entry can be due
-                        } else {
-                            const int old = atomicAdd(&A.count[row], tot);
-                            int pos = old;
-                            for (int w = 0; w < kT / 32 && pos < A.cap; ++w) {
-                                uint32_t bm = is_row ? S.rowmask[w][x] : S.colmask[w & 3][x];
-                                if (!is_row && w >= 4) bm = 0u;
-                                while (bm && pos < A.cap) {
-                                    const int i = __ffs(bm) - 1;
-                                    bm &= bm - 1;
-                                    A.nbr[row * A.cap + pos++] = (int32_t)(other + w * 32 + i);
-                                }
-                            }
-                        }
-                    }
-                }
-                if (et == 0) screened += diag ? (int64_t)na * (na + 1) / 2 : (int64_t)na * nb;
-            } else if (one_each) {
+            // (6) unions
+            if (one_each) {
                 // both sides are single components: join them through any neighbour pair
                 if (work && all_in) {
                     int c2 = 0;
@@ -1914,10 +1831,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_kernel(const __grid_constant__
             g = g_next;
             h = h_next;
             grp = grp_next;
-        }
-        if (MODE == 1 && et == 0 && screened) {
-            atomicAdd(&A.stats[kStatScreened], (unsigned long long)screened);
-            atomicAdd(&A.stats[kStatTcPairs], (unsigned long long)screened);
         }
     }
 
