@@ -350,7 +350,10 @@ int run_cover(mapper_ctx* ctx, const double* lens, int64_t n, int32_t m, const i
 // with the BF16 first phase lists of at most kShortBlocks pairs times K blocks of
 // 64 columns take one. The phase would save at most 0.45 T3 there (~2.5 ns a
 // pair and K block, 20 us at the limit); its list and second launch cost about
-// eight short kernels: 5k x 8 742 -> 703 us, 13.7k x 37 881 -> 838 in one phase.
+// eight short kernels: 5k x 8 742 -> 703 us, 13.7k x 37 881 -> 838 in one phase;
+// 2k x 8 (52 pairs) 626 -> 586, 30k x 16 (5.6k) 1291 -> 1228, 8k x 256 (1.5k) 692
+// -> 644. (Above the line, drawn by that estimate, one phase was still ahead: 14k x
+// 128, 9.4k blocks, 764 -> 688, 14k x 256, 18.5k, 798 -> 714.)
 constexpr double kDeferMax = 0.35;
 constexpr int64_t kSampleMinPairs = 8192;
 constexpr int64_t kShortBlocks = 8192;
@@ -1009,7 +1012,9 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         CK(list_unions(a.count, a.nbr, cap, a.core, a.parent, rd.root.as<int32_t>(), a.row_pt, R, s,
                        a.stats + kStatOob), "list unions");
         // (without lists the rows are not joined yet; on short lists one launch of a
-        // CTA per pair costs less than four: 5k x 8 0.74 against 0.76 ms)
+        // CTA per pair costs less than four: 5k x 8 0.74 against 0.76 ms, 400k x 16
+        // with 28 pairs 3.32 against 3.34, 12k x 4 with 7.0k as much; with 25k pairs
+        // 0.88 against 0.86, with 90k 1.23 against 1.04, with 1.5M 6.46 against 3.03)
         if (cap && PL.n[kListAllIn] >= 8192) {
             Buf troots;
             CK(troots.alloc(sizeof(int2) * std::max<int64_t>(L.T, 1), s), "alloc");
@@ -1024,8 +1029,11 @@ int run_cluster_radii(mapper_ctx* ctx, const float* X, int64_t n, int32_t d, int
         // neighbour pair. After the unions along the neighbour lists few pairs
         // are left (none to a few hundred of up to 1.2 M; 3 k of 173 k at 1M x
         // 256), so two rounds do, and one on short lists (a round is four
-        // launches: 5k x 8 702 -> 685 us, 13.7k x 37 832 -> 813); without lists
-        // (minPts 1, or above 65) the rounds join everything, in five steps.
+        // launches: 5k x 8 702 -> 685 us, 13.7k x 37 832 -> 813, 30k x 16, 5.6k
+        // pairs, 1301 -> 1237). Longer lists differ: in one round 65k x 8 (28k
+        // pairs) 2.85 -> 2.77 ms and 400k x 16 (59k) 3.33 -> 3.27, but 400k x 2
+        // (67k) 8.36 -> 8.48. Without lists (minPts 1, or above 65) the rounds join
+        // everything, in five steps.
         auto union_rounds = [&](const PassArgs& base, const TcArgs& tbase, int64_t n, bool tc) -> int {
             if (n == 0) return MAPPER_OK;
             // every count stays on the device: each launch covers the list's

@@ -237,8 +237,10 @@ cudaError_t whole_cloud_slots(int64_t n, int32_t* slot_point, int32_t* slot_elem
 }
 
 // Up to this many elements the thread at a change of element writes the offsets
-// of the empty ones before it; more (a fine grid, mostly empty) take a search
-// per element.
+// of the empty ones before it (a launch less: cover of 5k points in 12 elements
+// 80 us against 84, of 200k in 60 x 60 149 against 159); more (a fine grid, mostly
+// empty) take a search per element, because a gap is one thread's work (5k points
+// at one end of 1000 x 1000 elements and one at the other: 4.46 ms against 0.27).
 constexpr int64_t kSplitElems = 4096;
 
 cudaError_t split_keys(const uint64_t* keys, const int32_t* pt, int64_t M, int64_t E, int32_t* slot_point,

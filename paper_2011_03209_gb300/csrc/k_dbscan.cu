@@ -845,6 +845,10 @@ cudaError_t border_from_lists(const int32_t* count, const int32_t* nbr, int cap,
     return cudaGetLastError();
 }
 
+// From this many rows on, roots hook twice more before the unions; below it the
+// two passes and their copies cost what they save. Graphs with and without them:
+// 90k points x 16 (112k memberships) 1.24 and 1.22 ms, 130k x 16 1.70 and 1.70,
+// 260k x 16 2.32 and 2.34, 400k x 16 3.32 and 3.38, 400k x 2 8.38 and 8.46.
 constexpr int64_t kHookRows = 1 << 17;
 
 cudaError_t list_unions(const int32_t* count, const int32_t* nbr, int cap, const uint8_t* core, int32_t* parent,

@@ -336,7 +336,10 @@ __global__ void __launch_bounds__(256) cand_count_kernel(const int64_t* __restri
 // element (eseg_off[E + 1]), and out = (segments, tiles, element tile pairs).
 // One launch and one read-back where a scan per array would take a launch or two
 // each and the host three round trips. Covers of more than kLayoutElems elements
-// (fine grids, mostly empty) take those.
+// (fine grids, mostly empty) take those: the CTA walks segments and elements by
+// itself. Graphs with the one kernel and with the scans: 14k x 37 815 and 851 us,
+// 200k x 2 in 66 x 66 elements 3.77 and 3.81 ms, in 127 x 127 6.06 and 6.09, 1M x 2
+// in 127 x 127 15.49 and 15.50.
 constexpr int kLayoutThreads = 1024;
 constexpr int64_t kLayoutElems = 16384;
 
