@@ -11,7 +11,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
-#include "common.cuh"
+#include "dbscan.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -417,26 +417,83 @@ __global__ void __launch_bounds__(32 * kEccWarps) col_sum_exp_kernel(const float
     }
 }
 
+// Two columns at a time (each half rounded as the scalar instruction).
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b)
+{
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_neg(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b)
+{
+    f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b)
+{
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
+{
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// a + b (a - b) = the result + e exactly
+__device__ __forceinline__ f2 two_sum(f2 a, f2 b, f2& e)
+{
+    const f2 s = f2_add(a, b), bb = f2_sub(s, a);
+    e = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
+    return s;
+}
+__device__ __forceinline__ f2 two_diff(f2 a, f2 b, f2& e)
+{
+    const f2 s = f2_sub(a, b), bb = f2_sub(s, a);
+    e = f2_sub(f2_sub(a, f2_sub(s, bb)), f2_add(b, bb));
+    return s;
+}
+// the same where |a| >= |b| or a = 0
+__device__ __forceinline__ f2 fast_sum(f2 a, f2 b, f2& e)
+{
+    const f2 s = f2_add(a, b);
+    e = f2_sub(b, f2_sub(s, a));
+    return s;
+}
+
 // |x - mu|^2 of every row for the eccentricity. In FP64 that is a subtract and
-// an FMA a value, which the FP64 pipe takes 0.84 ms for at 1M x 256; here a value
-// takes ~65 FP32 instructions. The mean's 53 bits are three floats, because what
-// is cut from it shifts a whole column by a part of |mu|, however small x - mu
-// is; t = x - mu as th + tl + t3 (two-sums, to 2^-72 of |t| and |mu|), th^2 = p + pe
-// and 2 th tl = q + qe exactly, qe + tl^2 + 2 th t3 in two FMAs, and a 32-column
-// sum of them as an FP32 expansion of three terms, added to the row's FP64 sum.
-// The roundings are below 2^-68 of a value's square, so a row's error is that of
-// its d / 32 FP64 adds, against two FP64 roundings a value (largest relative
-// error over 3000 rows, means 0 to 1e6: 1.1e-16 at 1 to 8 columns, 3.2e-16 at 256;
-// the FP64 form 4.7e-16 and 1.7e-15). A chunk where some |t| is not zero or in
-// [2^-40, 2^55) is summed in FP64 instead (subtract and FMA, columns in order).
-// One thread a row, as lens_rows_kernel.
+// an FMA a value, which the FP64 pipe takes 0.84 ms for at 1M x 256; here two
+// columns at a time take ~51 packed FP32 instructions, bound by the FP32 pipe. The
+// mean's 53 bits are three floats, because what is cut from it shifts a whole
+// column by a part of |mu|, however small x - mu is. t = x - mu as th + tl + t3 (to
+// 2^-72 of |t| and |mu|):
+//   x - m1 = y + a and a - m2 = v + b exactly; |y| >= |v| or y = 0 (x and m1 within
+//   a factor of 2: a = 0 and y is a multiple of half an ulp of m1 or 0; else |y| is
+//   half the larger of them or more), so y + v = th + c by the short sum; c + (b - m3)
+//   likewise, up to 2^-24 of b, which is 2^-48 of |x| and |mu|.
+// th^2 = p + pe and 2 th tl = q + qe exactly, qe + tl^2 + 2 th t3 in two FMAs, and a
+// 32-column sum of them as an FP32 expansion of three terms a half, added to the
+// row's FP64 sum. The roundings are below 2^-68 of a value's square, so a row's error
+// is that of its d / 32 FP64 adds, against two FP64 roundings a value (largest
+// relative error over 3000 rows, means 0 to 1e6: 1.1e-16 at 1 to 8 columns, 3.2e-16
+// at 256; the FP64 form 4.7e-16 and 1.7e-15). A chunk where some |t| is not zero or
+// in [2^-40, 2^55) is summed in FP64 instead (subtract and FMA, columns in order).
+// One thread a row, as lens_rows_kernel. One column at a time, with two-sums
+// throughout, the call of 1M x 256 took 990 us, now 900.
+constexpr int kEccPitch = kChunk + 2;          // (a thread's pairs of columns: no bank conflicts)
+
 __global__ void __launch_bounds__(kRows) ecc_rows_kernel(const float* __restrict__ X, int64_t n, int32_t d, int64_t ld,
                                                          const double* __restrict__ mu, double* __restrict__ f, int m,
                                                          int j)
 {
-    __shared__ float tile[kRows][kChunk + 1];
+    __shared__ __align__(16) float tile[kRows][kEccPitch];
     __shared__ double smu[kChunk];
-    __shared__ __align__(16) float4 smf[kChunk];                   // the mean as three floats
+    __shared__ __align__(16) float sm12[kChunk / 2][4];        // the mean's floats: m1 of two columns, m2 of two
+    __shared__ __align__(8) float sm3[kChunk];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t row0 = (int64_t)blockIdx.x * kRows;
     const bool vec = ld % 4 == 0 && ((uintptr_t)X & 15) == 0;
@@ -451,10 +508,8 @@ __global__ void __launch_bounds__(kRows) ecc_rows_kernel(const float* __restrict
                 const int64_t row = row0 + r;
                 float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (row < n) x = __ldg(reinterpret_cast<const float4*>(X + row * ld + k0 + c4));
-                tile[r][c4] = x.x;
-                tile[r][c4 + 1] = x.y;
-                tile[r][c4 + 2] = x.z;
-                tile[r][c4 + 3] = x.w;
+                *reinterpret_cast<float2*>(&tile[r][c4]) = make_float2(x.x, x.y);
+                *reinterpret_cast<float2*>(&tile[r][c4 + 2]) = make_float2(x.z, x.w);
             }
         } else {
 #pragma unroll 8
@@ -465,41 +520,57 @@ __global__ void __launch_bounds__(kRows) ecc_rows_kernel(const float* __restrict
                 tile[r][lane] = x;
             }
         }
-        if (tid < kc) {
-            const double mk = mu[k0 + tid];
+        if (tid < kChunk) {                                        // (columns past d: x = mu = 0)
+            const double mk = tid < kc ? mu[k0 + tid] : 0.0;
             const float m1 = (float)mk;
             const double rest = mk - (double)m1;                   // (exact)
             const float m2 = (float)rest;
             smu[tid] = mk;
-            smf[tid] = make_float4(m1, m2, (float)(rest - (double)m2), 0.f);
+            sm12[tid >> 1][tid & 1] = m1;
+            sm12[tid >> 1][2 + (tid & 1)] = m2;
+            sm3[tid] = (float)(rest - (double)m2);
         }
         __syncthreads();
-        float s = 0.f, e = 0.f, e2 = 0.f;
+        f2 s = 0ull, e = 0ull, e2 = 0ull;
         unsigned lo = ~0u, hi = 0u;                                // 2 |th| as bits: smallest (not 0) less 1, largest
-#pragma unroll 4
-        for (int k = 0; k < kc; ++k) {
-            const float4 mk = smf[k];
-            float a, c, t3, err, b;
-            const float y = two_sum(tile[tid][k], -mk.x, a);        // x - m1 = y + a
-            const float v = two_sum(a, -mk.y, b);                   // a - m2 = v + b
-            const float th = two_sum(y, v, c);
-            const float tl = two_sum(c, __fsub_rn(b, mk.z), t3);
-            const unsigned t = __float_as_uint(th) << 1;
-            hi = max(hi, t);
-            lo = min(lo, t - 1u);
-            const float p = __fmul_rn(th, th), h2 = __fadd_rn(th, th), q = __fmul_rn(h2, tl);
-            const float rest = __fmaf_rn(h2, t3, __fmaf_rn(tl, tl, __fmaf_rn(h2, tl, -q)));
-            s = two_sum(s, p, err);
+        const int pairs = (kc + 1) / 2;
+#pragma unroll 2
+        for (int k = 0; k < pairs; ++k) {
+            const ulonglong2 m12 = *reinterpret_cast<const ulonglong2*>(sm12[k]);
+            const f2 m3 = *reinterpret_cast<const f2*>(&sm3[2 * k]);
+            f2 a, b, c, t3, err;
+            const f2 y = two_diff(*reinterpret_cast<const f2*>(&tile[tid][2 * k]), m12.x, a);
+            const f2 v = two_diff(a, m12.y, b);
+            const f2 th = fast_sum(y, v, c);
+            const f2 tl = fast_sum(c, f2_sub(b, m3), t3);
+            const f2 p = f2_mul(th, th), h2 = f2_add(th, th), q = f2_mul(h2, tl);
+            const f2 pe = f2_fma(th, th, f2_neg(p));
+            const f2 rest = f2_fma(h2, t3, f2_fma(tl, tl, f2_fma(h2, tl, f2_neg(q))));
+            float th0, th1, s0, s1, p0, p1;
+            f2_unpack(th, th0, th1);
+            const unsigned b0 = __float_as_uint(th0) << 1, b1 = __float_as_uint(th1) << 1;
+            hi = max(hi, max(b0, b1));
+            lo = min(lo, min(b0 - 1u, b1 - 1u));
+            // (both are sums of squares: the larger one first)
+            f2_unpack(s, s0, s1);
+            f2_unpack(p, p0, p1);
+            s = fast_sum(f2_pack(fmaxf(s0, p0), fmaxf(s1, p1)), f2_pack(fminf(s0, p0), fminf(s1, p1)), err);
             e = two_sum(e, err, b);
-            e2 = __fadd_rn(e2, b);
-            e = two_sum(e, __fmaf_rn(th, th, -p), b);
-            e2 = __fadd_rn(e2, b);
+            e2 = f2_add(e2, b);
+            e = two_sum(e, pe, b);
+            e2 = f2_add(e2, b);
             e = two_sum(e, q, b);
-            e2 = __fadd_rn(e2, __fadd_rn(b, rest));
+            e2 = f2_add(e2, f2_add(b, rest));
         }
         // 2^-40 and 2^55 as bits
         if (lo >= (87u << 24) - 1u && hi < (182u << 24)) {
-            acc += (double)s + ((double)e + (double)e2);
+            float s0, s1, e0, e1, l0, l1, err, b0, b1;
+            f2_unpack(s, s0, s1);
+            f2_unpack(e, e0, e1);
+            f2_unpack(e2, l0, l1);
+            const float sum = two_sum(s0, s1, err);
+            const float low = two_sum(two_sum(e0, e1, b0), err, b1);
+            acc += (double)sum + ((double)low + (double)__fadd_rn(__fadd_rn(l0, l1), __fadd_rn(b0, b1)));
         } else {
             for (int k = 0; k < kc; ++k) {
                 const double t = __dsub_rn((double)tile[tid][k], smu[k]);
@@ -1103,7 +1174,7 @@ cudaError_t column_means(const float* X, int64_t n, int32_t d, int64_t ld, doubl
 // sqrt(|x - mu|^2 + V) without any pair of points: column means as FP64 sums
 // give them, |x - mu|^2 more exactly than FP64 sums do (ecc_rows_kernel), V their
 // mean (fixed-order sums). 1M x 256 through mapper_lens: 3024 us with FP64
-// arithmetic throughout and a pass of its own for the finite check, 990 us now;
+// arithmetic throughout and a pass of its own for the finite check, 900 us now;
 // with the mean as two floats 832, but on 3000 rows of mean 1e6 and spread 1 in
 // 2 columns up to 2.5e-10 off, where FP64 arithmetic and this form are off by 8e-15.
 cudaError_t lens_ecc2(const float* X, int64_t n, int32_t d, int64_t ld, double* f, int m, int j, cudaStream_t s,
