@@ -1228,11 +1228,13 @@ int run_nerve(mapper_ctx* ctx, const std::shared_ptr<ClusterData>& cl, mapper_gr
         CK(rb.get(h, dc, sizeof(h)), "copy");
         CK(rb.wait(), "sync");
         edges_done = h[1] == 0;
-        // the graph keeps the edges, not a list far longer than them (a copy that
-        // small graphs, of up to 64 nodes, do without: 10 us of 680 at 5k x 8)
+        // The graph keeps the list as it is where that is small (up to 64 nodes)
+        // or small beside what it keeps of its memberships anyway (42 bytes each);
+        // else the edges move to an array of their own (alloc and copy: 4 to 5 us
+        // of 690 at 5k x 8 with 100 intervals, 776 at 14k x 37 with 121).
         const size_t bytes = sizeof(int32_t) * 2 * (size_t)h[0];
         g->Eg = (int64_t)h[0];
-        if (edges_done && list.bytes <= std::max<size_t>(2 * bytes, 16 << 10)) {
+        if (edges_done && list.bytes <= std::max<size_t>({2 * bytes, 16 << 10, 16 * (size_t)M})) {
             g->edges = std::move(list);
         } else if (edges_done) {
             CK(g->edges.alloc(bytes, s), "alloc");
